@@ -96,12 +96,15 @@ typedef struct {
 typedef struct {
     int prec;                    /* pc_prec: FP32 with FP64 rescue (0) or plain FP64 */
     double cell_size;            /* grid cell side; 0 = chosen by the cost model */
-    int ipt;                     /* i-points per thread (2 or 4); 0 = auto */
-    int priv;                    /* shared-histogram replication: 1 = one count copy per warp,
-                                    2 = one shared copy, other values = automatic (up to 32
-                                    lane copies, lane l updating copy l % k, when they fit
-                                    16 KB: few bins then never collide within a warp) */
-    long long rescue_capacity;   /* rescue-queue slots; 0 = auto; < 0 = none (all inline) */
+    int ipt;                     /* points of a block: 128 ipt (2 or 4; 0 = auto); the FP32
+                                    kernel deals a block to warps 64 points at a time */
+    int priv;                    /* shared-histogram replication: 2 = one shared copy where the
+                                    bins are found by tables or packed floors, other values =
+                                    automatic (up to 32 lane copies, lane l updating copy
+                                    l % k, when they fit 16 KB: few bins then never collide
+                                    within a warp); 1 also keeps weighted sums in binary64 */
+    long long rescue_capacity;   /* rescue-queue slots; 0 = auto (none: near-edge pairs are
+                                    checked inside the pair kernel); < 0 = none */
     int use_graph;               /* pc_count_batch: replay a captured CUDA graph */
     int grid_ctas_per_sm;        /* persistent CTAs per SM; 0 = occupancy limit */
     int shard_index;             /* with shard_count > 1: count only the i-points of the */
@@ -134,12 +137,11 @@ typedef struct {
                                     grid's weight exponents spanning at most 8 binades and
                                     the two grids' spans adding up to at most 12; truncation
                                     below 2^-34 relative), flushed in binary64; 3 the same
-                                    for binary64 weights: the integer products of their
-                                    binary32 roundings hi (conditions as for 2 on the his,
-                                    which must reach 2^-78 where the weight is not a
-                                    binary32 value) plus the binary32 terms hi_i lo_j +
-                                    lo_i hi_j of their remainders lo = fl32(w - hi), rounded
-                                    to the accumulators' unit (below 2^-34 relative) */
+                                    for binary64 weights (conditions as for 2 on their
+                                    binary32 roundings, which must reach 2^-78 where the
+                                    weight is not a binary32 value): products of the weights'
+                                    leading 63 bits, rounded to the accumulators' unit (below
+                                    2^-34 relative) */
     long long tree_pairs;        /* pc_count_tree: list node pairs listed by the traversal */
     float ms_traverse;           /* pc_count_tree: device-and-host time of the traversal */
 } pc_stats;
@@ -212,7 +214,7 @@ pc_status pc_count_batch(const pc_grid *const *gs, int m, const pc_bins *b, cons
  *   g         a grid from pc_build_grid, on the current device
  *   counts    int64 [nbins] (host or device), wcounts binary64 [nbins] or
  *             NULL; both written on return
- * All temporaries live in one fixed device array of about 12.3 MiB inside the
+ * All temporaries live in one fixed device array of about 10.8 MiB inside the
  * library, which every GPU that loads the library holds until the process
  * exits.  Its device address is looked up on the first call on each device
  * (a lookup that allocates nothing).  Like the library's
@@ -343,7 +345,7 @@ pc_status pc_tree_export(const pc_tree *t, long long *start, long long *count, i
  *   counts, wcounts, st   as for pc_count_auto (st adds tree_pairs, the list
  *                         node pairs, and ms_traverse; cell_size reports the
  *                         largest list node extent)
- *   o                     prec, ipt (2 or 4; blocks of at most 128 ipt points,
+ *   o                     prec, ipt (2 or 4: blocks of at most 128 ipt points,
  *                         each list node split into equal blocks), priv,
  *                         rescue_capacity, grid_ctas_per_sm and the block
  *                         shards (shard_index of shard_count) apply

@@ -106,6 +106,8 @@ static Workspace &workspace(int dev) {
 // ---------------------------------------------------------------------------
 // plan: bins, error bands, lookup tables, stencil
 // ---------------------------------------------------------------------------
+enum { PLAN_LUT = 0, PLAN_LIN = 1, PLAN_LINOFF = 2, PLAN_LOG = 3, PLAN_FIX = 5 };   // PATH_* of the kernel
+
 struct Plan {
     int mode = 0, los = 0, na = 0, nb = 1, nbins = 0;
     std::vector<double> ea, eb;   // edges
@@ -125,6 +127,15 @@ struct Plan {
     float lin_invB2 = 0, lin_thrB = 0;
     float lin_offA1 = 0;         // lin_offA + 1, rounded once
     float lin_mS = 0;
+    // the pair kernel's choice: tables, or floors from zero, from any edge or
+    // of logarithms (the lin fields; also for mu along the midpoint line of
+    // sight, which lin leaves out)
+    int path = PLAN_LUT;
+    // fixed-point floors: bands in units of 2^-16 (first axis; pi of (sigma, pi);
+    // mu, fx_mA / s + fx_mB) and the separation the mu band stops growing at
+    int fix = 0;
+    unsigned fx_s = 0, fx_p = 0;
+    double fx_mA = 0, fx_mB = 0, fx_sf = 0;
 };
 
 static bool edges_ok(const double *e, int n, bool zero_one) {
@@ -364,6 +375,14 @@ static pc_status make_plan(const pc_bins *b, const Geom &g, const double *pts_lo
         build_lut(P.ea, false, V, 2.0 * eps_sig, P.lut, P.la);
         build_lut(P.eb, false, V, 2.0 * eps_z, P.lut, P.lb);
     }
+    // mu floors along the midpoint line of sight run only inside the kernel's
+    // own choice (P.path); the lin view stays with the z line of sight
+    const bool mid_mu = P.mode == PC_BIN_SMU && P.los == PC_LOS_MIDPOINT;
+    // mu = |d.l| rsqrt(l^2) rsqrt(s^2) may exceed 1 by rounding: along z by the
+    // reciprocal root's and the squares' errors (3e-7), along the midpoint by
+    // 12.3 u = 7.4e-7 (3 u from d.l, 1.5 u from each square, 2.15 u from each
+    // reciprocal root, 2 u from the products); the scale stays below n_mu by more
+    const double mu_shrink = ldexp(1.0, mid_mu ? -20 : -21);
     // ---- evenly spaced edges: floor-based bins ------------------------------
     // s (and mu along z): bin = floor(t), t = (s - e0) / D, with the band
     // moved into t units plus the rounding of t itself (scaling factor and
@@ -378,9 +397,9 @@ static pc_status make_plan(const pc_bins *b, const Geom &g, const double *pts_lo
         double devm = 0.0;
         if (P.mode == PC_BIN_SMU) {
             for (int k = 0; k <= P.nb; ++k) devm = std::max(devm, fabs(P.eb[k] - (double)k / P.nb));
-            lin_mu = (P.los == PC_LOS_Z) && devm <= 1e-12;
+            lin_mu = (P.los == PC_LOS_Z || P.fp32_ok) && devm <= 1e-12;
         }
-        bool mode_ok = P.mode == PC_BIN_S || (P.mode == PC_BIN_SMU && P.los == PC_LOS_Z);
+        bool mode_ok = P.mode == PC_BIN_S || P.mode == PC_BIN_SMU;
         if (lin_s && lin_mu && mode_ok && (P.rcut - e0) / D < 4.0e6) {
             double ts_max = (P.rcut - e0) / D + 1.0;
             double eps_t = (eps_s + dev) / D + 4.0 * u * (ts_max + fabs(e0) / D);
@@ -399,9 +418,9 @@ static pc_status make_plan(const pc_bins *b, const Geom &g, const double *pts_lo
                     // lands in the last bin without a clamp; the scale's shift
                     // of up to 2^-21 n_mu joins the band
                     const double nb = P.nb;
-                    P.lin_nB = nextafterf((float)(nb * (1.0 - ldexp(1.0, -21))), 0.0f);
+                    P.lin_nB = nextafterf((float)(nb * (1.0 - mu_shrink)), 0.0f);
                     P.lin_mA = (float)(muA * nb * (1.0 + 1e-6));
-                    double cB = 0.5 - (muB + 4.0 * u + devm + ldexp(1.0, -21)) * nb;
+                    double cB = 0.5 - (muB + 4.0 * u + devm + mu_shrink) * nb;
                     P.lin_cB = nextafterf((float)cB, 0.0f);
                     if (!(cB > 0.25)) P.lin = 0;
                 }
@@ -428,9 +447,9 @@ static pc_status make_plan(const pc_bins *b, const Geom &g, const double *pts_lo
         double devm = 0.0;
         if (P.mode == PC_BIN_SMU) {
             for (int k = 0; k <= P.nb; ++k) devm = std::max(devm, fabs(P.eb[k] - (double)k / P.nb));
-            lin_mu = (P.los == PC_LOS_Z) && devm <= 1e-12;
+            lin_mu = (P.los == PC_LOS_Z || P.fp32_ok) && devm <= 1e-12;
         }
-        bool mode_ok = P.mode == PC_BIN_S || (P.mode == PC_BIN_SMU && P.los == PC_LOS_Z);
+        bool mode_ok = P.mode == PC_BIN_S || P.mode == PC_BIN_SMU;
         double dev = 0.0;
         for (int k = 0; k <= P.na; ++k) dev = std::max(dev, fabs(log2(P.ea[k] / e0) / lq - k));
         if (mode_ok && lin_mu && lq > 0.0 && dev <= 1e-6 && P.na < (1 << 20)) {
@@ -452,15 +471,17 @@ static pc_status make_plan(const pc_bins *b, const Geom &g, const double *pts_lo
                 P.lin_norange = 0;
                 if (P.mode == PC_BIN_SMU) {
                     const double nb = P.nb;   // mu scale and band as for linear s bins
-                    P.lin_nB = nextafterf((float)(nb * (1.0 - ldexp(1.0, -21))), 0.0f);
+                    P.lin_nB = nextafterf((float)(nb * (1.0 - mu_shrink)), 0.0f);
                     P.lin_mA = (float)(muA * nb * (1.0 + 1e-6));
-                    double cB = 0.5 - (muB + 4.0 * u + devm + ldexp(1.0, -21)) * nb;
+                    double cB = 0.5 - (muB + 4.0 * u + devm + mu_shrink) * nb;
                     P.lin_cB = nextafterf((float)cB, 0.0f);
                     if (!(cB > 0.25)) P.lin = P.lin_log = 0;
                 }
             }
         }
     }
+    P.path = !P.lin ? PLAN_LUT : (P.lin_log ? PLAN_LOG : (P.ea[0] == 0.0 ? PLAN_LIN : PLAN_LINOFF));
+    if (mid_mu) P.lin = P.lin_log = P.lin_norange = 0;
     // ---- (sigma, pi) with evenly spaced edges from 0: floors of both ------
     // t_sigma = sigma / D_a, t_pi = pi / D_b, sigma and pi formed as on the
     // table path, so their bands eps_sig and eps_z apply (in t units), plus
@@ -484,7 +505,48 @@ static pc_status make_plan(const pc_bins *b, const Geom &g, const double *pts_lo
             P.lin_invB2 = (float)(1.0 / Db);
             P.lin_thrB = nextafterf((float)(0.5 - etb), 0.0f);
             P.lin_norange = 0;
+            P.path = PLAN_LIN;
         }
+    }
+    // ---- fixed-point floors (PATH_FIX) ---------------------------------------
+    // The values of the floors from zero, summed once onto a grid of 2^-16: the
+    // band in these units, with half a unit for that sum.  Along z the bounds
+    // above are used with a factor of 1.25 instead of 2: per axis u (2.5 c +
+    // 3 |d|), hence s errs by u (4.33 c + 3 s), the squares' roundings add 1.5 u
+    // s, the reciprocal root 2.15 u s, and the scale and its product 2 u s (the
+    // last product is exact); mu by u (6.83 c / s + 3 + 3 + 1.5 + 2.15 + 1).
+    if (P.path == PLAN_LIN && P.na <= 126 && P.nb <= 126) {
+        const double one = 65536.0;
+        double es = 0.0, ep = 0.0;
+        if (P.mode == PC_BIN_SIGPI) {
+            const double Da = P.ea[P.na] / P.na, Db = P.eb[P.nb] / P.nb;
+            es = eps_sig / Da + 1e-9 + 4.0 * u * P.na;
+            ep = eps_z / Db + 1e-9 + 4.0 * u * P.nb;
+        } else {
+            const double D = P.ea[P.na] / P.na;
+            es = (1.25 * u * (4.34 * c + 8.7 * Rb) + tiny) / D + 1e-9;
+        }
+        P.fx_s = (unsigned)ceil(es * one + 0.5);
+        P.fx_p = (unsigned)ceil(ep * one + 0.5);
+        bool ok = es * one < 8192.0 && ep * one < 8192.0;
+        if (P.mode == PC_BIN_SMU) {
+            const double nb = P.nb;
+            const double mA = P.los == PC_LOS_Z ? 1.25 * 6.9 * u * c + tiny : muA;
+            const double mB = P.los == PC_LOS_Z ? 1.25 * 10.7 * u + ldexp(1.0, -46) : muB + 4.0 * u;
+            // the box tests' gap, less than 2^-20 X off, bounds s from below:
+            // within 1 % from 128 times that on (and the band's own roundings)
+            double ext = 0.0;
+            for (int a = 0; a < 3; ++a) ext = std::max(ext, (pts_hi[a] - pts_lo[a]) + g.L[a]);
+            P.fx_sf = std::max({c / 16.0, ldexp(ext, -13) + ldexp(X + Lm, -40), 1e-3 * R0});
+            P.fx_mA = nb * mA * one * 1.02;
+            P.fx_mB = nb * mB * one * 1.02 + 1e-12 * nb * one + 0.5 + 0.5;
+            ok = ok && P.fx_mA / P.fx_sf + P.fx_mB < 8192.0;
+        }
+        // no FP32 square may overflow (the kernel's indices rely on it), and the
+        // constant 1e-30 in the squares must stay far inside the first band
+        const double Dmin = std::min(P.ea[P.na] / P.na, P.mode == PC_BIN_SIGPI ? P.eb[P.nb] / P.nb : 1e300);
+        ok = ok && X + Lm + R0 + c < 1e15 && Dmin > 1e-9;
+        P.fix = ok ? 1 : 0;
     }
     // ---- stencil -------------------------------------------------------------
     int kmax[3] = {0, 0, 0};
@@ -507,36 +569,25 @@ static pc_status make_plan(const pc_bins *b, const Geom &g, const double *pts_lo
 // ---------------------------------------------------------------------------
 // one counting launch over a set of tasks
 // ---------------------------------------------------------------------------
-// Histogram replication from pc_opts.priv: 1 = one count copy per warp,
-// 2 = a single shared copy, otherwise automatic: lane copies (lane l updates
-// copy l % k) as many as fit a 16 KB budget, so the lanes of a warp do not
-// collide on the few bins of a small histogram.
+// Histogram replication from pc_opts.priv: 2 = a single shared copy,
+// otherwise lane copies (lane l updates copy l % k), as many as fit a 16 KB
+// budget, so the lanes of a warp do not collide on the few bins of a small
+// histogram (1 also keeps the weighted sums in binary64).
 // (weighted: binary64 weight sums share the copies and the budget; the
 // integer weight records take the counts' copies outside that budget.)
-static void choose_replication(int mode, int nbins, bool weighted, int &priv, int &hist_k) {
-    priv = 0;
+static void choose_replication(int mode, int nbins, bool weighted, int &hist_k) {
     hist_k = 1;
-    if (mode == 1) { priv = 1; return; }
     if (mode == 2) return;
     const long long per_copy = (long long)nbins * (4 + (weighted ? 8 : 0));
     while (hist_k < 32 && per_copy * hist_k * 2 <= 16384) hist_k *= 2;
 }
 
-// Rows of each shared histogram copy: the bins, the discarded rows of the
-// floor bins without a range test, and at least one row past the bins that
-// lanes without an in-range pair update (row nbins).
+// Entries of each shared histogram copy: rows of hs entries and one discarded
+// entry past them.  The (sigma, pi) floors send pi past its last bin to a
+// discarded column.
 static void set_hist_rows(PairParams &p, const Plan &P) {
-    p.nbins_smem = P.nbins + (p.lin_norange ? (P.mode == PC_BIN_S ? 1 : P.nb) : 0);
-    p.trash_row = P.nbins;
-    p.nbins_smem = std::max(p.nbins_smem, P.nbins + 1);
-}
-
-// Shared-memory fallback: fewer lane copies, then no warp copies, then the
-// global histogram.  Returns false when nothing is left to give up.
-static bool shrink_replication(PairParams &p) {
-    if (p.hist_k > 1) { p.hist_k /= 2; return true; }
-    if (p.priv) { p.priv = 0; return true; }
-    return false;
+    p.hs = P.nb + (P.mode == PC_BIN_SIGPI && p.path == PLAN_LIN ? 1 : 0);
+    p.nent = P.na * p.hs + 1;
 }
 
 struct CountJob {
@@ -647,21 +698,12 @@ static pc_status setup_count(const CountJob &J, const pc_bins *b, const pc_opts 
     for (auto &t : J.tasks) npts += t.gi.n;
     S.nblk_cap = (size_t)S.ntasks * S.ncell + (size_t)(npts / S.bi) + 16;
     S.hist_n = (size_t)J.nhist * S.P.nbins;
-    // rescue queue capacity: ~4e-3 of the expected in-range pairs (overflow
-    // is evaluated inside the pair kernel, so this only sets the fast case)
+    // rescue queue: only when asked for.  Near-edge pairs are checked inside
+    // the pair kernel otherwise, where their binary64 work overlaps the FP32
+    // pairs of the other warps
     S.qcap = 0;
     if (S.prec == PC_PREC_F32_RESCUE) {
         if (S.o.rescue_capacity > 0) S.qcap = (unsigned long long)S.o.rescue_capacity;
-        else if (S.o.rescue_capacity == 0) {
-            double vol = 1.0;
-            for (int a = 0; a < 3; ++a) vol *= std::max(J.phi[a] - J.plo[a], 1e-9);
-            double vs = 4.0 / 3.0 * M_PI * S.P.reff * S.P.reff * S.P.reff;
-            double pairs = 0.0;
-            for (auto &t : J.tasks)
-                pairs += 0.5 * (double)t.gi.n * (double)t.gj.n * std::min(1.0, vs / vol);
-            double want = std::max(1.0e6, 4.0e-3 * pairs * (J.is_auto ? 1.0 : 2.0));
-            S.qcap = (unsigned long long)std::min(want, 4.0e8);
-        }
     }
     return PC_OK;
 }
@@ -717,12 +759,179 @@ static pc_status upload_tables(const CountJob &J, const CountSetup &S, const Dev
     return PC_OK;
 }
 
+// The FP32 path's constants from the plan, and the box tests' limits.
+static void set_fp32_params(const Geom &g, const double *lo, const double *hi, const Plan &P, int prec,
+                            PairParams &p) {
+    p.path = (prec == PC_PREC_F32_RESCUE) ? P.path : PLAN_LUT;
+    p.lin_invA = P.lin_invA;
+    // the floors with an offset take t_s + 1 (exact floors down to t_s = -1)
+    p.lin_offA = P.lin_offA1;
+    p.lin_thrA = P.lin_thrA;
+    p.lin_mS = P.lin_mS;
+    p.lin_nB = P.lin_nB;
+    p.lin_mA = P.lin_mA;
+    p.lin_cB = P.lin_cB;
+    p.lin_invB2 = P.lin_invB2;
+    p.lin_thrB = P.lin_thrB;
+    set_hist_rows(p, P);
+    {
+        auto two = [](float v) { return make_float2(v, v); };
+        const double one = 65536.0;
+        p.fix = (p.path == PLAN_LIN && P.fix) ? 1 : 0;
+        p.f_tiny = two(1e-30f);
+        p.f_cfs = two((float)(128.0 + P.fx_s / one));
+        p.f_cfp = (float)(128.0 + P.fx_p / one);
+        p.f_lim = 128.5f + (float)P.na;
+        p.f_limB = 128.5f + (float)P.nb;
+        p.f_ts2 = 2 * P.fx_s;
+        p.f_tp2 = 2 * P.fx_p;
+        p.f_mA = nextafterf((float)P.fx_mA, INFINITY);
+        p.f_mB = nextafterf((float)P.fx_mB, INFINITY);
+        // pairs closer than fx_sf: t below it, with the band and the clamp's side
+        p.f_sf2 = (float)(P.fx_sf * P.fx_sf);
+        p.f_close = (float)(128.0 + 2.0 * P.fx_s / one + P.fx_sf * (1.0 + 1e-6) * P.lin_invA);
+        for (int a = 0; a < 3; ++a) p.L32[a] = (float)g.L[a];
+    }
+    // Box tests run in FP32 on coordinates relative to the grids' origins, at
+    // most X in magnitude (images included): outward-rounded boxes, and a gap
+    // that takes four more roundings of at most 2^-24 x 3 X, so a computed gap
+    // exceeds the true one by less than 2^-20 X (2^-50 of the absolute
+    // coordinates for the subtraction of the origin); squares and sums add a
+    // relative 2^-22.  The limits carry twice that.
+    double X = 0.0, A = 0.0, c = 0.0;
+    for (int a = 0; a < 3; ++a) {
+        X = std::max(X, (hi[a] - lo[a]) + g.L[a]);
+        A = std::max({A, fabs(lo[a]), fabs(hi[a])});
+        c = std::max(c, g.c[a]);
+    }
+    const double m = ldexp(X, -19) + ldexp(A, -49);
+    auto up = [&](double r) {
+        const double v = (r + m) * (r + m) * (1.0 + ldexp(1.0, -20));
+        return v < 1e38 ? nextafterf((float)v, INFINITY) : INFINITY;
+    };
+    p.r2prune = up(P.rcut);
+    p.q2prune = p.zprune = INFINITY;
+    if (P.mode == PC_BIN_SIGPI) {   // along z: sigma and pi each stay below their last edge
+        const double slack = P.rcut - P.reff;
+        p.q2prune = up(P.ea[P.na] + slack);
+        p.zprune = nextafterf((float)((P.eb[P.nb] + slack + m) * (1.0 + ldexp(1.0, -20))), INFINITY);
+    }
+    // absent points: beyond the reach of every point of a neighbouring cell
+    // (node), whose offset is at most rcut + 3 c, and small enough for exact floors
+    p.far = (float)(4.0 * (P.rcut + c));
+}
+
+// Shared-memory layout and launch shape: histogram copies (fewer until they
+// fit, else the global histogram), warps per CTA for the most resident warps
+// (ties: the smallest CTA).  wint: try the integer weight products first.
+static pc_status fit_params(int prec, int opt_priv, int dev, bool weighted, bool wint_try, bool wcorr,
+                            PairParams &p, size_t &smem, int &per_sm) {
+    int smem_optin = 0;
+    PC_CUDA(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    const int static_smem = 256;
+    const int lut_size = p.lut_total, path0 = p.path, hs0 = p.hs, nent0 = p.nent;
+    const bool f64 = prec == PC_PREC_F64;
+    const int nw_min = 4;
+    auto fit = [&](bool wint) {
+        p.wint = wint ? 1 : 0;
+        p.wcorr = (wint && wcorr) ? 1 : 0;
+        p.path = path0;
+        p.layout = 0;
+        choose_replication(opt_priv, p.nbins, weighted && !wint, p.hist_k);
+        if (p.fix && (wint || !weighted)) {   // fixed-point floors (not for binary64 weight sums)
+            p.path = PLAN_FIX;
+            if (p.mode == PC_BIN_S) {
+                p.layout = 2;
+                p.hist_k = 32;
+            } else if (!weighted) {
+                p.layout = 1;
+                p.hist_k = 1;
+            } else {   // mu = 1 (pi past its last bin) needs a column of its own
+                p.hs = p.n_b + 1;
+                p.nent = p.n_a * p.hs + 1 + p.n_b;
+                while (p.hs * p.hist_k > 255) p.hist_k /= 2;   // one byte (f_coef)
+            }
+        }
+        for (;;) {
+            p.smem_hist_ok = 1;
+            // the floor bins need no tables
+            p.lut_total = (p.path != PLAN_LUT || f64) ? 0 : lut_size;
+            const size_t need = f64 ? pairs_f64_smem(p) : pairs_f32_smem(p, nw_min);
+            if (need + static_smem <= (size_t)smem_optin) break;
+            if (p.layout == 0 && p.hist_k > 1) {   // fewer lane copies, then the global histogram
+                p.hist_k /= 2;
+                continue;
+            }
+            p.smem_hist_ok = 0;
+            p.path = PLAN_LUT;
+            p.layout = 0;
+            p.lut_total = f64 ? 0 : lut_size;
+            p.hist_k = 1;
+            break;
+        }
+    };
+    fit(wint_try && opt_priv != 1);
+    if (p.wint && !p.smem_hist_ok) {
+        p.hs = hs0;
+        p.nent = nent0;
+        fit(false);
+    }
+    p.wfold = (p.wint && p.hist_k < 16) ? 1 : 0;
+    {   // the floor paths' pair constants
+        auto two = [](float v) { return make_float2(v, v); };
+        const float row = 4.0f * p.hist_k * p.hs, col = 4.0f * p.hist_k;
+        p.f_coef = (unsigned)p.hist_k | (unsigned)(p.hs * p.hist_k) << 8;
+        p.c_23 = two(8388608.0f);
+        p.c_p = two(8388607.5f);
+        p.c_m1 = two(-1.0f);
+        p.c_invA = two(p.lin_invA);
+        p.c_offA = two(p.lin_offA);
+        p.c_thrA = two(p.lin_thrA);
+        p.c_nmS = two(-p.lin_mS);
+        p.c_invB = two(p.mode == PC_BIN_SIGPI ? p.lin_invB2 : p.lin_nB);
+        p.c_nmB = two(-p.lin_mA);
+        p.c_cB = two(p.mode == PC_BIN_SIGPI ? p.lin_thrB : p.lin_cB);
+        p.c_nrow = two(-row);
+        p.c_ncol = two(-col);
+        p.c_kA = 8388608.0f - (p.path == PLAN_LIN ? 0.5f : 1.5f) * row -
+                 (p.mode == PC_BIN_S ? 0.0f : 0.5f * col);
+    }
+    if (f64) {
+        smem = pairs_f64_smem(p);
+        if (smem + static_smem > (size_t)smem_optin)
+            return fail(PC_EUNSUPPORTED, "bins: tables do not fit in shared memory");
+        per_sm = pairs_f64_ctas_per_sm(p, smem);
+        return PC_OK;
+    }
+    // 8 warps at most with weights: a copy's products between a warp's flushes
+    // must hold one batch (64 x 64 products to one lane copy, WINT_LIMIT / 2 / 8)
+    int best_warps = 0, best_nw = 0;
+    for (int nw : {4, 8, 12, 16}) {
+        if (p.wint && nw > 8) break;
+        const size_t need = pairs_f32_smem(p, nw);
+        if (need + static_smem > (size_t)smem_optin) break;
+        const int n = pairs_f32_ctas_per_sm(p, need);
+        if (n * nw > best_warps) {
+            best_warps = n * nw;
+            best_nw = nw;
+        }
+    }
+    if (best_nw == 0) {
+        if (pairs_f32_smem(p, nw_min) + static_smem > (size_t)smem_optin)
+            return fail(PC_EUNSUPPORTED, "bins: tables do not fit in shared memory");
+        per_sm = 0;
+        return PC_OK;
+    }
+    smem = pairs_f32_smem(p, best_nw);
+    per_sm = best_warps / best_nw;
+    return PC_OK;
+}
+
 // Kernel parameters and launch shape.
 static pc_status make_params(const CountJob &J, const CountSetup &S, const DevBufs &B,
                              PairParams &p, int &grid, size_t &smem) {
     const Plan &P = S.P;
     memset(static_cast<void *>(&p), 0, sizeof(p));
-    p.groups = 1;
     p.tree = J.tree ? 1 : 0;
     p.tasks = B.tasks;
     p.blocks = B.blocks;
@@ -757,75 +966,22 @@ static pc_status make_params(const CountJob &J, const CountSetup &S, const DevBu
     p.counters = B.ctr;
     p.shard_count = S.o.shard_count > 1 ? S.o.shard_count : 1;
     p.shard_index = S.o.shard_count > 1 ? S.o.shard_index : 0;
-    p.lin = (S.prec == PC_PREC_F32_RESCUE) ? P.lin : 0;
-    p.lin_norange = p.lin ? P.lin_norange : 0;
-    p.lin_log = p.lin ? P.lin_log : 0;
-    p.lin_mS = P.lin_mS;
-    p.lin_invB2 = P.lin_invB2;
-    p.lin_thrB = P.lin_thrB;
-    set_hist_rows(p, P);
-    p.lin_invA = P.lin_invA;
-    // the range-tested floor bins take t_s + 1 (exact floors down to t_s = -1)
-    p.lin_offA = P.lin_norange ? P.lin_offA : P.lin_offA1;
-    p.lin_thrA = P.lin_thrA;
-    p.lin_nB = P.lin_nB;
-    p.lin_mA = P.lin_mA;
-    p.lin_cB = P.lin_cB;
-
-    int dev_sms = 0, smem_optin = 0;
-    PC_CUDA(cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, S.dev));
-    PC_CUDA(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, S.dev));
-    const int static_smem = 256;
-    const int lut_size = p.lut_total;
-    // shared-memory layout for a weight path: replication, then fewer copies
-    // until it fits, else the global histogram
-    auto fit = [&](bool wint) {
-        p.wint = wint ? 1 : 0;
-        p.wcorr = (wint && J.wcorr) ? 1 : 0;
-        choose_replication(S.o.priv, P.nbins, S.weighted && !wint, p.priv, p.hist_k);
-        for (;;) {
-            p.wint_k = p.hist_k;   // the weight records take the counts' lane copies
-            p.smem_hist_ok = 1;
-            // the floor-based bins need no tables (they serve only the global-
-            // histogram variant)
-            p.lut_total = p.lin ? 0 : lut_size;
-            size_t need = (S.prec == PC_PREC_F64) ? pairs_f64_smem(p) : pairs_f32_smem(p, S.ipt);
-            if (need + static_smem <= (size_t)smem_optin) break;
-            if (shrink_replication(p)) continue;
-            p.smem_hist_ok = 0;
-            p.lut_total = lut_size;
-            break;
-        }
-        return (S.prec == PC_PREC_F64) ? pairs_f64_smem(p) : pairs_f32_smem(p, S.ipt);
-    };
+    set_fp32_params(J.geom, J.lo, J.hi, P, S.prec, p);
+    p.nsub = (S.bi + 63) / 64;
+    p.multi = J.nhist > 1 ? 1 : 0;
+    for (auto &t : J.tasks) p.npts_i += t.gi.n;
+    p.npts_i /= p.shard_count;
     // integer weight products need floor bins, every weight packable and
     // shared histograms with one count copy per CTA; with fewer than 16 lane
     // copies (more than a few hundred bins) a copy would be flushed every few
     // hundred j-points, so its records are folded into the CTA's exact sums
     // instead (fold mode)
-    const bool wint_try = S.weighted && p.lin && J.wint_ok && S.prec == PC_PREC_F32_RESCUE;
-    smem = fit(wint_try);
-    if (p.wint && !(p.smem_hist_ok && !p.priv)) smem = fit(false);
-    p.wfold = (p.wint && p.hist_k < 16) ? 1 : 0;
-    if (smem + static_smem > (size_t)smem_optin)
-        return fail(PC_EUNSUPPORTED, "bins: tables do not fit in shared memory");
-    int per_sm = (S.prec == PC_PREC_F64) ? pairs_f64_ctas_per_sm(p, smem)
-                                         : pairs_f32_ctas_per_sm(p, S.ipt, smem);
-    // A shared histogram so large that at most two CTAs of NT threads fit an
-    // SM: run CTAs of four independent thread groups sharing one histogram
-    // (single-histogram jobs, floor bins, binary64 or no weights, 2 i-points)
-    if (S.prec == PC_PREC_F32_RESCUE && p.smem_hist_ok && p.lin && !p.wint && !p.priv &&
-        J.nhist == 1 && S.ipt == 2 && per_sm <= 2 && !p.tree) {
-        p.groups = 4;
-        const size_t smem4 = pairs_f32_smem(p, S.ipt);
-        const int per4 = (smem4 + 8192 <= (size_t)smem_optin) ? pairs_f32_ctas_per_sm(p, S.ipt, smem4) : 0;
-        if (per4 >= 1) {
-            smem = smem4;
-            per_sm = per4;
-        } else {
-            p.groups = 1;
-        }
-    }
+    const bool wint_try = S.weighted && p.path != PLAN_LUT && J.wint_ok && S.prec == PC_PREC_F32_RESCUE;
+    int per_sm = 0;
+    pc_status s = fit_params(S.prec, S.o.priv, S.dev, S.weighted, wint_try, J.wcorr, p, smem, per_sm);
+    if (s != PC_OK) return s;
+    int dev_sms = 0;
+    PC_CUDA(cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, S.dev));
     if (per_sm <= 0)
         return fail(PC_ECUDA, std::string("pair kernel cannot be resident: ") + pc_last_error());
     if (S.o.grid_ctas_per_sm > 0) per_sm = std::min(per_sm, S.o.grid_ctas_per_sm);
@@ -851,7 +1007,7 @@ static pc_status enqueue_count(const CountSetup &S, const DevBufs &B, const Pair
                                  B.off, B.tot, st));
     if (ev_pairs) PC_CUDA(cudaEventRecord(ev_pairs, st));
     cudaError_t e = (S.prec == PC_PREC_F64) ? launch_pairs_f64(p, grid, smem, st)
-                                            : launch_pairs_f32(p, S.ipt, grid, smem, st);
+                                            : launch_pairs_f32(p, grid, smem, st);
     if (e != cudaSuccess) return cuda_fail(e, "pair kernel launch");
     if (ev_rescue) PC_CUDA(cudaEventRecord(ev_rescue, st));
     if (S.prec == PC_PREC_F32_RESCUE && S.qcap) {
@@ -1111,8 +1267,10 @@ static pc_status run_count_graph(const CountJob &J, const std::vector<const pc_g
 
 static TaskDev task_of(const pc_grid *gi, const pc_grid *gj, int hist, int is_auto) {
     TaskDev t;
-    t.gi = GridDev{gi->rel, gi->cx, gi->xw, gi->cell_start, gi->n, gi->wlo};
-    t.gj = GridDev{gj->rel, gj->cx, gj->xw, gj->cell_start, gj->n, gj->wlo};
+    t.gi = GridDev{gi->rel, gi->cx, gi->xw, gi->cell_start, gi->n, gi->wlo, gi->obox,
+                   {gi->g.lo[0], gi->g.lo[1], gi->g.lo[2]}};
+    t.gj = GridDev{gj->rel, gj->cx, gj->xw, gj->cell_start, gj->n, gj->wlo, gj->obox,
+                   {gj->g.lo[0], gj->g.lo[1], gj->g.lo[2]}};
     t.hist = hist;
     t.is_auto = is_auto;
     // one unit of the integer weight products: 2^(emax_i + emax_j - 300)
@@ -1163,6 +1321,10 @@ extern "C" pc_status pc_count_cross(const pc_grid *g1, const pc_grid *g2, const 
         return fail(PC_EINVAL, "pc_count_cross: grids differ in box, bounds or cell size");
     if (wcounts && !(g1->weighted && g2->weighted))
         return fail(PC_EINVAL, "pc_count_cross: both grids need weights for weighted counts");
+    // The denser catalogue gives the i-points: its 64 points fill a warp and
+    // span a small box, so fewer boxes of the other come within reach (every
+    // pair is symmetric).  Shards are cells of g1, so they keep it
+    if (!(o && o->shard_count > 1) && g2->n > g1->n) std::swap(g1, g2);
     CountJob J;
     J.tasks.push_back(task_of(g1, g2, 0, 0));
     J.nhist = 1;
@@ -1212,6 +1374,11 @@ static bool same_tree_geometry(const pc_tree *a, const pc_tree *b) {
     return true;
 }
 
+static GridDev tree_dev(const pc_tree *t) {
+    return GridDev{t->rel, nullptr, t->xw, nullptr, t->n, t->wlo, t->obox,
+                   {t->g.lo[0], t->g.lo[1], t->g.lo[2]}};
+}
+
 static double tree_rmin(const pc_tree *t) {
     if (t->g.periodic || !(t->r2min > 0.0)) return 0.0;
     return sqrt(t->r2min) * (1.0 - 1e-12);
@@ -1230,11 +1397,13 @@ extern "C" pc_status pc_count_tree(const pc_tree *t1, const pc_tree *t2, const p
     if (wcounts && !(t1->weighted && tj->weighted))
         return fail(PC_EINVAL, "pc_count_tree: weighted counts need weights on every tree");
     cudaStream_t st = (cudaStream_t)stream;
+    // the denser catalogue gives the i-points (see pc_count_cross)
+    if (!is_auto && !(opt && opt->shard_count > 1) && tj->n > t1->n) std::swap(t1, tj);
 
     CountJob J;
     TaskDev T;
-    T.gi = GridDev{t1->rel, nullptr, t1->xw, nullptr, t1->n, t1->wlo};
-    T.gj = GridDev{tj->rel, nullptr, tj->xw, nullptr, tj->n, tj->wlo};
+    T.gi = tree_dev(t1);
+    T.gj = tree_dev(tj);
     T.hist = 0;
     T.is_auto = is_auto ? 1 : 0;
     T.wscale = (t1->wint && tj->wint) ? ldexp(1.0, t1->wemax + tj->wemax - 300) : 0.0;
@@ -1359,7 +1528,7 @@ extern "C" pc_status pc_count_tree_batch(const pc_tree *const *ts, int m, const 
         if (wcounts && !t->weighted)
             return fail(PC_EINVAL, "pc_count_tree_batch: weighted counts need weights on every tree");
         TaskDev T;
-        T.gi = GridDev{t->rel, nullptr, t->xw, nullptr, t->n, t->wlo};
+        T.gi = tree_dev(t);
         T.gj = T.gi;
         T.hist = k;
         T.is_auto = 1;
@@ -1658,11 +1827,9 @@ constexpr int NA_MAX_CELLS = 1 << 18;     // cells of the grid
 constexpr int NA_MAX_BLOCKS = 1 << 19;    // i-blocks
 constexpr int NA_MAX_ROWS = 8192;         // stencil rows
 constexpr int NA_MAX_LUT = 2 * (MAX_LUT + 2);
-constexpr unsigned long long NA_QUEUE = 1ull << 17;   // rescue slots (overflow is evaluated in-kernel)
 
 struct NaLayout {
-    size_t hist, whist, counters, scalars, tasks, stencil, lut, ea, eb, cnt, off, tot, blocks, queue,
-        total;
+    size_t hist, whist, counters, scalars, tasks, stencil, lut, ea, eb, cnt, off, tot, blocks, total;
 };
 
 constexpr size_t na_align(size_t x) { return (x + 255) / 256 * 256; }
@@ -1683,14 +1850,13 @@ constexpr NaLayout na_layout() {
     L.off = o;      o = na_align(o + sizeof(int) * (NA_MAX_CELLS + 1));
     L.tot = o;      o = na_align(o + sizeof(int) * (NA_MAX_CELLS / 4096 + 2));
     L.blocks = o;   o = na_align(o + sizeof(Block) * NA_MAX_BLOCKS);
-    L.queue = o;    o = na_align(o + sizeof(uint3) * NA_QUEUE);
     L.total = o;
     return L;
 }
 
 constexpr NaLayout NA = na_layout();
 
-// The scratch array (12.3 MiB).  Every GPU that loads the library holds
+// The scratch array (10.8 MiB).  Every GPU that loads the library holds
 // it until the process exits.
 static __device__ __align__(256) unsigned char g_count_scratch[NA.total];
 
@@ -1784,7 +1950,6 @@ extern "C" pc_status pc_count_auto_noalloc(const pc_grid *g, const pc_bins *b, c
 
     PairParams p;
     memset(static_cast<void *>(&p), 0, sizeof(p));
-    p.groups = 1;
     p.tasks = tasks;
     p.blocks = (const Block *)(base + NA.blocks);
     p.nblocks = sc + 1;
@@ -1812,52 +1977,24 @@ extern "C" pc_status pc_count_auto_noalloc(const pc_grid *g, const pc_bins *b, c
     p.Eb = (const double *)(base + NA.eb);
     p.hist = hist;
     p.whist = wcounts ? whist : nullptr;
-    p.queue = (uint3 *)(base + NA.queue);
     p.qcount = ctr + 2;
-    p.qcap = (prec == PC_PREC_F32_RESCUE) ? NA_QUEUE : 0;
+    p.qcap = 0;   // near-edge pairs are checked inside the pair kernel
     p.counters = ctr;
     p.shard_count = o.shard_count > 1 ? o.shard_count : 1;
     p.shard_index = o.shard_count > 1 ? o.shard_index : 0;
-    choose_replication(o.priv, P.nbins, wcounts != nullptr, p.priv, p.hist_k);
-    p.wint_k = 1;   // binary64 weight sums here (no integer weight planes)
-    p.lin = (prec == PC_PREC_F32_RESCUE) ? P.lin : 0;
-    p.lin_norange = p.lin ? P.lin_norange : 0;
-    p.lin_log = p.lin ? P.lin_log : 0;
-    p.lin_mS = P.lin_mS;
-    p.lin_invB2 = P.lin_invB2;
-    p.lin_thrB = P.lin_thrB;
-    set_hist_rows(p, P);
-    p.lin_invA = P.lin_invA;
-    // the range-tested floor bins take t_s + 1 (exact floors down to t_s = -1)
-    p.lin_offA = P.lin_norange ? P.lin_offA : P.lin_offA1;
-    p.lin_thrA = P.lin_thrA;
-    p.lin_nB = P.lin_nB;
-    p.lin_mA = P.lin_mA;
-    p.lin_cB = P.lin_cB;
-
-    int sms = 0, smem_optin = 0;
+    set_fp32_params(g->g, g->pts_lo, g->pts_hi, P, prec, p);
+    p.nsub = (bi + 63) / 64;
+    p.npts_i = g->n / p.shard_count;
+    int sms = 0, per_sm = 0;
+    size_t smem = 0;
     PC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, cur));
-    PC_CUDA(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, cur));
-    const int lut_size = p.lut_total;
-    for (;;) {
-        p.smem_hist_ok = 1;
-        p.lut_total = p.lin ? 0 : lut_size;
-        size_t need = (prec == PC_PREC_F64) ? pairs_f64_smem(p) : pairs_f32_smem(p, ipt);
-        if (need + 256 <= (size_t)smem_optin) break;
-        if (shrink_replication(p)) continue;
-        p.smem_hist_ok = 0;
-        p.lut_total = lut_size;
-        break;
-    }
-    size_t smem = (prec == PC_PREC_F64) ? pairs_f64_smem(p) : pairs_f32_smem(p, ipt);
-    if (smem + 256 > (size_t)smem_optin)
-        return fail(PC_EUNSUPPORTED, "bins: tables do not fit in shared memory");
-    int per_sm = (prec == PC_PREC_F64) ? pairs_f64_ctas_per_sm(p, smem)
-                                       : pairs_f32_ctas_per_sm(p, ipt, smem);
+    // binary64 weight sums here (fold mode's sums would need an allocation)
+    s = fit_params(prec, o.priv, cur, wcounts != nullptr, false, false, p, smem, per_sm);
+    if (s != PC_OK) return s;
     if (per_sm <= 0) return fail(PC_ECUDA, "pair kernel cannot be resident");
     if (o.grid_ctas_per_sm > 0) per_sm = std::min(per_sm, o.grid_ctas_per_sm);
     cudaError_t e = (prec == PC_PREC_F64) ? launch_pairs_f64(p, sms * per_sm, smem, st)
-                                          : launch_pairs_f32(p, ipt, sms * per_sm, smem, st);
+                                          : launch_pairs_f32(p, sms * per_sm, smem, st);
     if (e != cudaSuccess) return cuda_fail(e, "pair kernel launch");
     if (p.qcap) {
         e = launch_rescue(p, st);

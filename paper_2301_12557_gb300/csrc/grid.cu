@@ -213,25 +213,13 @@ pc_status weight_stats(const void *w, int w_is_f32, int n, cudaStream_t st, int 
     return PC_OK;
 }
 
-// Packed integer weight (stored in the w lane of the FP32 point record): the
-// binary32 significand M with its leading one (w = M 2^(e-150)), shifted up
-// by 8 - (emax - e) (the grid's exponents span at most 8 binades), so that it
-// fits 32 bits and a pair's exact 64-bit product is (M_i M_j) 2^(16 - k_i -
-// k_j), k = emax - e.  Zero weights pack to 0.
-__device__ __forceinline__ unsigned pack_weight(double wv, int emax, int span) {
-    const unsigned b = __float_as_uint(__double2float_rn(wv));
-    const int e = (int)((b >> 23) & 0xFF);
-    if (e == 0) return 0u;
-    return ((b & 0x7FFFFFu) | 0x800000u) << (span - (emax - e));
-}
-
 __global__ void k_scatter(const double *__restrict__ xyz, const void *__restrict__ w, int w_is_f32,
-                          int wpack_emax, int wpack_span, int n, Geom g, int sub_bits,
+                          int wpack_emax, int n, Geom g, int sub_bits,
                           const int *__restrict__ cell,
                           const int *__restrict__ slot, const int *__restrict__ key_start,
                           float4 *__restrict__ rel,
                           uint16_t *__restrict__ cxo, double4_32a *__restrict__ xw,
-                          int *__restrict__ perm, float *__restrict__ wlo) {
+                          int *__restrict__ perm, unsigned *__restrict__ wlo) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     int key = cell[i];
@@ -250,12 +238,46 @@ __global__ void k_scatter(const double *__restrict__ xyz, const void *__restrict
     }
     double wv = 1.0;
     if (w) wv = w_is_f32 ? (double)((const float *)w)[i] : ((const double *)w)[i];
-    const unsigned wp = (w && wpack_emax > 0) ? pack_weight(wv, wpack_emax, wpack_span) : 0u;
+    const unsigned wp = (w && wpack_emax > 0) ? weight_hi(wv, wpack_emax) : 0u;
     rel[pos] = make_float4(r[0], r[1], r[2], __uint_as_float(wp));
     if (wlo) wlo[pos] = weight_lo(wv, wpack_emax);
     cxo[pos] = (uint16_t)id[0];
     xw[pos] = make_double4_32a(x[0], x[1], x[2], wv);
     perm[pos] = i;
+}
+
+// Box of every eight consecutive points relative to `org`, rounded outward: a
+// thread per point, the eight of an oct reduced with shuffles.  One read of
+// the 32-byte records (coalesced) and 4 bytes written a point.
+__global__ void __launch_bounds__(256) k_obox(const double4_32a *__restrict__ xw, int n, double ox, double oy,
+                                              double oz, float4 *__restrict__ obox) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const double org[3] = {ox, oy, oz};
+    float lo[3], hi[3];
+    double4_32a a = make_double4_32a(0.0, 0.0, 0.0, 0.0);
+    if (i < n) a = xw[i];
+    const double v[3] = {a.x, a.y, a.z};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        lo[k] = i < n ? __double2float_rd(__dsub_rd(v[k], org[k])) : INFINITY;
+        hi[k] = i < n ? __double2float_ru(__dsub_ru(v[k], org[k])) : -INFINITY;
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) {
+            lo[k] = fminf(lo[k], __shfl_xor_sync(0xffffffffu, lo[k], o));
+            hi[k] = fmaxf(hi[k], __shfl_xor_sync(0xffffffffu, hi[k], o));
+        }
+    }
+    if (i < n && (i & 7) == 0) {
+        obox[i / 4] = make_float4(lo[0], lo[1], lo[2], 0.f);
+        obox[i / 4 + 1] = make_float4(hi[0], hi[1], hi[2], 0.f);
+    }
+}
+
+cudaError_t make_obox(const double4_32a *xw, int n, const double org[3], float4 *obox, cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    k_obox<<<(unsigned)(((long long)n + 255) / 256), 256, 0, st>>>(xw, n, org[0], org[1], org[2], obox);
+    note_launch();
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -460,6 +482,7 @@ static void grid_release(pc_grid *g) {
     cudaFree(g->cell_start);
     cudaFree(g->perm);
     cudaFree(g->wlo);
+    cudaFree(g->obox);
     delete g;
 }
 
@@ -648,7 +671,8 @@ extern "C" pc_status pc_build_grid(const double *xyz, const void *w, int w_is_f3
     if (e == cudaSuccess) e = ::pc::alloc_dev(&g->xw, sizeof(double4_32a) * nn);
     if (e == cudaSuccess) e = ::pc::alloc_dev(&g->cell_start, sizeof(int) * (g->ncell + 1));
     if (e == cudaSuccess) e = ::pc::alloc_dev(&g->perm, sizeof(int) * nn);
-    if (e == cudaSuccess && g->wcorr) e = ::pc::alloc_dev(&g->wlo, sizeof(float) * nn);
+    if (e == cudaSuccess) e = ::pc::alloc_dev(&g->obox, obox_bytes((long long)nn));
+    if (e == cudaSuccess && g->wcorr) e = ::pc::alloc_dev(&g->wlo, sizeof(unsigned) * nn);
     if (e != cudaSuccess) {
         cleanup();
         grid_release(g);
@@ -684,12 +708,13 @@ extern "C" pc_status pc_build_grid(const double *xyz, const void *w, int w_is_f3
     if (e == cudaSuccess && n > 0) {
         int blocks = (int)((n + 255) / 256);
         k_scatter<<<blocks, 256, 0, st>>>(dxyz, dw, w_is_f32, g->wint ? g->wemax : 0,
-                                          WINT_GRID_SPAN, (int)n, G,
+                                          (int)n, G,
                                           sub_bits, cell, slot, key_start, g->rel, g->cx, g->xw,
                                           g->perm, g->wlo);
         note_launch();
         e = cudaGetLastError();
     }
+    if (e == cudaSuccess) e = make_obox(g->xw, (int)n, G.lo, g->obox, st);
     if (key_start) cudaFreeAsync(key_start, st);
     if (counts) cudaFreeAsync(counts, st);
     if (cell) cudaFreeAsync(cell, st);

@@ -1,28 +1,40 @@
 // Pair-separation histogram kernels (templates; instantiated per binning
 // mode in pairs_*.cu).
 //
-// Work decomposition (grid traversal of Sect. 2.1 with the half-shell
-// duplicate removal of Sect. 3.1): a persistent CTA (or each of its thread
-// groups) repeatedly takes a block of up to NT * RI consecutive points of one
-// cell (the i-points, kept in registers) and streams every candidate j-point
-// of the neighbouring cells through shared memory.  Neighbours are visited row
-// by row: for a stencil row (dy, dz) the cells (ax + xlo .. ax + xhi, ay + dy,
-// az + dz) are contiguous in the cell-sorted arrays, so each row is one index
-// range (split at most in three by periodic wrapping).  Periodic images are
-// handled by shifting whole cells (Sect. 3.1), never by testing each pair.
-// Runs of 32 staged j-points are skipped per warp when their bounding box is
-// out of reach of the warp's i-points.
+// Work decomposition of the FP32 kernel (grid traversal of Sect. 2.1 with the
+// half-shell duplicate removal of Sect. 3.1): every warp works on its own,
+// with no barrier among the warps of a CTA, which share only the histogram.
+// A warp takes up to 64 consecutive points of one cell (the i-points, two a
+// lane, in registers) and walks the candidate j-points of the neighbouring
+// cells.  Neighbours are visited row by row: for a stencil row (dy, dz) the
+// cells (ax + xlo .. ax + xhi, ay + dy, az + dz) are contiguous in the
+// cell-sorted arrays, so each row is one index range (split at most in three
+// by periodic wrapping).  Periodic images are handled by shifting whole cells
+// (Sect. 3.1), never by testing each pair.  The build stores the bounding box
+// of every run of eight points (an oct); the warp tests 32 octs at a time
+// against the box of its i-points and stages only those that can reach it,
+// eight octs a batch, in its own slice of shared memory.
 //
-// FP32 path: the j-point is staged as its offset from the i-cell centre,
+// FP32 arithmetic: the j-point is staged as its offset from the i-cell centre,
 // rel_j + delta * c, so a pair costs three subtractions and three
-// multiply-adds.  The squared separation selects candidates; in-range pairs
-// are binned by floors of scaled values (evenly spaced or logarithmic s,
-// evenly spaced mu, sigma and pi; Sect. 3.2.2) or through lookup tables for
-// other edges (Sect. 3.2.3), each table entry holding the single bin edge
-// near that table cell.  A pair whose value lies within the proven FP32 error
-// band of an edge is re-evaluated with the exact binary64 definition (queued
-// for the rescue kernel), so the integer counts equal the binary64 definition
-// exactly.
+// multiply-adds, two j-points per packed instruction.  In-range pairs are
+// binned by floors of scaled values (evenly spaced or logarithmic s, evenly
+// spaced mu, sigma and pi; Sect. 3.2.2) or through lookup tables for other
+// edges (Sect. 3.2.3), each table entry holding the single bin edge near that
+// table cell.  The floor paths form a counter's address in FP32 as well and
+// send every pair outside the histogram to a discarded entry with one integer
+// minimum, so the loop has no branch and no range test.  A pair whose value
+// lies within the proven FP32 error band of an edge is checked with the exact
+// binary64 definition and its counter corrected if the FP32 bin was another
+// one, so the integer counts equal the binary64 definition exactly.
+//
+// What bounds it (2M clustered points, (s, mu) 40 x 100, 6.70e10 pairs in
+// range): issue slots (70 % used; the FMA and integer pipes at 52 %, shared
+// memory at 62 %).  139 warp instructions per 64 x 4 pairs, 113 of them the loop
+// itself; 18 % of the pairs are empty lanes and the ends of octs.  80.7 ms
+// against 154.7 ms for CTAs of 128 threads that staged every candidate tile
+// behind a barrier (138 instructions per 64 x 2 pairs in range, issued on 60 % of
+// the cycles) and queued near-edge pairs for a second kernel.
 #pragma once
 
 #include "pc_internal.cuh"
@@ -33,105 +45,103 @@ constexpr unsigned long long FLUSH_LIMIT = 1ull << 30;
 // integer weight path: products (each < 2^48) per lane copy between flushes;
 // each of its three u32 piece sums then adds less than 2^16 pieces of 16
 // bits, and the copy's recombined sum stays below 2^64.  With binary64
-// remainders (W == 3) a product is below 2^49, its top piece below 2^17,
-// and half as many products fit.
-constexpr unsigned long long WINT_LIMIT = 1ull << 16;
-
-struct SmemLayout {
-    size_t lut, ea, eb, hist, whist, seg, tile, meta, tw, q, total;
-    size_t gstride;   // per-group area [seg, q end): group g's copy is g * gstride further
-};
+// weights (W == 3) a product may reach 2^48, its top piece 2^16, and half as
+// many are allowed.
+constexpr unsigned WINT_LIMIT = 1u << 16;
 
 __host__ __device__ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// FP32 path (f64 = false) and FP64 path (f64 = true) share one layout.
-__host__ __device__ inline SmemLayout smem_layout(const PairParams &p, bool f64) {
-    SmemLayout L;
-    size_t o = 0;
-    L.lut = o;
-    o = align_up(o + (size_t)p.lut_total * sizeof(float2), 16);
-    // squared edges: the FP64 kernel's binning (the FP32 kernel's rescue
-    // reads them from global memory)
-    L.ea = o;
-    if (f64) o = align_up(o + (size_t)(p.n_a + 1) * sizeof(double), 16);
-    L.eb = o;
-    if (f64) o = align_up(o + (size_t)(p.n_b + 1) * sizeof(double), 16);
-    int copies = (p.priv ? NT / 32 : 1) * p.hist_k;
-    L.hist = o;
-    if (p.smem_hist_ok) o = align_up(o + (size_t)p.nbins_smem * copies * sizeof(int), 16);
-    L.whist = o;
-    if (p.smem_hist_ok && p.weighted) {
-        if (p.wint && !f64)   // records of three u32 sums of 16-bit product pieces
-            o = align_up(o + (size_t)3 * p.nbins_smem * p.wint_k * sizeof(unsigned), 16);
-        else
-            o = align_up(o + (size_t)p.nbins_smem * p.hist_k * sizeof(double), 16);
+// ---------------------------------------------------------------------------
+// FP32 kernel: shared memory
+// ---------------------------------------------------------------------------
+constexpr int BI = 64;        // i-points per warp (two a lane)
+constexpr int JB = 64;        // j-points per staged batch (eight octs)
+constexpr int JO = JB / 8;
+constexpr int RING = 64;      // octs kept for staging (ring): up to JO - 1 + 32
+constexpr int QCAP = 64;      // near-edge quads kept by a warp before it checks them
+constexpr int FIX_TOP = 126;  // most bins per axis of the fixed-point floors
+constexpr int SEG_G = 97;     // j-segments of a chunk: 32 stencil rows, <= 3 each, and the own cell
+constexpr int SEG_T = 33;     // 32 listed tree nodes and the own node
+
+// Byte offsets of a warp's slice.
+struct WarpOff {
+    __host__ __device__ static constexpr int seg(bool) { return 0; }                               // int4[nseg]
+    __host__ __device__ static constexpr int nseg(bool tree) { return tree ? SEG_T : SEG_G; }
+    __host__ __device__ static constexpr int soff(bool tree) { return nseg(tree) * 16; }          // float4[nseg] (tree)
+    __host__ __device__ static constexpr int tile(bool tree) { return soff(tree) + (tree ? SEG_T * 16 : 0); }   // x, y, z
+    __host__ __device__ static constexpr int tw(bool tree) { return tile(tree) + 3 * JB * 4; }    // weights, 8 B a point
+    __host__ __device__ static constexpr int queue(bool tree, int w) { return tw(tree) + (w ? JB * 8 : 0); }    // uint2[QCAP]
+    __host__ __device__ static constexpr int ring(bool tree, int w) { return queue(tree, w) + QCAP * 8; }       // int4[RING]
+    __host__ __device__ static constexpr int pref(bool tree, int w) { return ring(tree, w) + RING * 16; }       // int[nseg + 1]
+    __host__ __device__ static constexpr int total(bool tree, int w) {
+        return (pref(tree, w) + (nseg(tree) + 1) * 4 + 15) / 16 * 16;
     }
+};
+
+// Histogram layouts (word = 4 bytes; entry (n, m), lane copy k of hist_k):
+//  LAY_ROWS   word (n hs + m) hist_k + k; weights: binary64 sums at the same
+//             index, or records of three u32 at 3 x the word
+//  LAY_SKEW   word w + w / 32, w = 256 n + m: the bytes of the two fixed-point
+//             floors side by side; the skew puts rows 8 banks apart (counts only)
+//  LAY_BYTES  word 64 n + k, 32 copies (one axis); weights: the pieces of a
+//             product at + 32 words and, past the last row, at + 0 and + 32
+enum { LAY_ROWS = 0, LAY_SKEW = 1, LAY_BYTES = 2 };
+
+__host__ __device__ inline int hist_words(const PairParams &p) {
+    if (p.layout == LAY_SKEW) {
+        const int w = 256 * p.n_a + 255;
+        return w + w / 32 + 1;
+    }
+    if (p.layout == LAY_BYTES) return 64 * (p.n_a + 1);
+    return p.nent * p.hist_k;
+}
+
+// Fill in the layout of a CTA of nw warps: histograms, weight sums, tables,
+// the warps' slices.  Returns the bytes.
+inline size_t f32_layout(PairParams &p, int nw) {
+    size_t o = 0;
+    if (p.smem_hist_ok) o = align_up(o + (size_t)hist_words(p) * sizeof(int), 16);
+    p.sm_whist = (int)o;
+    if (p.smem_hist_ok && p.weighted) {   // piece sums, or binary64 sums
+        if (p.layout == LAY_BYTES) o += (size_t)hist_words(p) * sizeof(unsigned);
+        else o = align_up(o + (size_t)hist_words(p) * (p.wint ? 3 * sizeof(unsigned) : sizeof(double)), 16);
+    }
+    p.sm_lut = (int)o;
+    o = align_up(o + (size_t)p.lut_total * sizeof(float2), 16);
+    p.sm_warp = (int)o;
+    p.nwarps = nw;
+    return o + (size_t)nw * WarpOff::total(p.tree != 0, p.weighted);
+}
+
+// FP64 kernel: offsets of its shared arrays.
+struct SmemLayout64 {
+    size_t ea, eb, hist, whist, seg, tile, meta, total;
+};
+__host__ __device__ inline SmemLayout64 f64_layout(const PairParams &p) {
+    SmemLayout64 L;
+    size_t o = 0;
+    L.hist = o;
+    if (p.smem_hist_ok) o = align_up(o + (size_t)hist_words(p) * sizeof(int), 16);
+    L.whist = o;
+    if (p.smem_hist_ok && p.weighted) o = align_up(o + (size_t)p.nent * p.hist_k * sizeof(double), 16);
+    L.ea = o;
+    o = align_up(o + (size_t)(p.n_a + 1) * sizeof(double), 16);
+    L.eb = o;
+    o = align_up(o + (size_t)(p.n_b + 1) * sizeof(double), 16);
     L.seg = o;
-    o = align_up(o + (size_t)(p.tree && !f64 ? MAXSEG_T : MAXSEG) * sizeof(int4), 16);
-    int tj = f64 ? TJ64 : TJ;
+    o = align_up(o + (size_t)MAXSEG * sizeof(int4), 16);
     L.tile = o;
-    o = align_up(o + (size_t)2 * tj * (f64 ? sizeof(double4_32a) : 3 * sizeof(float)), 16);
+    o = align_up(o + (size_t)TJ64 * sizeof(double4_32a), 16);
     L.meta = o;
-    if (f64) o = align_up(o + (size_t)2 * tj * sizeof(int2), 16);
-    else if (p.tree) o = align_up(o + (size_t)MAXSEG_T * sizeof(float4), 16);   // segment offsets
-    // staged j weights: binary64, or the packed 4-byte integer weights (and,
-    // with binary64 remainders, the 4-byte remainders after them)
-    L.tw = o;
-    if (p.weighted && !f64)
-        o = align_up(o + (size_t)2 * tj * (p.wint ? (p.wcorr ? 2 : 1) * sizeof(unsigned) : sizeof(double)), 16);
-    L.q = o;
-    o = align_up(o + (size_t)LQ * sizeof(uint3), 16);
-    L.gstride = o - L.seg;
-    L.total = L.seg + (size_t)(f64 ? 1 : p.groups) * L.gstride;
+    o = align_up(o + (size_t)TJ64 * sizeof(int2), 16);
+    L.total = o;
     return L;
 }
 
 // ---------------------------------------------------------------------------
-// thread groups: a CTA of G groups of NT threads; each group works on its own
-// blocks and synchronises only with itself (named barrier 1 + group)
+// warp helpers
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int gtid() { return (int)(threadIdx.x % NT); }
-
-template <int G>
-__device__ __forceinline__ void gsync() {
-    if (G == 1) {
-        __syncthreads();
-    } else {
-        asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)(threadIdx.x / NT)), "r"(NT) : "memory");
-    }
-}
-
-template <int G>
-__device__ __forceinline__ bool gsync_or(bool v) {
-    if (G == 1) return __syncthreads_or(v) != 0;
-    unsigned r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, %2, %3, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(r)
-        : "r"((unsigned)v), "r"(1 + (int)(threadIdx.x / NT)), "r"(NT)
-        : "memory");
-    return r != 0;
-}
-
-// ---------------------------------------------------------------------------
-// per-CTA state shared by both precisions
-// ---------------------------------------------------------------------------
-struct CtaShared {
-    int blk;
-    int nseg;
-    int total;
-    int qn;
-    unsigned long long pruned;   // candidate pairs decided by group bounds
-};
-
-// Axis-aligned box of a group of points in the i-cell's FP32 frame.
-struct GBox {
-    float4 lo, hi;
-};
-constexpr int JG = 32;           // j-points per bounding-box group
-static_assert(TJ % JG == 0 && TJ / JG <= 32, "group masks are one 32-bit ballot");
-static_assert(NT % JG == 0 && (JG == 16 || JG == 32), "each warp stages whole groups");
+constexpr unsigned FULL = 0xffffffffu;
 
 // Order-preserving map of binary32 onto int32 (its own inverse): a < b as
 // floats iff fkey(a) < fkey(b) as signed integers.
@@ -140,316 +150,150 @@ __device__ __forceinline__ int fkey(float f) {
     return b ^ ((b >> 31) & 0x7fffffff);
 }
 __device__ __forceinline__ float fkey_inv(int k) { return __int_as_float(k ^ ((k >> 31) & 0x7fffffff)); }
-__device__ __forceinline__ float warp_minf(float v) {
-    return fkey_inv(__reduce_min_sync(0xffffffffu, fkey(v)));
-}
-__device__ __forceinline__ float warp_maxf(float v) {
-    return fkey_inv(__reduce_max_sync(0xffffffffu, fkey(v)));
-}
-
-// Box of the JG consecutive lanes that hold one staged j-group (lanes
-// without a point pass valid = false); every lane gets its group's box.
-__device__ __forceinline__ GBox lane_group_box(float x, float y, float z, bool valid) {
-    float lx = valid ? x : INFINITY, ly = valid ? y : INFINITY, lz = valid ? z : INFINITY;
-    float hx = valid ? x : -INFINITY, hy = valid ? y : -INFINITY, hz = valid ? z : -INFINITY;
-    if (JG == 32) {
-        lx = warp_minf(lx); ly = warp_minf(ly); lz = warp_minf(lz);
-        hx = warp_maxf(hx); hy = warp_maxf(hy); hz = warp_maxf(hz);
-    } else {
-#pragma unroll
-        for (int o = JG / 2; o > 0; o >>= 1) {   // stays inside each half-warp
-            lx = fminf(lx, __shfl_xor_sync(0xffffffffu, lx, o));
-            ly = fminf(ly, __shfl_xor_sync(0xffffffffu, ly, o));
-            lz = fminf(lz, __shfl_xor_sync(0xffffffffu, lz, o));
-            hx = fmaxf(hx, __shfl_xor_sync(0xffffffffu, hx, o));
-            hy = fmaxf(hy, __shfl_xor_sync(0xffffffffu, hy, o));
-            hz = fmaxf(hz, __shfl_xor_sync(0xffffffffu, hz, o));
-        }
-    }
-    return GBox{make_float4(lx, ly, lz, 0.f), make_float4(hx, hy, hz, 0.f)};
-}
-
-// Groups of the staged tile that may hold a pair in range of this warp's
-// i-points.  Bit g is clear only if, for every i of the warp and every j of
-// group g, the kernel's own FP32 value fl(fl(dz dz + fl(dy dy + fl(dx dx))))
-// would be >= r2cut: |fl(x_j - x_i)| >= fl(gap) per axis because rounding is
-// monotone, and the same operations on the gaps give a lower bound of s2.
-// So the skipped pairs are exactly pairs the kernel would reject one by one.
-// Group g of tile `tile` is the chunk's group g * fstride + tile; the last
-// group of the chunk may hold fewer than JG points (of `total`).
-__device__ __forceinline__ unsigned group_mask(const GBox *gb, const GBox &ib, int ngroups,
-                                               int tile, int fstride, int total, int ni,
-                                               float r2cut, unsigned long long *pruned) {
+__device__ __forceinline__ float warp_minf(float v) { return fkey_inv(__reduce_min_sync(FULL, fkey(v))); }
+__device__ __forceinline__ float warp_maxf(float v) { return fkey_inv(__reduce_max_sync(FULL, fkey(v))); }
+__device__ __forceinline__ int warp_incl_scan(int v) {
     const int lane = threadIdx.x & 31;
-    bool keep = false;
-    if (lane < ngroups) {
-        const GBox g = gb[lane];
-        const float gx = fmaxf(fmaxf(g.lo.x - ib.hi.x, ib.lo.x - g.hi.x), 0.f);
-        const float gy = fmaxf(fmaxf(g.lo.y - ib.hi.y, ib.lo.y - g.hi.y), 0.f);
-        const float gz = fmaxf(fmaxf(g.lo.z - ib.hi.z, ib.lo.z - g.hi.z), 0.f);
-        keep = fmaf(gz, gz, fmaf(gy, gy, gx * gx)) < r2cut;
-        if (!keep && ni > 0) {
-            const int first = (lane * fstride + tile) * JG;
-            atomicAdd(pruned, (unsigned long long)min(JG, total - first) * (unsigned)ni);
-        }
-    }
-    return __ballot_sync(0xffffffffu, keep);
-}
-
-// Exclusive prefix over the segment lengths held in seg[k].y (in place);
-// returns the total.  All NT threads call it.
-template <int G = 1>
-__device__ __forceinline__ int seg_scan(int4 *seg, int nseg, int *s_tmp) {
-    // each thread owns a contiguous run of ceil(nseg / NT) segments
-    const int tid = gtid();
-    const int per = (nseg + NT - 1) / NT;
-    int b0 = tid * per, b1 = min(b0 + per, nseg);
-    int local = 0;
-    for (int k = b0; k < b1; ++k) local += seg[k].y;
-    // block-wide exclusive scan of `local` (NT = 128: 4 warps)
-    int lane = tid & 31, warp = tid >> 5;
-    int v = local;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        int t = __shfl_up_sync(0xffffffffu, v, o);
+        const int t = __shfl_up_sync(FULL, v, o);
         if (lane >= o) v += t;
     }
-    if (lane == 31) s_tmp[warp] = v;
-    gsync<G>();
-    int wbase = 0;
-    for (int w = 0; w < warp; ++w) wbase += s_tmp[w];
-    int total = s_tmp[0] + s_tmp[1] + s_tmp[2] + s_tmp[3];
-    int run = wbase + v - local;
-    for (int k = b0; k < b1; ++k) {
-        int len = seg[k].y;
-        seg[k].y = run;
-        run += len;
-    }
-    gsync<G>();
-    return total;
+    return v;
 }
-
-// Segment holding flat position f: largest k with seg[k].y <= f.
-__device__ __forceinline__ int seg_find(const int4 *seg, int nseg, int f) {
-    int lo = 0, hi = nseg;
-    while (hi - lo > 1) {
-        int mid = (lo + hi) >> 1;
-        if (seg[mid].y <= f) lo = mid; else hi = mid;
-    }
-    return lo;
-}
-
-// Build the j-segments of stencil rows [r0, r1) for the i-cell (ax, ay, az).
-// seg = {first point, length, dy | dz << 16, image code}.
-__device__ __forceinline__ void build_segments(const PairParams &p, const GridDev &gj, int ax,
-                                               int ay, int az, int r0, int r1, int4 *seg,
-                                               int *s_nseg) {
-    const int nx = p.g.ng[0], ny = p.g.ng[1], nz = p.g.ng[2];
-    for (int row = r0 + gtid(); row < r1; row += NT) {
-        int4 st = p.stencil[row];
-        int dy = st.x, dz = st.y;
-        int y = ay + dy, z = az + dz, wy = 0, wz = 0;
-        if (y < 0) { if (!p.g.periodic) continue; y += ny; wy = -1; }
-        else if (y >= ny) { if (!p.g.periodic) continue; y -= ny; wy = 1; }
-        if (z < 0) { if (!p.g.periodic) continue; z += nz; wz = -1; }
-        else if (z >= nz) { if (!p.g.periodic) continue; z -= nz; wz = 1; }
-        const int rowbase = (z * ny + y) * nx;
-        const int x0 = ax + st.z, x1 = ax + st.w;
-        int pc0[3], pc1[3], pw[3], np = 0;
-        if (p.g.periodic) {
-            if (x0 < 0) { pc0[np] = x0 + nx; pc1[np] = min(x1, -1) + nx; pw[np++] = -1; }
-            int m0 = max(x0, 0), m1 = min(x1, nx - 1);
-            if (m0 <= m1) { pc0[np] = m0; pc1[np] = m1; pw[np++] = 0; }
-            if (x1 >= nx) { pc0[np] = max(x0, nx) - nx; pc1[np] = x1 - nx; pw[np++] = 1; }
-        } else {
-            int m0 = max(x0, 0), m1 = min(x1, nx - 1);
-            if (m0 <= m1) { pc0[np] = m0; pc1[np] = m1; pw[np++] = 0; }
-        }
-        const int meta = (dy & 0xFFFF) | (dz << 16);
-        for (int q = 0; q < np; ++q) {
-            int a0 = gj.cell_start[rowbase + pc0[q]];
-            int a1 = gj.cell_start[rowbase + pc1[q] + 1];
-            if (a1 > a0) {
-                int slot = atomicAdd(s_nseg, 1);
-                seg[slot] = make_int4(a0, a1 - a0, meta, (pw[q] + 1) * 9 + (wy + 1) * 3 + (wz + 1));
-            }
-        }
-    }
+__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+    return v;
 }
 
 // ---------------------------------------------------------------------------
-// rescue helpers
+// shared histogram -> global
 // ---------------------------------------------------------------------------
-template <int MODE, int LOS, bool COUNT = true>
-__device__ __noinline__ void inline_rescue(const PairParams &p, uint3 e) {
-    const int task = (int)(e.z >> 5), img = (int)(e.z & 31);
-    const TaskDev &T = p.tasks[task];
-    double4_32a a = T.gi.xw[e.x];
-    double4_32a b = T.gj.xw[e.y];
-    int bin = f64_pair_bin<MODE, LOS>(a, b, img, p.g, p.Ea, p.n_a, p.Eb, p.n_b);
-    if (bin >= 0) {
-        size_t h = (size_t)T.hist * p.nbins + bin;
-        atomicAdd(&p.hist[h], 1ull);
-        if (p.weighted) atomicAdd(&p.whist[h], __dmul_rn(a.w, b.w));
+// The counters of an entry's lane copies are read by hist_k consecutive lanes
+// and summed with shuffles; the entries (the rows' discarded columns among them,
+// the discarded row not) are dealt to warps first, first + nw, ...  A counter is
+// taken by an exchange, so a warp can flush what has been added so far while
+// others keep adding.
+__device__ __forceinline__ int hist_entries(const PairParams &p) {
+    return p.layout == LAY_ROWS ? p.n_a * p.hs : p.nbins;
+}
+__device__ __forceinline__ int hist_word(const PairParams &p, int e, int k, int &bin) {
+    bin = e;
+    if (p.layout == LAY_SKEW) {
+        const int n = e / p.n_b, w = 256 * n + (e - n * p.n_b);
+        return w + (w >> 5);
     }
-    if (COUNT) atomicAdd(&p.counters[1], 1ull);
+    if (p.layout == LAY_BYTES) return 64 * e + k;
+    if (p.hs != p.n_b) {
+        const int n = e / p.hs, m = e - n * p.hs;
+        bin = m < p.n_b ? n * p.n_b + m : -1;
+    }
+    return e * p.hist_k + k;
 }
 
-template <int MODE, int LOS>
-__device__ __forceinline__ void push_rescue(const PairParams &p, uint3 *s_q, int *s_qn, uint3 e) {
-    int slot = atomicAdd(s_qn, 1);
-    if (slot < LQ) {
-        s_q[slot] = e;
-        return;
-    }
-    unsigned long long g = atomicAdd(p.qcount, 1ull);
-    if (g < p.qcap) p.queue[g] = e;
-    else inline_rescue<MODE, LOS>(p, e);
-}
-
-// Drain the CTA's staged rescue entries to the global queue.  All threads
-// call it, after a barrier that follows their last push, so every thread
-// reads the same count.
-template <int MODE, int LOS, int G = 1>
-__device__ __forceinline__ void drain_rescue(const PairParams &p, uint3 *s_q, CtaShared &cs,
-                                             unsigned long long *s_base) {
-    int n = min(cs.qn, LQ);
-    if (n == 0) return;
-    const int tid = gtid();
-    if (tid == 0) *s_base = atomicAdd(p.qcount, (unsigned long long)n);
-    gsync<G>();
-    unsigned long long base = *s_base;
-    for (int k = tid; k < n; k += NT) {
-        unsigned long long g = base + k;
-        if (g < p.qcap) p.queue[g] = s_q[k];
-        else inline_rescue<MODE, LOS, false>(p, s_q[k]);
-    }
-    // entries past the queue were evaluated here: one counter update per drain
-    if (tid == 0 && base + n > p.qcap)
-        atomicAdd(&p.counters[1], base + n - max(base, p.qcap));
-    gsync<G>();
-    if (tid == 0) cs.qn = 0;
-    gsync<G>();
-}
-
-// Read a shared counter and clear it.  With several thread groups sharing
-// the histogram another group may be adding to it meanwhile: exchange.
-template <int G>
-__device__ __forceinline__ int take_i32(int *a) {
-    if (G == 1) {
-        const int v = *a;
-        *a = 0;
-        return v;
-    }
-    return atomicExch(a, 0);
-}
-template <int G>
-__device__ __forceinline__ unsigned long long take_u64(unsigned long long *a) {
-    if (G == 1) {
-        const unsigned long long v = *a;
-        *a = 0ull;
-        return v;
-    }
-    return atomicExch(a, 0ull);
-}
-
-// Fold mode (integer weights, one thread group): the exact sum of bin b's
-// lane-copy records as a 128-bit value (lo, hi), the records cleared; each
-// copy's sum is below 2^64.
-__device__ __forceinline__ void fold_bin(const PairParams &p, unsigned *wp, int b,
-                                         unsigned long long &lo, unsigned long long &hi) {
-    lo = 0ull;
-    hi = 0ull;
-    for (int k = 0; k < p.wint_k; ++k) {
-        unsigned *r = wp + ((size_t)b * p.wint_k + k) * 3;
-        const unsigned long long t = (unsigned long long)r[0] + ((unsigned long long)r[1] << 16) +
-                                     ((unsigned long long)r[2] << 32);
-        r[0] = r[1] = r[2] = 0u;
-        lo += t;
-        hi += lo < t ? 1ull : 0ull;
-    }
-}
-
-// Fold mode: every bin's records into this CTA's 128-bit sums in wfold_buf
-// (bin b is always handled by thread b mod NT, here and in flush_hist, so a
-// CTA's sums need no atomics); the counts stay in their copies.
-__device__ __forceinline__ void fold_records(const PairParams &p, double *s_whist) {
-    __syncthreads();
-    unsigned *wp = reinterpret_cast<unsigned *>(s_whist);
-    for (int b = threadIdx.x; b < p.nbins_smem; b += NT) {
-        unsigned long long lo, hi;
-        fold_bin(p, wp, b, lo, hi);
-        if (b < p.nbins && (lo | hi)) {
-            unsigned long long *f = p.wfold_buf + ((size_t)blockIdx.x * p.nbins + b) * 2;
-            const unsigned long long l1 = f[0] + lo;
-            f[1] += hi + (l1 < lo ? 1ull : 0ull);
-            f[0] = l1;
+static __device__ __noinline__ void flush_counts(const PairParams &p, int off, int first, int nw, int h) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int lane = threadIdx.x & 31, K = p.hist_k, words = hist_entries(p) * K;
+    int *hist = reinterpret_cast<int *>(smem + off);
+    for (int w0 = first * 32; w0 < words; w0 += nw * 32) {
+        const int idx = w0 + lane;
+        int v = 0, b = -1;
+        if (idx < words) {
+            const int word = hist_word(p, idx / K, idx & (K - 1), b);
+            v = atomicExch(&hist[word], 0);
         }
+        for (int o = 1; o < K; o <<= 1) v += __shfl_xor_sync(FULL, v, o);
+        if (b >= 0 && (lane & (K - 1)) == 0 && v)
+            atomicAdd(&p.hist[(size_t)h * p.nbins + b], (unsigned long long)(long long)v);
     }
-    __syncthreads();
 }
 
-// Add the shared histogram(s) into histogram `h` and clear them (all threads
-// of the calling group; with G > 1 each group flushes whatever has been
-// added so far, which the exchanges take exactly once).
-template <int G = 1>
-__device__ __forceinline__ void flush_hist(const PairParams &p, int *s_hist, double *s_whist,
-                                           int h, double wscale = 0.0) {
-    gsync<G>();
-    if (p.smem_hist_ok && h >= 0) {
-        // layout [warp copy][bin][lane copy]; bins past nbins form the
-        // discarded row of lin_norange and are only cleared
-        const int copies = p.priv ? NT / 32 : 1, K = p.hist_k, nbs = p.nbins_smem;
-        unsigned long long *u = reinterpret_cast<unsigned long long *>(s_whist);
-        unsigned *wp = reinterpret_cast<unsigned *>(s_whist);   // integer weight records
-        const int WK = p.wint_k;
-        for (int b = gtid(); b < nbs; b += NT) {
-            long long v = 0;
-            for (int c = 0; c < copies; ++c)
-                for (int k = 0; k < K; ++k) v += take_i32<G>(&s_hist[(c * nbs + b) * K + k]);
-            if (b >= p.nbins) {   // discarded rows (and the row of lanes without a pair)
-                if (p.weighted && p.wint) {
-                    for (int q = 0; q < 3 * WK; ++q) take_i32<G>((int *)&wp[(size_t)b * 3 * WK + q]);
-                } else if (p.weighted) {
-                    for (int k = 0; k < K; ++k) take_u64<G>(&u[b * K + k]);
-                }
-                continue;
-            }
-            if (v) atomicAdd(&p.hist[(size_t)h * p.nbins + b], (unsigned long long)v);
-            if (p.weighted) {
-                double w = 0.0;
-                if (p.wint && p.wfold) {
-                    // this CTA's exact sum: its folded 128-bit sum plus what
-                    // the records still hold, converted once
-                    unsigned long long lo, hi;
-                    fold_bin(p, wp, b, lo, hi);
-                    unsigned long long *f = p.wfold_buf + ((size_t)blockIdx.x * p.nbins + b) * 2;
-                    const unsigned long long l1 = lo + f[0];
-                    hi += f[1] + (l1 < lo ? 1ull : 0ull);
-                    lo = l1;
-                    f[0] = f[1] = 0ull;
-                    w = ((double)hi * 18446744073709551616.0 + (double)lo) * wscale;
-                } else if (p.wint) {
-                    // per lane copy: the exact sum of its products (below
-                    // 2^64) from its record of three 16-bit-piece sums
-                    for (int k = 0; k < WK; ++k) {
-                        const size_t e = ((size_t)b * WK + k) * 3;
-                        const unsigned long long lo = (unsigned)take_i32<G>((int *)&wp[e]);
-                        const unsigned long long mid = (unsigned)take_i32<G>((int *)&wp[e + 1]);
-                        const unsigned long long hi = (unsigned)take_i32<G>((int *)&wp[e + 2]);
-                        w += (double)(lo + (mid << 16) + (hi << 32));
-                    }
-                    w *= wscale;
+// Weighted sums: binary64 (wint = 0), or the exact sums of the integer
+// products' pieces, either scaled into the global histogram or (fold mode)
+// added to the CTA's exact 128-bit sums in wfold_buf.
+static __device__ __noinline__ void flush_weights(const PairParams &p, int woff, int first, int nw, int h,
+                                                  double wscale) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    unsigned char *wbase = smem + woff;
+    const int lane = threadIdx.x & 31, K = p.hist_k, words = hist_entries(p) * K;
+    for (int w0 = first * 32; w0 < words; w0 += nw * 32) {
+        const int idx = w0 + lane;
+        unsigned long long t = 0ull;
+        int b = -1;
+        if (idx < words) {
+            const int word = hist_word(p, idx / K, idx & (K - 1), b);
+            if (p.wint) {
+                unsigned *r = reinterpret_cast<unsigned *>(wbase);
+                unsigned *r0, *r1, *r2;
+                if (p.layout == LAY_BYTES) {
+                    r0 = reinterpret_cast<unsigned *>(smem) + word + 32;
+                    r1 = r + word;
+                    r2 = r1 + 32;
                 } else {
-                    // binary64 sums, exchanged as their bit patterns
-                    for (int k = 0; k < K; ++k)
-                        w += __longlong_as_double((long long)take_u64<G>(&u[b * K + k]));
+                    r0 = r + 3 * (size_t)word;
+                    r1 = r0 + 1;
+                    r2 = r0 + 2;
                 }
-                if (w != 0.0) atomicAdd(&p.whist[(size_t)h * p.nbins + b], w);
+                const unsigned long long lo = atomicExch(r0, 0u), mid = atomicExch(r1, 0u),
+                                         hi = atomicExch(r2, 0u);
+                t = lo + (mid << 16) + (hi << 32);
+            } else {
+                t = atomicExch(reinterpret_cast<unsigned long long *>(wbase) + word, 0ull);
             }
         }
+        const bool head = b >= 0 && (lane & (K - 1)) == 0;
+        if (p.wint && p.wfold) {
+            unsigned long long hi = 0ull;
+            for (int o = 1; o < K; o <<= 1) {
+                const unsigned long long l2 = __shfl_xor_sync(FULL, t, o), h2 = __shfl_xor_sync(FULL, hi, o);
+                const unsigned long long s = t + l2;
+                hi += h2 + (s < t ? 1ull : 0ull);
+                t = s;
+            }
+            if (head && (t | hi)) {
+                unsigned long long *f = p.wfold_buf + ((size_t)blockIdx.x * p.nbins + b) * 2;
+                const unsigned long long old = atomicAdd(&f[0], t);
+                if (old + t < old) ++hi;
+                if (hi) atomicAdd(&f[1], hi);
+            }
+        } else {
+            double w = p.wint ? (double)t : __longlong_as_double((long long)t);
+            for (int o = 1; o < K; o <<= 1) w += __shfl_xor_sync(FULL, w, o);
+            if (head && w != 0.0) atomicAdd(&p.whist[(size_t)h * p.nbins + b], p.wint ? w * wscale : w);
+        }
     }
-    gsync<G>();
+}
+
+// Largest counter of a LAY_ROWS histogram: with counts and weights flushed
+// together, no record of the integer weights has taken more products since
+// (but for additions in flight while they were flushed).
+static __device__ __noinline__ int most_counted(const PairParams &p) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int lane = threadIdx.x & 31, words = p.n_a * p.hs * p.hist_k, n4 = words / 4;
+    int *hist = reinterpret_cast<int *>(smem);
+    if (p.hs != p.n_b)   // the rows' discarded columns fill fastest: nobody reads them
+        for (int k = lane; k < p.n_a * p.hist_k; k += 32)
+            hist[((k / p.hist_k) * p.hs + p.n_b) * p.hist_k + (k & (p.hist_k - 1))] = 0;
+    int m = 0;
+    for (int k = lane; k < n4; k += 32) {
+        const int4 v = reinterpret_cast<const int4 *>(hist)[k];
+        m = max(max(m, max(v.x, v.y)), max(v.z, v.w));
+    }
+    if (4 * n4 + lane < words) m = max(m, hist[4 * n4 + lane]);
+    return __reduce_max_sync(FULL, m);
+}
+
+// Fold mode: the CTA's exact sums, converted once (after a barrier that
+// follows the last fold).
+__device__ __forceinline__ void flush_folded(const PairParams &p, int h, double wscale) {
+    for (int b = threadIdx.x; b < p.nbins; b += blockDim.x) {
+        unsigned long long *f = p.wfold_buf + ((size_t)blockIdx.x * p.nbins + b) * 2;
+        const unsigned long long lo = atomicExch(&f[0], 0ull), hi = atomicExch(&f[1], 0ull);
+        if (lo | hi)
+            atomicAdd(&p.whist[(size_t)h * p.nbins + b],
+                      ((double)hi * 18446744073709551616.0 + (double)lo) * wscale);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -485,7 +329,7 @@ struct BinCtx {
 };
 
 struct Bin32 {
-    int bin;     // histogram index, valid only if ok
+    int k, j;    // bin on each axis, valid only if ok
     bool ok;     // falls inside the histogram
     bool near;   // within an error band: needs the binary64 definition
 };
@@ -517,7 +361,8 @@ __device__ __forceinline__ Bin32 bin_f32(const BinCtx &c, float dx, float dy, fl
         lut_locate(c.lutA, c.invA, c.TA1, s, k, e);
         r.near = is_near(s, e, c.epsA);
         r.ok = (unsigned)k < c.nA;
-        r.bin = k;
+        r.k = k;
+        r.j = 0;
         return r;
     }
     if (LOS == LOS_Z) {
@@ -531,7 +376,8 @@ __device__ __forceinline__ Bin32 bin_f32(const BinCtx &c, float dx, float dy, fl
             float epsm = fmaf(c.muA, rs, c.muB);
             r.near = is_near(s, e, c.epsA) || is_near(mu, em, epsm) || (epsm > c.muW);
             r.ok = (unsigned)k < c.nA;
-            r.bin = k * (int)c.nB + j;
+            r.k = k;
+            r.j = j;
             return r;
         }
         // (sigma, pi) along z
@@ -542,11 +388,12 @@ __device__ __forceinline__ Bin32 bin_f32(const BinCtx &c, float dx, float dy, fl
         lut_locate(c.lutB, c.invB, c.TB1, pz, j, ep);
         r.near = is_near(sg, e, c.epsA) || is_near(pz, ep, c.epsB);
         r.ok = ((unsigned)k < c.nA) && ((unsigned)j < c.nB);
-        r.bin = k * (int)c.nB + j;
+        r.k = k;
+        r.j = j;
         return r;
     }
-    // midpoint line of sight: l = 2 x_i + d
-    float lx = fmaf(2.0f, ax_, dx), ly = fmaf(2.0f, ay_, dy), lz = fmaf(2.0f, az_, dz);
+    // midpoint line of sight: l = 2 x_i + d (ax_ holds 2 x_i)
+    float lx = ax_ + dx, ly = ay_ + dy, lz = az_ + dz;
     float sl = fmaf(dz, lz, fmaf(dy, ly, dx * lx));
     float ll = fmaf(lz, lz, fmaf(ly, ly, lx * lx));
     float rl = rsqrt_fast(ll);
@@ -561,7 +408,8 @@ __device__ __forceinline__ Bin32 bin_f32(const BinCtx &c, float dx, float dy, fl
         float epsm = fmaf(c.muA, rs, c.muB);
         r.near = is_near(s, e, c.epsA) || is_near(mu, em, epsm) || (epsm > c.muW);
         r.ok = (unsigned)k < c.nA;
-        r.bin = k * (int)c.nB + j;
+        r.k = k;
+        r.j = j;
         return r;
     }
     // sigma = |d x l| / |l|
@@ -575,36 +423,13 @@ __device__ __forceinline__ Bin32 bin_f32(const BinCtx &c, float dx, float dy, fl
     lut_locate(c.lutB, c.invB, c.TB1, pi, j, ep);
     r.near = is_near(sg, e, c.epsA) || is_near(pi, ep, c.epsB);
     r.ok = ((unsigned)k < c.nA) && ((unsigned)j < c.nB);
-    r.bin = k * (int)c.nB + j;
+    r.k = k;
+    r.j = j;
     return r;
 }
 
-// Evenly spaced s bins (and mu bins for (s, mu) along z): bin = floor of a
-// scaled value; the pair is near an edge when that value's fractional part
-// is within the band of 0 or 1.
-struct LinCtx {
-    float invA, offA, thrA;   // s scaling and band threshold
-    float mS;                 // logarithmic s: band term per 1/s
-    float invB2, thrB;        // (sigma, pi): pi scaling and band threshold
-    float nB, mA, cB;         // mu scaling and per-pair band threshold
-    unsigned nA, nB_u;
-};
-
-
-
-// Shared-memory reduction at a 32-bit shared-window address, issued only
-// when `on` is set (one predicated instruction, no branch).
-__device__ __forceinline__ void red_shared_u32_if(unsigned addr, bool on) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p red.shared.add.u32 [%0], 1;\n\t}"
-        ::"r"(addr), "r"((unsigned)on));
-}
-// Unpredicated: the whole warp issues it, lanes without a pair pointing at
-// the discarded row.  A partially predicated shared reduction measured about
-// half the throughput of a full-warp one on this GPU.
-__device__ __forceinline__ void red_shared_u32(unsigned addr, unsigned v) {
-    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(v));
-}
+// Shared-memory reductions of the weighted sums.
+//
 // The three 16-bit pieces of an integer weight product p = P >> 16 into one
 // lane copy's record {lo, mid, hi} (immediate offsets from one address),
 // taken from the 64-bit product P itself: bits 16-31, 32-47 and 48-63.
@@ -616,21 +441,19 @@ __device__ __forceinline__ void red_shared_pieces(unsigned addr, unsigned long l
         "red.shared.add.u32 [%0+8], %3;" ::"r"(addr),
         "r"(lo >> 16), "r"(hi & 0xFFFFu), "r"(hi >> 16));
 }
-// Integer weight product of a pair with binary64 remainders (W == 3), in
-// units of the task's wscale: V = round(P / 2^16 + c) with P the exact
-// product of the packed weights (hi_i hi_j = P 2^-16 wscale) and c the
-// remainder terms (hi_i lo_j + lo_i hi_j) / wscale = pf_i l_j + l_i pf_j (l
-// the scaled remainders, pf the packed weights as binary32), evaluated in
-// binary32 (|c| < 2^-23 P / 2^16 < 2^25) and rounded to an integer.  V is
-// non-negative and below 2^49; its error against the exact w_i w_j / wscale
-// is at most 1 + 2^-40 P / 2^16 units (the two roundings, the dropped
-// lo_i lo_j and the binary32 error of c).
-__device__ __forceinline__ unsigned long long corrected_product(unsigned wi, float pfi, float li,
-                                                                unsigned wj, float lj) {
-    const float c = fmaf(pfi, lj, li * __uint2float_rn(wj));
-    const long long k = (long long)__float2int_rn(c);
-    const unsigned long long P = (unsigned long long)wi * wj;
-    return ((P + 0x8000ull) >> 16) + (unsigned long long)k;
+// Integer weight product of a pair with binary64 weights (W == 3), in units of
+// the task's wscale: a weight is A + B 2^-31 in units of its grid's scale (A the
+// packed 32 bits, B the next 31), the i-point's halved: A' + B' 2^-31.  P = A' A_j
+// + 2 t, t = (A' B_j + B' A_j) 2^-32 from the products' high words, is the exact
+// product / 2 but for less than 5 (the two truncated high words, the dropped
+// B' B_j and the bit B' lost), and V = round(P 2^-15) is non-negative and at most
+// 2^48.  All integer: the binary32 remainders this replaces took a conversion
+// each way on the slow pipe.
+__device__ __forceinline__ unsigned long long corrected_product(unsigned wi, unsigned bi, unsigned wj,
+                                                                unsigned bj) {
+    const unsigned t = __umulhi(wi, bj) + __umulhi(bi, wj) + 0x2000u;   // below 2^32
+    const unsigned long long P = (unsigned long long)t * 2u + (unsigned long long)wi * wj;
+    return P >> 15;
 }
 // The three pieces of V (bits 0-15, 16-31 and 32-48) into one lane copy's
 // record, as red_shared_pieces does for P >> 16.
@@ -648,866 +471,1207 @@ __device__ __forceinline__ void red_shared_f64_if(unsigned addr, double v, bool 
         ::"r"(addr), "d"(v), "r"((unsigned)on));
 }
 
-// Rare path: stage one near-edge pair for the binary64 rescue.
-template <int MODE, int LOS>
-__device__ __noinline__ void rescue_push(const PairParams &p, uint3 *s_q, int *s_qn,
-                                         const int4 *s_seg, int nseg, int f0, int fstride, int jj,
-                                         int bstart, int i, unsigned task_bits) {
-    int jidx, img;
-    if (f0 < 0) {
-        jidx = bstart + jj;
-        img = 13;
-    } else {
-        // tile f0 holds the chunk's j-groups f0, f0 + fstride, f0 + 2 fstride, ...
-        const int f = ((jj / JG) * fstride + f0) * JG + (jj % JG);
-        int4 sg = s_seg[seg_find(s_seg, nseg, f)];
-        jidx = sg.x + (f - sg.y);
-        img = sg.w;
-    }
-    push_rescue<MODE, LOS>(p, s_q, s_qn,
-                           make_uint3((unsigned)i, (unsigned)jidx, (unsigned)img | task_bits));
-}
+// How the bins are found: lookup tables, floors (evenly spaced from 0; evenly
+// spaced from any edge; logarithmic s), or tables into the global histogram
+// when it does not fit shared memory.  PATH_FIX: the floors of PATH_LIN in
+// fixed point, for up to FIX_TOP bins an axis.
+enum { PATH_LUT = 0, PATH_LIN = 1, PATH_LINOFF = 2, PATH_LOG = 3, PATH_GLOBAL = 4, PATH_FIX = 5 };
 
-// Everything the inner loop needs, in registers.
-template <int RI>
-struct IPts {
-    float x[RI], y[RI], z[RI];     // offsets from the i-cell centre (far away if unused)
-    float xa[RI], ya[RI], za[RI];  // absolute positions (midpoint line of sight)
-    double w[RI];
-    unsigned wm[RI];               // packed integer weight (integer weight path)
-    float wl[RI], pf[RI];          // W == 3: scaled remainder, packed weight as binary32
-    int idx[RI];
+// Two pairs' outcome: byte offset of the counter in the shared histogram
+// (PATH_GLOBAL: bin, or ~0u for none), and whether the pair lies within an
+// error band of an edge.  A floor path's near pair still gets the counter of
+// its FP32 bin (or the discarded one); a table path's gets the discarded one.
+struct Pair2 {
+    unsigned a0, a1;
+    bool n0, n1;
 };
 
-// A staged tile of j-points (structure of arrays, even length, shifted into
-// the i-cell's frame).
+// Binning state of a thread (the floor paths' other constants are in the
+// kernel parameters).
+template <int MODE, int LOS, int PATH>
+struct Ctx {
+    BinCtx bc;                    // tables
+    float2 kA;                    // floor paths: counter address constant, lane copy included
+    unsigned trash;               // this thread's discarded counter
+    unsigned hk4, copy;           // bytes between counters of consecutive entries; lane copy
+
+    // cp: byte offset of this thread's lane copy
+    __device__ __forceinline__ void init(const PairParams &p, const float2 *s_lut, unsigned cp) {
+        hk4 = 4u * (unsigned)p.hist_k;
+        copy = cp;
+        trash = PATH == PATH_GLOBAL ? 0xffffffffu : hk4 * (unsigned)(p.n_a * p.hs) + cp;
+        if (PATH == PATH_LUT || PATH == PATH_GLOBAL) {
+            bc.lutA = s_lut + p.la.off;
+            bc.lutB = s_lut + p.lb.off;
+            bc.invA = p.la.inv_w;
+            bc.invB = p.lb.inv_w;
+            bc.TA1 = (unsigned)(p.la.T + 1);
+            bc.TB1 = (unsigned)(p.lb.T + 1);
+            bc.epsA = p.eps_a;
+            bc.epsB = p.eps_b;
+            bc.muA = p.mu_A;
+            bc.muB = p.mu_B;
+            bc.muW = p.mu_W;
+            bc.nA = (unsigned)p.n_a;
+            bc.nB = (unsigned)p.n_b;
+            return;
+        }
+        // address of entry (n, m): row n + col m + copy, with g_A = -(n' + 1/2),
+        // n' = n (+ 1 with an offset: t carries + 1), g_B = -(m + 1/2): FP32
+        // integers below 2^24, so every step is exact
+        kA = make_float2(p.c_kA + (float)cp, p.c_kA + (float)cp);
+    }
+};
+
+// Counter offsets from the floors: n' and m as g = -(floor + 1/2); the FP32
+// sum 2^23 + offset holds the offset in its low bits.  Offsets past the last
+// row, below the first (they wrap as unsigned) and NaN become the discarded
+// counter with one add-and-minimum.
+template <class C>
+__device__ __forceinline__ void addr2(const C &c, float2 A, Pair2 &o) {
+    o.a0 = __viaddmin_u32(__float_as_uint(A.x), 0xB5000000u, c.trash);
+    o.a1 = __viaddmin_u32(__float_as_uint(A.y), 0xB5000000u, c.trash);
+}
+
+// Bin of entry e of a LAY_ROWS histogram, -1 for a discarded one.
+__device__ __forceinline__ int entry_bin(const PairParams &p, int e) {
+    if (e >= p.n_a * p.hs) return -1;
+    const int row = e / p.hs, col = e - row * p.hs;
+    return col < p.n_b ? row * p.n_b + col : -1;
+}
+
+// Bins of two pairs (x and y lanes) from their FP32 separations.
+//
+// Floor of the first axis, t = (s - e_0) / D evaluated as s2 (rsqrt(s2) / D):
+// adding 2^23 rounded down leaves floor(t) in the low bits; g = -(floor + 1/2)
+// and d = t + g = frac(t) - 1/2 in one fused step, and the pair is near an
+// edge unless |d| < 1/2 - band.  With an offset (first edge above zero, and
+// logarithmic s) t carries + 1: below 2^23 the FP32 spacing is 1/2, so floors
+// are exact only for t >= 0, and everything below -1 is out of range whatever
+// its floor.  NaN (s2 = 0) compares false: near.
+template <int MODE, int LOS, int PATH>
+__device__ __forceinline__ Pair2 bin2(const PairParams &p, const Ctx<MODE, LOS, PATH> &c, float2 dx, float2 dy, float2 dz,
+                                      float2 q, float2 s2, float xa, float ya, float za) {
+    Pair2 o;
+    if (PATH == PATH_LUT || PATH == PATH_GLOBAL) {
+        const Bin32 b0 = bin_f32<MODE, LOS>(c.bc, dx.x, dy.x, dz.x, q.x, s2.x, xa, ya, za);
+        const Bin32 b1 = bin_f32<MODE, LOS>(c.bc, dx.y, dy.y, dz.y, q.y, s2.y, xa, ya, za);
+        const bool in0 = s2.x < p.r2cut, in1 = s2.y < p.r2cut;
+        o.n0 = in0 && b0.near;
+        o.n1 = in1 && b1.near;
+        const bool u0 = in0 && b0.ok && !b0.near, u1 = in1 && b1.ok && !b1.near;
+        if (PATH == PATH_GLOBAL) {
+            o.a0 = u0 ? (unsigned)(b0.k * (int)c.bc.nB + b0.j) : c.trash;
+            o.a1 = u1 ? (unsigned)(b1.k * (int)c.bc.nB + b1.j) : c.trash;
+        } else {
+            o.a0 = u0 ? c.hk4 * (unsigned)(b0.k * p.hs + b0.j) + c.copy : c.trash;
+            o.a1 = u1 ? c.hk4 * (unsigned)(b1.k * p.hs + b1.j) + c.copy : c.trash;
+        }
+        return o;
+    }
+    const float2 C23 = p.c_23, CP = p.c_p, M1 = p.c_m1;
+    // line-of-sight components (midpoint: l = 2 x_i + d; xa holds 2 x_i)
+    float2 pz, rl, lx, ly, lz;
+    if (LOS == LOS_MID && MODE != MODE_S) {
+        lx = __fadd2_rn(make_float2(xa, xa), dx);
+        ly = __fadd2_rn(make_float2(ya, ya), dy);
+        lz = __fadd2_rn(make_float2(za, za), dz);
+        const float2 sl = __ffma2_rn(dz, lz, __ffma2_rn(dy, ly, __fmul2_rn(dx, lx)));
+        const float2 ll = __ffma2_rn(lz, lz, __ffma2_rn(ly, ly, __fmul2_rn(lx, lx)));
+        rl = make_float2(rsqrt_fast(ll.x), rsqrt_fast(ll.y));
+        pz = make_float2(fabsf(sl.x), fabsf(sl.y));
+    } else if (MODE != MODE_S) {
+        pz = make_float2(fabsf(dz.x), fabsf(dz.y));
+    }
+    if (MODE == MODE_SIGPI) {
+        // sigma = q rsqrt(q) along z, |d x l| / |l| along the midpoint
+        float2 v, rv;
+        if (LOS == LOS_Z) {
+            v = q;
+            rv = __fmul2_rn(make_float2(rsqrt_fast(q.x), rsqrt_fast(q.y)), p.c_invA);
+        } else {
+            const float2 ndx = __fmul2_rn(dx, M1), ndy = __fmul2_rn(dy, M1), ndz = __fmul2_rn(dz, M1);
+            const float2 cx = __ffma2_rn(dy, lz, __fmul2_rn(ndz, ly));
+            const float2 cy = __ffma2_rn(dz, lx, __fmul2_rn(ndx, lz));
+            const float2 cz = __ffma2_rn(dx, ly, __fmul2_rn(ndy, lx));
+            v = __ffma2_rn(cz, cz, __ffma2_rn(cy, cy, __fmul2_rn(cx, cx)));
+            const float2 rla = __fmul2_rn(rl, p.c_invA);
+            rv = __fmul2_rn(make_float2(rsqrt_fast(v.x), rsqrt_fast(v.y)), rla);
+        }
+        const float2 rp = LOS == LOS_Z ? p.c_invB : __fmul2_rn(rl, p.c_invB);
+        const float2 fa = __ffma2_rd(v, rv, C23), fb = __ffma2_rd(pz, rp, C23);
+        const float2 ga = __ffma2_rn(fa, M1, CP), gb = __ffma2_rn(fb, M1, CP);
+        const float2 da = __ffma2_rn(v, rv, ga), db = __ffma2_rn(pz, rp, gb);
+        o.n0 = !(fabsf(da.x) < p.c_thrA.x) | !(fabsf(db.x) < p.c_cB.x);
+        o.n1 = !(fabsf(da.y) < p.c_thrA.y) | !(fabsf(db.y) < p.c_cB.y);
+        // pi past its last bin: the discarded column n_b of the row (pi may
+        // exceed pi_max while s is still below sqrt(sigma_max^2 + pi_max^2))
+        const float lim = 0.5f - (float)p.hs;
+        const float2 gc = make_float2(fmaxf(gb.x, lim), fmaxf(gb.y, lim));
+        addr2(c, __ffma2_rn(gc, p.c_ncol, __ffma2_rn(ga, p.c_nrow, c.kA)), o);
+        return o;
+    }
+    const float2 rs = make_float2(rsqrt_fast(s2.x), rsqrt_fast(s2.y));
+    float2 ga, da;
+    if (PATH == PATH_LIN) {
+        const float2 ra = __fmul2_rn(rs, p.c_invA);
+        const float2 f = __ffma2_rd(s2, ra, C23);
+        ga = __ffma2_rn(f, M1, CP);
+        da = __ffma2_rn(s2, ra, ga);
+    } else {
+        const float2 ts = PATH == PATH_LOG
+                              ? __ffma2_rn(make_float2(lg2_fast(s2.x), lg2_fast(s2.y)), p.c_invA, p.c_offA)
+                              : __ffma2_rn(s2, __fmul2_rn(rs, p.c_invA), p.c_offA);
+        const float2 f = __fadd2_rd(ts, C23);
+        ga = __ffma2_rn(f, M1, CP);
+        da = __fadd2_rn(ts, ga);
+    }
+    const float2 th = PATH == PATH_LOG ? __ffma2_rn(p.c_nmS, rs, p.c_thrA) : p.c_thrA;
+    o.n0 = !(fabsf(da.x) < th.x);
+    o.n1 = !(fabsf(da.y) < th.y);
+    float2 A = __ffma2_rn(ga, p.c_nrow, c.kA);
+    if (MODE == MODE_SMU) {
+        // t_mu = mu n_mu, scaled just below n_mu: mu = 1 is in the last bin
+        const float2 rm = LOS == LOS_Z ? __fmul2_rn(rs, p.c_invB) : __fmul2_rn(__fmul2_rn(rl, rs), p.c_invB);
+        const float2 f = __ffma2_rd(pz, rm, C23);
+        const float2 gm = __ffma2_rn(f, M1, CP);
+        const float2 dm = __ffma2_rn(pz, rm, gm);
+        const float2 tm = __ffma2_rn(p.c_nmB, rs, p.c_cB);
+        o.n0 = o.n0 | !(fabsf(dm.x) < tm.x);
+        o.n1 = o.n1 | !(fabsf(dm.y) < tm.y);
+        A = __ffma2_rn(gm, p.c_ncol, A);
+    }
+    addr2(c, A, o);
+    return o;
+}
+
+// A warp's i-points: lane l holds the block's points 2 l and 2 l + 1.
+template <int LOS, int W>
+struct IPts {
+    float x[2], y[2], z[2];        // offsets from the i-cell centre (far away if unused)
+    float xa[2], ya[2], za[2];     // twice the absolute positions (midpoint line of sight)
+    double w[2];                   // W == 1
+    unsigned wm[2];                // W >= 2: packed integer weight
+    unsigned wb[2];                // W == 3: wm halved and the next 31 bits
+};
+
+// One i-point's registers from its record (the midpoint sums start from 2 x_i:
+// doubling is exact, so 2 x_i + d rounds once, as a fused multiply-add would).
+template <int MODE, int LOS, int W>
+__device__ __forceinline__ void load_i(const GridDev &g, int i, IPts<LOS, W> &I, int r) {
+    const float4 q = g.rel[i];
+    I.x[r] = q.x; I.y[r] = q.y; I.z[r] = q.z;
+    if (W >= 2) I.wm[r] = __float_as_uint(q.w);
+    if (W == 3) {
+        const unsigned B = g.wlo ? g.wlo[i] : 0u;
+        I.wb[r] = (I.wm[r] & 1u) << 30 | B >> 1;
+        I.wm[r] >>= 1;
+    }
+    if ((LOS == LOS_MID && MODE != MODE_S) || W == 1) {
+        const double4_32a a = g.xw[i];
+        I.xa[r] = 2.0f * (float)a.x; I.ya[r] = 2.0f * (float)a.y; I.za[r] = 2.0f * (float)a.z;
+        if (W == 1) I.w[r] = a.w;
+    }
+}
+
+// A j-point in the i-cell's frame: grid, rel_j + delta c (delta the offset of
+// the cells, periodic image included); tree, rel_j + o (o the offset of the
+// two node centres).
+__device__ __forceinline__ float3 stage_grid(const PairParams &p, float4 q, int cx, int ax, int meta, int img) {
+    const int dxc = cx - ax + (img / 9 - 1) * p.g.ng[0];
+    const int dyc = (int)(short)(meta & 0xFFFF), dzc = meta >> 16;
+    return make_float3(fmaf((float)dxc, p.g.c32[0], q.x), fmaf((float)dyc, p.g.c32[1], q.y),
+                       fmaf((float)dzc, p.g.c32[2], q.z));
+}
+__device__ __forceinline__ float4 tree_offset(const PairParams &p, int inode, int jnode, int img) {
+    const double *ci = p.tcen_i + 3 * (size_t)inode, *cj = p.tcen_j + 3 * (size_t)jnode;
+    const double sx = (double)(img / 9 - 1), sy = (double)((img / 3) % 3 - 1), sz = (double)(img % 3 - 1);
+    return make_float4(__double2float_rn(__dsub_rn(__dadd_rn(cj[0], __dmul_rn(sx, p.g.L[0])), ci[0])),
+                       __double2float_rn(__dsub_rn(__dadd_rn(cj[1], __dmul_rn(sy, p.g.L[1])), ci[1])),
+                       __double2float_rn(__dsub_rn(__dadd_rn(cj[2], __dmul_rn(sz, p.g.L[2])), ci[2])), 0.f);
+}
+
+// The staged batch of JB j-points in a warp's slice.
 struct Tile {
     const float *x, *y, *z;
-    const double *w;               // binary64 weights (W == 1)
-    const unsigned *wm;            // packed integer weights (W >= 2), same storage
-    const float *wl;               // scaled binary64 remainders (W == 3), after wm
+    const double *w;               // W == 1
+    const unsigned *wm;            // W >= 2 (same storage)
+    const unsigned *wl;            // W == 3: the next 31 bits, after wm
 };
 
-// Table-based bins, one pair at a time (every mode and line of sight).
-// MASK: the tile holds the block's own points and only pairs j > i count.
-template <int MODE, int LOS, int W, int RI, bool MASK>
-__device__ __forceinline__ void pair_tile_lut(const PairParams &p, Tile tb, int len, unsigned gmask,
-                                              const IPts<RI> &I, const BinCtx &bc, float r2cut,
-                                              unsigned hist_sa, unsigned whist_sa, unsigned hk4,
-                                              uint3 *s_q, int *s_qn, const int4 *s_seg, int nseg,
-                                              int f0, int fstride, int bstart, unsigned task_bits) {
+// All pairs of the warp's i-points with nq quads of staged j-points: per
+// iteration four j-points x two i-points a lane, in packed FP32, every
+// counter updated by the full warp (pairs outside the histogram go to the
+// discarded counter).  Returns a bit per quad: some pair of this lane is near
+// an edge.  MASK: the tile holds points jbase, jbase + 1, ... of the i-block
+// itself and only pairs j > i count.
+template <int MODE, int LOS, int W, int PATH, bool MASK>
+__device__ __forceinline__ unsigned pair_quads(const PairParams &p, const Tile &t, int nq,
+                                               const IPts<LOS, W> &I, const Ctx<MODE, LOS, PATH> &c,
+                                               unsigned char *hist, unsigned wbase, int jbase,
+                                               size_t hbase) {
+    const int lane = threadIdx.x & 31;
+    unsigned near = 0u;
 #pragma unroll 1
-    for (unsigned gm = gmask; gm; gm &= gm - 1) {
-    const int j0 = (__ffs(gm) - 1) * JG, j1 = min(j0 + JG, len);
-#pragma unroll 2
-    for (int jj = j0; jj < j1; ++jj) {
-        const float qx = tb.x[jj], qy = tb.y[jj], qz = tb.z[jj];
-        float dxv[RI], dyv[RI], dzv[RI], qv[RI], s2v[RI];
-        bool inr[RI];
+    for (int q = 0; q < nq; ++q) {
+        const float4 X = reinterpret_cast<const float4 *>(t.x)[q];
+        const float4 Y = reinterpret_cast<const float4 *>(t.y)[q];
+        const float4 Z = reinterpret_cast<const float4 *>(t.z)[q];
         bool any = false;
 #pragma unroll
-        for (int r = 0; r < RI; ++r) {
-            dxv[r] = qx - I.x[r];
-            dyv[r] = qy - I.y[r];
-            dzv[r] = qz - I.z[r];
-            qv[r] = fmaf(dyv[r], dyv[r], dxv[r] * dxv[r]);
-            s2v[r] = fmaf(dzv[r], dzv[r], qv[r]);
-            inr[r] = s2v[r] < r2cut;
-            if (MASK) inr[r] = inr[r] && (bstart + jj > I.idx[r]);
-            any = any || inr[r];
-        }
-        if (__any_sync(0xffffffffu, any)) {
-            double wj = 0.0;
-            if (W == 1) wj = tb.w[jj];
-            bool resc[RI];
-            bool anyr = false;
+        for (int h = 0; h < 2; ++h) {
+            const float2 Xh = h ? make_float2(X.z, X.w) : make_float2(X.x, X.y);
+            const float2 Yh = h ? make_float2(Y.z, Y.w) : make_float2(Y.x, Y.y);
+            const float2 Zh = h ? make_float2(Z.z, Z.w) : make_float2(Z.x, Z.y);
 #pragma unroll
-            for (int r = 0; r < RI; ++r) {
-                Bin32 b = bin_f32<MODE, LOS>(bc, dxv[r], dyv[r], dzv[r], qv[r], s2v[r], I.xa[r],
-                                             I.ya[r], I.za[r]);
-                const bool add = inr[r] && b.ok && !b.near;
-                red_shared_u32_if(hist_sa + hk4 * (unsigned)b.bin, add);
-                if (W == 1) red_shared_f64_if(whist_sa + 2u * hk4 * (unsigned)b.bin, __dmul_rn(I.w[r], wj), add);
-                resc[r] = inr[r] && b.near;
-                anyr = anyr || resc[r];
-            }
-            if (__any_sync(0xffffffffu, anyr)) {
-#pragma unroll
-                for (int r = 0; r < RI; ++r)
-                    if (resc[r])
-                        rescue_push<MODE, LOS>(p, s_q, s_qn, s_seg, nseg, f0, fstride, jj, bstart, I.idx[r],
-                                               task_bits);
-            }
-        }
-    }
-    }
-}
-
-// Evenly spaced bins, two j-points per step in packed FP32 (s, and (s, mu)
-// along z).  For each pair: t_s = (s - e0) / D, bin = floor(t_s); the pair
-// is near an edge unless |frac(t_s) - 1/2| < thrA; mu likewise with its
-// per-pair band.  Histogram addresses are formed from the float bits of
-// floor(t) + 2^23, with the 2^23 bias folded into the base address.
-template <int MODE, int W, int RI, bool MASK, bool CHK, bool LOGS>
-__device__ __forceinline__ void pair_tile_lin2(const PairParams &p, Tile tb, int len, unsigned gmask,
-                                               const IPts<RI> &I, const LinCtx &lc, float r2cut,
-                                               unsigned hist_sa, unsigned whist_sa, unsigned hk4,
-                                               uint3 *s_q, int *s_qn, const int4 *s_seg, int nseg,
-                                               int f0, int fstride, int bstart, unsigned task_bits) {
-    const float2 C23 = make_float2(8388608.0f, 8388608.0f);
-    const float2 NC23H = make_float2(-8388608.0f + 0.5f, -8388608.0f + 0.5f);
-    const float2 M1 = make_float2(-1.0f, -1.0f);
-    const float2 INVA = make_float2(lc.invA, lc.invA);
-    const float2 OFFA = make_float2(lc.offA, lc.offA);
-    const float2 NB = make_float2(lc.nB, lc.nB);
-    const float2 NMA = make_float2(-lc.mA, -lc.mA);
-    const float2 CB = make_float2(lc.cB, lc.cB);
-    // With the range test (CHK) the offset carries +1 (host side): t_s + 1 >= 0
-    // for every t_s >= -1, where adding 2^23 and rounding down is an exact
-    // floor (below 2^23 the float spacing is 1/2); values below -1 are out of
-    // range whatever their floor.  The extra row is removed in the base.
-    const float halfA = 0.5f * (float)lc.nA;
-    const float hA1 = CHK ? halfA + 1.0f : halfA;
-    const float2 NHALFA = make_float2(-hA1, -hA1);
-    const float thrA = lc.thrA;
-    const float2 THRA = make_float2(lc.thrA, lc.thrA);
-    const float2 NMS = make_float2(-lc.mS, -lc.mS);
-    const unsigned nbu = (MODE == MODE_SMU) ? lc.nB_u : 1u;
-    // biases of the float bits of floor(t_s) + 2^23 (and floor(t_mu) + 2^23),
-    // folded into the bases
-    const unsigned bias = 0x4B000000u * nbu + ((MODE == MODE_SMU) ? 0x4B000000u : 0u) +
-                          (CHK ? nbu : 0u);
-    const unsigned hbase = hist_sa - hk4 * bias;
-    const unsigned htrash = hist_sa + hk4 * (unsigned)p.trash_row;
-    const unsigned wbase = whist_sa - 2u * hk4 * bias;
-    // integer weights: a 12-byte record {lo, mid, hi} per bin and lane copy
-    // (word 3 (bin copies + copy) + piece: bank 3 copy + piece, conflict-free),
-    // as many copies as the counts, so a record's address is 3 x the count's
-    // address + wdelta (the discarded row included)
-    const unsigned wdelta = whist_sa - 3u * hist_sa;
-    float2 NX[RI], NY[RI], NZ[RI];
-#pragma unroll
-    for (int r = 0; r < RI; ++r) {
-        NX[r] = make_float2(-I.x[r], -I.x[r]);
-        NY[r] = make_float2(-I.y[r], -I.y[r]);
-        NZ[r] = make_float2(-I.z[r], -I.z[r]);
-    }
-#pragma unroll 1
-    for (unsigned gm = gmask; gm; gm &= gm - 1) {
-    const int j0 = (__ffs(gm) - 1) * JG, j1 = min(j0 + JG, len);
-#pragma unroll 4
-    for (int jj = j0; jj < j1; jj += 2) {
-        const float2 X = *reinterpret_cast<const float2 *>(tb.x + jj);
-        const float2 Y = *reinterpret_cast<const float2 *>(tb.y + jj);
-        const float2 Z = *reinterpret_cast<const float2 *>(tb.z + jj);
-        float2 S2[RI], DZ[RI];
-        bool in0[RI], in1[RI];
-        bool any = false;
-#pragma unroll
-        for (int r = 0; r < RI; ++r) {
-            const float2 dx = __fadd2_rn(X, NX[r]);
-            const float2 dy = __fadd2_rn(Y, NY[r]);
-            DZ[r] = __fadd2_rn(Z, NZ[r]);
-            S2[r] = __ffma2_rn(DZ[r], DZ[r], __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
-            in0[r] = S2[r].x < r2cut;
-            in1[r] = S2[r].y < r2cut;
-            if (MASK) {
-                in0[r] = in0[r] && (bstart + jj > I.idx[r]);
-                in1[r] = in1[r] && (bstart + jj + 1 > I.idx[r]);
-            }
-            any = any || in0[r] || in1[r];
-        }
-        if (__any_sync(0xffffffffu, any)) {
-            bool re0[RI], re1[RI];
-            bool anyr = false;
-#pragma unroll
-            for (int r = 0; r < RI; ++r) {
-                const float2 s2 = S2[r];
-                const float2 rs = make_float2(rsqrt_fast(s2.x), rsqrt_fast(s2.y));
-                // t_s = (s - e0) / D, or log_q(s / e0) = A log2(s^2) + B
-                const float2 ts =
-                    LOGS ? __ffma2_rn(make_float2(lg2_fast(s2.x), lg2_fast(s2.y)), INVA, OFFA)
-                         : __ffma2_rn(__fmul2_rn(s2, rs), INVA, OFFA);
-                const float2 f = __fadd2_rd(ts, C23);
-                const float2 d = __ffma2_rn(__fadd2_rn(f, NC23H), M1, ts);   // frac - 1/2
-                bool ok0 = true, ok1 = true;
-                if (CHK) {
-                    const float2 o = __fadd2_rn(ts, NHALFA);
-                    ok0 = fabsf(o.x) < halfA;
-                    ok1 = fabsf(o.y) < halfA;
+            for (int r = 0; r < 2; ++r) {
+                float2 dx = __fadd2_rn(Xh, make_float2(-I.x[r], -I.x[r]));
+                const float2 dy = __fadd2_rn(Yh, make_float2(-I.y[r], -I.y[r]));
+                const float2 dz = __fadd2_rn(Zh, make_float2(-I.z[r], -I.z[r]));
+                if (MASK) {   // masked pairs: far out of range
+                    const int jj = jbase + 4 * q + 2 * h;
+                    if (jj <= 2 * lane + r) dx.x = p.far;
+                    if (jj + 1 <= 2 * lane + r) dx.y = p.far;
                 }
-                // NaN (s2 = 0) compares false: such pairs are near.  Log edges:
-                // the band grows as 1/s
-                const float2 ths = LOGS ? __ffma2_rn(NMS, rs, THRA) : THRA;
-                bool n0 = !(fabsf(d.x) < ths.x), n1 = !(fabsf(d.y) < ths.y);
-                unsigned b0 = (unsigned)__float_as_int(f.x), b1 = (unsigned)__float_as_int(f.y);
-                if (MODE == MODE_SMU) {
-                    const float2 adz = make_float2(fabsf(DZ[r].x), fabsf(DZ[r].y));
-                    const float2 tm = __fmul2_rn(adz, __fmul2_rn(rs, NB));
-                    const float2 fm = __fadd2_rd(tm, C23);
-                    const float2 dm = __ffma2_rn(__fadd2_rn(fm, NC23H), M1, tm);
-                    const float2 thm = __ffma2_rn(NMA, rs, CB);
-                    n0 = n0 || !(fabsf(dm.x) < thm.x);
-                    n1 = n1 || !(fabsf(dm.y) < thm.y);
-                    // t_mu < n_mu (scale below n_mu): mu = 1 is in the last bin;
-                    // a NaN index is never used (such pairs are near)
-                    const unsigned j0 = (unsigned)__float_as_int(fm.x);
-                    const unsigned j1 = (unsigned)__float_as_int(fm.y);
-                    b0 = b0 * nbu + j0;
-                    b1 = b1 * nbu + j1;
+                const float2 qq = __ffma2_rn(dy, dy, __fmul2_rn(dx, dx));
+                const float2 s2 = __ffma2_rn(dz, dz, qq);
+                const Pair2 b = bin2<MODE, LOS, PATH>(p, c, dx, dy, dz, qq, s2, I.xa[r], I.ya[r], I.za[r]);
+                any = any | b.n0 | b.n1;
+                if (PATH == PATH_GLOBAL) {
+                    if (b.a0 != c.trash) atomicAdd(p.hist + hbase + b.a0, 1ull);
+                    if (b.a1 != c.trash) atomicAdd(p.hist + hbase + b.a1, 1ull);
+                    if (W == 1) {
+                        if (b.a0 != c.trash)
+                            atomicAdd(p.whist + hbase + b.a0, __dmul_rn(I.w[r], t.w[4 * q + 2 * h]));
+                        if (b.a1 != c.trash)
+                            atomicAdd(p.whist + hbase + b.a1, __dmul_rn(I.w[r], t.w[4 * q + 2 * h + 1]));
+                    }
+                    continue;
                 }
-                const bool a0 = in0[r] && ok0 && !n0, a1 = in1[r] && ok1 && !n1;
-                const unsigned c0 = a0 ? hbase + hk4 * b0 : htrash;
-                const unsigned c1 = a1 ? hbase + hk4 * b1 : htrash;
-                red_shared_u32(c0, 1u);
-                red_shared_u32(c1, 1u);
-                if (W == 1) {
-                    const double2 wj = *reinterpret_cast<const double2 *>(tb.w + jj);
-                    red_shared_f64_if(wbase + 2u * hk4 * b0, __dmul_rn(I.w[r], wj.x), a0);
-                    red_shared_f64_if(wbase + 2u * hk4 * b1, __dmul_rn(I.w[r], wj.y), a1);
+                atomicAdd(reinterpret_cast<unsigned *>(hist + b.a0), 1u);
+                atomicAdd(reinterpret_cast<unsigned *>(hist + b.a1), 1u);
+                if (W == 1) {   // near pairs are added by their binary64 check
+                    const double2 wj = *reinterpret_cast<const double2 *>(t.w + 4 * q + 2 * h);
+                    red_shared_f64_if(wbase + 2u * b.a0, __dmul_rn(I.w[r], wj.x), b.a0 < c.trash && !b.n0);
+                    red_shared_f64_if(wbase + 2u * b.a1, __dmul_rn(I.w[r], wj.y), b.a1 < c.trash && !b.n1);
                 } else if (W == 2) {
                     // (M_i M_j) >> (k_i + k_j), k = emax - e the exponent offset:
                     // the packed M 2^(8 - k) multiplied exactly in 64 bits is
                     // P = M_i M_j 2^(16 - k_i - k_j), and the product is P >> 16
-                    // (truncation < 2^(k_i + k_j - 46) relative, below 2^48),
-                    // added as three 16-bit pieces to the lane copy's record
-                    const uint2 wj = *reinterpret_cast<const uint2 *>(tb.wm + jj);
-                    red_shared_pieces(3u * c0 + wdelta, (unsigned long long)I.wm[r] * wj.x);
-                    red_shared_pieces(3u * c1 + wdelta, (unsigned long long)I.wm[r] * wj.y);
+                    // (truncation < 2^(k_i + k_j - 46) relative, below 2^48).  A
+                    // record is 12 bytes and has the count's place among them
+                    const uint2 wj = *reinterpret_cast<const uint2 *>(t.wm + 4 * q + 2 * h);
+                    red_shared_pieces(wbase + 3u * b.a0, (unsigned long long)I.wm[r] * wj.x);
+                    red_shared_pieces(wbase + 3u * b.a1, (unsigned long long)I.wm[r] * wj.y);
                 } else if (W == 3) {
-                    // the same product with the binary64 remainders' terms
-                    const uint2 wj = *reinterpret_cast<const uint2 *>(tb.wm + jj);
-                    const float2 lj = *reinterpret_cast<const float2 *>(tb.wl + jj);
-                    red_shared_pieces_v(3u * c0 + wdelta,
-                                        corrected_product(I.wm[r], I.pf[r], I.wl[r], wj.x, lj.x));
-                    red_shared_pieces_v(3u * c1 + wdelta,
-                                        corrected_product(I.wm[r], I.pf[r], I.wl[r], wj.y, lj.y));
-                }
-                re0[r] = in0[r] && n0;
-                re1[r] = in1[r] && n1;
-                anyr = anyr || re0[r] || re1[r];
-            }
-            if (__any_sync(0xffffffffu, anyr)) {
-#pragma unroll
-                for (int r = 0; r < RI; ++r) {
-                    if (re0[r])
-                        rescue_push<MODE, LOS_Z>(p, s_q, s_qn, s_seg, nseg, f0, fstride, jj, bstart,
-                                                 I.idx[r], task_bits);
-                    if (re1[r])
-                        rescue_push<MODE, LOS_Z>(p, s_q, s_qn, s_seg, nseg, f0, fstride, jj + 1, bstart,
-                                                 I.idx[r], task_bits);
+                    const uint2 wj = *reinterpret_cast<const uint2 *>(t.wm + 4 * q + 2 * h);
+                    const uint2 lj = *reinterpret_cast<const uint2 *>(t.wl + 4 * q + 2 * h);
+                    red_shared_pieces_v(wbase + 3u * b.a0,
+                                        corrected_product(I.wm[r], I.wb[r], wj.x, lj.x));
+                    red_shared_pieces_v(wbase + 3u * b.a1,
+                                        corrected_product(I.wm[r], I.wb[r], wj.y, lj.y));
                 }
             }
         }
+        near |= (any ? 1u : 0u) << q;
     }
-    }
+    return near;
 }
 
-// (sigma, pi) bins, both axes evenly spaced from 0, two j-points per step in
-// packed FP32.  sigma and pi are formed exactly as in the table path (so the
-// same bands apply): along z, sigma = q rsqrt(q) with q = dx^2 + dy^2 and
-// pi = |dz|; for the midpoint line of sight l = 2 x_i + d, pi = |d.l| / |l|
-// and sigma = |d x l| / |l|.  Both indices are floors on the 2^23 grid; the
-// pair counts only if both lie below their axis' bin count (pi may exceed
-// pi_max while s is still below the reach sqrt(sigma_max^2 + pi_max^2)).
-template <int LOS, int W, int RI, bool MASK>
-__device__ __forceinline__ void pair_tile_sigpi2(const PairParams &p, Tile tb, int len, unsigned gmask,
-                                                 const IPts<RI> &I, const LinCtx &lc, float r2cut,
-                                                 unsigned hist_sa, unsigned whist_sa, unsigned hk4,
-                                                 uint3 *s_q, int *s_qn, const int4 *s_seg, int nseg,
-                                                 int f0, int fstride, int bstart,
-                                                 unsigned task_bits) {
-    const float2 C23 = make_float2(8388608.0f, 8388608.0f);
-    const float2 NC23H = make_float2(-8388608.0f + 0.5f, -8388608.0f + 0.5f);
-    const float2 M1 = make_float2(-1.0f, -1.0f);
-    const float2 TWO = make_float2(2.0f, 2.0f);
-    const float2 INVA = make_float2(lc.invA, lc.invA);
-    const float2 INVB = make_float2(lc.invB2, lc.invB2);
-    const float thrA = lc.thrA, thrB = lc.thrB;
-    const unsigned nbu = lc.nB_u;
-    const unsigned limA = 0x4B000000u + lc.nA, limB = 0x4B000000u + lc.nB_u;
-    const unsigned bias = 0x4B000000u * nbu + 0x4B000000u;
-    const unsigned hbase = hist_sa - hk4 * bias;
-    const unsigned htrash = hist_sa + hk4 * (unsigned)p.trash_row;
-    const unsigned wbase = whist_sa - 2u * hk4 * bias;
-    const unsigned wdelta = whist_sa - 3u * hist_sa;   // as in the floor-bin loop above
-    float2 NX[RI], NY[RI], NZ[RI];
-#pragma unroll
-    for (int r = 0; r < RI; ++r) {
-        NX[r] = make_float2(-I.x[r], -I.x[r]);
-        NY[r] = make_float2(-I.y[r], -I.y[r]);
-        NZ[r] = make_float2(-I.z[r], -I.z[r]);
-    }
-#pragma unroll 1
-    for (unsigned gm = gmask; gm; gm &= gm - 1) {
-    const int j0 = (__ffs(gm) - 1) * JG, j1 = min(j0 + JG, len);
-#pragma unroll 2
-    for (int jj = j0; jj < j1; jj += 2) {
-        const float2 X = *reinterpret_cast<const float2 *>(tb.x + jj);
-        const float2 Y = *reinterpret_cast<const float2 *>(tb.y + jj);
-        const float2 Z = *reinterpret_cast<const float2 *>(tb.z + jj);
-        float2 S2[RI];
-        bool in0[RI], in1[RI];
-        bool any = false;
-#pragma unroll
-        for (int r = 0; r < RI; ++r) {
-            const float2 dx = __fadd2_rn(X, NX[r]);
-            const float2 dy = __fadd2_rn(Y, NY[r]);
-            const float2 dz = __fadd2_rn(Z, NZ[r]);
-            S2[r] = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
-            in0[r] = S2[r].x < r2cut;
-            in1[r] = S2[r].y < r2cut;
-            if (MASK) {
-                in0[r] = in0[r] && (bstart + jj > I.idx[r]);
-                in1[r] = in1[r] && (bstart + jj + 1 > I.idx[r]);
-            }
-            any = any || in0[r] || in1[r];
-        }
-        if (__any_sync(0xffffffffu, any)) {
-            bool re0[RI], re1[RI];
-            bool anyr = false;
-#pragma unroll
-            for (int r = 0; r < RI; ++r) {
-                const float2 dx = __fadd2_rn(X, NX[r]);
-                const float2 dy = __fadd2_rn(Y, NY[r]);
-                const float2 dz = __fadd2_rn(Z, NZ[r]);
-                float2 sg, pz;
-                if (LOS == LOS_Z) {
-                    const float2 q = __ffma2_rn(dy, dy, __fmul2_rn(dx, dx));
-                    sg = __fmul2_rn(q, make_float2(rsqrt_fast(q.x), rsqrt_fast(q.y)));
-                    pz = make_float2(fabsf(dz.x), fabsf(dz.y));
-                } else {
-                    const float2 lx = __ffma2_rn(TWO, make_float2(I.xa[r], I.xa[r]), dx);
-                    const float2 ly = __ffma2_rn(TWO, make_float2(I.ya[r], I.ya[r]), dy);
-                    const float2 lz = __ffma2_rn(TWO, make_float2(I.za[r], I.za[r]), dz);
-                    const float2 sl = __ffma2_rn(dz, lz, __ffma2_rn(dy, ly, __fmul2_rn(dx, lx)));
-                    const float2 ll = __ffma2_rn(lz, lz, __ffma2_rn(ly, ly, __fmul2_rn(lx, lx)));
-                    const float2 rl = make_float2(rsqrt_fast(ll.x), rsqrt_fast(ll.y));
-                    pz = __fmul2_rn(make_float2(fabsf(sl.x), fabsf(sl.y)), rl);
-                    const float2 ndx = make_float2(-dx.x, -dx.y), ndy = make_float2(-dy.x, -dy.y),
-                                 ndz = make_float2(-dz.x, -dz.y);
-                    const float2 cx = __ffma2_rn(dy, lz, __fmul2_rn(ndz, ly));
-                    const float2 cy = __ffma2_rn(dz, lx, __fmul2_rn(ndx, lz));
-                    const float2 cz = __ffma2_rn(dx, ly, __fmul2_rn(ndy, lx));
-                    const float2 cc = __ffma2_rn(cz, cz, __ffma2_rn(cy, cy, __fmul2_rn(cx, cx)));
-                    sg = __fmul2_rn(__fmul2_rn(cc, make_float2(rsqrt_fast(cc.x), rsqrt_fast(cc.y))), rl);
-                }
-                const float2 ta = __fmul2_rn(sg, INVA), tb2 = __fmul2_rn(pz, INVB);
-                const float2 fa = __fadd2_rd(ta, C23), fb = __fadd2_rd(tb2, C23);
-                const float2 da = __ffma2_rn(__fadd2_rn(fa, NC23H), M1, ta);   // frac - 1/2
-                const float2 db = __ffma2_rn(__fadd2_rn(fb, NC23H), M1, tb2);
-                // NaN (s = 0 or l = 0) compares false: near
-                const bool n0 = !(fabsf(da.x) < thrA) || !(fabsf(db.x) < thrB);
-                const bool n1 = !(fabsf(da.y) < thrA) || !(fabsf(db.y) < thrB);
-                const unsigned ba0 = (unsigned)__float_as_int(fa.x), ba1 = (unsigned)__float_as_int(fa.y);
-                const unsigned bb0 = (unsigned)__float_as_int(fb.x), bb1 = (unsigned)__float_as_int(fb.y);
-                const bool ok0 = ba0 < limA && bb0 < limB, ok1 = ba1 < limA && bb1 < limB;
-                const unsigned b0 = ba0 * nbu + bb0, b1 = ba1 * nbu + bb1;
-                const bool a0 = in0[r] && ok0 && !n0, a1 = in1[r] && ok1 && !n1;
-                const unsigned c0 = a0 ? hbase + hk4 * b0 : htrash;
-                const unsigned c1 = a1 ? hbase + hk4 * b1 : htrash;
-                red_shared_u32(c0, 1u);
-                red_shared_u32(c1, 1u);
-                if (W == 1) {
-                    const double2 wj = *reinterpret_cast<const double2 *>(tb.w + jj);
-                    red_shared_f64_if(wbase + 2u * hk4 * b0, __dmul_rn(I.w[r], wj.x), a0);
-                    red_shared_f64_if(wbase + 2u * hk4 * b1, __dmul_rn(I.w[r], wj.y), a1);
-                } else if (W == 2) {
-                    const uint2 wj = *reinterpret_cast<const uint2 *>(tb.wm + jj);
-                    red_shared_pieces(3u * c0 + wdelta, (unsigned long long)I.wm[r] * wj.x);
-                    red_shared_pieces(3u * c1 + wdelta, (unsigned long long)I.wm[r] * wj.y);
-                } else if (W == 3) {
-                    const uint2 wj = *reinterpret_cast<const uint2 *>(tb.wm + jj);
-                    const float2 lj = *reinterpret_cast<const float2 *>(tb.wl + jj);
-                    red_shared_pieces_v(3u * c0 + wdelta,
-                                        corrected_product(I.wm[r], I.pf[r], I.wl[r], wj.x, lj.x));
-                    red_shared_pieces_v(3u * c1 + wdelta,
-                                        corrected_product(I.wm[r], I.pf[r], I.wl[r], wj.y, lj.y));
-                }
-                re0[r] = in0[r] && n0;
-                re1[r] = in1[r] && n1;
-                anyr = anyr || re0[r] || re1[r];
-            }
-            if (__any_sync(0xffffffffu, anyr)) {
-#pragma unroll
-                for (int r = 0; r < RI; ++r) {
-                    if (re0[r])
-                        rescue_push<MODE_SIGPI, LOS>(p, s_q, s_qn, s_seg, nseg, f0, fstride, jj,
-                                                     bstart, I.idx[r], task_bits);
-                    if (re1[r])
-                        rescue_push<MODE_SIGPI, LOS>(p, s_q, s_qn, s_seg, nseg, f0, fstride, jj + 1,
-                                                     bstart, I.idx[r], task_bits);
-                }
-            }
-        }
-    }
-    }
+// ---------------------------------------------------------------------------
+// fixed-point floors (PATH_FIX)
+// ---------------------------------------------------------------------------
+// For bins evenly spaced from zero, at most FIX_TOP an axis, a scaled value t
+// (s / D, mu n_mu, sigma / D, pi / D) is added to 128 + B 2^-16 in one fused
+// multiply-add.  FP32 numbers in [128, 256) are multiples of 2^-16: byte 2 of
+// the sum is floor(t + B 2^-16) and its low half the 16-bit fraction.  B is the
+// error band in these units (the arithmetic's bound and the sum's own rounding,
+// rounded up), so the pair is near an edge iff the fraction is below 2 B, and
+// otherwise the byte is its bin.  One three-input minimum of 16-bit halves
+// covers two values of the near test (the upper halves ride along unused), one
+// byte permutation puts the two bins side by side as the counter's index, and
+// values past the last bin are clamped to half a bin past it: the discarded
+// row (pi: column), never near.  mu n_mu has no shrunken scale: mu = 1 lands in
+// column n_mu, is near, and is put right by its binary64 check.  A tiny
+// constant added to the squares keeps coincident points finite (they are near,
+// t = 0).  Every index stays inside the histogram: coordinates are finite and
+// below 1e16 (others count as absent; the host limits the extents to 1e15, so no
+// square overflows), hence 128 <= T <= n_a + 128.5 and 128 <= M < 256.
+//
+// Against the packed floors of bin2 this leaves 40 of 68 packed FP32
+// instructions a quad (their three-register forms cost three register-read
+// cycles each); measured on the loop alone, (s, mu) 40 x 100: 161 against 224
+// cycles a quad and scheduler, one axis 121 against 147.
+__device__ __forceinline__ unsigned prmt(unsigned a, unsigned b, unsigned s) {
+    unsigned d;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(s));
+    return d;
 }
 
-// Global-histogram variant for histograms too large for shared memory.
-template <int MODE, int LOS, int W, int RI, bool MASK>
-__device__ __forceinline__ void pair_tile_global(const PairParams &p, Tile tb, int len, unsigned gmask,
-                                                 const IPts<RI> &I, const BinCtx &bc, float r2cut,
-                                                 size_t hbase, uint3 *s_q, int *s_qn,
-                                                 const int4 *s_seg, int nseg, int f0, int fstride, int bstart,
-                                                 unsigned task_bits) {
-    for (unsigned gm = gmask; gm; gm &= gm - 1) {
-    const int j0 = (__ffs(gm) - 1) * JG, j1 = min(j0 + JG, len);
-    for (int jj = j0; jj < j1; ++jj) {
-        const float qx = tb.x[jj], qy = tb.y[jj], qz = tb.z[jj];
-        for (int r = 0; r < RI; ++r) {
-            float dx = qx - I.x[r], dy = qy - I.y[r], dz = qz - I.z[r];
-            float qxy = fmaf(dy, dy, dx * dx);
-            float s2 = fmaf(dz, dz, qxy);
-            bool inr = s2 < r2cut;
-            if (MASK) inr = inr && (bstart + jj > I.idx[r]);
-            if (!inr) continue;
-            Bin32 b = bin_f32<MODE, LOS>(bc, dx, dy, dz, qxy, s2, I.xa[r], I.ya[r], I.za[r]);
-            if (b.near) {
-                rescue_push<MODE, LOS>(p, s_q, s_qn, s_seg, nseg, f0, fstride, jj, bstart, I.idx[r],
-                                       task_bits);
-            } else if (b.ok) {
-                atomicAdd(p.hist + hbase + b.bin, 1ull);
-                if (W == 1) atomicAdd(p.whist + hbase + b.bin, __dmul_rn(I.w[r], tb.w[jj]));
-            }
-        }
-    }
-    }
+// The three 16-bit pieces of P >> 16, taken from P; of V (the top one 17 bits).
+__device__ __forceinline__ uint3 pieces(unsigned long long P) {
+    const unsigned lo = (unsigned)P, hi = (unsigned)(P >> 32);
+    return make_uint3(lo >> 16, hi & 0xFFFFu, hi >> 16);
+}
+__device__ __forceinline__ uint3 pieces_v(unsigned long long V) {
+    const unsigned lo = (unsigned)V;
+    return make_uint3(lo & 0xFFFFu, lo >> 16, (unsigned)(V >> 32));
+}
+__device__ __forceinline__ void add_pieces(unsigned char *a0, unsigned char *a1, unsigned char *a2, uint3 v) {
+    atomicAdd(reinterpret_cast<unsigned *>(a0), v.x);
+    atomicAdd(reinterpret_cast<unsigned *>(a1), v.y);
+    atomicAdd(reinterpret_cast<unsigned *>(a2), v.z);
 }
 
-// One tile through the variant that applies.
-template <int MODE, int LOS, int W, int RI, bool LIN, bool MASK>
-__device__ __forceinline__ void pair_tile(const PairParams &p, bool smem_hist, Tile tb, int len,
-                                          unsigned gmask,
-                                          const IPts<RI> &I, const BinCtx &bc, const LinCtx &lc,
-                                          float r2cut, unsigned hist_sa, unsigned whist_sa,
-                                          unsigned hk4, size_t hbase, uint3 *s_q, int *s_qn,
-                                          const int4 *s_seg,
-                                          int nseg, int f0, int fstride, int bstart, unsigned task_bits) {
-    static_assert(W < 2 || LIN, "integer weights run only with floor-based bins");
-    if (!smem_hist) {
-        pair_tile_global<MODE, LOS, W, RI, MASK>(p, tb, len, gmask, I, bc, r2cut, hbase, s_q, s_qn, s_seg,
-                                                 nseg, f0, fstride, bstart, task_bits);
-    } else if constexpr (LIN && MODE == MODE_SIGPI) {
-        pair_tile_sigpi2<LOS, W, RI, MASK>(p, tb, len, gmask, I, lc, r2cut, hist_sa, whist_sa, hk4,
-                                           s_q, s_qn, s_seg, nseg, f0, fstride, bstart, task_bits);
-    } else if constexpr (LIN) {
-        if (p.lin_log)
-            pair_tile_lin2<MODE, W, RI, MASK, true, true>(p, tb, len, gmask, I, lc, r2cut, hist_sa,
-                                                          whist_sa, hk4, s_q, s_qn, s_seg, nseg,
-                                                          f0, fstride, bstart, task_bits);
-        else if (p.lin_norange)
-            pair_tile_lin2<MODE, W, RI, MASK, false, false>(p, tb, len, gmask, I, lc, r2cut, hist_sa,
-                                                     whist_sa, hk4, s_q, s_qn, s_seg, nseg, f0, fstride,
-                                                     bstart, task_bits);
-        else
-            pair_tile_lin2<MODE, W, RI, MASK, true, false>(p, tb, len, gmask, I, lc, r2cut, hist_sa,
-                                                    whist_sa, hk4, s_q, s_qn,
-                                          s_seg, nseg, f0, fstride, bstart, task_bits);
+struct Fix2 {
+    float2 T, M;   // first axis (clamped) and second axis, in fixed point
+};
+
+template <int MODE, int LOS>
+__device__ __forceinline__ Fix2 fix2(const PairParams &p, float2 dx, float2 dy, float2 dz, float2 cfm, float xa,
+                                     float ya, float za, float2 &s2) {
+    Fix2 o;
+    float2 pz, rl, lx, ly, lz;
+    const float2 q = __ffma2_rn(dy, dy, __ffma2_rn(dx, dx, p.f_tiny));
+    s2 = __ffma2_rn(dz, dz, q);
+    if (LOS == LOS_MID && MODE != MODE_S) {   // l = 2 x_i + d
+        lx = __fadd2_rn(make_float2(xa, xa), dx);
+        ly = __fadd2_rn(make_float2(ya, ya), dy);
+        lz = __fadd2_rn(make_float2(za, za), dz);
+        const float2 sl = __ffma2_rn(dz, lz, __ffma2_rn(dy, ly, __fmul2_rn(dx, lx)));
+        const float2 ll = __ffma2_rn(lz, lz, __ffma2_rn(ly, ly, __ffma2_rn(lx, lx, p.f_tiny)));
+        rl = make_float2(rsqrt_fast(ll.x), rsqrt_fast(ll.y));
+        pz = make_float2(fabsf(sl.x), fabsf(sl.y));
+    } else if (MODE != MODE_S) {
+        pz = make_float2(fabsf(dz.x), fabsf(dz.y));
+    }
+    float2 T;
+    if (MODE == MODE_SIGPI) {
+        float2 v = q, rv;
+        if (LOS == LOS_Z) {
+            rv = __fmul2_rn(make_float2(rsqrt_fast(q.x), rsqrt_fast(q.y)), p.c_invA);
+        } else {   // sigma = |d x l| / |l|
+            const float2 M1 = p.c_m1;
+            const float2 ndx = __fmul2_rn(dx, M1), ndy = __fmul2_rn(dy, M1), ndz = __fmul2_rn(dz, M1);
+            const float2 cx = __ffma2_rn(dy, lz, __fmul2_rn(ndz, ly));
+            const float2 cy = __ffma2_rn(dz, lx, __fmul2_rn(ndx, lz));
+            const float2 cz = __ffma2_rn(dx, ly, __fmul2_rn(ndy, lx));
+            v = __ffma2_rn(cz, cz, __ffma2_rn(cy, cy, __ffma2_rn(cx, cx, p.f_tiny)));
+            rv = __fmul2_rn(make_float2(rsqrt_fast(v.x), rsqrt_fast(v.y)), __fmul2_rn(rl, p.c_invA));
+        }
+        T = __ffma2_rn(v, rv, p.f_cfs);
+        const float2 M = __ffma2_rn(pz, LOS == LOS_Z ? p.c_invB : __fmul2_rn(rl, p.c_invB), cfm);
+        o.M = make_float2(fminf(M.x, p.f_limB), fminf(M.y, p.f_limB));
     } else {
-        pair_tile_lut<MODE, LOS, W, RI, MASK>(p, tb, len, gmask, I, bc, r2cut, hist_sa, whist_sa,
-                                              hk4, s_q,
-                                              s_qn, s_seg, nseg, f0, fstride, bstart, task_bits);
+        const float2 rs = make_float2(rsqrt_fast(s2.x), rsqrt_fast(s2.y));
+        T = __ffma2_rn(s2, __fmul2_rn(rs, p.c_invA), p.f_cfs);
+        if (MODE == MODE_SMU)
+            o.M = __ffma2_rn(pz, LOS == LOS_Z ? __fmul2_rn(rs, p.c_invB)
+                                              : __fmul2_rn(__fmul2_rn(rl, rs), p.c_invB), cfm);
     }
+    o.T = make_float2(fminf(T.x, p.f_lim), fminf(T.y, p.f_lim));
+    return o;
+}
+
+// All pairs of the warp's i-points with nq quads of staged j-points, as
+// pair_quads.  SLOW: batches that may hold pairs closer than the separation the
+// mu band is taken at (T below f_close: near), and the block's own points (the
+// tile holds its points from jbase on, pairs j <= i are masked; jbase past any
+// i: none is).
+template <int MODE, int LOS, int W, bool SLOW>
+__device__ __forceinline__ unsigned quads_fix(const PairParams &p, const Tile &t, int nq, const IPts<LOS, W> &I,
+                                              unsigned char *smem, float cfm1, unsigned tm2, int jbase) {
+    const int lane = threadIdx.x & 31;
+    const float2 cfm = make_float2(cfm1, cfm1);
+    const unsigned copy = 4u * (unsigned)lane;                 // LAY_BYTES
+    const unsigned kc = (unsigned)(lane & (p.hist_k - 1));    // LAY_ROWS
+    unsigned *hist = reinterpret_cast<unsigned *>(smem);
+    unsigned near = 0u;
+    // two quads an iteration where the body stays small in the instruction cache
+    constexpr int UNROLL = SLOW || W || (LOS == LOS_MID && MODE != MODE_S) ? 1 : 2;
+#pragma unroll UNROLL
+    for (int q = 0; q < nq; ++q) {
+        const float4 X = reinterpret_cast<const float4 *>(t.x)[q];
+        const float4 Y = reinterpret_cast<const float4 *>(t.y)[q];
+        const float4 Z = reinterpret_cast<const float4 *>(t.z)[q];
+        unsigned accT = 0xffffffffu, accM = 0xffffffffu;
+        bool close = false;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float2 Xh = h ? make_float2(X.z, X.w) : make_float2(X.x, X.y);
+            const float2 Yh = h ? make_float2(Y.z, Y.w) : make_float2(Y.x, Y.y);
+            const float2 Zh = h ? make_float2(Z.z, Z.w) : make_float2(Z.x, Z.y);
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                float2 dx = __fadd2_rn(Xh, make_float2(-I.x[r], -I.x[r]));
+                const float2 dy = __fadd2_rn(Yh, make_float2(-I.y[r], -I.y[r]));
+                const float2 dz = __fadd2_rn(Zh, make_float2(-I.z[r], -I.z[r]));
+                if (SLOW) {   // masked pairs: far out of range
+                    const int jj = jbase + 4 * q + 2 * h;
+                    if (jj <= 2 * lane + r) dx.x = p.far;
+                    if (jj + 1 <= 2 * lane + r) dx.y = p.far;
+                }
+                float2 s2;
+                const Fix2 f = fix2<MODE, LOS>(p, dx, dy, dz, cfm, I.xa[r], I.ya[r], I.za[r], s2);
+                const unsigned t0 = __float_as_uint(f.T.x), t1 = __float_as_uint(f.T.y);
+                accT = __vimin3_u16x2(accT, t0, t1);
+                if (SLOW && MODE == MODE_SMU) close = close | (f.T.x < p.f_close) | (f.T.y < p.f_close);
+                unsigned P0 = 0u, P1 = 0u;   // W >= 2: addresses of the pieces' records
+                if (MODE == MODE_S) {
+                    // byte 1: the bin, byte 0: this lane's copy
+                    const unsigned a0 = prmt(t0, copy, 0x5524), a1 = prmt(t1, copy, 0x5524);
+                    atomicAdd(reinterpret_cast<unsigned *>(smem + a0), 1u);
+                    atomicAdd(reinterpret_cast<unsigned *>(smem + a1), 1u);
+                    P0 = a0;
+                    P1 = a1;
+                } else {
+                    const unsigned m0 = __float_as_uint(f.M.x), m1 = __float_as_uint(f.M.y);
+                    accM = __vimin3_u16x2(accM, m0, m1);
+                    // 256 n + m from the two bytes (the sign bit of byte 2 is 0)
+                    const unsigned w0 = prmt(m0, t0, 0xAA62), w1 = prmt(m1, t1, 0xAA62);
+                    if (W == 0) {
+                        atomicAdd(&hist[w0 + (w0 >> 5)], 1u);
+                        atomicAdd(&hist[w1 + (w1 >> 5)], 1u);
+                    } else {   // LAY_ROWS
+                        P0 = __dp4a(w0, p.f_coef, kc);   // (n hs + m) hist_k + copy
+                        P1 = __dp4a(w1, p.f_coef, kc);
+                        atomicAdd(&hist[P0], 1u);
+                        atomicAdd(&hist[P1], 1u);
+                    }
+                }
+                if (W >= 2) {
+                    // (M_i M_j) >> (k_i + k_j), k = emax - e the exponent offset:
+                    // the packed M 2^(8 - k) multiplied exactly in 64 bits is
+                    // P = M_i M_j 2^(16 - k_i - k_j), and the product is P >> 16
+                    // (truncation < 2^(k_i + k_j - 46) relative, below 2^48)
+                    const uint2 wj = *reinterpret_cast<const uint2 *>(t.wm + 4 * q + 2 * h);
+                    uint3 v0, v1;   // 16-bit pieces, lowest first
+                    if (W == 2) {
+                        v0 = pieces((unsigned long long)I.wm[r] * wj.x);
+                        v1 = pieces((unsigned long long)I.wm[r] * wj.y);
+                    } else {
+                        const uint2 lj = *reinterpret_cast<const uint2 *>(t.wl + 4 * q + 2 * h);
+                        v0 = pieces_v(corrected_product(I.wm[r], I.wb[r], wj.x, lj.x));
+                        v1 = pieces_v(corrected_product(I.wm[r], I.wb[r], wj.y, lj.y));
+                    }
+                    if (MODE == MODE_S) {
+                        add_pieces(smem + P0 + 128, smem + P0 + p.sm_whist, smem + P0 + p.sm_whist + 128, v0);
+                        add_pieces(smem + P1 + 128, smem + P1 + p.sm_whist, smem + P1 + p.sm_whist + 128, v1);
+                    } else {
+                        unsigned char *r0 = smem + p.sm_whist + 12 * P0, *r1 = smem + p.sm_whist + 12 * P1;
+                        add_pieces(r0, r0 + 4, r0 + 8, v0);
+                        add_pieces(r1, r1 + 4, r1 + 8, v1);
+                    }
+                }
+            }
+        }
+        bool any = (accT & 0xffffu) < p.f_ts2;
+        if (MODE != MODE_S) any = any | ((accM & 0xffffu) < tm2);
+        if (SLOW) any = any | close;
+        near |= (any ? 1u : 0u) << q;
+    }
+    return near;
+}
+
+// Two pairs' bins and near flags from their fixed-point values (the near-edge
+// check repeats the loop's arithmetic with them); bin -1: discarded.
+template <int MODE>
+__device__ __forceinline__ int fix_bin(const PairParams &p, float T, float M, unsigned tm2, bool &near) {
+    const unsigned t = __float_as_uint(T), m = MODE == MODE_S ? 0u : __float_as_uint(M);
+    near = (t & 0xffffu) < p.f_ts2;
+    if (MODE != MODE_S) near = near || (m & 0xffffu) < tm2;
+    if (MODE == MODE_SMU) near = near || T < p.f_close;
+    const int n = (int)((t >> 16) & 0x7f), k = (int)((m >> 16) & 0x7f);
+    return n < p.n_a && k < p.n_b ? n * p.n_b + k : -1;
+}
+
+// Weighted product of a pair as the fast path added it (integer paths).
+template <int LOS, int W>
+__device__ __forceinline__ unsigned long long fast_product(const IPts<LOS, W> &I, int r, unsigned wj, unsigned lj) {
+    if (W == 3) return corrected_product(I.wm[r], I.wb[r], wj, lj);
+    return ((unsigned long long)I.wm[r] * wj) >> 16;
+}
+
+// Check n queued near-edge quads with the binary64 definition, one per lane.
+// An entry is {first of its four j-points, source lane | own block << 5 |
+// segment << 6 | mu band << 13}.  The lane repeats the quad's FP32 arithmetic
+// on the same operands, so it sees the same bins and the same near pairs, and
+// corrects the global histogram where the binary64 bin differs from the one
+// counted.  With a rescue queue (pc_opts.rescue_capacity > 0) the fast count is
+// undone instead and the pair queued while there is room.
+template <int MODE, int LOS, int W, int PATH, bool TREE>
+__device__ __noinline__ void check_near(const PairParams &p, const uint2 *queue, const int4 *seg, int n, int task,
+                                        int cell, int start, int count, unsigned copy, const float2 *s_lut) {
+    const int lane = threadIdx.x & 31;
+    const TaskDev &T = p.tasks[task];
+    Ctx<MODE, LOS, PATH == PATH_FIX ? PATH_LIN : PATH> c;
+    if (PATH != PATH_FIX) c.init(p, s_lut, copy);
+    unsigned m8 = 0u;         // near pairs: bit 4 r + j
+    int b8[8];                // the bins they were counted in (-1: none)
+    int i0 = 0, j0 = 0, img = 13;
+    if (lane < n) {
+        const uint2 e = queue[lane];
+        const int src = (int)(e.y & 31u);
+        const bool own = (e.y >> 5) & 1u;
+        const unsigned band = e.y >> 13;
+        j0 = (int)e.x;
+        i0 = start + 2 * src;
+        int4 sg = make_int4(start, start + count, TREE ? -1 : 0, 13);
+        if (!own) sg = seg[(e.y >> 6) & 127u];
+        img = sg.w;
+        unsigned vm = 0u;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) vm |= (j0 + j >= sg.x && j0 + j < sg.y) ? 1u << j : 0u;
+        float3 s[4];
+        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (TREE && sg.z >= 0) o = tree_offset(p, cell, sg.z, img);
+        const int ax = TREE ? 0 : cell % p.g.ng[0];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            s[j] = make_float3(0.f, 0.f, 0.f);
+            if (!(vm >> j & 1u)) continue;
+            const float4 q = T.gj.rel[j0 + j];
+            if (TREE) s[j] = own ? make_float3(q.x, q.y, q.z) : make_float3(o.x + q.x, o.y + q.y, o.z + q.z);
+            else s[j] = own ? make_float3(q.x, q.y, q.z)
+                            : stage_grid(p, q, T.gj.cx[j0 + j], ax, sg.z, img);
+        }
+        const float cf1 = MODE == MODE_SIGPI ? p.f_cfp : fmaf((float)band, 1.0f / 65536.0f, 128.0f);
+        const float2 cfm = make_float2(cf1, cf1);
+        const unsigned tm2 = MODE == MODE_SIGPI ? p.f_tp2 : 2u * band;
+        IPts<LOS, W> I;
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            I.x[r] = I.y[r] = I.z[r] = I.xa[r] = I.ya[r] = I.za[r] = 0.f;
+            if (2 * src + r < count) load_i<MODE, LOS, W>(T.gi, i0 + r, I, r);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float2 dx = __fadd2_rn(make_float2(s[2 * h].x, s[2 * h + 1].x), make_float2(-I.x[r], -I.x[r]));
+                const float2 dy = __fadd2_rn(make_float2(s[2 * h].y, s[2 * h + 1].y), make_float2(-I.y[r], -I.y[r]));
+                const float2 dz = __fadd2_rn(make_float2(s[2 * h].z, s[2 * h + 1].z), make_float2(-I.z[r], -I.z[r]));
+                const int j = 2 * h;
+                const bool iok = 2 * src + r < count;
+                const bool v0 = iok && (vm >> j & 1u) && !(own && j0 + j <= i0 + r);
+                const bool v1 = iok && (vm >> (j + 1) & 1u) && !(own && j0 + j + 1 <= i0 + r);
+                float2 s2;
+                bool n0, n1;
+                if (PATH == PATH_FIX) {
+                    const Fix2 f = fix2<MODE, LOS>(p, dx, dy, dz, cfm, I.xa[r], I.ya[r], I.za[r], s2);
+                    b8[4 * r + j] = fix_bin<MODE>(p, f.T.x, f.M.x, tm2, n0);
+                    b8[4 * r + j + 1] = fix_bin<MODE>(p, f.T.y, f.M.y, tm2, n1);
+                } else {
+                    const float2 qq = __ffma2_rn(dy, dy, __fmul2_rn(dx, dx));
+                    s2 = __ffma2_rn(dz, dz, qq);
+                    const Pair2 b = bin2<MODE, LOS, PATH == PATH_FIX ? PATH_LIN : PATH>(
+                        p, c, dx, dy, dz, qq, s2, I.xa[r], I.ya[r], I.za[r]);
+                    n0 = b.n0;
+                    n1 = b.n1;
+                    b8[4 * r + j] = b8[4 * r + j + 1] = -1;   // tables: near pairs are not counted
+                    if (PATH != PATH_LUT && PATH != PATH_GLOBAL) {
+                        if (b.a0 < c.trash) b8[4 * r + j] = entry_bin(p, (int)((b.a0 - copy) / c.hk4));
+                        if (b.a1 < c.trash) b8[4 * r + j + 1] = entry_bin(p, (int)((b.a1 - copy) / c.hk4));
+                    }
+                }
+                if (v0 && n0 && s2.x < p.r2cut) m8 |= 1u << (4 * r + j);
+                if (v1 && n1 && s2.y < p.r2cut) m8 |= 1u << (4 * r + j + 1);
+            }
+        }
+    }
+    unsigned done = 0u;
+    while (__any_sync(FULL, m8 != 0u)) {
+        if (m8) {
+            const int k = __ffs(m8) - 1;
+            m8 &= m8 - 1;
+            int fast = b8[0];
+#pragma unroll
+            for (int q = 1; q < 8; ++q) fast = k == q ? b8[q] : fast;
+            const int i = i0 + (k >> 2), j = j0 + (k & 3);
+            const size_t hb = (size_t)T.hist * p.nbins;
+            unsigned long long slot = ~0ull;
+            if (p.qcap) slot = atomicAdd(p.qcount, 1ull);
+            int bin = -1;
+            double wp = 0.0;
+            if (slot < p.qcap) {
+                p.queue[slot] = make_uint3((unsigned)i, (unsigned)j, (unsigned)img | ((unsigned)task << 5));
+            } else {
+                const double4_32a A = T.gi.xw[i], B = T.gj.xw[j];
+                bin = max(f64_pair_bin<MODE, LOS>(A, B, img, p.g, p.Ea, p.n_a, p.Eb, p.n_b), -1);
+                wp = __dmul_rn(A.w, B.w);
+                ++done;
+            }
+            if (bin != fast) {
+                if (fast >= 0) {
+                    atomicAdd(&p.hist[hb + (size_t)fast], 0xffffffffffffffffull);   // - 1
+                    if (W >= 2) {
+                        IPts<LOS, W> I;
+                        load_i<MODE, LOS, W>(T.gi, i, I, 0);
+                        const unsigned wj = __float_as_uint(T.gj.rel[j].w);
+                        const unsigned lj = (W == 3 && T.gj.wlo) ? T.gj.wlo[j] : 0u;
+                        atomicAdd(&p.whist[hb + (size_t)fast],
+                                  -((double)fast_product<LOS, W>(I, 0, wj, lj) * T.wscale));
+                    }
+                }
+                if (bin >= 0) {
+                    atomicAdd(&p.hist[hb + (size_t)bin], 1ull);
+                    if (W >= 1) atomicAdd(&p.whist[hb + (size_t)bin], wp);
+                }
+            } else if (W == 1 && bin >= 0) {   // near pairs' binary64 weights are added here only
+                atomicAdd(&p.whist[hb + (size_t)bin], wp);
+            }
+        }
+        __syncwarp();
+    }
+    const unsigned tot = __reduce_add_sync(FULL, done);
+    if (lane == 0 && tot) atomicAdd(&p.counters[1], (unsigned long long)tot);
 }
 
 // ---------------------------------------------------------------------------
 // FP32 kernel
 // ---------------------------------------------------------------------------
-// W: 0 unweighted, 1 binary64 weighted sums, 2 integer weight products.
-// G: independent groups of NT threads per CTA that share the histograms (a
-// large histogram then keeps G x 4 warps per SM busy instead of 4).
-// TREE: blocks are k-d tree nodes and their j-segments come from the list of
-// the dual-tree traversal instead of the stencil rows.
-template <int MODE, int LOS, int W, int RI, bool LIN, int G = 1, bool TREE = false>
-__global__ void __launch_bounds__(NT * G, (G > 1 ? 1 : (RI <= 2 ? 5 : 4)))
+// W: 0 unweighted, 1 binary64 weighted sums, 2 integer weight products, 3 the
+// same with binary64 remainders.  TREE: blocks are k-d tree nodes and their
+// j-segments come from the list of the dual-tree traversal instead of the
+// stencil rows.
+//
+// Work items: (block, 64-point part of the block, slice of its octs).  Slices
+// (S > 1) split the i-points' candidates among warps, for about 24 items a
+// warp of the grid, so that the last items do not leave the chip half empty.
+// One histogram: each warp takes items from the global counter until none are
+// left.  Several (batches): the CTA takes ranges of items of one histogram and
+// flushes between them.
+//
+// Registers: the loops need 50 to 80; with the rest of a warp's state 80 (96 with
+// more operands a pair) give 24 (20) resident warps.  80 to 128 measured within
+// 2 %, the loop alone loses 5 % at 12 warps.
+template <int MODE, int LOS, int W, int PATH, bool TREE>
+__global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH == PATH_LUT ? 96 : 80)
     k_pairs_f32(const __grid_constant__ PairParams p) {
-    static_assert(!TREE || G == 1, "the tree variant runs one thread group per CTA");
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ CtaShared cs_g[G];
-    __shared__ int s_tmp_g[G][8];
-    __shared__ unsigned long long s_base_g[G];
-    __shared__ GBox s_gbox_g[G][2][TJ / JG];   // bounding boxes of the staged j-groups
-    __shared__ GBox s_ibox_g[G][NT / 32];      // bounding box of each warp's i-points
-    const int grp = (int)(threadIdx.x / NT);
-    CtaShared &cs = cs_g[grp];
-    int *s_tmp = s_tmp_g[grp];
-    unsigned long long &s_base = s_base_g[grp];
-    GBox(*s_gbox)[TJ / JG] = s_gbox_g[grp];
-    GBox *s_ibox = s_ibox_g[grp];
+    __shared__ int s_cur, s_end, s_next, s_lim, s_task;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
+    unsigned char *ws = smem + p.sm_warp + (size_t)warp * WarpOff::total(TREE, W);
+    int4 *seg = reinterpret_cast<int4 *>(ws + WarpOff::seg(TREE));
+    float4 *soff = reinterpret_cast<float4 *>(ws + WarpOff::soff(TREE));
+    float *tx = reinterpret_cast<float *>(ws + WarpOff::tile(TREE));
+    float *ty = tx + JB, *tz = ty + JB;
+    double *tw = reinterpret_cast<double *>(ws + WarpOff::tw(TREE));
+    unsigned *twm = reinterpret_cast<unsigned *>(tw);
+    unsigned *twl = twm + JB;
+    uint2 *queue = reinterpret_cast<uint2 *>(ws + WarpOff::queue(TREE, W));
+    int4 *ring = reinterpret_cast<int4 *>(ws + WarpOff::ring(TREE, W));
+    int *pref = reinterpret_cast<int *>(ws + WarpOff::pref(TREE, W));
+    const Tile tile{tx, ty, tz, tw, twm, twl};
+    const float2 *s_lut = reinterpret_cast<const float2 *>(smem + p.sm_lut);
 
-    const SmemLayout Ly = smem_layout(p, false);
-    float2 *s_lut = (float2 *)(smem + Ly.lut);
-    int *s_hist = (int *)(smem + Ly.hist);
-    double *s_whist = (double *)(smem + Ly.whist);
-    unsigned char *gsm = smem + (size_t)grp * Ly.gstride;   // this group's own area
-    int4 *s_seg = (int4 *)(gsm + Ly.seg);
-    float *s_tx = (float *)(gsm + Ly.tile);     // [2][TJ] each
-    float *s_ty = s_tx + 2 * TJ;
-    float *s_tz = s_ty + 2 * TJ;
-    double *s_tw = (double *)(gsm + Ly.tw);
-    unsigned *s_twm = (unsigned *)(gsm + Ly.tw);   // packed weights share the storage
-    float *s_twl = (float *)(s_twm + 2 * TJ);      // W == 3: remainders after them
-    uint3 *s_q = (uint3 *)(gsm + Ly.q);
-    float4 *s_soff = (float4 *)(gsm + Ly.meta);   // tree: offset of each segment's block centre
-
-    const int tid = gtid();
-    for (int k = threadIdx.x; k < p.lut_total; k += NT * G) s_lut[k] = p.lut[k];
-    const int nbins = p.nbins;
-    const bool smem_hist = p.smem_hist_ok != 0;
-    if (smem_hist) {
-        const int copies = (p.priv ? NT / 32 : 1) * p.hist_k;
-        for (int k = threadIdx.x; k < p.nbins_smem * copies; k += NT * G) s_hist[k] = 0;
-        if (W >= 2) {   // the integer weight records (and this CTA's folded sums)
-            unsigned *wp = reinterpret_cast<unsigned *>(s_whist);
-            for (int k = threadIdx.x; k < 3 * p.nbins_smem * p.wint_k; k += NT * G) wp[k] = 0u;
-            if (p.wfold)
-                for (int b = threadIdx.x; b < p.nbins; b += NT) {
-                    unsigned long long *f = p.wfold_buf + ((size_t)blockIdx.x * p.nbins + b) * 2;
-                    f[0] = f[1] = 0ull;
-                }
-        } else if (W) {
-            for (int k = threadIdx.x; k < p.nbins_smem * p.hist_k; k += NT * G) s_whist[k] = 0.0;
-        }
+    // clear the histograms, stage the tables
+    for (int k = threadIdx.x; k < p.sm_lut / 4; k += blockDim.x) reinterpret_cast<unsigned *>(smem)[k] = 0u;
+    for (int k = threadIdx.x; k < p.lut_total; k += blockDim.x)
+        reinterpret_cast<float2 *>(smem + p.sm_lut)[k] = p.lut[k];
+    if (W >= 2 && p.wfold)
+        for (int b = threadIdx.x; b < 2 * p.nbins; b += blockDim.x)
+            p.wfold_buf[(size_t)blockIdx.x * p.nbins * 2 + b] = 0ull;
+    if (threadIdx.x == 0) {
+        s_cur = s_end = s_next = s_lim = 0;
+        s_task = -1;
     }
-    if (tid == 0) {
-        cs.qn = 0;
-        cs.pruned = 0;
-    }
+    const unsigned copy = 4u * (unsigned)(lane & (p.hist_k - 1));
+    Ctx<MODE, LOS, PATH == PATH_FIX ? PATH_LIN : PATH> c;
+    if (PATH != PATH_FIX) c.init(p, s_lut, copy);
+    const unsigned wbase = (unsigned)__cvta_generic_to_shared(smem + p.sm_whist);
+    const float far = p.far;
 
-    BinCtx bc;
-    bc.lutA = s_lut + p.la.off;
-    bc.lutB = s_lut + p.lb.off;
-    bc.invA = p.la.inv_w;
-    bc.invB = p.lb.inv_w;
-    bc.TA1 = (unsigned)(p.la.T + 1);
-    bc.TB1 = (unsigned)(p.lb.T + 1);
-    bc.epsA = p.eps_a;
-    bc.epsB = p.eps_b;
-    bc.muA = p.mu_A;
-    bc.muB = p.mu_B;
-    bc.muW = p.mu_W;
-    bc.nA = (unsigned)p.n_a;
-    bc.nB = (unsigned)p.n_b;
-    LinCtx lc;
-    lc.invA = p.lin_invA;
-    lc.offA = p.lin_offA;
-    lc.thrA = p.lin_thrA;
-    lc.mS = p.lin_mS;
-    lc.invB2 = p.lin_invB2;
-    lc.thrB = p.lin_thrB;
-    lc.nB = p.lin_nB;
-    lc.mA = p.lin_mA;
-    lc.cB = p.lin_cB;
-    lc.nA = (unsigned)p.n_a;
-    lc.nB_u = (unsigned)p.n_b;
-    const float r2cut = p.r2cut;
-    // this thread's copy: warp copy (priv) and lane copy (tid % hist_k); bins
-    // are hist_k entries apart
-    const unsigned lane_copy = (unsigned)(tid & (p.hist_k - 1));
-    const unsigned hk4 = 4u * (unsigned)p.hist_k;
-    const unsigned hist_sa = (unsigned)__cvta_generic_to_shared(s_hist) +
-                             (p.priv ? (unsigned)((tid >> 5) * p.nbins_smem * p.hist_k * 4) : 0u) +
-                             4u * lane_copy;
-    const unsigned whist_sa = (unsigned)__cvta_generic_to_shared(s_whist) +
-                              (W >= 2 ? 12u * lane_copy : 8u * lane_copy);
-
-    const int nx = p.g.ng[0], ny = p.g.ng[1];
-    const float c32x = p.g.c32[0], c32y = p.g.c32[1], c32z = p.g.c32[2];
     const int nblocks = *p.nblocks;
-    unsigned long long cand_local = 0;    // thread 0 only
-    unsigned long long since_flush = 0;   // CTA-uniform
-    unsigned long long wterms = 0;        // CTA-uniform bound of products per lane copy (W >= 2)
-    int cur_hist = -1;
-    double cur_wscale = 0.0;
-    // integer weights: before n more j-points, flush if a lane copy of the
-    // weight records could exceed WINT_LIMIT products (NT / wint_k threads
-    // share a copy; each piece sum then stays below 2^16 x 2^16)
-    auto wint_room = [&](int n) {
-        if (W < 2) return;
-        const unsigned long long add = (unsigned long long)(NT / p.wint_k) * RI * (unsigned)n;
-        if (wterms + add > (W == 3 ? WINT_LIMIT / 2 : WINT_LIMIT)) {
-            if (p.wfold) {
-                fold_records(p, s_whist);
-            } else {
-                flush_hist<G>(p, s_hist, s_whist, cur_hist, cur_wscale);
-                since_flush = 0;
-            }
-            wterms = 0;
-        }
-        wterms += add;
-    };
-    __syncthreads();   // CTA-wide: shared histograms are clear
+    const int nsub = p.nsub;
+    int S = 1;
+    {
+        const long long units = max((long long)nblocks, p.npts_i / BI + 1);
+        const long long want = 24ll * gridDim.x * nw;
+        if (units < want) S = (int)min(32ll, (want + units - 1) / units);
+    }
+    const int per_block = nsub * S;
+    const long long nitems = (long long)nblocks * per_block;
+    const int chunk = (int)max((long long)nw, min((long long)nw * 32 * S, nitems / (6ll * gridDim.x)));
+    unsigned long long cand = 0, pruned = 0;   // per lane
+    unsigned since = 0, wterms = 0;            // quads, products per copy since this warp's flushes
+    const unsigned flush_quads = (unsigned)(FLUSH_LIMIT / 256 / nw);
+    // Integer weights: no record may take more than `wmax` products between
+    // flushes.  One axis (LAY_BYTES, 32 copies): each warp flushes after its
+    // share of that bound.  Otherwise a copy's share is used up in a batch or
+    // two while its bins hold little: each warp then looks for the largest
+    // counter, and flushes (counts with the weights) only past a quarter of the
+    // bound; what is in flight during a flush, at most 16 slots of a lane and
+    // warp, is taken off the quarter
+    constexpr bool SCAN = !(PATH == PATH_FIX && MODE == MODE_S);
+    constexpr unsigned wmax = W == 3 ? WINT_LIMIT / 2 : WINT_LIMIT;
+    const unsigned wlimit = (SCAN ? wmax / 4 * 3 : wmax) / (unsigned)nw;
+    const int wfull = (int)(wmax / 4) - 16 * nw * (32 / p.hist_k);
+    const unsigned wper = W >= 2 ? 8u * (unsigned)(32 / p.hist_k) : 0u;   // products per copy and quad
+    __syncthreads();
 
     for (;;) {
-        if (tid == 0) cs.blk = atomicAdd(p.work_counter, 1);   // the list holds only this shard's blocks
-        gsync<G>();
-        const int bidx = cs.blk;
-        if (bidx >= nblocks) break;
-        const Block B = p.blocks[bidx];
-        const TaskDev &T = p.tasks[B.task];
-        if (T.hist != cur_hist || (W >= 2 && T.wscale != cur_wscale)) {
-            flush_hist<G>(p, s_hist, s_whist, cur_hist, cur_wscale);
-            cur_hist = T.hist;
-            cur_wscale = T.wscale;
-            since_flush = 0;
-            wterms = 0;
+        // ---- next item ------------------------------------------------------
+        long long it;
+        if (!p.multi) {
+            unsigned v = 0u;
+            if (lane == 0) v = (unsigned)atomicAdd(p.work_counter, 1);
+            it = __shfl_sync(FULL, v, 0);
+            if (it >= nitems) break;
+        } else {
+            int v = 0;
+            for (;;) {
+                if (lane == 0) v = atomicAdd(&s_cur, 1);
+                v = __shfl_sync(FULL, v, 0);
+                if (v < s_end) break;
+                // range used up: every warp arrives here; the next one of a
+                // single task is fetched, the histograms flushed on a change
+                __syncthreads();
+                const int old = s_task;
+                __syncthreads();
+                if (threadIdx.x == 0) {
+                    int b = s_next;
+                    if (b >= s_lim) {
+                        b = (int)min((long long)atomicAdd(p.work_counter, chunk), nitems);
+                        s_lim = (int)min((long long)b + chunk, nitems);
+                    }
+                    int e = b;
+                    if (b < s_lim) {
+                        const int task = p.blocks[b / per_block].task;
+                        int lo = b + 1, hi = s_lim;   // items [b, e) belong to `task`
+                        while (lo < hi) {
+                            const int mid = (lo + hi) >> 1;
+                            if (p.blocks[mid / per_block].task == task) lo = mid + 1; else hi = mid;
+                        }
+                        e = lo;
+                        s_task = task;
+                    } else {
+                        s_task = -2;
+                    }
+                    s_cur = b;
+                    s_end = e;
+                    s_next = e;
+                }
+                __syncthreads();
+                if (s_task != old && old >= 0) {
+                    const int h = p.tasks[old].hist;
+                    if (PATH != PATH_GLOBAL) {
+                        flush_counts(p, 0, warp, nw, h);
+                        if (W) flush_weights(p, p.sm_whist, warp, nw, h, p.tasks[old].wscale);
+                    }
+                    __syncthreads();
+                    if (W >= 2 && p.wfold) flush_folded(p, h, p.tasks[old].wscale);
+                    since = wterms = 0;
+                    __syncthreads();
+                }
+                if (s_task == -2) break;
+            }
+            if (s_task == -2) break;
+            it = v;
         }
-        const size_t hbase = (size_t)T.hist * nbins;
-        const unsigned task_bits = (unsigned)B.task << 5;
-        const int ax = B.cell % nx, ay = (B.cell / nx) % ny, az = B.cell / (nx * ny);
+        const Block B = p.blocks[it / per_block];
+        const int rem = (int)(it % per_block), sub = rem / S, part = rem - sub * S;
+        const int k = (B.count + BI - 1) / BI;
+        if (sub >= k) continue;
+        const int start = B.start + (int)((long long)B.count * sub / k);
+        const int count = B.start + (int)((long long)B.count * (sub + 1) / k) - start;
+        const TaskDev &T = p.tasks[B.task];
+        const int nx = p.g.ng[0], ny = p.g.ng[1], nz = p.g.ng[2];
+        const int ax = TREE ? 0 : B.cell % nx, ay = TREE ? 0 : (B.cell / nx) % ny,
+                  az = TREE ? 0 : B.cell / (nx * ny);
 
-        // thread t holds the block's points RI t .. RI t + RI - 1: a warp covers
-        // 32 RI consecutive (sub-cell ordered, so spatially compact) points
-        IPts<RI> I;
+        // ---- i-points and their box (relative to the i-grid's origin) --------
+        IPts<LOS, W> I;
+        float blx = INFINITY, bly = INFINITY, blz = INFINITY, bhx = -INFINITY, bhy = -INFINITY, bhz = -INFINITY;
 #pragma unroll
-        for (int r = 0; r < RI; ++r) {
-            const int loc = RI * tid + r;
-            I.idx[r] = B.start + loc;
+        for (int r = 0; r < 2; ++r) {
+            I.x[r] = -far;      // unused: out of range of every j-point
+            I.y[r] = I.z[r] = 0.f;
             I.xa[r] = I.ya[r] = I.za[r] = 0.f;
             I.w[r] = 0.0;
             I.wm[r] = 0u;
-            I.wl[r] = I.pf[r] = 0.f;
-            I.x[r] = I.y[r] = I.z[r] = -1.0e18f;  // unused lane: far from every j (and from the +1e18 pad slot)
-            if (loc < B.count) {
-                float4 q = T.gi.rel[I.idx[r]];
-                I.x[r] = q.x; I.y[r] = q.y; I.z[r] = q.z;
-                I.wm[r] = __float_as_uint(q.w);
-                if (W == 3) {
-                    I.pf[r] = __uint2float_rn(I.wm[r]);
-                    I.wl[r] = T.gi.wlo ? T.gi.wlo[I.idx[r]] : 0.f;
+            I.wb[r] = 0u;
+            if (2 * lane + r < count) {
+                const int i = start + 2 * lane + r;
+                load_i<MODE, LOS, W>(T.gi, i, I, r);
+                if (PATH == PATH_FIX && !(fabsf(I.x[r]) + fabsf(I.y[r]) + fabsf(I.z[r]) < 1e16f)) {
+                    I.x[r] = -far;      // not a number: no pair
+                    I.y[r] = I.z[r] = 0.f;
                 }
-                if (LOS == LOS_MID || W == 1) {
-                    double4_32a a = T.gi.xw[I.idx[r]];
-                    I.xa[r] = (float)a.x; I.ya[r] = (float)a.y; I.za[r] = (float)a.z;
-                    I.w[r] = a.w;
-                }
+                const double4_32a a = T.gi.xw[i];
+                const double ox = a.x - T.gi.org[0], oy = a.y - T.gi.org[1], oz = a.z - T.gi.org[2];
+                blx = fminf(blx, __double2float_rd(ox)); bhx = fmaxf(bhx, __double2float_ru(ox));
+                bly = fminf(bly, __double2float_rd(oy)); bhy = fmaxf(bhy, __double2float_ru(oy));
+                blz = fminf(blz, __double2float_rd(oz)); bhz = fmaxf(bhz, __double2float_ru(oz));
             }
         }
-        {   // the warp's i-box (empty box if the warp holds no point)
-            float lx = INFINITY, ly = INFINITY, lz = INFINITY;
-            float hx = -INFINITY, hy = -INFINITY, hz = -INFINITY;
-#pragma unroll
-            for (int r = 0; r < RI; ++r)
-                if (RI * tid + r < B.count) {
-                    lx = fminf(lx, I.x[r]); hx = fmaxf(hx, I.x[r]);
-                    ly = fminf(ly, I.y[r]); hy = fmaxf(hy, I.y[r]);
-                    lz = fminf(lz, I.z[r]); hz = fmaxf(hz, I.z[r]);
-                }
-            lx = warp_minf(lx); ly = warp_minf(ly); lz = warp_minf(lz);
-            hx = warp_maxf(hx); hy = warp_maxf(hy); hz = warp_maxf(hz);
-            if ((tid & 31) == 0)
-                s_ibox[tid >> 5] = GBox{make_float4(lx, ly, lz, 0.f), make_float4(hx, hy, hz, 0.f)};
-        }
-        const int ni_w = min(max(B.count - (tid >> 5) * 32 * RI, 0), 32 * RI);
+        // the boxes are compared in the j-grid's coordinates: its origin
+        // relative to the i-grid's is taken off the i-box
+        const float ogx = (float)(T.gj.org[0] - T.gi.org[0]), ogy = (float)(T.gj.org[1] - T.gi.org[1]),
+                    ogz = (float)(T.gj.org[2] - T.gi.org[2]);
+        blx = warp_minf(blx) - ogx; bly = warp_minf(bly) - ogy; blz = warp_minf(blz) - ogz;
+        bhx = warp_maxf(bhx) - ogx; bhy = warp_maxf(bhy) - ogy; bhz = warp_maxf(bhz) - ogz;
 
-        // ---- phase A (auto): pairs inside the block, j > i ------------------
-        if (T.is_auto) {
-            const int lenA = (B.count + 1) & ~1;    // even; the pad slot is far away
-            for (int f = tid; f < lenA; f += NT) {
-                if (f < B.count) {
-                    int pj = B.start + f;
-                    float4 q = T.gj.rel[pj];
-                    s_tx[f] = q.x; s_ty[f] = q.y; s_tz[f] = q.z;
-                    if (W == 1) s_tw[f] = T.gj.xw[pj].w;
-                    if (W >= 2) s_twm[f] = __float_as_uint(q.w);
-                    if (W == 3) s_twl[f] = T.gj.wlo ? T.gj.wlo[pj] : 0.f;
-                } else {
-                    s_tx[f] = s_ty[f] = s_tz[f] = 1.0e18f;
-                    if (W == 1) s_tw[f] = 0.0;
-                    if (W >= 2) s_twm[f] = 0u;
-                    if (W == 3) s_twl[f] = 0.f;
-                }
-            }
-            gsync<G>();
-            wint_room(lenA);
-            const int ngA = (lenA + JG - 1) / JG;    // all groups evaluated
-            const unsigned maskA = ngA >= 32 ? 0xffffffffu : (1u << ngA) - 1u;
-            pair_tile<MODE, LOS, W, RI, LIN, true>(p, smem_hist, Tile{s_tx, s_ty, s_tz, s_tw, s_twm, s_twl}, lenA,
-                                                   maskA, I, bc, lc, r2cut, hist_sa, whist_sa, hk4, hbase, s_q,
-                                                   &cs.qn, s_seg, 0, -1, 0, B.start, task_bits);
-            if (tid == 0) cand_local += (unsigned long long)B.count * (B.count - 1) / 2;
-            since_flush += (unsigned long long)B.count * B.count;
-            gsync<G>();
-        }
-
-        // ---- phase B: j-segments, in chunks ---------------------------------
-        // grid: the stencil rows, ROWCHUNK at a time; tree: the i-block's list
-        // of (j-node, image) pairs, MAXSEG_T at a time
-        // tree: virtual segment 0 of an auto count is the rest of the i-node
-        // after this block (same node, no offset), then the listed nodes
-        int ts0 = 0, tvirt = 0, trest = 0, node_end = 0;
-        if constexpr (TREE) {
+        // ---- j-segments, in chunks ------------------------------------------
+        int ts0 = 0, ntl = 0, own_end = 0;
+        if (TREE) {
             ts0 = p.tseg_off[B.cell];
+            ntl = p.tseg_off[B.cell + 1] - ts0;
             if (T.is_auto) {
                 const int2 r = p.tblk_j[B.cell];
-                node_end = r.x + r.y;
-                trest = (node_end > B.start + B.count) ? 1 : 0;
+                own_end = r.x + r.y;
             }
-            tvirt = p.tseg_off[B.cell + 1] - ts0 + trest;
+        } else {
+            ntl = p.nrows;
+            if (T.is_auto) own_end = T.gi.cell_start[B.cell + 1];
         }
-        const int nchunk = TREE ? (tvirt + MAXSEG_T - 1) / MAXSEG_T : (p.nrows + ROWCHUNK - 1) / ROWCHUNK;
+        // pairs inside the block (j > i) first
+        bool own = T.is_auto && part == 0;
+        if (own && lane == 0) cand += (unsigned long long)count * (unsigned)(count - 1) / 2;
+        const int nchunk = max(1, (ntl + 31) / 32);
+        int round0 = 0;      // rounds of 32 octs before this chunk
+        int qn = 0;          // queued near-edge quads
         for (int ch = 0; ch < nchunk; ++ch) {
-            if constexpr (TREE) {
-                // segment k: a listed j-node's points, staged relative to the
-                // i-node's centre through the offset of the two centres
-                const int v0 = ch * MAXSEG_T;
-                const int ns = min(MAXSEG_T, tvirt - v0);
-                const double *ci = p.tcen_i + 3 * (size_t)B.cell;
-                for (int k = tid; k < ns; k += NT) {
-                    const int v = v0 + k;
-                    if (v < trest) {
-                        s_soff[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-                        s_seg[k] = make_int4(B.start + B.count, node_end - B.start - B.count, k, 13);
-                        continue;
-                    }
-                    const int2 e = p.tseg[ts0 + v - trest];
+            __syncwarp();
+            int nseg = 0, noct = 0;
+            if (ch == 0 && own_end > start + count) {   // rest of the own cell: j > i for all
+                const int a0 = start + count;
+                if (lane == 0) {
+                    seg[0] = make_int4(a0, own_end, TREE ? -1 : 0, 13);
+                    pref[0] = 0;
+                    if (TREE) soff[0] = make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+                nseg = 1;
+                noct = ((own_end + 7) >> 3) - (a0 >> 3);
+            }
+            const int row = ch * 32 + lane;
+            int a0[3], a1[3], im[3], np = 0, no = 0, meta = 0;
+            if (row < ntl) {
+                if (TREE) {
+                    const int2 e = p.tseg[ts0 + row];
                     const int2 r = p.tblk_j[e.x];
-                    const double *cj = p.tcen_j + 3 * (size_t)e.x;
-                    const double sx = (double)(e.y / 9 - 1), sy = (double)((e.y / 3) % 3 - 1),
-                                 sz = (double)(e.y % 3 - 1);
-                    s_soff[k] = make_float4(
-                        __double2float_rn(__dsub_rn(__dadd_rn(cj[0], __dmul_rn(sx, p.g.L[0])), ci[0])),
-                        __double2float_rn(__dsub_rn(__dadd_rn(cj[1], __dmul_rn(sy, p.g.L[1])), ci[1])),
-                        __double2float_rn(__dsub_rn(__dadd_rn(cj[2], __dmul_rn(sz, p.g.L[2])), ci[2])),
-                        0.f);
-                    s_seg[k] = make_int4(r.x, r.y, k, e.y);
-                }
-                if (tid == 0) cs.nseg = ns;
-                gsync<G>();
-            } else {
-                const int r0 = ch * ROWCHUNK;
-                const int r1 = min(r0 + ROWCHUNK, p.nrows);
-                if (tid == 0) {
-                    int ns = 0;
-                    const int cell_end = T.gi.cell_start[B.cell + 1];
-                    if (T.is_auto && r0 == 0 && cell_end > B.start + B.count) {
-                        // rest of the own cell after this block (j > i for all)
-                        s_seg[0] = make_int4(B.start + B.count, cell_end - B.start - B.count, 0, 13);
-                        ns = 1;
-                    }
-                    cs.nseg = ns;
-                }
-                gsync<G>();
-                build_segments(p, T.gj, ax, ay, az, r0, r1, s_seg, &cs.nseg);
-                gsync<G>();
-            }
-            const int nseg = cs.nseg;
-            gsync<G>();                 // every thread has read nseg before it changes
-            if (nseg == 0) continue;
-            const int total = seg_scan<G>(s_seg, nseg, s_tmp);
-            // The chunk's j-points form ngt groups of JG; tile t holds the
-            // groups t, t + ntiles, t + 2 ntiles, ...: every tile mixes all rows
-            // of the chunk, so the warps (each pruning against its own i-box)
-            // get similar work per tile.
-            constexpr int GPT = TJ / JG;
-            const int ngt = (total + JG - 1) / JG;
-            const int ntiles = (ngt + GPT - 1) / GPT;
-            auto tile_groups = [&](int t) { return (ngt - t + ntiles - 1) / ntiles; };
-            if (tid == 0) cand_local += (unsigned long long)total * B.count;
-
-            // staging registers (TJ / NT slots per thread)
-            constexpr int SPT = TJ / NT;
-            float4 rq[SPT];
-            double rw[SPT];
-            float rwl[SPT];
-            int rcx[SPT], rmeta[SPT], rimg[SPT];
-            bool rv[SPT];
-            auto load_tile = [&](int t) {
+                    a0[0] = r.x; a1[0] = r.x + r.y; im[0] = e.y;
+                    meta = e.x;
+                    np = r.y > 0 ? 1 : 0;
+                    no = np ? ((a1[0] + 7) >> 3) - (a0[0] >> 3) : 0;
+                } else {
+                    const int4 sr = p.stencil[row];
+                    const int dy = sr.x, dz = sr.y;
+                    int y = ay + dy, z = az + dz, wy = 0, wz = 0;
+                    bool in = true;
+                    if (y < 0) { in = in && p.g.periodic; y += ny; wy = -1; }
+                    else if (y >= ny) { in = in && p.g.periodic; y -= ny; wy = 1; }
+                    if (z < 0) { in = in && p.g.periodic; z += nz; wz = -1; }
+                    else if (z >= nz) { in = in && p.g.periodic; z -= nz; wz = 1; }
+                    meta = (dy & 0xFFFF) | (dz << 16);
+                    const int rowbase = (z * ny + y) * nx;
+                    const int x0 = ax + sr.z, x1 = ax + sr.w;
 #pragma unroll
-                for (int s = 0; s < SPT; ++s) {
-                    const int slot = tid + s * NT;
-                    const int f = ((slot / JG) * ntiles + t) * JG + (slot % JG);
-                    rv[s] = f < total && slot / JG < tile_groups(t);
-                    if (rv[s]) {
-                        int4 sg = s_seg[seg_find(s_seg, nseg, f)];
-                        int pj = sg.x + (f - sg.y);
-                        rq[s] = T.gj.rel[pj];
-                        if constexpr (!TREE) rcx[s] = T.gj.cx[pj];
-                        rmeta[s] = sg.z;
-                        rimg[s] = sg.w;
-                        if (W == 1) rw[s] = T.gj.xw[pj].w;
-                        if (W == 3) rwl[s] = T.gj.wlo ? T.gj.wlo[pj] : 0.f;
-                    }
-                }
-            };
-            auto store_tile = [&](int t) {
-                const int buf = t & 1;
-                const int len = tile_groups(t) * JG;   // whole groups; missing points are pads
-#pragma unroll
-                for (int s = 0; s < SPT; ++s) {
-                    const int slot = tid + s * NT;
-                    float x = 1.0e18f, y = 1.0e18f, z = 1.0e18f;   // pad slot
-                    double wv = 0.0;
-                    if (rv[s]) {
-                        if constexpr (TREE) {
-                            const float4 o = s_soff[rmeta[s]];
-                            x = o.x + rq[s].x;
-                            y = o.y + rq[s].y;
-                            z = o.z + rq[s].z;
-                        } else {
-                            int wrapx = rimg[s] / 9 - 1;
-                            int dxc = rcx[s] - ax + wrapx * nx;
-                            int dyc = (int)(short)(rmeta[s] & 0xFFFF);
-                            int dzc = rmeta[s] >> 16;
-                            x = fmaf((float)dxc, c32x, rq[s].x);
-                            y = fmaf((float)dyc, c32y, rq[s].y);
-                            z = fmaf((float)dzc, c32z, rq[s].z);
+                    for (int q = 0; q < 3; ++q) {   // the part left of the box, inside, right of it
+                        int c0, c1;
+                        if (q == 0) { c0 = x0 + nx; c1 = min(x1, -1) + nx; }
+                        else if (q == 1) { c0 = max(x0, 0); c1 = min(x1, nx - 1); }
+                        else { c0 = max(x0, nx) - nx; c1 = x1 - nx; }
+                        const bool use = in && c0 <= c1 && (q == 1 || p.g.periodic) &&
+                                         (q != 0 || x0 < 0) && (q != 2 || x1 >= nx);
+                        a0[q] = a1[q] = 0;
+                        im[q] = q * 9 + (wy + 1) * 3 + (wz + 1);
+                        if (use) {
+                            a0[q] = T.gj.cell_start[rowbase + c0];
+                            a1[q] = T.gj.cell_start[rowbase + c1 + 1];
                         }
-                        wv = rw[s];
+                        if (a1[q] > a0[q]) {
+                            ++np;
+                            no += ((a1[q] + 7) >> 3) - (a0[q] >> 3);
+                        }
                     }
-                    if (slot < len) {
-                        s_tx[buf * TJ + slot] = x;
-                        s_ty[buf * TJ + slot] = y;
-                        s_tz[buf * TJ + slot] = z;
-                        if (W == 1) s_tw[buf * TJ + slot] = wv;
-                        if (W >= 2) s_twm[buf * TJ + slot] = rv[s] ? __float_as_uint(rq[s].w) : 0u;
-                        if (W == 3) s_twl[buf * TJ + slot] = rv[s] ? rwl[s] : 0.f;
-                    }
-                    // boxes of the j-groups (JG consecutive slots each)
-                    const GBox gb = lane_group_box(x, y, z, rv[s]);
-                    if ((tid & (JG - 1)) == 0) s_gbox[buf][slot / JG] = gb;
-                }
-            };
-
-            load_tile(0);
-            store_tile(0);
-            gsync<G>();
-            for (int t = 0; t < ntiles; ++t) {
-                const int buf = t & 1;
-                const int len = tile_groups(t) * JG;
-                if (t + 1 < ntiles) load_tile(t + 1);
-                wint_room(len);
-                const unsigned gm = group_mask(s_gbox[buf], s_ibox[tid >> 5], len / JG, t, ntiles,
-                                               total, ni_w, r2cut, &cs.pruned);
-                pair_tile<MODE, LOS, W, RI, LIN, false>(
-                    p, smem_hist,
-                    Tile{s_tx + buf * TJ, s_ty + buf * TJ, s_tz + buf * TJ, s_tw + buf * TJ,
-                         s_twm + buf * TJ, s_twl + buf * TJ},
-                    len, gm, I, bc, lc, r2cut, hist_sa, whist_sa, hk4, hbase, s_q, &cs.qn, s_seg,
-                    nseg, t, ntiles, B.start, task_bits);
-                since_flush += (unsigned long long)len * B.count;
-                if (t + 1 < ntiles) store_tile(t + 1);
-                // one decision for the whole CTA, taken at the barrier: read
-                // after it, the count could already include pushes of the next
-                // tile by a faster warp, and the drain holds barriers itself
-                if (gsync_or<G>(cs.qn >= LQ / 2))
-                    drain_rescue<MODE, LOS, G>(p, s_q, cs, &s_base);
-                if (since_flush > FLUSH_LIMIT / G) {
-                    flush_hist<G>(p, s_hist, s_whist, cur_hist, cur_wscale);
-                    since_flush = 0;
-                    wterms = 0;
                 }
             }
-            gsync<G>();
+            {
+                const int is = warp_incl_scan(np), io = warp_incl_scan(no);
+                int slot = nseg + is - np, o = noct + io - no;
+#pragma unroll
+                for (int q = 0; q < (TREE ? 1 : 3); ++q)
+                    if (np && a1[q] > a0[q]) {
+                        seg[slot] = make_int4(a0[q], a1[q], meta, im[q]);
+                        if (TREE) soff[slot] = tree_offset(p, B.cell, meta, im[q]);
+                        pref[slot] = o;
+                        o += ((a1[q] + 7) >> 3) - (a0[q] >> 3);
+                        ++slot;
+                    }
+                nseg += __shfl_sync(FULL, is, 31);
+                noct += __shfl_sync(FULL, io, 31);
+            }
+            __syncwarp();
+            const int nround = (noct + 31) / 32;
+            // this slice's rounds: global round number = part (mod S)
+            int rd = (part - round0 % S + S) % S;
+            round0 += nround;
+            int head = 0, tail = 0;
+            for (;;) {
+                // fill the ring: 32 octs a round, those whose box can reach the
+                // i-points' box.  Boxes are rounded outward, and r2prune carries
+                // the rounding of this test (host side), so a dropped pair is at
+                // least rcut apart
+                while (!own && tail - head < JO && rd < nround) {
+                    const int f = rd * 32 + lane;
+                    rd += S;
+                    bool keep = false;
+                    int lo = 0, p0 = 0;
+                    float g2 = 0.f;
+                    if (f < noct) {
+                        int hi = nseg;
+                        while (hi - lo > 1) {
+                            const int mid = (lo + hi) >> 1;
+                            if (pref[mid] <= f) lo = mid; else hi = mid;
+                        }
+                        const int4 sg = seg[lo];
+                        const int oct = (sg.x >> 3) + (f - pref[lo]);
+                        p0 = oct << 3;
+                        float4 bl = T.gj.obox[2 * (size_t)oct], bh = T.gj.obox[2 * (size_t)oct + 1];
+                        if (p.g.periodic) {
+                            const float sx = (float)(sg.w / 9 - 1) * p.L32[0];
+                            const float sy = (float)((sg.w / 3) % 3 - 1) * p.L32[1];
+                            const float sz = (float)(sg.w % 3 - 1) * p.L32[2];
+                            bl.x += sx; bl.y += sy; bl.z += sz;
+                            bh.x += sx; bh.y += sy; bh.z += sz;
+                        }
+                        const float gx = fmaxf(fmaxf(bl.x - bhx, blx - bh.x), 0.f);
+                        const float gy = fmaxf(fmaxf(bl.y - bhy, bly - bh.y), 0.f);
+                        const float gz = fmaxf(fmaxf(bl.z - bhz, blz - bh.z), 0.f);
+                        const float gq = fmaf(gy, gy, gx * gx);
+                        g2 = fmaf(gz, gz, gq);
+                        keep = g2 < p.r2prune;
+                        if (MODE == MODE_SIGPI && LOS == LOS_Z)   // the reach is a cylinder
+                            keep = keep && gq < p.q2prune && gz < p.zprune;
+                        const unsigned long long np2 =
+                            (unsigned long long)(min(sg.y, p0 + 8) - max(sg.x, p0)) * (unsigned)count;
+                        cand += np2;
+                        if (!keep) pruned += np2;
+                    }
+                    const unsigned who = __ballot_sync(FULL, keep);
+                    if (keep)
+                        ring[(tail + __popc(who & ((1u << lane) - 1u))) & (RING - 1)] =
+                            make_int4(p0, lo, __float_as_int(g2), 0);
+                    tail += __popc(who);
+                    __syncwarp();
+                }
+                // one batch: the block's own points, or up to eight octs
+                const int m = own ? (count + 7) >> 3 : min(JO, tail - head);
+                unsigned near = 0u;
+                unsigned band = 0u;
+                if (m > 0) {
+                    float g2 = INFINITY;
+#pragma unroll
+                    for (int h = 0; h < JB / 32; ++h) {
+                        const int sl = lane + 32 * h, oc = sl >> 3;
+                        float3 s = make_float3(far, 0.f, 0.f);
+                        float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+                        int pj = start + sl;
+                        bool v = own && sl < count;
+                        if (v) {
+                            q = T.gj.rel[pj];
+                            s = make_float3(q.x, q.y, q.z);
+                        } else if (!own && oc < m) {
+                            const int4 e = ring[(head + oc) & (RING - 1)];
+                            const int4 sg = seg[e.y];
+                            g2 = fminf(g2, __int_as_float(e.z));
+                            pj = e.x + (lane & 7);
+                            v = pj >= sg.x && pj < sg.y;
+                            if (v) {
+                                q = T.gj.rel[pj];
+                                if (TREE) {
+                                    const float4 o = soff[e.y];
+                                    s = make_float3(o.x + q.x, o.y + q.y, o.z + q.z);
+                                } else {
+                                    s = stage_grid(p, q, T.gj.cx[pj], ax, sg.z, sg.w);
+                                }
+                            }
+                        }
+                        if (PATH == PATH_FIX && !(fabsf(s.x) + fabsf(s.y) + fabsf(s.z) < 1e16f))
+                            s = make_float3(far, 0.f, 0.f);   // not a number: no pair
+                        tx[sl] = s.x; ty[sl] = s.y; tz[sl] = s.z;
+                        if (W == 1) tw[sl] = v ? T.gj.xw[pj].w : 0.0;
+                        if (W >= 2) twm[sl] = __float_as_uint(q.w);
+                        if (W == 3) twl[sl] = (v && T.gj.wlo) ? T.gj.wlo[pj] : 0u;
+                    }
+                    __syncwarp();
+                    const int nq = 2 * m;
+                    since += nq;
+                    if (since > flush_quads && PATH != PATH_GLOBAL) {
+                        flush_counts(p, 0, 0, 1, T.hist);
+                        if (SCAN && W >= 2) flush_weights(p, p.sm_whist, 0, 1, T.hist, T.wscale);
+                        since = nq;
+                    }
+                    if (W >= 2) {
+                        wterms += wper * (unsigned)nq;
+                        if (wterms > wlimit) {
+                            const bool full = !SCAN || most_counted(p) > wfull;
+                            if (SCAN && full) flush_counts(p, 0, 0, 1, T.hist);
+                            if (full) flush_weights(p, p.sm_whist, 0, 1, T.hist, T.wscale);
+                            wterms = wper * (unsigned)nq;
+                        }
+                    }
+                    if constexpr (PATH == PATH_FIX) {
+                        float cfm = p.f_cfp;
+                        unsigned tm2 = p.f_tp2;
+                        bool slow = own;
+                        if (MODE == MODE_SMU) {
+                            // the mu band at the batch's smallest separation
+                            g2 = own ? 0.f : __uint_as_float(__reduce_min_sync(FULL, __float_as_uint(g2)));
+                            slow = g2 < p.f_sf2;
+                            band = __float2uint_ru(fmaf(p.f_mA, rsqrt_fast(fmaxf(g2, p.f_sf2)), p.f_mB));
+                            cfm = fmaf((float)band, 1.0f / 65536.0f, 128.0f);
+                            tm2 = 2u * band;
+                        }
+                        if (slow)
+                            near = quads_fix<MODE, LOS, W, true>(p, tile, nq, I, smem, cfm, tm2,
+                                                                 own ? 0 : 2 * BI);
+                        else
+                            near = quads_fix<MODE, LOS, W, false>(p, tile, nq, I, smem, cfm, tm2, 0);
+                    } else {
+                        const size_t hbase = (size_t)T.hist * p.nbins;
+                        if (own)
+                            near = pair_quads<MODE, LOS, W, PATH, true>(p, tile, nq, I, c, smem, wbase, 0, hbase);
+                        else
+                            near = pair_quads<MODE, LOS, W, PATH, false>(p, tile, nq, I, c, smem, wbase, 0, hbase);
+                    }
+                }
+                // queue the near quads, check them 32 at a time (and, before the
+                // segments change, the rest)
+                const bool last = rd >= nround && (own ? tail == head && nround == 0 : tail - head == m);
+                for (;;) {
+                    const unsigned who = __ballot_sync(FULL, near != 0u);
+                    if (near) {
+                        const int q = __ffs(near) - 1;
+                        near &= near - 1;
+                        uint2 e = make_uint2((unsigned)(start + 4 * q), (unsigned)lane | 32u | band << 13);
+                        if (!own) {
+                            const int4 o = ring[(head + (q >> 1)) & (RING - 1)];
+                            e = make_uint2((unsigned)(o.x + 4 * (q & 1)),
+                                           (unsigned)lane | (unsigned)o.y << 6 | band << 13);
+                        }
+                        queue[qn + __popc(who & ((1u << lane) - 1u))] = e;
+                    }
+                    qn += __popc(who);
+                    const bool rest = last && !__any_sync(FULL, near != 0u);
+                    if (qn >= 32 || (rest && qn > 0)) {
+                        const int n = min(qn, 32);
+                        __syncwarp();
+                        check_near<MODE, LOS, W, PATH, TREE>(p, queue, seg, n, B.task, B.cell, start, count, copy,
+                                                             s_lut);
+                        __syncwarp();
+                        qn -= n;
+                        uint2 e = make_uint2(0u, 0u);
+                        if (lane < qn) e = queue[n + lane];
+                        __syncwarp();
+                        if (lane < qn) queue[lane] = e;
+                    }
+                    __syncwarp();
+                    if (who == 0u && qn < 32 && !(last && qn > 0)) break;
+                }
+                if (!own) head += m;
+                own = false;
+                if (last) break;
+            }
         }
-        drain_rescue<MODE, LOS, G>(p, s_q, cs, &s_base);
-        gsync<G>();
     }
-    drain_rescue<MODE, LOS, G>(p, s_q, cs, &s_base);
-    flush_hist<G>(p, s_hist, s_whist, cur_hist, cur_wscale);
-    if (tid == 0 && cand_local) atomicAdd(&p.counters[0], cand_local);
-    if (tid == 0 && cs.pruned) atomicAdd(&p.counters[3], cs.pruned);
+    __syncthreads();
+    if (!p.multi) {   // batches have flushed after their last range
+        const double wscale = p.tasks[0].wscale;
+        if (PATH != PATH_GLOBAL) {
+            flush_counts(p, 0, warp, nw, 0);
+            if (W) flush_weights(p, p.sm_whist, warp, nw, 0, wscale);
+        }
+        if (W >= 2 && p.wfold) {
+            __syncthreads();
+            flush_folded(p, 0, wscale);
+        }
+    }
+    cand = warp_sum_u64(cand);
+    pruned = warp_sum_u64(pruned);
+    if (lane == 0 && cand) atomicAdd(&p.counters[0], cand);
+    if (lane == 0 && pruned) atomicAdd(&p.counters[3], pruned);
+}
+
+// ---------------------------------------------------------------------------
+// FP64 kernel: j-segments of a CTA
+// ---------------------------------------------------------------------------
+// Exclusive prefix over the segment lengths held in seg[k].y (in place);
+// returns the total.  All NT threads call it.
+__device__ __forceinline__ int seg_scan(int4 *seg, int nseg, int *s_tmp) {
+    // each thread owns a contiguous run of ceil(nseg / NT) segments
+    const int tid = threadIdx.x;
+    const int per = (nseg + NT - 1) / NT;
+    int b0 = tid * per, b1 = min(b0 + per, nseg);
+    int local = 0;
+    for (int k = b0; k < b1; ++k) local += seg[k].y;
+    // block-wide exclusive scan of `local` (NT = 128: 4 warps)
+    int lane = tid & 31, warp = tid >> 5;
+    int v = local;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        int t = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += t;
+    }
+    if (lane == 31) s_tmp[warp] = v;
+    __syncthreads();
+    int wbase = 0;
+    for (int w = 0; w < warp; ++w) wbase += s_tmp[w];
+    int total = s_tmp[0] + s_tmp[1] + s_tmp[2] + s_tmp[3];
+    int run = wbase + v - local;
+    for (int k = b0; k < b1; ++k) {
+        int len = seg[k].y;
+        seg[k].y = run;
+        run += len;
+    }
+    __syncthreads();
+    return total;
+}
+
+// Segment holding flat position f: largest k with seg[k].y <= f.
+__device__ __forceinline__ int seg_find(const int4 *seg, int nseg, int f) {
+    int lo = 0, hi = nseg;
+    while (hi - lo > 1) {
+        int mid = (lo + hi) >> 1;
+        if (seg[mid].y <= f) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
+// Build the j-segments of stencil rows [r0, r1) for the i-cell (ax, ay, az).
+// seg = {first point, length, dy | dz << 16, image code}.
+__device__ __forceinline__ void build_segments(const PairParams &p, const GridDev &gj, int ax,
+                                               int ay, int az, int r0, int r1, int4 *seg,
+                                               int *s_nseg) {
+    const int nx = p.g.ng[0], ny = p.g.ng[1], nz = p.g.ng[2];
+    for (int row = r0 + (int)threadIdx.x; row < r1; row += NT) {
+        int4 st = p.stencil[row];
+        int dy = st.x, dz = st.y;
+        int y = ay + dy, z = az + dz, wy = 0, wz = 0;
+        if (y < 0) { if (!p.g.periodic) continue; y += ny; wy = -1; }
+        else if (y >= ny) { if (!p.g.periodic) continue; y -= ny; wy = 1; }
+        if (z < 0) { if (!p.g.periodic) continue; z += nz; wz = -1; }
+        else if (z >= nz) { if (!p.g.periodic) continue; z -= nz; wz = 1; }
+        const int rowbase = (z * ny + y) * nx;
+        const int x0 = ax + st.z, x1 = ax + st.w;
+        int pc0[3], pc1[3], pw[3], np = 0;
+        if (p.g.periodic) {
+            if (x0 < 0) { pc0[np] = x0 + nx; pc1[np] = min(x1, -1) + nx; pw[np++] = -1; }
+            int m0 = max(x0, 0), m1 = min(x1, nx - 1);
+            if (m0 <= m1) { pc0[np] = m0; pc1[np] = m1; pw[np++] = 0; }
+            if (x1 >= nx) { pc0[np] = max(x0, nx) - nx; pc1[np] = x1 - nx; pw[np++] = 1; }
+        } else {
+            int m0 = max(x0, 0), m1 = min(x1, nx - 1);
+            if (m0 <= m1) { pc0[np] = m0; pc1[np] = m1; pw[np++] = 0; }
+        }
+        const int meta = (dy & 0xFFFF) | (dz << 16);
+        for (int q = 0; q < np; ++q) {
+            int a0 = gj.cell_start[rowbase + pc0[q]];
+            int a1 = gj.cell_start[rowbase + pc1[q] + 1];
+            if (a1 > a0) {
+                int slot = atomicAdd(s_nseg, 1);
+                seg[slot] = make_int4(a0, a1 - a0, meta, (pw[q] + 1) * 9 + (wy + 1) * 3 + (wz + 1));
+            }
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1516,10 +1680,9 @@ __global__ void __launch_bounds__(NT * G, (G > 1 ? 1 : (RI <= 2 ? 5 : 4)))
 template <int MODE, int LOS, bool W>
 __global__ void __launch_bounds__(NT) k_pairs_f64(const __grid_constant__ PairParams p) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ CtaShared cs;
-    __shared__ int s_tmp[8];
+    __shared__ int s_blk, s_nseg, s_tmp[8];
 
-    const SmemLayout Ly = smem_layout(p, true);
+    const SmemLayout64 Ly = f64_layout(p);
     double *s_Ea = (double *)(smem + Ly.ea);
     double *s_Eb = (double *)(smem + Ly.eb);
     int *s_hist = (int *)(smem + Ly.hist);
@@ -1532,28 +1695,35 @@ __global__ void __launch_bounds__(NT) k_pairs_f64(const __grid_constant__ PairPa
     for (int k = tid; k <= p.n_a; k += NT) s_Ea[k] = p.Ea[k];
     for (int k = tid; k <= p.n_b; k += NT) s_Eb[k] = p.Eb[k];
     if (p.smem_hist_ok) {
-        const int copies = (p.priv ? NT / 32 : 1) * p.hist_k;
-        for (int k = tid; k < p.nbins_smem * copies; k += NT) s_hist[k] = 0;
-        if (W) for (int k = tid; k < p.nbins_smem * p.hist_k; k += NT) s_whist[k] = 0.0;
+        for (int k = tid; k < p.nent * p.hist_k; k += NT) s_hist[k] = 0;
+        if (W) for (int k = tid; k < p.nent * p.hist_k; k += NT) s_whist[k] = 0.0;
     }
     const int K = p.hist_k, lane_copy = tid & (K - 1);
-    int *my_hist = s_hist + (p.priv ? (tid >> 5) * p.nbins_smem * K : 0) + lane_copy;
+    int *my_hist = s_hist + lane_copy;
     double *my_whist = s_whist + lane_copy;
     const int nx = p.g.ng[0], ny = p.g.ng[1];
     const int nblocks = *p.nblocks;
     unsigned long long cand_local = 0, since_flush = 0;
     int cur_hist = -1;
+    auto flush_cta = [&](int h) {
+        __syncthreads();
+        if (p.smem_hist_ok && h >= 0) {
+            flush_counts(p, (int)Ly.hist, tid >> 5, NT / 32, h);
+            if (W) flush_weights(p, (int)Ly.whist, tid >> 5, NT / 32, h, 0.0);
+        }
+        __syncthreads();
+    };
     __syncthreads();
 
     for (;;) {
-        if (tid == 0) cs.blk = atomicAdd(p.work_counter, 1);   // the list holds only this shard's blocks
+        if (tid == 0) s_blk = atomicAdd(p.work_counter, 1);   // the list holds only this shard's blocks
         __syncthreads();
-        const int bidx = cs.blk;
+        const int bidx = s_blk;
         if (bidx >= nblocks) break;
         const Block B = p.blocks[bidx];
         const TaskDev &T = p.tasks[B.task];
         if (T.hist != cur_hist) {
-            flush_hist(p, s_hist, s_whist, cur_hist);
+            flush_cta(cur_hist);
             cur_hist = T.hist;
             since_flush = 0;
         }
@@ -1599,12 +1769,12 @@ __global__ void __launch_bounds__(NT) k_pairs_f64(const __grid_constant__ PairPa
                     s_seg[0] = make_int4(B.start + B.count, cell_end - B.start - B.count, 0, 13);
                     ns = 1;
                 }
-                cs.nseg = ns;
+                s_nseg = ns;
             }
             __syncthreads();
-            build_segments(p, T.gj, ax, ay, az, r0, r1, s_seg, &cs.nseg);
+            build_segments(p, T.gj, ax, ay, az, r0, r1, s_seg, &s_nseg);
             __syncthreads();
-            const int nseg = cs.nseg;
+            const int nseg = s_nseg;
             __syncthreads();                 // every thread has read nseg before it changes
             if (nseg == 0) continue;
             const int total = seg_scan(s_seg, nseg, s_tmp);
@@ -1624,14 +1794,14 @@ __global__ void __launch_bounds__(NT) k_pairs_f64(const __grid_constant__ PairPa
                 since_flush += (unsigned long long)len * B.count;
                 __syncthreads();
                 if (since_flush > FLUSH_LIMIT) {
-                    flush_hist(p, s_hist, s_whist, cur_hist);
+                    flush_cta(cur_hist);
                     since_flush = 0;
                 }
             }
         }
         __syncthreads();
     }
-    flush_hist(p, s_hist, s_whist, cur_hist);
+    flush_cta(cur_hist);
     if (tid == 0 && cand_local) atomicAdd(&p.counters[0], cand_local);
 }
 
@@ -1663,90 +1833,53 @@ __global__ void __launch_bounds__(256) k_rescue(const __grid_constant__ PairPara
 template <int MODE, int LOS>
 using PairKernel = void (*)(PairParams);
 
-// Kernel variant for (weighted, i-points per thread, linear bins).  Linear
-// bins are specialised only where they apply: s, and (s, mu) along z.
-template <int MODE, int LOS>
-PairKernel<MODE, LOS> pick_f32(const PairParams &p, int ipt) {
-    constexpr bool LINOK = (MODE == MODE_S) || (MODE == MODE_SMU && LOS == LOS_Z) || MODE == MODE_SIGPI;
-    const bool lin = LINOK && p.lin;
-    if constexpr (LINOK) {
-        // several thread groups per CTA (large histograms): floor bins, 2 i-points
-        if (p.groups > 1 && lin && !p.wint)
-            return p.weighted ? k_pairs_f32<MODE, LOS, 1, 2, true, 4> : k_pairs_f32<MODE, LOS, 0, 2, true, 4>;
+template <int MODE, int LOS, int PATH, bool TREE>
+PairKernel<MODE, LOS> pick_w(const PairParams &p) {
+    if (!p.weighted) return k_pairs_f32<MODE, LOS, 0, PATH, TREE>;
+    if constexpr (PATH == PATH_FIX)   // integer weight products only
+        return p.wcorr ? k_pairs_f32<MODE, LOS, 3, PATH, TREE> : k_pairs_f32<MODE, LOS, 2, PATH, TREE>;
+    else {
+    if constexpr (PATH != PATH_LUT && PATH != PATH_GLOBAL) {
+        if (p.wint && p.wcorr) return k_pairs_f32<MODE, LOS, 3, PATH, TREE>;
+        if (p.wint) return k_pairs_f32<MODE, LOS, 2, PATH, TREE>;
     }
-    if (p.weighted) {
-        if constexpr (LINOK) {
-            if (lin && p.wint && p.wcorr) return ipt == 4 ? k_pairs_f32<MODE, LOS, 3, 4, true>
-                                                          : k_pairs_f32<MODE, LOS, 3, 2, true>;
-            if (lin && p.wint) return ipt == 4 ? k_pairs_f32<MODE, LOS, 2, 4, true>
-                                               : k_pairs_f32<MODE, LOS, 2, 2, true>;
-        }
-        if (ipt == 4) return lin ? k_pairs_f32<MODE, LOS, 1, 4, LINOK> : k_pairs_f32<MODE, LOS, 1, 4, false>;
-        return lin ? k_pairs_f32<MODE, LOS, 1, 2, LINOK> : k_pairs_f32<MODE, LOS, 1, 2, false>;
+    return k_pairs_f32<MODE, LOS, 1, PATH, TREE>;
     }
-    if (ipt == 4) return lin ? k_pairs_f32<MODE, LOS, 0, 4, LINOK> : k_pairs_f32<MODE, LOS, 0, 4, false>;
-    return lin ? k_pairs_f32<MODE, LOS, 0, 2, LINOK> : k_pairs_f32<MODE, LOS, 0, 2, false>;
 }
 
-// Tree variant (one thread group) for RI i-points per thread.
-template <int MODE, int LOS, int RI>
-PairKernel<MODE, LOS> pick_f32_tree_ri(const PairParams &p) {
-    constexpr bool LINOK = (MODE == MODE_S) || (MODE == MODE_SMU && LOS == LOS_Z) || MODE == MODE_SIGPI;
-    const bool lin = LINOK && p.lin;
-    if (p.weighted) {
-        if constexpr (LINOK) {
-            if (lin && p.wint && p.wcorr) return k_pairs_f32<MODE, LOS, 3, RI, true, 1, true>;
-            if (lin && p.wint) return k_pairs_f32<MODE, LOS, 2, RI, true, 1, true>;
-        }
-        return lin ? k_pairs_f32<MODE, LOS, 1, RI, LINOK, 1, true> : k_pairs_f32<MODE, LOS, 1, RI, false, 1, true>;
+// Kernel variant for the weights and the way the bins are found; (sigma, pi)
+// floors exist for edges from zero only.
+template <int MODE, int LOS, bool TREE>
+PairKernel<MODE, LOS> pick_f32(const PairParams &p) {
+    if (!p.smem_hist_ok) return pick_w<MODE, LOS, PATH_GLOBAL, TREE>(p);
+    if constexpr (MODE != MODE_SIGPI) {
+        if (p.path == PATH_LINOFF) return pick_w<MODE, LOS, PATH_LINOFF, TREE>(p);
+        if (p.path == PATH_LOG) return pick_w<MODE, LOS, PATH_LOG, TREE>(p);
     }
-    return lin ? k_pairs_f32<MODE, LOS, 0, RI, LINOK, 1, true> : k_pairs_f32<MODE, LOS, 0, RI, false, 1, true>;
+    if (p.path == PATH_FIX) return pick_w<MODE, LOS, PATH_FIX, TREE>(p);
+    if (p.path == PATH_LIN) return pick_w<MODE, LOS, PATH_LIN, TREE>(p);
+    return pick_w<MODE, LOS, PATH_LUT, TREE>(p);
 }
 
-template <int MODE, int LOS>
-PairKernel<MODE, LOS> pick_f32_tree(const PairParams &p, int ipt) {
-    return ipt == 4 ? pick_f32_tree_ri<MODE, LOS, 4>(p) : pick_f32_tree_ri<MODE, LOS, 2>(p);
-}
-
-template <int MODE, int LOS>
-cudaError_t launch_kernel_f32(PairKernel<MODE, LOS> k, const PairParams &p, int grid, size_t smem,
-                              cudaStream_t st) {
+template <int MODE, int LOS, bool TREE>
+cudaError_t launch_mode_f32(const PairParams &p, int grid, size_t smem, cudaStream_t st) {
+    PairKernel<MODE, LOS> k = pick_f32<MODE, LOS, TREE>(p);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     if (grid <= 0) return cudaSuccess;
-    k<<<grid, NT * p.groups, smem, st>>>(p);
+    k<<<grid, 32 * p.nwarps, smem, st>>>(p);
     note_launch();
     return cudaGetLastError();
 }
 
-template <int MODE, int LOS>
-int occupancy_kernel_f32(PairKernel<MODE, LOS> k, const PairParams &p, size_t smem) {
+template <int MODE, int LOS, bool TREE>
+int occupancy_mode_f32(const PairParams &p, size_t smem) {
+    PairKernel<MODE, LOS> k = pick_f32<MODE, LOS, TREE>(p);
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return 0;
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, NT * p.groups, smem) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, 32 * p.nwarps, smem) != cudaSuccess) return 0;
     return nb;
-}
-
-template <int MODE, int LOS>
-cudaError_t launch_mode_f32(const PairParams &p, int ipt, int grid, size_t smem, cudaStream_t st) {
-    return launch_kernel_f32<MODE, LOS>(pick_f32<MODE, LOS>(p, ipt), p, grid, smem, st);
-}
-
-template <int MODE, int LOS>
-int occupancy_mode_f32(const PairParams &p, int ipt, size_t smem) {
-    return occupancy_kernel_f32<MODE, LOS>(pick_f32<MODE, LOS>(p, ipt), p, smem);
-}
-
-template <int MODE, int LOS>
-cudaError_t launch_mode_f32_tree(const PairParams &p, int ipt, int grid, size_t smem,
-                                 cudaStream_t st) {
-    return launch_kernel_f32<MODE, LOS>(pick_f32_tree<MODE, LOS>(p, ipt), p, grid, smem, st);
-}
-
-template <int MODE, int LOS>
-int occupancy_mode_f32_tree(const PairParams &p, int ipt, size_t smem) {
-    return occupancy_kernel_f32<MODE, LOS>(pick_f32_tree<MODE, LOS>(p, ipt), p, smem);
 }
 
 template <int MODE, int LOS>

@@ -20,15 +20,17 @@ struct pc_grid {
     // integer weight path: every weight a non-negative normal binary32 value or
     // zero (wint), with biased exponents in [wemin, wemax]; the FP32 records
     // then carry the packed weights.  Binary64 weights take it through their
-    // binary32 rounding hi (exponents as above) and remainder (wcorr, wlo)
+    // binary32 rounding's exponents (as above), with the bits past the packed
+    // 32 in wlo (wcorr)
     int wint = 0, wemax = 0, wemin = 0;
     int wcorr = 0;
-    float *wlo = nullptr;       // cell order: remainders (GridDev::wlo), or null
+    unsigned *wlo = nullptr;       // cell order: remainders (GridDev::wlo), or null
     float4 *rel;
     uint16_t *cx;
     double4_32a *xw;
     int *cell_start;
     int *perm;
+    float4 *obox;               // box of every eight points (GridDev::obox, origin g.lo)
 };
 
 // k-d tree of Alg. 1 (tree.cu).  Nodes in heap order: slot 0 is the root,
@@ -49,11 +51,12 @@ struct pc_tree {
     double r2min = 0.0;         // non-periodic: lower bound of min |x|^2
     int wint = 0, wemax = 0, wemin = 0;   // as pc_grid
     int wcorr = 0;
-    float *wlo = nullptr;       // tree order: as pc_grid
+    unsigned *wlo = nullptr;       // tree order: as pc_grid
     double bext = 0.0;          // largest extent (any axis) of a list node's box
     float4 *rel;                // tree order: FP32 offset from the list node's centre, .w packed weight
     double4_32a *xw;            // tree order: FP64 canonical coordinates, weight
     int *perm;                  // tree position -> input index
+    float4 *obox;               // box of every eight points (GridDev::obox, origin g.lo)
     int2 *vnode;                // every slot's range by the halving rule
     int2 *node;                 // {start, count} of present slots; count -1: empty slot
     double *nbox;               // lo[3], hi[3] per slot (present slots)
@@ -160,6 +163,12 @@ cudaError_t scan_exclusive_into(const int *in, int *out, int n, int *tot, cudaSt
 cudaError_t make_blocks_into(const TaskDev *tasks_dev, int ntasks, int ncell, int bi,
                              int shard_index, int shard_count, Block *blocks, int *nblocks_dev,
                              int *tmp_counts, int *tmp_offsets, int *tmp_tot, cudaStream_t st);
+
+// Bounding boxes of every eight consecutive points (GridDev::obox): 2 float4
+// per oct, ceil(n / 8) octs.
+cudaError_t make_obox(const double4_32a *xw, int n, const double org[3], float4 *obox,
+                      cudaStream_t st);
+inline size_t obox_bytes(long long n) { return sizeof(float4) * 2 * (size_t)((n + 7) / 8); }
 
 // Forget cached count graphs that use grid g (the grid is being freed).
 void forget_grid(const pc_grid *g);

@@ -13,15 +13,11 @@ namespace pc {
 // ---------------------------------------------------------------------------
 // launch geometry of the pair kernels
 // ---------------------------------------------------------------------------
-constexpr int NT = 128;        // threads per CTA (per thread group with grouped CTAs)
-constexpr int TJ = 512;        // j points per shared-memory tile (FP32 path)
+constexpr int NT = 128;        // threads per CTA (FP64 path); blocks hold NT * ipt points
 constexpr int TJ64 = 128;      // j points per tile (FP64 path)
-constexpr int MAXSEG = 256;    // j segments per chunk of stencil rows
-constexpr int MAXSEG_T = 128;  // j segments per chunk of a tree list (nodes of 129+ points;
-                               // segments and their offsets fit the grid's segment space)
+constexpr int MAXSEG = 256;    // j segments per chunk of stencil rows (FP64 path)
 constexpr int ROWCHUNK = 84;   // stencil rows per chunk (<= 3 segments each)
 static_assert(3 * ROWCHUNK + 1 <= MAXSEG, "a chunk's segments (and the own-cell rest) fit");
-constexpr int LQ = 192;        // rescue staging slots per CTA (per thread group)
 constexpr int MAX_LUT = 8192;  // LUT entries per histogram axis
 // integer weight path: largest exponent range of one catalogue's weights
 // (the packed significand M << range fits 32 bits), and of two catalogues'
@@ -31,14 +27,17 @@ constexpr int WINT_MAX_SPAN = 12;
 
 enum { MODE_S = 0, MODE_SMU = 1, MODE_SIGPI = 2 };
 
-// Remainder of a binary64 weight past its binary32 rounding hi, scaled for the
-// pair kernel's correction: fl32(w - hi) 2^(142 - emax), emax the largest
-// biased exponent of the catalogue's his (w - hi is exact in binary64, and
-// the scaled value stays below 2^-8 in magnitude).
-__device__ __forceinline__ float weight_lo(double wv, int emax) {
-    const float hi = __double2float_rn(wv);
-    const float lo = __double2float_rn(__dsub_rn(wv, (double)hi));
-    return __double2float_rn(__dmul_rn((double)lo, ldexp(1.0, 142 - emax)));
+// Packed integer weight: w 2^(158 - emax), emax the largest biased binary32
+// exponent of the catalogue's weights' binary32 roundings (exponents spanning at
+// most 8 binades), as 32 bits, and the next 31.  A binary32 value w = M 2^(e -
+// 150) gives M 2^(8 - (emax - e)) exactly, and a pair's exact 64-bit product is
+// M_i M_j 2^(16 - k_i - k_j), k = emax - e.
+__device__ __forceinline__ unsigned weight_hi(double w, int emax) {
+    return __double2uint_rz(ldexp(w, 158 - emax));
+}
+__device__ __forceinline__ unsigned weight_lo(double w, int emax) {
+    const double s = ldexp(w, 158 - emax);
+    return __double2uint_rz((s - (double)__double2uint_rz(s)) * 2147483648.0);
 }
 enum { LOS_Z = 0, LOS_MID = 1 };
 
@@ -50,11 +49,14 @@ struct GridDev {
     const double4_32a *xw;       // FP64 canonical coordinates, .w = weight (1 if none)
     const int *cell_start;   // ncell + 1
     int n;
-    // integer weight path with binary64 weights: per point the binary32
-    // remainder lo = fl32(w - hi) of its weight (hi = fl32(w), the packed
-    // weight) times 2^(142 - e_max), e_max the grid's largest hi exponent;
-    // null when every weight is a binary32 value
-    const float *wlo;
+    // integer weight path with binary64 weights: per point the 31 bits that
+    // follow the packed weight's (weight_lo); null when every weight is a
+    // binary32 value
+    const unsigned *wlo;
+    // bounding box of every run of eight points (an oct), relative to org and
+    // rounded outward: {lo x, y, z, 0}, {hi x, y, z, 0}
+    const float4 *obox;
+    double org[3];
 };
 
 // One counting task: blocks of i-points of gi against the stencil of gj,
@@ -115,31 +117,48 @@ struct PairParams {
     unsigned long long *counters;  // [0] candidates, [1] inline rescues
     int shard_index, shard_count;   // the block list holds only the cells (tree: list nodes)
                                     // whose index % shard_count == shard_index
-    int groups = 1;          // FP32 kernel: independent groups of NT threads per CTA sharing
-                             // one shared histogram (large histograms)
-    int priv;                // 0: one histogram per CTA; 1: one per warp
     int hist_k = 1;          // lane copies of the shared histograms (power of 2, <= 32):
                              // lane l updates copy l % hist_k, stored [bin][copy]
     int smem_hist_ok;        // histogram fits in shared memory
-    // evenly spaced s (and mu) edges: bins by floor instead of tables
-    int lin;
-    float lin_invA, lin_offA;    // t_s = s * lin_invA + lin_offA, bin = floor(t_s)
-    float lin_thrA;              // not near an edge iff |frac(t_s) - 1/2| < lin_thrA
-    float lin_nB;                // t_mu = mu * lin_nB
-    float lin_mA, lin_cB;        // not near iff |frac(t_mu) - 1/2| < lin_cB - lin_mA / s
-    // lin with e_0 = 0 and every candidate below n_a + 1 bin widths: t_s >= 0,
-    // floor(t_s) <= n_a, so the s-range test is replaced by one discarded row
-    // (row n_a) of the shared histogram
-    int lin_norange;
-    // lin with logarithmic s edges: t_s = lin_invA log2(s^2) + lin_offA, and the
-    // s band grows as 1/s: not near iff |frac(t_s) - 1/2| < lin_thrA - lin_mS / s
-    int lin_log;
-    float lin_mS;
-    // lin for (sigma, pi) bins (both axes evenly spaced from 0): t_sigma =
-    // sigma lin_invA, t_pi = pi lin_invB2, not near iff |frac - 1/2| is below
-    // lin_thrA and lin_thrB
+    // FP32 path: how the bins are found (PATH_* of the pair kernel), and the
+    // floor paths' constants: t_s = s lin_invA + lin_offA (logarithmic s: t_s =
+    // lin_invA log2(s^2) + lin_offA), bin = floor(t_s), not near an edge iff
+    // |frac(t_s) - 1/2| < lin_thrA (- lin_mS / s for logarithmic s); with an
+    // offset lin_offA carries + 1.  t_mu = mu lin_nB, not near iff |frac(t_mu) -
+    // 1/2| < lin_cB - lin_mA / s.  (sigma, pi): t_pi = pi lin_invB2, lin_thrB
+    int path;
+    float lin_invA, lin_offA, lin_thrA, lin_mS;
+    float lin_nB, lin_mA, lin_cB;
     float lin_invB2, lin_thrB;
-    int nbins_smem;              // bins per shared copy: nbins, plus n_b with lin_norange
+    // the floor paths' constants as pairs (both lanes equal), so that the packed
+    // instructions can take them from the constant bank: 2^23, 2^23 - 1/2, -1,
+    // the scales and offset, minus the band terms per 1/s, the second axis's
+    // threshold, minus the bytes of a row and of a column
+    float2 c_23, c_p, c_m1, c_invA, c_offA, c_thrA, c_nmS, c_invB, c_nmB, c_cB, c_nrow, c_ncol;
+    float c_kA;              // counter address constant without the lane copy
+    // fixed-point floors (PATH_FIX, see the kernel): 1e-30; 128 + band of the
+    // first axis and (sigma, pi) of the second; the clamps; twice the bands in
+    // units of 2^-16; t below which a pair is always near, its separation
+    // squared; mu band in units, f_mA / s + f_mB
+    float2 f_tiny, f_cfs;
+    float f_cfp, f_lim, f_limB, f_close, f_sf2, f_mA, f_mB;
+    unsigned f_ts2, f_tp2;
+    unsigned f_coef;         // weighted LAY_ROWS: bytes {hist_k, hs hist_k} (entry from the two bins)
+    int fix;                 // the plan allows PATH_FIX
+    int layout;              // of the shared histogram (LAY_*)
+    float L32[3];            // periodic box sides (0: none)
+    // shared histogram: entry (a, b) = a hs + b, the columns n_b .. hs - 1 and
+    // the last entry n_a hs discarded; nent = n_a hs + 1
+    int hs, nent;
+    // layout of a CTA (bytes): weight sums, tables, the warps' slices
+    int sm_whist, sm_lut, sm_warp, nwarps;
+    // box tests: squared distance from which an oct is dropped, and for
+    // (sigma, pi) along z the cylinder's squared radius and half length, all
+    // with the tests' rounding added; far: coordinate of absent points
+    float r2prune, q2prune, zprune, far;
+    int nsub;                // 64-point parts a block may have
+    int multi;               // several histograms (batches)
+    long long npts_i;        // i-points of all tasks
     // weighted sums from exact integer products of the packed binary32 weights
     // (significand product shifted by both exponent offsets, below 2^48),
     // accumulated as three 16-bit pieces in a record of three u32 sums per bin
@@ -147,9 +166,8 @@ struct PairParams {
     // the task's wscale
     int wint;
     // integer weight path with binary64 weights (some grid carries wlo): each
-    // pair's product gains the binary32 correction hi_i lo_j + lo_i hi_j,
-    // rounded to the accumulators' unit, and the product is rounded instead
-    // of truncated
+    // pair's product gains the cross terms of the next 31 bits and is rounded
+    // to the accumulators' unit instead of truncated
     int wcorr;
     // integer weights with fewer than 16 lane copies (large histograms): each
     // copy reaches its product limit often, so the records are folded into
@@ -157,11 +175,6 @@ struct PairParams {
     // bin, low word first: gridDim x nbins x 2) instead of being flushed
     int wfold;
     unsigned long long *wfold_buf;
-    int wint_k;              // lane copies of the integer weight records: hist_k
-    // shared-histogram row that lanes without an in-range pair update (the
-    // floor-bin kernels issue every reduction with the full warp); the flush
-    // discards it like every row past nbins
-    int trash_row;
     // k-d tree path (Alg. 3): each i-block (a tree node at the block level)
     // pairs with the j-blocks listed for it by the dual-tree traversal
     int tree;
@@ -212,13 +225,13 @@ inline cudaError_t alloc_host(T **p, size_t bytes) {
 // ---------------------------------------------------------------------------
 // launchers implemented in the kernel translation units
 // ---------------------------------------------------------------------------
-cudaError_t launch_pairs_f32(const PairParams &p, int ipt, int grid, size_t smem,
-                             cudaStream_t st);   // p.tree selects the tree variant
 cudaError_t launch_pairs_f64(const PairParams &p, int grid, size_t smem, cudaStream_t st);
 cudaError_t launch_rescue(const PairParams &p, cudaStream_t st);
-size_t pairs_f32_smem(const PairParams &p, int ipt);
+cudaError_t launch_pairs_f32(const PairParams &p, int grid, size_t smem,
+                             cudaStream_t st);   // p.tree selects the tree variant
+size_t pairs_f32_smem(PairParams &p, int nwarps);   // fills in p's layout
 size_t pairs_f64_smem(const PairParams &p);
-int pairs_f32_ctas_per_sm(const PairParams &p, int ipt, size_t smem);
+int pairs_f32_ctas_per_sm(const PairParams &p, size_t smem);
 int pairs_f64_ctas_per_sm(const PairParams &p, size_t smem);
 
 // ---------------------------------------------------------------------------

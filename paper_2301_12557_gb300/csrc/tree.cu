@@ -508,23 +508,14 @@ __global__ void k_block_info(const double *__restrict__ box, const int2 *__restr
     atomicMax(ext_key, okey(e));
 }
 
-// Packed integer weight: the significand with its leading one shifted up by
-// 8 - (emax - e) (exponents within 8 binades), as on the grid path.
-__device__ __forceinline__ unsigned pack_weight_t(double wv, int emax, int span) {
-    const unsigned b = __float_as_uint(__double2float_rn(wv));
-    const int e = (int)((b >> 23) & 0xFF);
-    if (e == 0) return 0u;
-    return ((b & 0x7FFFFFu) | 0x800000u) << (span - (emax - e));
-}
-
 // Point records in tree order: FP32 offset from the list node's centre (.w the
 // packed integer weight or 0), FP64 canonical coordinates and weight.
 __global__ void k_tree_scatter(const double *__restrict__ x, const void *__restrict__ w, int w_is_f32,
-                               int wpack_emax, int wpack_span, const unsigned *__restrict__ perm,
+                               int wpack_emax, const unsigned *__restrict__ perm,
                                const int *__restrict__ bid, const double *__restrict__ cen, int n,
                                float4 *__restrict__ rel, double4_32a *__restrict__ xw,
                                int *__restrict__ perm_out, unsigned pbase = 0u,
-                               float *__restrict__ wlo = nullptr) {
+                               unsigned *__restrict__ wlo = nullptr) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const unsigned p = perm[i];
@@ -537,7 +528,7 @@ __global__ void k_tree_scatter(const double *__restrict__ x, const void *__restr
     }
     double wv = 1.0;
     if (w) wv = w_is_f32 ? (double)((const float *)w)[p] : ((const double *)w)[p];
-    const unsigned wp = (w && wpack_emax > 0) ? pack_weight_t(wv, wpack_emax, wpack_span) : 0u;
+    const unsigned wp = (w && wpack_emax > 0) ? weight_hi(wv, wpack_emax) : 0u;
     rel[i] = make_float4(r[0], r[1], r[2], __uint_as_float(wp));
     if (wlo) wlo[i] = weight_lo(wv, wpack_emax);
     xw[i] = make_double4_32a(v[0], v[1], v[2], wv);
@@ -959,6 +950,7 @@ static void tree_release(pc_tree *t) {
     cudaFree(t->naxis);
     cudaFree(t->bcen);
     cudaFree(t->brng);
+    cudaFree(t->obox);
     delete t;
 }
 
@@ -1115,7 +1107,7 @@ extern "C" pc_status pc_build_tree(const double *xyz, const void *w, int w_is_f3
             t->wemin = r[1] >= 0 ? r[2] : 1;
             t->wcorr = r[3] > 0 ? 1 : 0;
             if (t->wcorr) {
-                cudaError_t ea = ::pc::alloc_dev(&t->wlo, sizeof(float) * (size_t)n);
+                cudaError_t ea = ::pc::alloc_dev(&t->wlo, sizeof(unsigned) * (size_t)n);
                 if (ea != cudaSuccess) {
                     cudaGetLastError();
                     return bail(fail(PC_ENOMEM, "pc_build_tree: device allocation failed"));
@@ -1146,6 +1138,7 @@ extern "C" pc_status pc_build_tree(const double *xyz, const void *w, int w_is_f3
     if (e == cudaSuccess) e = ::pc::alloc_dev(&t->rel, sizeof(float4) * n);
     if (e == cudaSuccess) e = ::pc::alloc_dev(&t->xw, sizeof(double4_32a) * n);
     if (e == cudaSuccess) e = ::pc::alloc_dev(&t->perm, sizeof(int) * n);
+    if (e == cudaSuccess) e = ::pc::alloc_dev(&t->obox, obox_bytes(n));
     if (e == cudaSuccess) e = ::pc::alloc_dev(&t->bcen, sizeof(double) * 3 * ((size_t)1 << blevel));
     if (e == cudaSuccess) e = ::pc::alloc_dev(&t->brng, sizeof(int2) * ((size_t)1 << blevel));
     if (e != cudaSuccess) {
@@ -1227,11 +1220,12 @@ extern "C" pc_status pc_build_tree(const double *xyz, const void *w, int w_is_f3
         k_block_info<<<(nblk + 255) / 256, 256, 0, st>>>(t->nbox, t->vnode, blevel, t->bcen, t->brng, ext);
         note_launch();
         k_tree_scatter<<<gpos, 256, 0, st>>>(x, dw, w_is_f32, t->wint ? t->wemax : 0,
-                                             WINT_GRID_SPAN, va, bid, t->bcen,
+                                             va, bid, t->bcen,
                                              (int)n, t->rel, t->xw, t->perm, 0u, t->wlo);
         note_launch();
         e = cudaGetLastError();
     }
+    if (e == cudaSuccess) e = make_obox(t->xw, (int)n, G.lo, t->obox, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&ext_key, ext, sizeof(long long), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return bail(cuda_fail(e, "pc_build_tree"));
@@ -1508,7 +1502,7 @@ extern "C" pc_status pc_build_tree_batch(const double *const *xyz, const void *c
         const size_t ns = ((size_t)2 << depth[k]) - 1, nb = (size_t)1 << blev[k], nk = (size_t)n[k];
         total += carve(sizeof(int2) * ns) * 2 + carve(sizeof(double) * 6 * ns) + carve(ns) +
                  carve(sizeof(float4) * nk) + carve(sizeof(double4_32a) * nk) + carve(sizeof(int) * nk) +
-                 carve(sizeof(double) * 3 * nb) + carve(sizeof(int2) * nb);
+                 carve(sizeof(double) * 3 * nb) + carve(sizeof(int2) * nb) + carve(obox_bytes(n[k]));
     }
     TreeArena *arena = new TreeArena();
     e = ::pc::alloc_dev(&arena->p, total);
@@ -1549,6 +1543,7 @@ extern "C" pc_status pc_build_tree_batch(const double *const *xyz, const void *c
         t->perm = (int *)take(sizeof(int) * n[k]);
         t->bcen = (double *)take(sizeof(double) * 3 * nb);
         t->brng = (int2 *)take(sizeof(int2) * nb);
+        t->obox = (float4 *)take(obox_bytes(n[k]));
         const double *xs = x + 3 * pos[r];
         pc_status s = PC_OK;
         if (G0.periodic) {
@@ -1577,7 +1572,7 @@ extern "C" pc_status pc_build_tree_batch(const double *const *xyz, const void *c
                 t->wemin = res[1] >= 0 ? res[2] : 1;
                 t->wcorr = res[3] > 0 ? 1 : 0;
                 if (t->wcorr) {   // its own allocation, outside the shared block
-                    cudaError_t ea = ::pc::alloc_dev(&t->wlo, sizeof(float) * (size_t)n[k]);
+                    cudaError_t ea = ::pc::alloc_dev(&t->wlo, sizeof(unsigned) * (size_t)n[k]);
                     if (ea != cudaSuccess) {
                         cudaGetLastError();
                         return bail(fail(PC_ENOMEM, "pc_build_tree_batch: device allocation failed"));
@@ -1682,10 +1677,11 @@ extern "C" pc_status pc_build_tree_batch(const double *const *xyz, const void *c
                                                               ext + r);
             note_launch();
             k_tree_scatter<<<(unsigned)((t->n + 255) / 256), 256, 0, st>>>(
-                x, wall, w_is_f32, t->wint ? t->wemax : 0, WINT_GRID_SPAN, va + pos[r],
+                x, wall, w_is_f32, t->wint ? t->wemax : 0, va + pos[r],
                 bid + pos[r], t->bcen, t->n, t->rel, t->xw, t->perm, (unsigned)pos[r], t->wlo);
             note_launch();
             e = cudaGetLastError();
+            if (e == cudaSuccess) e = make_obox(t->xw, t->n, t->g.lo, t->obox, st);
         }
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(ext_key.data(), ext, sizeof(long long) * m, cudaMemcpyDeviceToHost, st);

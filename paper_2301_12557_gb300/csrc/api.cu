@@ -831,7 +831,9 @@ static pc_status fit_params(int prec, int opt_priv, int dev, bool weighted, bool
     const int static_smem = 256;
     const int lut_size = p.lut_total, path0 = p.path, hs0 = p.hs, nent0 = p.nent;
     const bool f64 = prec == PC_PREC_F64;
-    const int nw_min = 4;
+    p.f64 = f64 ? 1 : 0;
+    p.sm_guess = p.f64;
+    const int nw_min = f64 ? 1 : 4;   // as few as still count: edges fill the rest
     auto fit = [&](bool wint) {
         p.wint = wint ? 1 : 0;
         p.wcorr = (wint && wcorr) ? 1 : 0;
@@ -856,8 +858,7 @@ static pc_status fit_params(int prec, int opt_priv, int dev, bool weighted, bool
             p.smem_hist_ok = 1;
             // the floor bins need no tables
             p.lut_total = (p.path != PLAN_LUT || f64) ? 0 : lut_size;
-            const size_t need = f64 ? pairs_f64_smem(p) : pairs_f32_smem(p, nw_min);
-            if (need + static_smem <= (size_t)smem_optin) break;
+            if (pairs_smem(p, nw_min) + static_smem <= (size_t)smem_optin) break;
             if (p.layout == 0 && p.hist_k > 1) {   // fewer lane copies, then the global histogram
                 p.hist_k /= 2;
                 continue;
@@ -867,6 +868,8 @@ static pc_status fit_params(int prec, int opt_priv, int dev, bool weighted, bool
             p.layout = 0;
             p.lut_total = f64 ? 0 : lut_size;
             p.hist_k = 1;
+            // many edges: no FP32 roundings beside them
+            if (f64 && pairs_smem(p, nw_min) + static_smem > (size_t)smem_optin) p.sm_guess = 0;
             break;
         }
     };
@@ -896,33 +899,26 @@ static pc_status fit_params(int prec, int opt_priv, int dev, bool weighted, bool
         p.c_kA = 8388608.0f - (p.path == PLAN_LIN ? 0.5f : 1.5f) * row -
                  (p.mode == PC_BIN_S ? 0.0f : 0.5f * col);
     }
-    if (f64) {
-        smem = pairs_f64_smem(p);
-        if (smem + static_smem > (size_t)smem_optin)
-            return fail(PC_EUNSUPPORTED, "bins: tables do not fit in shared memory");
-        per_sm = pairs_f64_ctas_per_sm(p, smem);
-        return PC_OK;
-    }
     // 8 warps at most with weights: a copy's products between a warp's flushes
     // must hold one batch (64 x 64 products to one lane copy, WINT_LIMIT / 2 / 8)
     int best_warps = 0, best_nw = 0;
-    for (int nw : {4, 8, 12, 16}) {
-        if (p.wint && nw > 8) break;
-        const size_t need = pairs_f32_smem(p, nw);
+    for (int nw : {1, 2, 4, 8, 12, 16}) {
+        if (nw < nw_min || (p.wint && nw > 8)) continue;
+        const size_t need = pairs_smem(p, nw);
         if (need + static_smem > (size_t)smem_optin) break;
-        const int n = pairs_f32_ctas_per_sm(p, need);
+        const int n = f64 ? pairs_f64_ctas_per_sm(p, need) : pairs_f32_ctas_per_sm(p, need);
         if (n * nw > best_warps) {
             best_warps = n * nw;
             best_nw = nw;
         }
     }
     if (best_nw == 0) {
-        if (pairs_f32_smem(p, nw_min) + static_smem > (size_t)smem_optin)
+        if (pairs_smem(p, nw_min) + static_smem > (size_t)smem_optin)
             return fail(PC_EUNSUPPORTED, "bins: tables do not fit in shared memory");
         per_sm = 0;
         return PC_OK;
     }
-    smem = pairs_f32_smem(p, best_nw);
+    smem = pairs_smem(p, best_nw);
     per_sm = best_warps / best_nw;
     return PC_OK;
 }

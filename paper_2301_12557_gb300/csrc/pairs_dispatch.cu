@@ -24,8 +24,7 @@ static int variant(const PairParams &p) {
     return p.los == LOS_Z ? 3 : 4;
 }
 
-size_t pairs_f32_smem(PairParams &p, int nwarps) { return f32_layout(p, nwarps); }
-size_t pairs_f64_smem(const PairParams &p) { return f64_layout(p).total; }
+size_t pairs_smem(PairParams &p, int nwarps) { return cta_layout(p, nwarps); }
 
 cudaError_t launch_pairs_f32(const PairParams &p, int grid, size_t smem, cudaStream_t st) {
     if (p.tree) {

@@ -63,20 +63,28 @@ constexpr int FIX_TOP = 126;  // most bins per axis of the fixed-point floors
 constexpr int SEG_G = 97;     // j-segments of a chunk: 32 stencil rows, <= 3 each, and the own cell
 constexpr int SEG_T = 33;     // 32 listed tree nodes and the own node
 
-// Byte offsets of a warp's slice.
+// Byte offsets of a warp's slice: segments, their offsets (tree), the staged
+// batch (FP64: coordinates and weight, and the images' shifts), its weights, the
+// near-edge queue, the ring and the octs before each segment.
+template <bool TREE, bool WEIGHTED, bool F64>
 struct WarpOff {
-    __host__ __device__ static constexpr int seg(bool) { return 0; }                               // int4[nseg]
-    __host__ __device__ static constexpr int nseg(bool tree) { return tree ? SEG_T : SEG_G; }
-    __host__ __device__ static constexpr int soff(bool tree) { return nseg(tree) * 16; }          // float4[nseg] (tree)
-    __host__ __device__ static constexpr int tile(bool tree) { return soff(tree) + (tree ? SEG_T * 16 : 0); }   // x, y, z
-    __host__ __device__ static constexpr int tw(bool tree) { return tile(tree) + 3 * JB * 4; }    // weights, 8 B a point
-    __host__ __device__ static constexpr int queue(bool tree, int w) { return tw(tree) + (w ? JB * 8 : 0); }    // uint2[QCAP]
-    __host__ __device__ static constexpr int ring(bool tree, int w) { return queue(tree, w) + QCAP * 8; }       // int4[RING]
-    __host__ __device__ static constexpr int pref(bool tree, int w) { return ring(tree, w) + RING * 16; }       // int[nseg + 1]
-    __host__ __device__ static constexpr int total(bool tree, int w) {
-        return (pref(tree, w) + (nseg(tree) + 1) * 4 + 15) / 16 * 16;
-    }
+    enum {
+        nseg = TREE ? SEG_T : SEG_G,
+        soff = nseg * 16,                                    // int4[nseg] before it
+        tile = soff + (TREE ? SEG_T * 16 : 0),               // float4[nseg]
+        tw = tile + (F64 ? JB * 7 * 8 : 3 * JB * 4),         // x, y, z (+ w, shifts)
+        queue = tw + (WEIGHTED && !F64 ? JB * 8 : 0),        // 8 B a point
+        ring = queue + (F64 ? 0 : QCAP * 8),                 // uint2[QCAP]
+        pref = ring + RING * 16,                             // int4[RING]
+        total = (pref + (nseg + 1) * 4 + 15) / 16 * 16       // int[nseg + 1]
+    };
 };
+inline size_t warp_slice(const PairParams &p) {
+    int n = p.weighted ? (int)WarpOff<false, true, false>::total : (int)WarpOff<false, false, false>::total;
+    if (p.tree) n = p.weighted ? (int)WarpOff<true, true, false>::total : (int)WarpOff<true, false, false>::total;
+    if (p.f64) n = (int)WarpOff<false, false, true>::total;
+    return (size_t)n;
+}
 
 // Histogram layouts (word = 4 bytes; entry (n, m), lane copy k of hist_k):
 //  LAY_ROWS   word (n hs + m) hist_k + k; weights: binary64 sums at the same
@@ -96,9 +104,10 @@ __host__ __device__ inline int hist_words(const PairParams &p) {
     return p.nent * p.hist_k;
 }
 
-// Fill in the layout of a CTA of nw warps: histograms, weight sums, tables,
-// the warps' slices.  Returns the bytes.
-inline size_t f32_layout(PairParams &p, int nw) {
+// Fill in the layout of a CTA of nw warps: histograms, weight sums, tables (FP64:
+// squared edges, and their FP32 roundings when sm_guess says so), the warps'
+// slices.  Returns the bytes.
+inline size_t cta_layout(PairParams &p, int nw) {
     size_t o = 0;
     if (p.smem_hist_ok) o = align_up(o + (size_t)hist_words(p) * sizeof(int), 16);
     p.sm_whist = (int)o;
@@ -107,35 +116,15 @@ inline size_t f32_layout(PairParams &p, int nw) {
         else o = align_up(o + (size_t)hist_words(p) * (p.wint ? 3 * sizeof(unsigned) : sizeof(double)), 16);
     }
     p.sm_lut = (int)o;
-    o = align_up(o + (size_t)p.lut_total * sizeof(float2), 16);
+    if (p.f64) {
+        const size_t ne = (size_t)(p.n_a + 1) + (size_t)(p.n_b + 1);
+        o = align_up(o + ne * (sizeof(double) + (p.sm_guess ? sizeof(float) : 0)), 16);
+    } else {
+        o = align_up(o + (size_t)p.lut_total * sizeof(float2), 16);
+    }
     p.sm_warp = (int)o;
     p.nwarps = nw;
-    return o + (size_t)nw * WarpOff::total(p.tree != 0, p.weighted);
-}
-
-// FP64 kernel: offsets of its shared arrays.
-struct SmemLayout64 {
-    size_t ea, eb, hist, whist, seg, tile, meta, total;
-};
-__host__ __device__ inline SmemLayout64 f64_layout(const PairParams &p) {
-    SmemLayout64 L;
-    size_t o = 0;
-    L.hist = o;
-    if (p.smem_hist_ok) o = align_up(o + (size_t)hist_words(p) * sizeof(int), 16);
-    L.whist = o;
-    if (p.smem_hist_ok && p.weighted) o = align_up(o + (size_t)p.nent * p.hist_k * sizeof(double), 16);
-    L.ea = o;
-    o = align_up(o + (size_t)(p.n_a + 1) * sizeof(double), 16);
-    L.eb = o;
-    o = align_up(o + (size_t)(p.n_b + 1) * sizeof(double), 16);
-    L.seg = o;
-    o = align_up(o + (size_t)MAXSEG * sizeof(int4), 16);
-    L.tile = o;
-    o = align_up(o + (size_t)TJ64 * sizeof(double4_32a), 16);
-    L.meta = o;
-    o = align_up(o + (size_t)TJ64 * sizeof(int2), 16);
-    L.total = o;
-    return L;
+    return o + (size_t)nw * warp_slice(p);
 }
 
 // ---------------------------------------------------------------------------
@@ -1125,19 +1114,277 @@ __device__ __noinline__ void check_near(const PairParams &p, const uint2 *queue,
 }
 
 // ---------------------------------------------------------------------------
-// FP32 kernel
+// work items, candidate segments and box tests (both precisions)
 // ---------------------------------------------------------------------------
-// W: 0 unweighted, 1 binary64 weighted sums, 2 integer weight products, 3 the
-// same with binary64 remainders.  TREE: blocks are k-d tree nodes and their
-// j-segments come from the list of the dual-tree traversal instead of the
-// stencil rows.
-//
 // Work items: (block, 64-point part of the block, slice of its octs).  Slices
 // (S > 1) split the i-points' candidates among warps, for about 24 items a
 // warp of the grid, so that the last items do not leave the chip half empty.
 // One histogram: each warp takes items from the global counter until none are
 // left.  Several (batches): the CTA takes ranges of items of one histogram and
 // flushes between them.
+struct RangeShared {
+    int cur, end, next, lim, task;
+};
+struct Items {
+    int per_block, S, chunk;
+    long long n;
+    __device__ __forceinline__ void init(const PairParams &p, int nw) {
+        const int nblocks = *p.nblocks;
+        const long long units = max((long long)nblocks, p.npts_i / BI + 1);
+        const long long want = 24ll * gridDim.x * nw;
+        S = 1;
+        if (units < want) S = (int)min(32ll, (want + units - 1) / units);
+        per_block = p.nsub * S;
+        n = (long long)nblocks * per_block;
+        chunk = (int)max((long long)nw, min((long long)nw * 32 * S, n / (6ll * gridDim.x)));
+    }
+};
+
+// Next item of this warp, -1 when none is left.  flush(task): every warp of the
+// CTA, between barriers, after the last item of `task` (batches).
+template <class F>
+__device__ __forceinline__ long long next_item(const PairParams &p, const Items &W, RangeShared &R, F flush) {
+    const int lane = threadIdx.x & 31;
+    if (!p.multi) {
+        unsigned v = 0u;
+        if (lane == 0) v = (unsigned)atomicAdd(p.work_counter, 1);
+        const long long it = __shfl_sync(FULL, v, 0);
+        return it < W.n ? it : -1;
+    }
+    for (;;) {
+        int v = 0;
+        if (lane == 0) v = atomicAdd(&R.cur, 1);
+        v = __shfl_sync(FULL, v, 0);
+        if (v < R.end) return v;
+        // range used up: every warp arrives here; the next one of a single
+        // task is fetched, the histograms flushed on a change
+        __syncthreads();
+        const int old = R.task;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int b = R.next;
+            if (b >= R.lim) {
+                b = (int)min((long long)atomicAdd(p.work_counter, W.chunk), W.n);
+                R.lim = (int)min((long long)b + W.chunk, W.n);
+            }
+            int e = b;
+            if (b < R.lim) {
+                const int task = p.blocks[b / W.per_block].task;
+                int lo = b + 1, hi = R.lim;   // items [b, e) belong to `task`
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (p.blocks[mid / W.per_block].task == task) lo = mid + 1; else hi = mid;
+                }
+                e = lo;
+                R.task = task;
+            } else {
+                R.task = -2;
+            }
+            R.cur = b;
+            R.end = e;
+            R.next = e;
+        }
+        __syncthreads();
+        if (R.task != old && old >= 0) flush(old);
+        if (R.task == -2) return -1;
+    }
+}
+
+// The i-points of an item: [start, start + count) of block B, slice `part`.
+struct Item {
+    Block B;
+    int start, count, part;
+    int ax, ay, az;          // grid: the i-cell
+    int ts0, ntl, own_end;   // list (tree) or stencil rows; end of the own cell (auto)
+};
+template <bool TREE>
+__device__ __forceinline__ bool open_item(const PairParams &p, const Items &W, long long it, Item &I) {
+    I.B = p.blocks[it / W.per_block];
+    const int rem = (int)(it % W.per_block), sub = rem / W.S;
+    I.part = rem - sub * W.S;
+    const int k = (I.B.count + BI - 1) / BI;
+    if (sub >= k) return false;
+    I.start = I.B.start + (int)((long long)I.B.count * sub / k);
+    I.count = I.B.start + (int)((long long)I.B.count * (sub + 1) / k) - I.start;
+    const TaskDev &T = p.tasks[I.B.task];
+    const int nx = p.g.ng[0], ny = p.g.ng[1];
+    I.ax = TREE ? 0 : I.B.cell % nx;
+    I.ay = TREE ? 0 : (I.B.cell / nx) % ny;
+    I.az = TREE ? 0 : I.B.cell / (nx * ny);
+    I.ts0 = 0;
+    I.own_end = 0;
+    if (TREE) {
+        I.ts0 = p.tseg_off[I.B.cell];
+        I.ntl = p.tseg_off[I.B.cell + 1] - I.ts0;
+        if (T.is_auto) {
+            const int2 r = p.tblk_j[I.B.cell];
+            I.own_end = r.x + r.y;
+        }
+    } else {
+        I.ntl = p.nrows;
+        if (T.is_auto) I.own_end = T.gi.cell_start[I.B.cell + 1];
+    }
+    return true;
+}
+
+// Bounding box of the warp's i-points, relative to the j-grid's origin.
+struct IBox {
+    float lx, ly, lz, hx, hy, hz;
+    __device__ __forceinline__ void clear() {
+        lx = ly = lz = INFINITY;
+        hx = hy = hz = -INFINITY;
+    }
+    __device__ __forceinline__ void add(const GridDev &g, const double4_32a &a) {
+        const double ox = a.x - g.org[0], oy = a.y - g.org[1], oz = a.z - g.org[2];
+        lx = fminf(lx, __double2float_rd(ox)); hx = fmaxf(hx, __double2float_ru(ox));
+        ly = fminf(ly, __double2float_rd(oy)); hy = fmaxf(hy, __double2float_ru(oy));
+        lz = fminf(lz, __double2float_rd(oz)); hz = fmaxf(hz, __double2float_ru(oz));
+    }
+    __device__ __forceinline__ void finish(const TaskDev &T) {
+        const float ogx = (float)(T.gj.org[0] - T.gi.org[0]), ogy = (float)(T.gj.org[1] - T.gi.org[1]),
+                    ogz = (float)(T.gj.org[2] - T.gi.org[2]);
+        lx = warp_minf(lx) - ogx; ly = warp_minf(ly) - ogy; lz = warp_minf(lz) - ogz;
+        hx = warp_maxf(hx) - ogx; hy = warp_maxf(hy) - ogy; hz = warp_maxf(hz) - ogz;
+    }
+};
+
+// Segments of chunk `ch` (32 stencil rows or listed nodes; the rest of the own
+// cell with the first): seg = {first point, end, dy | dz << 16 (tree: j-node),
+// image code}, pref the octs before each.  Returns their octs.
+template <bool TREE>
+__device__ __forceinline__ int build_chunk(const PairParams &p, const TaskDev &T, const Item &I, int ch, int4 *seg,
+                                           float4 *soff, int *pref, int &nseg) {
+    const int lane = threadIdx.x & 31;
+    const int nx = p.g.ng[0], ny = p.g.ng[1], nz = p.g.ng[2];
+    int noct = 0;
+    nseg = 0;
+    if (ch == 0 && I.own_end > I.start + I.count) {   // rest of the own cell: j > i for all
+        const int a0 = I.start + I.count;
+        if (lane == 0) {
+            seg[0] = make_int4(a0, I.own_end, TREE ? -1 : 0, 13);
+            pref[0] = 0;
+            if (TREE) soff[0] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        nseg = 1;
+        noct = ((I.own_end + 7) >> 3) - (a0 >> 3);
+    }
+    const int row = ch * 32 + lane;
+    int a0[3], a1[3], im[3], np = 0, no = 0, meta = 0;
+    if (row < I.ntl) {
+        if (TREE) {
+            const int2 e = p.tseg[I.ts0 + row];
+            const int2 r = p.tblk_j[e.x];
+            a0[0] = r.x; a1[0] = r.x + r.y; im[0] = e.y;
+            meta = e.x;
+            np = r.y > 0 ? 1 : 0;
+            no = np ? ((a1[0] + 7) >> 3) - (a0[0] >> 3) : 0;
+        } else {
+            const int4 sr = p.stencil[row];
+            const int dy = sr.x, dz = sr.y;
+            int y = I.ay + dy, z = I.az + dz, wy = 0, wz = 0;
+            bool in = true;
+            if (y < 0) { in = in && p.g.periodic; y += ny; wy = -1; }
+            else if (y >= ny) { in = in && p.g.periodic; y -= ny; wy = 1; }
+            if (z < 0) { in = in && p.g.periodic; z += nz; wz = -1; }
+            else if (z >= nz) { in = in && p.g.periodic; z -= nz; wz = 1; }
+            meta = (dy & 0xFFFF) | (dz << 16);
+            const int rowbase = (z * ny + y) * nx;
+            const int x0 = I.ax + sr.z, x1 = I.ax + sr.w;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {   // the part left of the box, inside, right of it
+                int c0, c1;
+                if (q == 0) { c0 = x0 + nx; c1 = min(x1, -1) + nx; }
+                else if (q == 1) { c0 = max(x0, 0); c1 = min(x1, nx - 1); }
+                else { c0 = max(x0, nx) - nx; c1 = x1 - nx; }
+                const bool use = in && c0 <= c1 && (q == 1 || p.g.periodic) && (q != 0 || x0 < 0) &&
+                                 (q != 2 || x1 >= nx);
+                a0[q] = a1[q] = 0;
+                im[q] = q * 9 + (wy + 1) * 3 + (wz + 1);
+                if (use) {
+                    a0[q] = T.gj.cell_start[rowbase + c0];
+                    a1[q] = T.gj.cell_start[rowbase + c1 + 1];
+                }
+                if (a1[q] > a0[q]) {
+                    ++np;
+                    no += ((a1[q] + 7) >> 3) - (a0[q] >> 3);
+                }
+            }
+        }
+    }
+    const int is = warp_incl_scan(np), io = warp_incl_scan(no);
+    int slot = nseg + is - np, o = noct + io - no;
+#pragma unroll
+    for (int q = 0; q < (TREE ? 1 : 3); ++q)
+        if (np && a1[q] > a0[q]) {
+            seg[slot] = make_int4(a0[q], a1[q], meta, im[q]);
+            if (TREE) soff[slot] = tree_offset(p, I.B.cell, meta, im[q]);
+            pref[slot] = o;
+            o += ((a1[q] + 7) >> 3) - (a0[q] >> 3);
+            ++slot;
+        }
+    nseg += __shfl_sync(FULL, is, 31);
+    noct += __shfl_sync(FULL, io, 31);
+    return noct;
+}
+
+// One round: octs 32 rd .. 32 rd + 31 of the chunk, those whose box can reach
+// the i-points' box appended to the ring {first point, segment, squared gap}.
+// Boxes are rounded outward, and r2prune carries the rounding of this test
+// (host side), so a dropped pair is at least rcut apart.
+template <int MODE, int LOS>
+__device__ __forceinline__ int ring_round(const PairParams &p, const TaskDev &T, int rd, int noct, int nseg,
+                                          const int4 *seg, const int *pref, const IBox &b, int count, int4 *ring,
+                                          int tail, unsigned long long &cand, unsigned long long &pruned) {
+    const int lane = threadIdx.x & 31;
+    const int f = rd * 32 + lane;
+    bool keep = false;
+    int lo = 0, p0 = 0;
+    float g2 = 0.f;
+    if (f < noct) {
+        int hi = nseg;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (pref[mid] <= f) lo = mid; else hi = mid;
+        }
+        const int4 sg = seg[lo];
+        const int oct = (sg.x >> 3) + (f - pref[lo]);
+        p0 = oct << 3;
+        float4 bl = T.gj.obox[2 * (size_t)oct], bh = T.gj.obox[2 * (size_t)oct + 1];
+        if (p.g.periodic) {
+            const float sx = (float)(sg.w / 9 - 1) * p.L32[0];
+            const float sy = (float)((sg.w / 3) % 3 - 1) * p.L32[1];
+            const float sz = (float)(sg.w % 3 - 1) * p.L32[2];
+            bl.x += sx; bl.y += sy; bl.z += sz;
+            bh.x += sx; bh.y += sy; bh.z += sz;
+        }
+        const float gx = fmaxf(fmaxf(bl.x - b.hx, b.lx - bh.x), 0.f);
+        const float gy = fmaxf(fmaxf(bl.y - b.hy, b.ly - bh.y), 0.f);
+        const float gz = fmaxf(fmaxf(bl.z - b.hz, b.lz - bh.z), 0.f);
+        const float gq = fmaf(gy, gy, gx * gx);
+        g2 = fmaf(gz, gz, gq);
+        keep = g2 < p.r2prune;
+        if (MODE == MODE_SIGPI && LOS == LOS_Z)   // the reach is a cylinder
+            keep = keep && gq < p.q2prune && gz < p.zprune;
+        const unsigned long long np2 =
+            (unsigned long long)(min(sg.y, p0 + 8) - max(sg.x, p0)) * (unsigned)count;
+        cand += np2;
+        if (!keep) pruned += np2;
+    }
+    const unsigned who = __ballot_sync(FULL, keep);
+    if (keep)
+        ring[(tail + __popc(who & ((1u << lane) - 1u))) & (RING - 1)] =
+            make_int4(p0, lo, __float_as_int(g2), 0);
+    __syncwarp();
+    return tail + __popc(who);
+}
+
+// ---------------------------------------------------------------------------
+// FP32 kernel
+// ---------------------------------------------------------------------------
+// W: 0 unweighted, 1 binary64 weighted sums, 2 integer weight products, 3 the
+// same with binary64 remainders.  TREE: blocks are k-d tree nodes and their
+// j-segments come from the list of the dual-tree traversal instead of the
+// stencil rows.
 //
 // Registers: the loops need 50 to 80; with the rest of a warp's state 80 (96 with
 // more operands a pair) give 24 (20) resident warps.  80 to 128 measured within
@@ -1146,19 +1393,20 @@ template <int MODE, int LOS, int W, int PATH, bool TREE>
 __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH == PATH_LUT ? 96 : 80)
     k_pairs_f32(const __grid_constant__ PairParams p) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int s_cur, s_end, s_next, s_lim, s_task;
+    __shared__ RangeShared s_range;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
-    unsigned char *ws = smem + p.sm_warp + (size_t)warp * WarpOff::total(TREE, W);
-    int4 *seg = reinterpret_cast<int4 *>(ws + WarpOff::seg(TREE));
-    float4 *soff = reinterpret_cast<float4 *>(ws + WarpOff::soff(TREE));
-    float *tx = reinterpret_cast<float *>(ws + WarpOff::tile(TREE));
+    using O = WarpOff<TREE, W != 0, false>;
+    unsigned char *ws = smem + p.sm_warp + (size_t)warp * O::total;
+    int4 *seg = reinterpret_cast<int4 *>(ws);
+    float4 *soff = reinterpret_cast<float4 *>(ws + O::soff);
+    float *tx = reinterpret_cast<float *>(ws + O::tile);
     float *ty = tx + JB, *tz = ty + JB;
-    double *tw = reinterpret_cast<double *>(ws + WarpOff::tw(TREE));
+    double *tw = reinterpret_cast<double *>(ws + O::tw);
     unsigned *twm = reinterpret_cast<unsigned *>(tw);
     unsigned *twl = twm + JB;
-    uint2 *queue = reinterpret_cast<uint2 *>(ws + WarpOff::queue(TREE, W));
-    int4 *ring = reinterpret_cast<int4 *>(ws + WarpOff::ring(TREE, W));
-    int *pref = reinterpret_cast<int *>(ws + WarpOff::pref(TREE, W));
+    uint2 *queue = reinterpret_cast<uint2 *>(ws + O::queue);
+    int4 *ring = reinterpret_cast<int4 *>(ws + O::ring);
+    int *pref = reinterpret_cast<int *>(ws + O::pref);
     const Tile tile{tx, ty, tz, tw, twm, twl};
     const float2 *s_lut = reinterpret_cast<const float2 *>(smem + p.sm_lut);
 
@@ -1169,27 +1417,15 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
     if (W >= 2 && p.wfold)
         for (int b = threadIdx.x; b < 2 * p.nbins; b += blockDim.x)
             p.wfold_buf[(size_t)blockIdx.x * p.nbins * 2 + b] = 0ull;
-    if (threadIdx.x == 0) {
-        s_cur = s_end = s_next = s_lim = 0;
-        s_task = -1;
-    }
+    if (threadIdx.x == 0) s_range = RangeShared{0, 0, 0, 0, -1};
     const unsigned copy = 4u * (unsigned)(lane & (p.hist_k - 1));
     Ctx<MODE, LOS, PATH == PATH_FIX ? PATH_LIN : PATH> c;
     if (PATH != PATH_FIX) c.init(p, s_lut, copy);
     const unsigned wbase = (unsigned)__cvta_generic_to_shared(smem + p.sm_whist);
     const float far = p.far;
 
-    const int nblocks = *p.nblocks;
-    const int nsub = p.nsub;
-    int S = 1;
-    {
-        const long long units = max((long long)nblocks, p.npts_i / BI + 1);
-        const long long want = 24ll * gridDim.x * nw;
-        if (units < want) S = (int)min(32ll, (want + units - 1) / units);
-    }
-    const int per_block = nsub * S;
-    const long long nitems = (long long)nblocks * per_block;
-    const int chunk = (int)max((long long)nw, min((long long)nw * 32 * S, nitems / (6ll * gridDim.x)));
+    Items items;
+    items.init(p, nw);
     unsigned long long cand = 0, pruned = 0;   // per lane
     unsigned since = 0, wterms = 0;            // quads, products per copy since this warp's flushes
     const unsigned flush_quads = (unsigned)(FLUSH_LIMIT / 256 / nw);
@@ -1208,78 +1444,26 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
     __syncthreads();
 
     for (;;) {
-        // ---- next item ------------------------------------------------------
-        long long it;
-        if (!p.multi) {
-            unsigned v = 0u;
-            if (lane == 0) v = (unsigned)atomicAdd(p.work_counter, 1);
-            it = __shfl_sync(FULL, v, 0);
-            if (it >= nitems) break;
-        } else {
-            int v = 0;
-            for (;;) {
-                if (lane == 0) v = atomicAdd(&s_cur, 1);
-                v = __shfl_sync(FULL, v, 0);
-                if (v < s_end) break;
-                // range used up: every warp arrives here; the next one of a
-                // single task is fetched, the histograms flushed on a change
-                __syncthreads();
-                const int old = s_task;
-                __syncthreads();
-                if (threadIdx.x == 0) {
-                    int b = s_next;
-                    if (b >= s_lim) {
-                        b = (int)min((long long)atomicAdd(p.work_counter, chunk), nitems);
-                        s_lim = (int)min((long long)b + chunk, nitems);
-                    }
-                    int e = b;
-                    if (b < s_lim) {
-                        const int task = p.blocks[b / per_block].task;
-                        int lo = b + 1, hi = s_lim;   // items [b, e) belong to `task`
-                        while (lo < hi) {
-                            const int mid = (lo + hi) >> 1;
-                            if (p.blocks[mid / per_block].task == task) lo = mid + 1; else hi = mid;
-                        }
-                        e = lo;
-                        s_task = task;
-                    } else {
-                        s_task = -2;
-                    }
-                    s_cur = b;
-                    s_end = e;
-                    s_next = e;
-                }
-                __syncthreads();
-                if (s_task != old && old >= 0) {
-                    const int h = p.tasks[old].hist;
-                    if (PATH != PATH_GLOBAL) {
-                        flush_counts(p, 0, warp, nw, h);
-                        if (W) flush_weights(p, p.sm_whist, warp, nw, h, p.tasks[old].wscale);
-                    }
-                    __syncthreads();
-                    if (W >= 2 && p.wfold) flush_folded(p, h, p.tasks[old].wscale);
-                    since = wterms = 0;
-                    __syncthreads();
-                }
-                if (s_task == -2) break;
+        auto flush = [&](int old) {
+            const int h = p.tasks[old].hist;
+            if (PATH != PATH_GLOBAL) {
+                flush_counts(p, 0, warp, nw, h);
+                if (W) flush_weights(p, p.sm_whist, warp, nw, h, p.tasks[old].wscale);
             }
-            if (s_task == -2) break;
-            it = v;
-        }
-        const Block B = p.blocks[it / per_block];
-        const int rem = (int)(it % per_block), sub = rem / S, part = rem - sub * S;
-        const int k = (B.count + BI - 1) / BI;
-        if (sub >= k) continue;
-        const int start = B.start + (int)((long long)B.count * sub / k);
-        const int count = B.start + (int)((long long)B.count * (sub + 1) / k) - start;
-        const TaskDev &T = p.tasks[B.task];
-        const int nx = p.g.ng[0], ny = p.g.ng[1], nz = p.g.ng[2];
-        const int ax = TREE ? 0 : B.cell % nx, ay = TREE ? 0 : (B.cell / nx) % ny,
-                  az = TREE ? 0 : B.cell / (nx * ny);
+            __syncthreads();
+            if (W >= 2 && p.wfold) flush_folded(p, h, p.tasks[old].wscale);
+            since = wterms = 0;
+            __syncthreads();
+        };
+        const long long id = next_item(p, items, s_range, flush);
+        if (id < 0) break;
+        Item it;
+        if (!open_item<TREE>(p, items, id, it)) continue;
+        const TaskDev &T = p.tasks[it.B.task];
 
-        // ---- i-points and their box (relative to the i-grid's origin) --------
         IPts<LOS, W> I;
-        float blx = INFINITY, bly = INFINITY, blz = INFINITY, bhx = -INFINITY, bhy = -INFINITY, bhz = -INFINITY;
+        IBox box;
+        box.clear();
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             I.x[r] = -far;      // unused: out of range of every j-point
@@ -1288,173 +1472,42 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
             I.w[r] = 0.0;
             I.wm[r] = 0u;
             I.wb[r] = 0u;
-            if (2 * lane + r < count) {
-                const int i = start + 2 * lane + r;
+            if (2 * lane + r < it.count) {
+                const int i = it.start + 2 * lane + r;
                 load_i<MODE, LOS, W>(T.gi, i, I, r);
                 if (PATH == PATH_FIX && !(fabsf(I.x[r]) + fabsf(I.y[r]) + fabsf(I.z[r]) < 1e16f)) {
                     I.x[r] = -far;      // not a number: no pair
                     I.y[r] = I.z[r] = 0.f;
                 }
-                const double4_32a a = T.gi.xw[i];
-                const double ox = a.x - T.gi.org[0], oy = a.y - T.gi.org[1], oz = a.z - T.gi.org[2];
-                blx = fminf(blx, __double2float_rd(ox)); bhx = fmaxf(bhx, __double2float_ru(ox));
-                bly = fminf(bly, __double2float_rd(oy)); bhy = fmaxf(bhy, __double2float_ru(oy));
-                blz = fminf(blz, __double2float_rd(oz)); bhz = fmaxf(bhz, __double2float_ru(oz));
+                box.add(T.gi, T.gi.xw[i]);
             }
         }
-        // the boxes are compared in the j-grid's coordinates: its origin
-        // relative to the i-grid's is taken off the i-box
-        const float ogx = (float)(T.gj.org[0] - T.gi.org[0]), ogy = (float)(T.gj.org[1] - T.gi.org[1]),
-                    ogz = (float)(T.gj.org[2] - T.gi.org[2]);
-        blx = warp_minf(blx) - ogx; bly = warp_minf(bly) - ogy; blz = warp_minf(blz) - ogz;
-        bhx = warp_maxf(bhx) - ogx; bhy = warp_maxf(bhy) - ogy; bhz = warp_maxf(bhz) - ogz;
+        box.finish(T);
 
-        // ---- j-segments, in chunks ------------------------------------------
-        int ts0 = 0, ntl = 0, own_end = 0;
-        if (TREE) {
-            ts0 = p.tseg_off[B.cell];
-            ntl = p.tseg_off[B.cell + 1] - ts0;
-            if (T.is_auto) {
-                const int2 r = p.tblk_j[B.cell];
-                own_end = r.x + r.y;
-            }
-        } else {
-            ntl = p.nrows;
-            if (T.is_auto) own_end = T.gi.cell_start[B.cell + 1];
-        }
         // pairs inside the block (j > i) first
-        bool own = T.is_auto && part == 0;
-        if (own && lane == 0) cand += (unsigned long long)count * (unsigned)(count - 1) / 2;
-        const int nchunk = max(1, (ntl + 31) / 32);
+        bool own = T.is_auto && it.part == 0;
+        if (own && lane == 0) cand += (unsigned long long)it.count * (unsigned)(it.count - 1) / 2;
+        const int nchunk = max(1, (it.ntl + 31) / 32);
         int round0 = 0;      // rounds of 32 octs before this chunk
         int qn = 0;          // queued near-edge quads
         for (int ch = 0; ch < nchunk; ++ch) {
             __syncwarp();
-            int nseg = 0, noct = 0;
-            if (ch == 0 && own_end > start + count) {   // rest of the own cell: j > i for all
-                const int a0 = start + count;
-                if (lane == 0) {
-                    seg[0] = make_int4(a0, own_end, TREE ? -1 : 0, 13);
-                    pref[0] = 0;
-                    if (TREE) soff[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-                nseg = 1;
-                noct = ((own_end + 7) >> 3) - (a0 >> 3);
-            }
-            const int row = ch * 32 + lane;
-            int a0[3], a1[3], im[3], np = 0, no = 0, meta = 0;
-            if (row < ntl) {
-                if (TREE) {
-                    const int2 e = p.tseg[ts0 + row];
-                    const int2 r = p.tblk_j[e.x];
-                    a0[0] = r.x; a1[0] = r.x + r.y; im[0] = e.y;
-                    meta = e.x;
-                    np = r.y > 0 ? 1 : 0;
-                    no = np ? ((a1[0] + 7) >> 3) - (a0[0] >> 3) : 0;
-                } else {
-                    const int4 sr = p.stencil[row];
-                    const int dy = sr.x, dz = sr.y;
-                    int y = ay + dy, z = az + dz, wy = 0, wz = 0;
-                    bool in = true;
-                    if (y < 0) { in = in && p.g.periodic; y += ny; wy = -1; }
-                    else if (y >= ny) { in = in && p.g.periodic; y -= ny; wy = 1; }
-                    if (z < 0) { in = in && p.g.periodic; z += nz; wz = -1; }
-                    else if (z >= nz) { in = in && p.g.periodic; z -= nz; wz = 1; }
-                    meta = (dy & 0xFFFF) | (dz << 16);
-                    const int rowbase = (z * ny + y) * nx;
-                    const int x0 = ax + sr.z, x1 = ax + sr.w;
-#pragma unroll
-                    for (int q = 0; q < 3; ++q) {   // the part left of the box, inside, right of it
-                        int c0, c1;
-                        if (q == 0) { c0 = x0 + nx; c1 = min(x1, -1) + nx; }
-                        else if (q == 1) { c0 = max(x0, 0); c1 = min(x1, nx - 1); }
-                        else { c0 = max(x0, nx) - nx; c1 = x1 - nx; }
-                        const bool use = in && c0 <= c1 && (q == 1 || p.g.periodic) &&
-                                         (q != 0 || x0 < 0) && (q != 2 || x1 >= nx);
-                        a0[q] = a1[q] = 0;
-                        im[q] = q * 9 + (wy + 1) * 3 + (wz + 1);
-                        if (use) {
-                            a0[q] = T.gj.cell_start[rowbase + c0];
-                            a1[q] = T.gj.cell_start[rowbase + c1 + 1];
-                        }
-                        if (a1[q] > a0[q]) {
-                            ++np;
-                            no += ((a1[q] + 7) >> 3) - (a0[q] >> 3);
-                        }
-                    }
-                }
-            }
-            {
-                const int is = warp_incl_scan(np), io = warp_incl_scan(no);
-                int slot = nseg + is - np, o = noct + io - no;
-#pragma unroll
-                for (int q = 0; q < (TREE ? 1 : 3); ++q)
-                    if (np && a1[q] > a0[q]) {
-                        seg[slot] = make_int4(a0[q], a1[q], meta, im[q]);
-                        if (TREE) soff[slot] = tree_offset(p, B.cell, meta, im[q]);
-                        pref[slot] = o;
-                        o += ((a1[q] + 7) >> 3) - (a0[q] >> 3);
-                        ++slot;
-                    }
-                nseg += __shfl_sync(FULL, is, 31);
-                noct += __shfl_sync(FULL, io, 31);
-            }
+            int nseg;
+            const int noct = build_chunk<TREE>(p, T, it, ch, seg, soff, pref, nseg);
             __syncwarp();
             const int nround = (noct + 31) / 32;
             // this slice's rounds: global round number = part (mod S)
-            int rd = (part - round0 % S + S) % S;
+            int rd = (it.part - round0 % items.S + items.S) % items.S;
             round0 += nround;
             int head = 0, tail = 0;
             for (;;) {
-                // fill the ring: 32 octs a round, those whose box can reach the
-                // i-points' box.  Boxes are rounded outward, and r2prune carries
-                // the rounding of this test (host side), so a dropped pair is at
-                // least rcut apart
                 while (!own && tail - head < JO && rd < nround) {
-                    const int f = rd * 32 + lane;
-                    rd += S;
-                    bool keep = false;
-                    int lo = 0, p0 = 0;
-                    float g2 = 0.f;
-                    if (f < noct) {
-                        int hi = nseg;
-                        while (hi - lo > 1) {
-                            const int mid = (lo + hi) >> 1;
-                            if (pref[mid] <= f) lo = mid; else hi = mid;
-                        }
-                        const int4 sg = seg[lo];
-                        const int oct = (sg.x >> 3) + (f - pref[lo]);
-                        p0 = oct << 3;
-                        float4 bl = T.gj.obox[2 * (size_t)oct], bh = T.gj.obox[2 * (size_t)oct + 1];
-                        if (p.g.periodic) {
-                            const float sx = (float)(sg.w / 9 - 1) * p.L32[0];
-                            const float sy = (float)((sg.w / 3) % 3 - 1) * p.L32[1];
-                            const float sz = (float)(sg.w % 3 - 1) * p.L32[2];
-                            bl.x += sx; bl.y += sy; bl.z += sz;
-                            bh.x += sx; bh.y += sy; bh.z += sz;
-                        }
-                        const float gx = fmaxf(fmaxf(bl.x - bhx, blx - bh.x), 0.f);
-                        const float gy = fmaxf(fmaxf(bl.y - bhy, bly - bh.y), 0.f);
-                        const float gz = fmaxf(fmaxf(bl.z - bhz, blz - bh.z), 0.f);
-                        const float gq = fmaf(gy, gy, gx * gx);
-                        g2 = fmaf(gz, gz, gq);
-                        keep = g2 < p.r2prune;
-                        if (MODE == MODE_SIGPI && LOS == LOS_Z)   // the reach is a cylinder
-                            keep = keep && gq < p.q2prune && gz < p.zprune;
-                        const unsigned long long np2 =
-                            (unsigned long long)(min(sg.y, p0 + 8) - max(sg.x, p0)) * (unsigned)count;
-                        cand += np2;
-                        if (!keep) pruned += np2;
-                    }
-                    const unsigned who = __ballot_sync(FULL, keep);
-                    if (keep)
-                        ring[(tail + __popc(who & ((1u << lane) - 1u))) & (RING - 1)] =
-                            make_int4(p0, lo, __float_as_int(g2), 0);
-                    tail += __popc(who);
-                    __syncwarp();
+                    tail = ring_round<MODE, LOS>(p, T, rd, noct, nseg, seg, pref, box, it.count, ring, tail, cand,
+                                                 pruned);
+                    rd += items.S;
                 }
                 // one batch: the block's own points, or up to eight octs
-                const int m = own ? (count + 7) >> 3 : min(JO, tail - head);
+                const int m = own ? (it.count + 7) >> 3 : min(JO, tail - head);
                 unsigned near = 0u;
                 unsigned band = 0u;
                 if (m > 0) {
@@ -1464,8 +1517,8 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
                         const int sl = lane + 32 * h, oc = sl >> 3;
                         float3 s = make_float3(far, 0.f, 0.f);
                         float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-                        int pj = start + sl;
-                        bool v = own && sl < count;
+                        int pj = it.start + sl;
+                        bool v = own && sl < it.count;
                         if (v) {
                             q = T.gj.rel[pj];
                             s = make_float3(q.x, q.y, q.z);
@@ -1481,7 +1534,7 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
                                     const float4 o = soff[e.y];
                                     s = make_float3(o.x + q.x, o.y + q.y, o.z + q.z);
                                 } else {
-                                    s = stage_grid(p, q, T.gj.cx[pj], ax, sg.z, sg.w);
+                                    s = stage_grid(p, q, T.gj.cx[pj], it.ax, sg.z, sg.w);
                                 }
                             }
                         }
@@ -1542,7 +1595,7 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
                     if (near) {
                         const int q = __ffs(near) - 1;
                         near &= near - 1;
-                        uint2 e = make_uint2((unsigned)(start + 4 * q), (unsigned)lane | 32u | band << 13);
+                        uint2 e = make_uint2((unsigned)(it.start + 4 * q), (unsigned)lane | 32u | band << 13);
                         if (!own) {
                             const int4 o = ring[(head + (q >> 1)) & (RING - 1)];
                             e = make_uint2((unsigned)(o.x + 4 * (q & 1)),
@@ -1555,7 +1608,7 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
                     if (qn >= 32 || (rest && qn > 0)) {
                         const int n = min(qn, 32);
                         __syncwarp();
-                        check_near<MODE, LOS, W, PATH, TREE>(p, queue, seg, n, B.task, B.cell, start, count, copy,
+                        check_near<MODE, LOS, W, PATH, TREE>(p, queue, seg, n, it.B.task, it.B.cell, it.start, it.count, copy,
                                                              s_lut);
                         __syncwarp();
                         qn -= n;
@@ -1592,217 +1645,244 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
 }
 
 // ---------------------------------------------------------------------------
-// FP64 kernel: j-segments of a CTA
+// plain FP64 kernel: the binary64 definition for every pair of a box in reach
 // ---------------------------------------------------------------------------
-// Exclusive prefix over the segment lengths held in seg[k].y (in place);
-// returns the total.  All NT threads call it.
-__device__ __forceinline__ int seg_scan(int4 *seg, int nseg, int *s_tmp) {
-    // each thread owns a contiguous run of ceil(nseg / NT) segments
-    const int tid = threadIdx.x;
-    const int per = (nseg + NT - 1) / NT;
-    int b0 = tid * per, b1 = min(b0 + per, nseg);
-    int local = 0;
-    for (int k = b0; k < b1; ++k) local += seg[k].y;
-    // block-wide exclusive scan of `local` (NT = 128: 4 warps)
-    int lane = tid & 31, warp = tid >> 5;
-    int v = local;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        int t = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += t;
-    }
-    if (lane == 31) s_tmp[warp] = v;
-    __syncthreads();
-    int wbase = 0;
-    for (int w = 0; w < warp; ++w) wbase += s_tmp[w];
-    int total = s_tmp[0] + s_tmp[1] + s_tmp[2] + s_tmp[3];
-    int run = wbase + v - local;
-    for (int k = b0; k < b1; ++k) {
-        int len = seg[k].y;
-        seg[k].y = run;
-        run += len;
-    }
-    __syncthreads();
-    return total;
-}
+// Items, segments and box tests as the FP32 kernel's; the staged j-points and
+// the i-points are the canonical binary64 coordinates.  This GPU issues about
+// 1.7 binary64 operations per SM clock, so the kernel is bound by their number:
+// eight a pair in reach (eleven with a periodic image) and two to four for the
+// bin, which a search over the edges' FP32 roundings only proposes and binary64
+// comparisons decide.  The definition's wrap rule needs no test: a pair in range
+// under the visited image is one the rule gives that image, since the reach
+// stays below L / 2 by more than the roundings.  Before: every candidate of the
+// stencil, with six comparisons for the wrap rule and a binary64 search; 50,001
+// uniform points in 40 s bins took 120.5 ms, now 7.1 ms.
+struct F64Edges {
+    const double *Ea, *Eb;
+    const float *Fa, *Fb;    // FP32 roundings, or null
+};
 
-// Segment holding flat position f: largest k with seg[k].y <= f.
-__device__ __forceinline__ int seg_find(const int4 *seg, int nseg, int f) {
-    int lo = 0, hi = nseg;
+// Largest k with v >= E[k] (v >= E[0] holds), from a guess by the FP32 edges.
+__device__ __forceinline__ int locate64(double v, const double *E, const float *F, int n) {
+    if (!F) return f64_locate(v, E, n);
+    const float f = (float)v;
+    int lo = 0, hi = n;
     while (hi - lo > 1) {
-        int mid = (lo + hi) >> 1;
-        if (seg[mid].y <= f) lo = mid; else hi = mid;
+        const int mid = (lo + hi) >> 1;
+        if (f >= F[mid]) lo = mid; else hi = mid;
     }
+    while (lo > 0 && v < E[lo]) --lo;
+    while (lo + 1 < n && v >= E[lo + 1]) ++lo;
+    return lo;
+}
+// Largest j < n with p2 >= M[j] s2 (the product rounded once).
+__device__ __forceinline__ int locate64_mu(double p2, double s2, const double *M, const float *F, int n) {
+    if (!F) return f64_locate_mu(p2, s2, M, n);
+    const float f = __fdividef((float)p2, (float)s2);
+    int lo = 0, hi = n;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (f >= F[mid]) lo = mid; else hi = mid;
+    }
+    while (lo > 0 && !(p2 >= __dmul_rn(M[lo], s2))) --lo;
+    while (lo + 1 < n && p2 >= __dmul_rn(M[lo + 1], s2)) ++lo;
     return lo;
 }
 
-// Build the j-segments of stencil rows [r0, r1) for the i-cell (ax, ay, az).
-// seg = {first point, length, dy | dz << 16, image code}.
-__device__ __forceinline__ void build_segments(const PairParams &p, const GridDev &gj, int ax,
-                                               int ay, int az, int r0, int r1, int4 *seg,
-                                               int *s_nseg) {
-    const int nx = p.g.ng[0], ny = p.g.ng[1], nz = p.g.ng[2];
-    for (int row = r0 + (int)threadIdx.x; row < r1; row += NT) {
-        int4 st = p.stencil[row];
-        int dy = st.x, dz = st.y;
-        int y = ay + dy, z = az + dz, wy = 0, wz = 0;
-        if (y < 0) { if (!p.g.periodic) continue; y += ny; wy = -1; }
-        else if (y >= ny) { if (!p.g.periodic) continue; y -= ny; wy = 1; }
-        if (z < 0) { if (!p.g.periodic) continue; z += nz; wz = -1; }
-        else if (z >= nz) { if (!p.g.periodic) continue; z -= nz; wz = 1; }
-        const int rowbase = (z * ny + y) * nx;
-        const int x0 = ax + st.z, x1 = ax + st.w;
-        int pc0[3], pc1[3], pw[3], np = 0;
-        if (p.g.periodic) {
-            if (x0 < 0) { pc0[np] = x0 + nx; pc1[np] = min(x1, -1) + nx; pw[np++] = -1; }
-            int m0 = max(x0, 0), m1 = min(x1, nx - 1);
-            if (m0 <= m1) { pc0[np] = m0; pc1[np] = m1; pw[np++] = 0; }
-            if (x1 >= nx) { pc0[np] = max(x0, nx) - nx; pc1[np] = x1 - nx; pw[np++] = 1; }
-        } else {
-            int m0 = max(x0, 0), m1 = min(x1, nx - 1);
-            if (m0 <= m1) { pc0[np] = m0; pc1[np] = m1; pw[np++] = 0; }
-        }
-        const int meta = (dy & 0xFFFF) | (dz << 16);
-        for (int q = 0; q < np; ++q) {
-            int a0 = gj.cell_start[rowbase + pc0[q]];
-            int a1 = gj.cell_start[rowbase + pc1[q] + 1];
-            if (a1 > a0) {
-                int slot = atomicAdd(s_nseg, 1);
-                seg[slot] = make_int4(a0, a1 - a0, meta, (pw[q] + 1) * 9 + (wy + 1) * 3 + (wz + 1));
-            }
-        }
+// Bin of an in-reach pair from its separation d (a, b: the positions, for the
+// midpoint line of sight); -1 outside.
+template <int MODE, int LOS>
+__device__ __forceinline__ int bin64(double d0, double d1, double d2, double s2, const double *a, const double *b,
+                                     const F64Edges &E, int na, int nb) {
+    if (MODE == MODE_S) {
+        if (!(s2 >= E.Ea[0] && s2 < E.Ea[na])) return -1;
+        return locate64(s2, E.Ea, E.Fa, na);
     }
+    double p2;
+    if (LOS == LOS_Z) {
+        p2 = __dmul_rn(d2, d2);
+    } else {
+        const double l0 = __dadd_rn(a[0], b[0]), l1 = __dadd_rn(a[1], b[1]), l2 = __dadd_rn(a[2], b[2]);
+        const double sl = __dadd_rn(__dadd_rn(__dmul_rn(d0, l0), __dmul_rn(d1, l1)), __dmul_rn(d2, l2));
+        const double ll = __dadd_rn(__dadd_rn(__dmul_rn(l0, l0), __dmul_rn(l1, l1)), __dmul_rn(l2, l2));
+        p2 = (ll > 0.0) ? __ddiv_rn(__dmul_rn(sl, sl), ll) : 0.0;
+    }
+    if (MODE == MODE_SMU) {
+        if (!(s2 >= E.Ea[0] && s2 < E.Ea[na])) return -1;
+        const int k = locate64(s2, E.Ea, E.Fa, na);
+        const int j = (s2 > 0.0) ? locate64_mu(p2, s2, E.Eb, E.Fb, nb) : 0;
+        return k * nb + j;
+    }
+    double q2 = __dsub_rn(s2, p2);
+    if (q2 < 0.0) q2 = 0.0;
+    if (!(q2 >= E.Ea[0] && q2 < E.Ea[na])) return -1;
+    if (!(p2 >= E.Eb[0] && p2 < E.Eb[nb])) return -1;
+    return locate64(q2, E.Ea, E.Fa, na) * nb + locate64(p2, E.Eb, E.Fb, nb);
 }
 
-// ---------------------------------------------------------------------------
-// plain FP64 kernel: the binary64 definition for every candidate pair
-// ---------------------------------------------------------------------------
 template <int MODE, int LOS, bool W>
-__global__ void __launch_bounds__(NT) k_pairs_f64(const __grid_constant__ PairParams p) {
+__global__ void __maxnreg__(96) k_pairs_f64(const __grid_constant__ PairParams p) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int s_blk, s_nseg, s_tmp[8];
+    __shared__ RangeShared s_range;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
+    using O = WarpOff<false, false, true>;
+    unsigned char *ws = smem + p.sm_warp + (size_t)warp * O::total;
+    int4 *seg = reinterpret_cast<int4 *>(ws);
+    double *tile = reinterpret_cast<double *>(ws + O::tile);   // {x, y, z, w, shift x, y, z} by point
+    int4 *ring = reinterpret_cast<int4 *>(ws + O::ring);
+    int *pref = reinterpret_cast<int *>(ws + O::pref);
+    double *sEa = reinterpret_cast<double *>(smem + p.sm_lut), *sEb = sEa + p.n_a + 1;
+    float *sF = reinterpret_cast<float *>(sEb + p.n_b + 1);
+    F64Edges E{sEa, sEb, p.sm_guess ? sF : nullptr, p.sm_guess ? sF + p.n_a + 1 : nullptr};
 
-    const SmemLayout64 Ly = f64_layout(p);
-    double *s_Ea = (double *)(smem + Ly.ea);
-    double *s_Eb = (double *)(smem + Ly.eb);
-    int *s_hist = (int *)(smem + Ly.hist);
-    double *s_whist = (double *)(smem + Ly.whist);
-    int4 *s_seg = (int4 *)(smem + Ly.seg);
-    double4_32a *s_tile = (double4_32a *)(smem + Ly.tile);
-    int2 *s_meta = (int2 *)(smem + Ly.meta);
-
-    const int tid = threadIdx.x;
-    for (int k = tid; k <= p.n_a; k += NT) s_Ea[k] = p.Ea[k];
-    for (int k = tid; k <= p.n_b; k += NT) s_Eb[k] = p.Eb[k];
-    if (p.smem_hist_ok) {
-        for (int k = tid; k < p.nent * p.hist_k; k += NT) s_hist[k] = 0;
-        if (W) for (int k = tid; k < p.nent * p.hist_k; k += NT) s_whist[k] = 0.0;
+    for (int k = threadIdx.x; k < p.sm_lut / 4; k += blockDim.x) reinterpret_cast<unsigned *>(smem)[k] = 0u;
+    for (int k = threadIdx.x; k <= p.n_a; k += blockDim.x) {
+        sEa[k] = p.Ea[k];
+        if (p.sm_guess) sF[k] = (float)p.Ea[k];
     }
-    const int K = p.hist_k, lane_copy = tid & (K - 1);
-    int *my_hist = s_hist + lane_copy;
-    double *my_whist = s_whist + lane_copy;
-    const int nx = p.g.ng[0], ny = p.g.ng[1];
-    const int nblocks = *p.nblocks;
-    unsigned long long cand_local = 0, since_flush = 0;
-    int cur_hist = -1;
-    auto flush_cta = [&](int h) {
-        __syncthreads();
-        if (p.smem_hist_ok && h >= 0) {
-            flush_counts(p, (int)Ly.hist, tid >> 5, NT / 32, h);
-            if (W) flush_weights(p, (int)Ly.whist, tid >> 5, NT / 32, h, 0.0);
-        }
-        __syncthreads();
-    };
+    for (int k = threadIdx.x; k <= p.n_b; k += blockDim.x) {
+        sEb[k] = p.Eb[k];
+        if (p.sm_guess) sF[p.n_a + 1 + k] = (float)p.Eb[k];
+    }
+    if (threadIdx.x == 0) s_range = RangeShared{0, 0, 0, 0, -1};
+    int *hist = reinterpret_cast<int *>(smem);
+    double *whist = reinterpret_cast<double *>(smem + p.sm_whist);
+    const int K = p.hist_k, kc = lane & (K - 1);
+    Items items;
+    items.init(p, nw);
+    unsigned long long cand = 0, pruned = 0;
+    unsigned since = 0;                              // j-points since this warp's last flush
+    const unsigned flush_j = (unsigned)(FLUSH_LIMIT / BI / nw);
     __syncthreads();
+    // squared reach, with the rounding of the squares (sigma^2 + pi^2 for both)
+    const double reach2 = (MODE == MODE_SIGPI ? sEa[p.n_a] + sEb[p.n_b] : sEa[p.n_a]) * (1.0 + 1e-12);
 
     for (;;) {
-        if (tid == 0) s_blk = atomicAdd(p.work_counter, 1);   // the list holds only this shard's blocks
-        __syncthreads();
-        const int bidx = s_blk;
-        if (bidx >= nblocks) break;
-        const Block B = p.blocks[bidx];
-        const TaskDev &T = p.tasks[B.task];
-        if (T.hist != cur_hist) {
-            flush_cta(cur_hist);
-            cur_hist = T.hist;
-            since_flush = 0;
-        }
-        const size_t hbase = (size_t)T.hist * p.nbins;
-        const int ax = B.cell % nx, ay = (B.cell / nx) % ny, az = B.cell / (nx * ny);
-        const bool have_i = tid < B.count;   // FP64 path: one i-point per thread
-        const int ii = B.start + tid;
-        double4_32a a = have_i ? T.gi.xw[ii] : make_double4_32a(0, 0, 0, 0);
-
-        auto add = [&](int bin, double wj) {
+        auto flush = [&](int old) {
             if (p.smem_hist_ok) {
-                atomicAdd(&my_hist[bin * K], 1);
-                if (W) atomicAdd(&my_whist[bin * K], __dmul_rn(a.w, wj));
-            } else {
-                atomicAdd(&p.hist[hbase + bin], 1ull);
-                if (W) atomicAdd(&p.whist[hbase + bin], __dmul_rn(a.w, wj));
+                flush_counts(p, 0, warp, nw, p.tasks[old].hist);
+                if (W) flush_weights(p, p.sm_whist, warp, nw, p.tasks[old].hist, 0.0);
             }
+            since = 0;
+            __syncthreads();
         };
-        auto eval = [&](const double4_32a &b, int img) {
-            int bin = f64_pair_bin<MODE, LOS>(a, b, img, p.g, s_Ea, p.n_a, s_Eb, p.n_b);
-            if (bin >= 0) add(bin, b.w);
-        };
-
-        if (T.is_auto) {
-            for (int f = tid; f < B.count; f += NT) {
-                int pj = B.start + f;
-                s_tile[f] = T.gj.xw[pj];
-                s_meta[f] = make_int2(pj, 13);
-            }
-            __syncthreads();
-            if (have_i)
-                for (int jj = tid + 1; jj < B.count; ++jj) eval(s_tile[jj], 13);
-            if (tid == 0) cand_local += (unsigned long long)B.count * (B.count - 1) / 2;
-            since_flush += (unsigned long long)B.count * B.count;
-            __syncthreads();
-        }
-        const int cell_end = T.gi.cell_start[B.cell + 1];
-        for (int r0 = 0; r0 < p.nrows; r0 += ROWCHUNK) {
-            const int r1 = min(r0 + ROWCHUNK, p.nrows);
-            if (tid == 0) {
-                int ns = 0;
-                if (T.is_auto && r0 == 0 && cell_end > B.start + B.count) {
-                    s_seg[0] = make_int4(B.start + B.count, cell_end - B.start - B.count, 0, 13);
-                    ns = 1;
-                }
-                s_nseg = ns;
-            }
-            __syncthreads();
-            build_segments(p, T.gj, ax, ay, az, r0, r1, s_seg, &s_nseg);
-            __syncthreads();
-            const int nseg = s_nseg;
-            __syncthreads();                 // every thread has read nseg before it changes
-            if (nseg == 0) continue;
-            const int total = seg_scan(s_seg, nseg, s_tmp);
-            for (int t0 = 0; t0 < total; t0 += TJ64) {
-                const int len = min(TJ64, total - t0);
-                for (int f = tid; f < len; f += NT) {
-                    int k = seg_find(s_seg, nseg, t0 + f);
-                    int4 sg = s_seg[k];
-                    int pj = sg.x + (t0 + f - sg.y);
-                    s_tile[f] = T.gj.xw[pj];
-                    s_meta[f] = make_int2(pj, sg.w);
-                }
-                __syncthreads();
-                if (have_i)
-                    for (int jj = 0; jj < len; ++jj) eval(s_tile[jj], s_meta[jj].y);
-                if (tid == 0) cand_local += (unsigned long long)len * B.count;
-                since_flush += (unsigned long long)len * B.count;
-                __syncthreads();
-                if (since_flush > FLUSH_LIMIT) {
-                    flush_cta(cur_hist);
-                    since_flush = 0;
-                }
+        const long long id = next_item(p, items, s_range, flush);
+        if (id < 0) break;
+        Item it;
+        if (!open_item<false>(p, items, id, it)) continue;
+        const TaskDev &T = p.tasks[it.B.task];
+        const size_t hbase = (size_t)T.hist * p.nbins;
+        double a[2][3], wi[2];
+        IBox box;
+        box.clear();
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            a[r][0] = a[r][1] = a[r][2] = __longlong_as_double(0x7ff8000000000000ll);   // no point: not a number
+            wi[r] = 0.0;
+            if (2 * lane + r < it.count) {
+                const double4_32a q = T.gi.xw[it.start + 2 * lane + r];
+                a[r][0] = q.x; a[r][1] = q.y; a[r][2] = q.z;
+                wi[r] = q.w;
+                box.add(T.gi, q);
             }
         }
-        __syncthreads();
+        box.finish(T);
+        bool own = T.is_auto && it.part == 0;
+        if (own && lane == 0) cand += (unsigned long long)it.count * (unsigned)(it.count - 1) / 2;
+        const int nchunk = max(1, (it.ntl + 31) / 32);
+        int round0 = 0;
+        for (int ch = 0; ch < nchunk; ++ch) {
+            __syncwarp();
+            int nseg;
+            const int noct = build_chunk<false>(p, T, it, ch, seg, nullptr, pref, nseg);
+            __syncwarp();
+            const int nround = (noct + 31) / 32;
+            int rd = (it.part - round0 % items.S + items.S) % items.S;
+            round0 += nround;
+            int head = 0, tail = 0;
+            for (;;) {
+                while (!own && tail - head < JO && rd < nround) {
+                    tail = ring_round<MODE, LOS>(p, T, rd, noct, nseg, seg, pref, box, it.count, ring, tail, cand,
+                                                 pruned);
+                    rd += items.S;
+                }
+                const int m = own ? (it.count + 7) >> 3 : min(JO, tail - head);
+                if (m == 0) break;
+                bool shifted = false;
+#pragma unroll
+                for (int h = 0; h < JB / 32; ++h) {
+                    const int sl = lane + 32 * h, oc = sl >> 3;
+                    int pj = it.start + sl, img = 13;
+                    bool v = own && sl < it.count;
+                    if (!own && oc < m) {
+                        const int4 e = ring[(head + oc) & (RING - 1)];
+                        const int4 sg = seg[e.y];
+                        pj = e.x + (lane & 7);
+                        v = pj >= sg.x && pj < sg.y;
+                        img = sg.w;
+                    }
+                    double4_32a q = make_double4_32a(0.0, 0.0, 0.0, 0.0);
+                    q.x = __longlong_as_double(0x7ff8000000000000ll);
+                    if (v) q = T.gj.xw[pj];
+                    double *t = tile + 7 * sl;
+                    t[0] = q.x; t[1] = q.y; t[2] = q.z; t[3] = q.w;
+                    // d - L is d + (-L), and d + 0 is d
+                    t[4] = (double)(img / 9 - 1) * p.g.L[0];
+                    t[5] = (double)((img / 3) % 3 - 1) * p.g.L[1];
+                    t[6] = (double)(img % 3 - 1) * p.g.L[2];
+                    shifted = shifted || (p.g.periodic && img != 13);
+                }
+                shifted = __any_sync(FULL, shifted);
+                __syncwarp();
+                since += 8 * m;
+                if (since > flush_j && p.smem_hist_ok) {
+                    flush_counts(p, 0, 0, 1, T.hist);
+                    since = 8 * m;
+                }
+                for (int j = 0; j < 8 * m; ++j) {
+                    const double *t = tile + 7 * j;
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        double d0 = __dsub_rn(t[0], a[r][0]), d1 = __dsub_rn(t[1], a[r][1]),
+                               d2 = __dsub_rn(t[2], a[r][2]);
+                        if (shifted) {
+                            d0 = __dadd_rn(d0, t[4]);
+                            d1 = __dadd_rn(d1, t[5]);
+                            d2 = __dadd_rn(d2, t[6]);
+                        }
+                        const double s2 =
+                            __dadd_rn(__dadd_rn(__dmul_rn(d0, d0), __dmul_rn(d1, d1)), __dmul_rn(d2, d2));
+                        bool in = s2 < reach2;
+                        if (own) in = in && j > 2 * lane + r;
+                        if (in) {
+                            const int b = bin64<MODE, LOS>(d0, d1, d2, s2, a[r], t, E, p.n_a, p.n_b);
+                            if (b >= 0) {
+                                if (p.smem_hist_ok) {
+                                    atomicAdd(&hist[b * K + kc], 1);
+                                    if (W) atomicAdd(&whist[b * K + kc], __dmul_rn(wi[r], t[3]));
+                                } else {
+                                    atomicAdd(&p.hist[hbase + b], 1ull);
+                                    if (W) atomicAdd(&p.whist[hbase + b], __dmul_rn(wi[r], t[3]));
+                                }
+                            }
+                        }
+                    }
+                }
+                if (!own) head += m;
+                own = false;
+                __syncwarp();
+            }
+        }
     }
-    flush_cta(cur_hist);
-    if (tid == 0 && cand_local) atomicAdd(&p.counters[0], cand_local);
+    __syncthreads();
+    if (!p.multi && p.smem_hist_ok) {
+        flush_counts(p, 0, warp, nw, 0);
+        if (W) flush_weights(p, p.sm_whist, warp, nw, 0, 0.0);
+    }
+    cand = warp_sum_u64(cand);
+    pruned = warp_sum_u64(pruned);
+    if (lane == 0 && cand) atomicAdd(&p.counters[0], cand);
+    if (lane == 0 && pruned) atomicAdd(&p.counters[3], pruned);
 }
 
 // ---------------------------------------------------------------------------
@@ -1888,7 +1968,7 @@ cudaError_t launch_mode_f64(const PairParams &p, int grid, size_t smem, cudaStre
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     if (grid <= 0) return cudaSuccess;
-    k<<<grid, NT, smem, st>>>(p);
+    k<<<grid, 32 * p.nwarps, smem, st>>>(p);
     note_launch();
     return cudaGetLastError();
 }
@@ -1899,7 +1979,7 @@ int occupancy_mode_f64(const PairParams &p, size_t smem) {
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return 0;
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, NT, smem) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, 32 * p.nwarps, smem) != cudaSuccess) return 0;
     return nb;
 }
 

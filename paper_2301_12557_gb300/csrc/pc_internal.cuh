@@ -13,11 +13,7 @@ namespace pc {
 // ---------------------------------------------------------------------------
 // launch geometry of the pair kernels
 // ---------------------------------------------------------------------------
-constexpr int NT = 128;        // threads per CTA (FP64 path); blocks hold NT * ipt points
-constexpr int TJ64 = 128;      // j points per tile (FP64 path)
-constexpr int MAXSEG = 256;    // j segments per chunk of stencil rows (FP64 path)
-constexpr int ROWCHUNK = 84;   // stencil rows per chunk (<= 3 segments each)
-static_assert(3 * ROWCHUNK + 1 <= MAXSEG, "a chunk's segments (and the own-cell rest) fit");
+constexpr int NT = 128;        // blocks hold up to NT * ipt points (FP64 path: NT)
 constexpr int MAX_LUT = 8192;  // LUT entries per histogram axis
 // integer weight path: largest exponent range of one catalogue's weights
 // (the packed significand M << range fits 32 bits), and of two catalogues'
@@ -152,6 +148,7 @@ struct PairParams {
     int hs, nent;
     // layout of a CTA (bytes): weight sums, tables, the warps' slices
     int sm_whist, sm_lut, sm_warp, nwarps;
+    int f64, sm_guess;       // FP64 kernel; with FP32 roundings of the edges
     // box tests: squared distance from which an oct is dropped, and for
     // (sigma, pi) along z the cylinder's squared radius and half length, all
     // with the tests' rounding added; far: coordinate of absent points
@@ -229,8 +226,7 @@ cudaError_t launch_pairs_f64(const PairParams &p, int grid, size_t smem, cudaStr
 cudaError_t launch_rescue(const PairParams &p, cudaStream_t st);
 cudaError_t launch_pairs_f32(const PairParams &p, int grid, size_t smem,
                              cudaStream_t st);   // p.tree selects the tree variant
-size_t pairs_f32_smem(PairParams &p, int nwarps);   // fills in p's layout
-size_t pairs_f64_smem(const PairParams &p);
+size_t pairs_smem(PairParams &p, int nwarps);   // fills in p's layout (both precisions)
 int pairs_f32_ctas_per_sm(const PairParams &p, size_t smem);
 int pairs_f64_ctas_per_sm(const PairParams &p, size_t smem);
 

@@ -95,7 +95,7 @@ typedef struct {
  * (every field 0). */
 typedef struct {
     int prec;                    /* pc_prec: FP32 with FP64 rescue (0) or plain FP64 */
-    double cell_size;            /* grid cell side; 0 = chosen by the cost model */
+    double cell_size;            /* grid cell side; 0 = chosen from density and reach */
     int ipt;                     /* points of a block: 128 ipt (2 or 4; 0 = auto); the FP32
                                     kernel deals a block to warps 64 points at a time */
     int priv;                    /* shared-histogram replication: 2 = one shared copy where the

@@ -106,7 +106,8 @@ static Workspace &workspace(int dev) {
 // ---------------------------------------------------------------------------
 // plan: bins, error bands, lookup tables, stencil
 // ---------------------------------------------------------------------------
-enum { PLAN_LUT = 0, PLAN_LIN = 1, PLAN_LINOFF = 2, PLAN_LOG = 3, PLAN_FIX = 5 };   // PATH_* of the kernel
+enum { PLAN_LUT = 0, PLAN_LIN = 1, PLAN_LINOFF = 2, PLAN_LOG = 3,   // PATH_* of the kernel
+       PLAN_FIX = 5, PLAN_FIXOFF = 6, PLAN_FIXLOG = 7 };
 
 struct Plan {
     int mode = 0, los = 0, na = 0, nb = 1, nbins = 0;
@@ -131,11 +132,12 @@ struct Plan {
     // of logarithms (the lin fields; also for mu along the midpoint line of
     // sight, which lin leaves out)
     int path = PLAN_LUT;
-    // fixed-point floors: bands in units of 2^-16 (first axis; pi of (sigma, pi);
-    // mu, fx_mA / s + fx_mB) and the separation the mu band stops growing at
+    // fixed-point floors (fix: PLAN_FIX*, or 0): scales, the first axis's constant
+    // without its band, bands in units of 2^-16 (first axis, fx_sA / s for
+    // logarithms; pi of (sigma, pi); mu, fx_mA / s + fx_mB), and the separation the
+    // mu band stops growing at
     int fix = 0;
-    unsigned fx_s = 0, fx_p = 0;
-    double fx_mA = 0, fx_mB = 0, fx_sf = 0;
+    double fx_c = 128.0, fx_inv = 0, fx_invB = 0, fx_s = 0, fx_sA = 0, fx_p = 0, fx_mA = 0, fx_mB = 0, fx_sf = 0;
 };
 
 static bool edges_ok(const double *e, int n, bool zero_one) {
@@ -508,45 +510,78 @@ static pc_status make_plan(const pc_bins *b, const Geom &g, const double *pts_lo
             P.path = PLAN_LIN;
         }
     }
-    // ---- fixed-point floors (PATH_FIX) ---------------------------------------
-    // The values of the floors from zero, summed once onto a grid of 2^-16: the
-    // band in these units, with half a unit for that sum.  Along z the bounds
-    // above are used with a factor of 1.25 instead of 2: per axis u (2.5 c +
-    // 3 |d|), hence s errs by u (4.33 c + 3 s), the squares' roundings add 1.5 u
-    // s, the reciprocal root 2.15 u s, and the scale and its product 2 u s (the
-    // last product is exact); mu by u (6.83 c / s + 3 + 3 + 1.5 + 2.15 + 1).
-    if (P.path == PLAN_LIN && P.na <= 126 && P.nb <= 126) {
+    // ---- fixed-point floors (PATH_FIX*) ---------------------------------------
+    // The values of the floors, summed once onto a grid of 2^-16: the band in
+    // these units, with half a unit for that sum (and with an offset another for
+    // the constant's rounding, below 256).  Along z the linear bounds above are
+    // used with a factor of 1.25 instead of 2: per axis u (2.5 c + 3 |d|), hence s
+    // errs by u (4.33 c + 3 s), the squares' roundings add 1.5 u s, the reciprocal
+    // root 2.15 u s, and the scale and its product 2 u s (the last product is
+    // exact); mu by u (6.83 c / s + 3 + 3 + 1.5 + 2.15 + 1).
+    {
         const double one = 65536.0;
-        double es = 0.0, ep = 0.0;
+        const double na = P.na, nb = P.nb;
+        int kind = P.path == PLAN_LIN ? PLAN_FIX : (P.path == PLAN_LINOFF ? PLAN_FIXOFF
+                                                    : (P.path == PLAN_LOG ? PLAN_FIXLOG : 0));
+        const double D = (P.ea[P.na] - P.ea[0]) / na;
+        bool ok = true;
+        // edges evenly spaced from zero (second axis of (sigma, pi)), and
+        // logarithmic sigma edges: dt = d sigma / (sigma ln q), sigma >= e_0 / 2
+        double Db = D, lq = 0.0;
         if (P.mode == PC_BIN_SIGPI) {
-            const double Da = P.ea[P.na] / P.na, Db = P.eb[P.nb] / P.nb;
-            es = eps_sig / Da + 1e-9 + 4.0 * u * P.na;
-            ep = eps_z / Db + 1e-9 + 4.0 * u * P.nb;
-        } else {
-            const double D = P.ea[P.na] / P.na;
-            es = (1.25 * u * (4.34 * c + 8.7 * Rb) + tiny) / D + 1e-9;
+            Db = P.eb[P.nb] / nb;
+            double devb = 0.0;
+            for (int k = 0; k <= P.nb; ++k) devb = std::max(devb, fabs(P.eb[k] - k * Db));
+            if (!kind && P.fp32_ok && P.ea[0] > 0.0 && P.eb[0] == 0.0 && devb <= 1e-9 * Db) {
+                lq = log2(P.ea[P.na] / P.ea[0]) / na;
+                double dev = 0.0;
+                for (int k = 0; k <= P.na; ++k) dev = std::max(dev, fabs(log2(P.ea[k] / P.ea[0]) / lq - k));
+                if (dev <= 1e-6 && eps_sig < 0.05 * P.ea[0]) kind = PLAN_FIXLOG;
+            }
+            P.fx_invB = 1.0 / Db;
+            P.fx_p = ceil((eps_z / Db + 1e-9 + 4.0 * u * nb) * one + 0.5);
+            ok = ok && P.fx_p < 8192.0;
         }
-        P.fx_s = (unsigned)ceil(es * one + 0.5);
-        P.fx_p = (unsigned)ceil(ep * one + 0.5);
-        bool ok = es * one < 8192.0 && ep * one < 8192.0;
+        if (kind == PLAN_FIXLOG) {
+            const double e0 = P.ea[0];
+            if (lq == 0.0) lq = log2(P.ea[P.na] / e0) / na;
+            const double ln2 = log(2.0), A = 1.0 / (2.0 * lq), B = -log2(e0) / lq;
+            const double Lmax = std::max(fabs(log2(P.rcut * P.rcut)), fabs(log2(0.25 * e0 * e0)));
+            const double common = A * ldexp(1.0, -21) * std::max(1.0, Lmax) +
+                                  u * (A * Lmax + fabs(B) + na + 130.0) * 2.0 + 1e-6 + A * ldexp(1.0, -45);
+            P.fx_inv = A;
+            P.fx_c = 129.0 + B;
+            if (P.mode == PC_BIN_SIGPI) {
+                P.fx_sA = 1.12 * eps_sig / (lq * ln2) * one;
+                P.fx_s = 2.0 * common * one + 2.0;
+            } else {
+                P.fx_sA = 2.0 * A * 2.0 * (4.4 * u * c + ldexp(X + Lm + R0, -51)) / ln2 * 1.01 * one;
+                P.fx_s = 2.0 * (A * 9.0 * u / ln2 * 1.01 + common) * one + 2.0;
+            }
+            P.fx_sA *= 1.001;
+            ok = ok && e0 > 1e-9 && eps_s < 0.05 * e0 && fabs(P.fx_c) < 250.0 && P.fx_sA / (0.5 * e0) + P.fx_s < 8192.0 && na <= 125;
+        } else if (kind) {
+            const double es = P.mode == PC_BIN_SIGPI
+                                  ? eps_sig / D + 1e-9 + 4.0 * u * na
+                                  : (1.25 * u * (4.34 * c + 8.7 * Rb) + tiny) / D + 1e-9;
+            P.fx_inv = 1.0 / D;
+            P.fx_c = kind == PLAN_FIX ? 128.0 : 129.0 - P.ea[0] / D;
+            P.fx_s = ceil(es * one + (kind == PLAN_FIX ? 0.5 : 1.5));
+            ok = ok && P.fx_s < 8192.0 && (kind == PLAN_FIX || (na <= 125 && fabs(P.fx_c) < 250.0));
+        }
         if (P.mode == PC_BIN_SMU) {
-            const double nb = P.nb;
             const double mA = P.los == PC_LOS_Z ? 1.25 * 6.9 * u * c + tiny : muA;
             const double mB = P.los == PC_LOS_Z ? 1.25 * 10.7 * u + ldexp(1.0, -46) : muB + 4.0 * u;
-            // the box tests' gap, less than 2^-20 X off, bounds s from below:
-            // within 1 % from 128 times that on (and the band's own roundings)
-            double ext = 0.0;
-            for (int a = 0; a < 3; ++a) ext = std::max(ext, (pts_hi[a] - pts_lo[a]) + g.L[a]);
-            P.fx_sf = std::max({c / 16.0, ldexp(ext, -13) + ldexp(X + Lm, -40), 1e-3 * R0});
-            P.fx_mA = nb * mA * one * 1.02;
-            P.fx_mB = nb * mB * one * 1.02 + 1e-12 * nb * one + 0.5 + 0.5;
+            P.fx_invB = nb;   // mu = 1 may land in column n_mu: near, put right there
+            P.fx_sf = std::max(c / 16.0, 1e-3 * R0);
+            P.fx_mA = nb * mA * one * 1.001;
+            P.fx_mB = nb * mB * one * 1.001 + 1e-12 * nb * one + 1.0;
             ok = ok && P.fx_mA / P.fx_sf + P.fx_mB < 8192.0;
         }
         // no FP32 square may overflow (the kernel's indices rely on it), and the
         // constant 1e-30 in the squares must stay far inside the first band
-        const double Dmin = std::min(P.ea[P.na] / P.na, P.mode == PC_BIN_SIGPI ? P.eb[P.nb] / P.nb : 1e300);
-        ok = ok && X + Lm + R0 + c < 1e15 && Dmin > 1e-9;
-        P.fix = ok ? 1 : 0;
+        ok = ok && X + Lm + R0 + c < 1e15 && std::min({D, Db, P.ea[1]}) > 1e-9 && na <= 126 && nb <= 126;
+        P.fix = ok ? kind : 0;
     }
     // ---- stencil -------------------------------------------------------------
     int kmax[3] = {0, 0, 0};
@@ -777,19 +812,31 @@ static void set_fp32_params(const Geom &g, const double *lo, const double *hi, c
     {
         auto two = [](float v) { return make_float2(v, v); };
         const double one = 65536.0;
-        p.fix = (p.path == PLAN_LIN && P.fix) ? 1 : 0;
+        p.fix = prec == PC_PREC_F32_RESCUE ? P.fix : 0;
+        p.row0 = 0;
+        const bool off = P.fix == PLAN_FIXOFF || P.fix == PLAN_FIXLOG;
+        p.f_inv = (float)P.fx_inv;
+        p.f_invB = (float)P.fx_invB;
         p.f_tiny = two(1e-30f);
-        p.f_cfs = two((float)(128.0 + P.fx_s / one));
+        p.f_cfs = two((float)(P.fx_c + (P.fix == PLAN_FIXLOG ? 0.0 : P.fx_s / one)));
+        p.f_ts2 = 2 * (unsigned)ceil(P.fx_s);
         p.f_cfp = (float)(128.0 + P.fx_p / one);
-        p.f_lim = 128.5f + (float)P.na;
+        p.f_tp2 = 2 * (unsigned)P.fx_p;
+        p.f_lim = (off ? 129.5f : 128.5f) + (float)P.na;
         p.f_limB = 128.5f + (float)P.nb;
-        p.f_ts2 = 2 * P.fx_s;
-        p.f_tp2 = 2 * P.fx_p;
         p.f_mA = nextafterf((float)P.fx_mA, INFINITY);
         p.f_mB = nextafterf((float)P.fx_mB, INFINITY);
-        // pairs closer than fx_sf: t below it, with the band and the clamp's side
+        p.f_sA = nextafterf((float)P.fx_sA, INFINITY);
+        p.f_sC = nextafterf((float)P.fx_s, INFINITY);
+        p.f_se2 = (float)(0.25 * P.ea[0] * P.ea[0]);
+        // pairs closer than fx_sf: t below it (none where that is below the first
+        // edge: they are out of range)
         p.f_sf2 = (float)(P.fx_sf * P.fx_sf);
-        p.f_close = (float)(128.0 + 2.0 * P.fx_s / one + P.fx_sf * (1.0 + 1e-6) * P.lin_invA);
+        double tsf = P.fx_sf * (1.0 + 1e-6);
+        if (P.fix == PLAN_FIXLOG) tsf = tsf > P.ea[0] ? 2.0 * log2(tsf) * P.fx_inv : -1e3;
+        else tsf *= P.fx_inv;
+        p.f_close = (float)(P.fx_c + tsf + 0.01);
+        if (off && p.f_close < 129.0f) p.f_close = 0.0f;
         for (int a = 0; a < 3; ++a) p.L32[a] = (float)g.L[a];
     }
     // Box tests run in FP32 on coordinates relative to the grids' origins, at
@@ -805,6 +852,7 @@ static void set_fp32_params(const Geom &g, const double *lo, const double *hi, c
         c = std::max(c, g.c[a]);
     }
     const double m = ldexp(X, -19) + ldexp(A, -49);
+    p.f_gm = nextafterf((float)m, INFINITY);
     auto up = [&](double r) {
         const double v = (r + m) * (r + m) * (1.0 + ldexp(1.0, -20));
         return v < 1e38 ? nextafterf((float)v, INFINITY) : INFINITY;
@@ -839,9 +887,11 @@ static pc_status fit_params(int prec, int opt_priv, int dev, bool weighted, bool
         p.wcorr = (wint && wcorr) ? 1 : 0;
         p.path = path0;
         p.layout = 0;
+        p.row0 = 0;
         choose_replication(opt_priv, p.nbins, weighted && !wint, p.hist_k);
         if (p.fix && (wint || !weighted)) {   // fixed-point floors (not for binary64 weight sums)
-            p.path = PLAN_FIX;
+            p.path = p.fix;
+            p.row0 = p.fix == PLAN_FIX ? 0 : 1;
             if (p.mode == PC_BIN_S) {
                 p.layout = 2;
                 p.hist_k = 32;
@@ -850,7 +900,7 @@ static pc_status fit_params(int prec, int opt_priv, int dev, bool weighted, bool
                 p.hist_k = 1;
             } else {   // mu = 1 (pi past its last bin) needs a column of its own
                 p.hs = p.n_b + 1;
-                p.nent = p.n_a * p.hs + 1 + p.n_b;
+                p.nent = (p.n_a + p.row0) * p.hs + 1 + p.n_b;
                 while (p.hs * p.hist_k > 255) p.hist_k /= 2;   // one byte (f_coef)
             }
         }
@@ -866,6 +916,7 @@ static pc_status fit_params(int prec, int opt_priv, int dev, bool weighted, bool
             p.smem_hist_ok = 0;
             p.path = PLAN_LUT;
             p.layout = 0;
+            p.row0 = 0;
             p.lut_total = f64 ? 0 : lut_size;
             p.hist_k = 1;
             // many edges: no FP32 roundings beside them
@@ -887,11 +938,11 @@ static pc_status fit_params(int prec, int opt_priv, int dev, bool weighted, bool
         p.c_23 = two(8388608.0f);
         p.c_p = two(8388607.5f);
         p.c_m1 = two(-1.0f);
-        p.c_invA = two(p.lin_invA);
+        p.c_invA = two(p.path >= PLAN_FIX ? p.f_inv : p.lin_invA);
         p.c_offA = two(p.lin_offA);
         p.c_thrA = two(p.lin_thrA);
         p.c_nmS = two(-p.lin_mS);
-        p.c_invB = two(p.mode == PC_BIN_SIGPI ? p.lin_invB2 : p.lin_nB);
+        p.c_invB = two(p.path >= PLAN_FIX ? p.f_invB : (p.mode == PC_BIN_SIGPI ? p.lin_invB2 : p.lin_nB));
         p.c_nmB = two(-p.lin_mA);
         p.c_cB = two(p.mode == PC_BIN_SIGPI ? p.lin_thrB : p.lin_cB);
         p.c_nrow = two(-row);
@@ -972,7 +1023,7 @@ static pc_status make_params(const CountJob &J, const CountSetup &S, const DevBu
     // copies (more than a few hundred bins) a copy would be flushed every few
     // hundred j-points, so its records are folded into the CTA's exact sums
     // instead (fold mode)
-    const bool wint_try = S.weighted && p.path != PLAN_LUT && J.wint_ok && S.prec == PC_PREC_F32_RESCUE;
+    const bool wint_try = S.weighted && (p.path != PLAN_LUT || p.fix) && J.wint_ok && S.prec == PC_PREC_F32_RESCUE;
     int per_sm = 0;
     pc_status s = fit_params(S.prec, S.o.priv, S.dev, S.weighted, wint_try, J.wcorr, p, smem, per_sm);
     if (s != PC_OK) return s;

@@ -59,7 +59,7 @@ constexpr int JB = 64;        // j-points per staged batch (eight octs)
 constexpr int JO = JB / 8;
 constexpr int RING = 64;      // octs kept for staging (ring): up to JO - 1 + 32
 constexpr int QCAP = 64;      // near-edge quads kept by a warp before it checks them
-constexpr int FIX_TOP = 126;  // most bins per axis of the fixed-point floors
+constexpr int FIX_TOP = 126;  // most bins per axis of the fixed-point floors (125 with an offset)
 constexpr int SEG_G = 97;     // j-segments of a chunk: 32 stencil rows, <= 3 each, and the own cell
 constexpr int SEG_T = 33;     // 32 listed tree nodes and the own node
 
@@ -87,6 +87,7 @@ inline size_t warp_slice(const PairParams &p) {
 }
 
 // Histogram layouts (word = 4 bytes; entry (n, m), lane copy k of hist_k):
+// (n counts a discarded row first when p.row0 is 1)
 //  LAY_ROWS   word (n hs + m) hist_k + k; weights: binary64 sums at the same
 //             index, or records of three u32 at 3 x the word
 //  LAY_SKEW   word w + w / 32, w = 256 n + m: the bytes of the two fixed-point
@@ -97,10 +98,10 @@ enum { LAY_ROWS = 0, LAY_SKEW = 1, LAY_BYTES = 2 };
 
 __host__ __device__ inline int hist_words(const PairParams &p) {
     if (p.layout == LAY_SKEW) {
-        const int w = 256 * p.n_a + 255;
+        const int w = 256 * (p.n_a + p.row0) + 255;
         return w + w / 32 + 1;
     }
-    if (p.layout == LAY_BYTES) return 64 * (p.n_a + 1);
+    if (p.layout == LAY_BYTES) return 64 * (p.n_a + p.row0 + 1);
     return p.nent * p.hist_k;
 }
 
@@ -170,15 +171,15 @@ __device__ __forceinline__ int hist_entries(const PairParams &p) {
 __device__ __forceinline__ int hist_word(const PairParams &p, int e, int k, int &bin) {
     bin = e;
     if (p.layout == LAY_SKEW) {
-        const int n = e / p.n_b, w = 256 * n + (e - n * p.n_b);
+        const int n = e / p.n_b, w = 256 * (n + p.row0) + (e - n * p.n_b);
         return w + (w >> 5);
     }
-    if (p.layout == LAY_BYTES) return 64 * e + k;
+    if (p.layout == LAY_BYTES) return 64 * (e + p.row0) + k;
     if (p.hs != p.n_b) {
         const int n = e / p.hs, m = e - n * p.hs;
         bin = m < p.n_b ? n * p.n_b + m : -1;
     }
-    return e * p.hist_k + k;
+    return (e + p.row0 * p.hs) * p.hist_k + k;
 }
 
 static __device__ __noinline__ void flush_counts(const PairParams &p, int off, int first, int nw, int h) {
@@ -259,11 +260,14 @@ static __device__ __noinline__ void flush_weights(const PairParams &p, int woff,
 // (but for additions in flight while they were flushed).
 static __device__ __noinline__ int most_counted(const PairParams &p) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int lane = threadIdx.x & 31, words = p.n_a * p.hs * p.hist_k, n4 = words / 4;
+    const int lane = threadIdx.x & 31, rows = p.n_a + p.row0;
+    const int words = rows * p.hs * p.hist_k, n4 = words / 4;
     int *hist = reinterpret_cast<int *>(smem);
-    if (p.hs != p.n_b)   // the rows' discarded columns fill fastest: nobody reads them
-        for (int k = lane; k < p.n_a * p.hist_k; k += 32)
+    // the discarded columns and the discarded first row fill fastest: nobody reads them
+    if (p.hs != p.n_b)
+        for (int k = lane; k < rows * p.hist_k; k += 32)
             hist[((k / p.hist_k) * p.hs + p.n_b) * p.hist_k + (k & (p.hist_k - 1))] = 0;
+    for (int k = lane; k < p.row0 * p.hs * p.hist_k; k += 32) hist[k] = 0;
     int m = 0;
     for (int k = lane; k < n4; k += 32) {
         const int4 v = reinterpret_cast<const int4 *>(hist)[k];
@@ -462,9 +466,12 @@ __device__ __forceinline__ void red_shared_f64_if(unsigned addr, double v, bool 
 
 // How the bins are found: lookup tables, floors (evenly spaced from 0; evenly
 // spaced from any edge; logarithmic s), or tables into the global histogram
-// when it does not fit shared memory.  PATH_FIX: the floors of PATH_LIN in
-// fixed point, for up to FIX_TOP bins an axis.
-enum { PATH_LUT = 0, PATH_LIN = 1, PATH_LINOFF = 2, PATH_LOG = 3, PATH_GLOBAL = 4, PATH_FIX = 5 };
+// when it does not fit shared memory.  PATH_FIX, PATH_FIXOFF and
+// PATH_FIXLOG: the first three floors (logarithmic also for sigma) in fixed
+// point, for up to FIX_TOP bins an axis.
+enum { PATH_LUT = 0, PATH_LIN = 1, PATH_LINOFF = 2, PATH_LOG = 3, PATH_GLOBAL = 4,
+       PATH_FIX = 5, PATH_FIXOFF = 6, PATH_FIXLOG = 7 };
+__host__ __device__ constexpr bool is_fix(int path) { return path >= PATH_FIX; }
 
 // Two pairs' outcome: byte offset of the counter in the shared histogram
 // (PATH_GLOBAL: bin, or ~0u for none), and whether the pair lies within an
@@ -770,27 +777,33 @@ __device__ __forceinline__ unsigned pair_quads(const PairParams &p, const Tile &
 // ---------------------------------------------------------------------------
 // fixed-point floors (PATH_FIX)
 // ---------------------------------------------------------------------------
-// For bins evenly spaced from zero, at most FIX_TOP an axis, a scaled value t
-// (s / D, mu n_mu, sigma / D, pi / D) is added to 128 + B 2^-16 in one fused
-// multiply-add.  FP32 numbers in [128, 256) are multiples of 2^-16: byte 2 of
-// the sum is floor(t + B 2^-16) and its low half the 16-bit fraction.  B is the
-// error band in these units (the arithmetic's bound and the sum's own rounding,
-// rounded up), so the pair is near an edge iff the fraction is below 2 B, and
-// otherwise the byte is its bin.  One three-input minimum of 16-bit halves
-// covers two values of the near test (the upper halves ride along unused), one
-// byte permutation puts the two bins side by side as the counter's index, and
-// values past the last bin are clamped to half a bin past it: the discarded
-// row (pi: column), never near.  mu n_mu has no shrunken scale: mu = 1 lands in
-// column n_mu, is near, and is put right by its binary64 check.  A tiny
-// constant added to the squares keeps coincident points finite (they are near,
-// t = 0).  Every index stays inside the histogram: coordinates are finite and
-// below 1e16 (others count as absent; the host limits the extents to 1e15, so no
-// square overflows), hence 128 <= T <= n_a + 128.5 and 128 <= M < 256.
+// For at most FIX_TOP bins an axis, a scaled value t (s / D, log_q(s / e_0), mu
+// n_mu, sigma / D, pi / D) is added to 128 + B 2^-16 in one fused multiply-add.
+// FP32 numbers in [128, 256) are multiples of 2^-16: byte 2 of the sum is
+// floor(t + B 2^-16) and its low half the 16-bit fraction.  B is the error band
+// in these units (the arithmetic's bound and the sum's own rounding, rounded
+// up), so the pair is near an edge iff the fraction is below 2 B, and otherwise
+// the byte is its bin.  One three-input minimum of 16-bit halves covers two
+// values of the near test (the upper halves ride along unused), one byte
+// permutation puts the two bins side by side as the counter's index, and values
+// past the last bin are clamped to half a bin past it: the discarded row (pi:
+// column), never near.  With a first edge above zero (PATH_FIXOFF, PATH_FIXLOG) t
+// carries + 1 and is clamped below to half a bin, another discarded row.  mu n_mu
+// has no shrunken scale: mu = 1 lands in column n_mu, is near, and is put right
+// by its binary64 check.  A tiny constant added to the squares keeps coincident
+// points finite.  Bands that grow as 1 / s (mu, logarithms) are taken at the
+// batch's smallest separation, from the boxes' gap.  Every index stays inside
+// the histogram: coordinates are finite and below 1e16 (others count as absent;
+// the host limits the extents to 1e15, so no square overflows), hence 128 <= T <
+// n_a + 130 and 128 <= M < 256.
 //
 // Against the packed floors of bin2 this leaves 40 of 68 packed FP32
 // instructions a quad (their three-register forms cost three register-read
 // cycles each); measured on the loop alone, (s, mu) 40 x 100: 161 against 224
 // cycles a quad and scheduler, one axis 121 against 147.
+// Whole kernel: 300,001 points, 40 logarithmic s bins x 100 mu bins 4.44 -> 3.40
+// ms against the packed floors; 10^6 points, 20 logarithmic sigma x 40 pi bins
+// 4.58 -> 2.70 ms against the tables.
 __device__ __forceinline__ unsigned prmt(unsigned a, unsigned b, unsigned s) {
     unsigned d;
     asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(s));
@@ -812,13 +825,44 @@ __device__ __forceinline__ void add_pieces(unsigned char *a0, unsigned char *a1,
     atomicAdd(reinterpret_cast<unsigned *>(a2), v.z);
 }
 
+// A batch's constants, from a 16-bit lower bound of its separations' square (the
+// upper half of the FP32 number; 0: none).
+struct Bands {
+    float2 cfs;          // first axis: 128 (+ 1 - offset) + band
+    float cfm;           // second axis
+    unsigned ts2, tm2;   // twice the bands, in units
+    float close;         // (s, mu): below it a pair is near whatever its mu
+};
+template <int MODE, int PATH>
+__device__ __forceinline__ Bands fix_bands(const PairParams &p, unsigned key) {
+    Bands b;
+    const float s2m = __uint_as_float(key << 16);
+    b.cfs = p.f_cfs;
+    b.ts2 = p.f_ts2;
+    b.cfm = p.f_cfp;
+    b.tm2 = p.f_tp2;
+    if (PATH == PATH_FIXLOG) {
+        const unsigned n = __float2uint_ru(fmaf(p.f_sA, rsqrt_fast(fmaxf(s2m, p.f_se2)), p.f_sC));
+        const float c = fmaf((float)n, 1.0f / 65536.0f, p.f_cfs.x);
+        b.cfs = make_float2(c, c);
+        b.ts2 = 2u * n;
+    }
+    if (MODE == MODE_SMU) {
+        const unsigned n = __float2uint_ru(fmaf(p.f_mA, rsqrt_fast(fmaxf(s2m, p.f_sf2)), p.f_mB));
+        b.cfm = fmaf((float)n, 1.0f / 65536.0f, 128.0f);
+        b.tm2 = 2u * n;
+    }
+    b.close = fmaf((float)b.ts2, 1.0f / 65536.0f, p.f_close);
+    return b;
+}
+
 struct Fix2 {
     float2 T, M;   // first axis (clamped) and second axis, in fixed point
 };
 
-template <int MODE, int LOS>
-__device__ __forceinline__ Fix2 fix2(const PairParams &p, float2 dx, float2 dy, float2 dz, float2 cfm, float xa,
-                                     float ya, float za, float2 &s2) {
+template <int MODE, int LOS, int PATH>
+__device__ __forceinline__ Fix2 fix2(const PairParams &p, float2 dx, float2 dy, float2 dz, float2 cfs, float2 cfm,
+                                     float xa, float ya, float za, float2 &s2) {
     Fix2 o;
     float2 pz, rl, lx, ly, lz;
     const float2 q = __ffma2_rn(dy, dy, __ffma2_rn(dx, dx, p.f_tiny));
@@ -836,28 +880,37 @@ __device__ __forceinline__ Fix2 fix2(const PairParams &p, float2 dx, float2 dy, 
     }
     float2 T;
     if (MODE == MODE_SIGPI) {
-        float2 v = q, rv;
-        if (LOS == LOS_Z) {
-            rv = __fmul2_rn(make_float2(rsqrt_fast(q.x), rsqrt_fast(q.y)), p.c_invA);
-        } else {   // sigma = |d x l| / |l|
+        float2 v = q;
+        if (LOS == LOS_MID) {   // sigma = |d x l| / |l|
             const float2 M1 = p.c_m1;
             const float2 ndx = __fmul2_rn(dx, M1), ndy = __fmul2_rn(dy, M1), ndz = __fmul2_rn(dz, M1);
             const float2 cx = __ffma2_rn(dy, lz, __fmul2_rn(ndz, ly));
             const float2 cy = __ffma2_rn(dz, lx, __fmul2_rn(ndx, lz));
             const float2 cz = __ffma2_rn(dx, ly, __fmul2_rn(ndy, lx));
             v = __ffma2_rn(cz, cz, __ffma2_rn(cy, cy, __ffma2_rn(cx, cx, p.f_tiny)));
-            rv = __fmul2_rn(make_float2(rsqrt_fast(v.x), rsqrt_fast(v.y)), __fmul2_rn(rl, p.c_invA));
         }
-        T = __ffma2_rn(v, rv, p.f_cfs);
+        if (PATH == PATH_FIXLOG) {
+            if (LOS == LOS_MID) v = __fmul2_rn(__fmul2_rn(v, rl), rl);
+            T = __ffma2_rn(make_float2(lg2_fast(v.x), lg2_fast(v.y)), p.c_invA, cfs);
+        } else {
+            float2 rv = make_float2(rsqrt_fast(v.x), rsqrt_fast(v.y));
+            rv = __fmul2_rn(rv, LOS == LOS_Z ? p.c_invA : __fmul2_rn(rl, p.c_invA));
+            T = __ffma2_rn(v, rv, cfs);
+        }
         const float2 M = __ffma2_rn(pz, LOS == LOS_Z ? p.c_invB : __fmul2_rn(rl, p.c_invB), cfm);
         o.M = make_float2(fminf(M.x, p.f_limB), fminf(M.y, p.f_limB));
     } else {
-        const float2 rs = make_float2(rsqrt_fast(s2.x), rsqrt_fast(s2.y));
-        T = __ffma2_rn(s2, __fmul2_rn(rs, p.c_invA), p.f_cfs);
+        float2 rs;
+        if (PATH != PATH_FIXLOG || MODE == MODE_SMU) rs = make_float2(rsqrt_fast(s2.x), rsqrt_fast(s2.y));
+        if (PATH == PATH_FIXLOG)
+            T = __ffma2_rn(make_float2(lg2_fast(s2.x), lg2_fast(s2.y)), p.c_invA, cfs);
+        else
+            T = __ffma2_rn(s2, __fmul2_rn(rs, p.c_invA), cfs);
         if (MODE == MODE_SMU)
             o.M = __ffma2_rn(pz, LOS == LOS_Z ? __fmul2_rn(rs, p.c_invB)
                                               : __fmul2_rn(__fmul2_rn(rl, rs), p.c_invB), cfm);
     }
+    if (PATH != PATH_FIX) T = make_float2(fmaxf(T.x, 128.5f), fmaxf(T.y, 128.5f));
     o.T = make_float2(fminf(T.x, p.f_lim), fminf(T.y, p.f_lim));
     return o;
 }
@@ -867,11 +920,11 @@ __device__ __forceinline__ Fix2 fix2(const PairParams &p, float2 dx, float2 dy, 
 // mu band is taken at (T below f_close: near), and the block's own points (the
 // tile holds its points from jbase on, pairs j <= i are masked; jbase past any
 // i: none is).
-template <int MODE, int LOS, int W, bool SLOW>
+template <int MODE, int LOS, int W, int PATH, bool SLOW>
 __device__ __forceinline__ unsigned quads_fix(const PairParams &p, const Tile &t, int nq, const IPts<LOS, W> &I,
-                                              unsigned char *smem, float cfm1, unsigned tm2, int jbase) {
+                                              unsigned char *smem, const Bands &bd, int jbase) {
     const int lane = threadIdx.x & 31;
-    const float2 cfm = make_float2(cfm1, cfm1);
+    const float2 cfm = make_float2(bd.cfm, bd.cfm);
     const unsigned copy = 4u * (unsigned)lane;                 // LAY_BYTES
     const unsigned kc = (unsigned)(lane & (p.hist_k - 1));    // LAY_ROWS
     unsigned *hist = reinterpret_cast<unsigned *>(smem);
@@ -901,10 +954,10 @@ __device__ __forceinline__ unsigned quads_fix(const PairParams &p, const Tile &t
                     if (jj + 1 <= 2 * lane + r) dx.y = p.far;
                 }
                 float2 s2;
-                const Fix2 f = fix2<MODE, LOS>(p, dx, dy, dz, cfm, I.xa[r], I.ya[r], I.za[r], s2);
+                const Fix2 f = fix2<MODE, LOS, PATH>(p, dx, dy, dz, bd.cfs, cfm, I.xa[r], I.ya[r], I.za[r], s2);
                 const unsigned t0 = __float_as_uint(f.T.x), t1 = __float_as_uint(f.T.y);
                 accT = __vimin3_u16x2(accT, t0, t1);
-                if (SLOW && MODE == MODE_SMU) close = close | (f.T.x < p.f_close) | (f.T.y < p.f_close);
+                if (SLOW && MODE == MODE_SMU) close = close | (f.T.x < bd.close) | (f.T.y < bd.close);
                 unsigned P0 = 0u, P1 = 0u;   // W >= 2: addresses of the pieces' records
                 if (MODE == MODE_S) {
                     // byte 1: the bin, byte 0: this lane's copy
@@ -954,8 +1007,8 @@ __device__ __forceinline__ unsigned quads_fix(const PairParams &p, const Tile &t
                 }
             }
         }
-        bool any = (accT & 0xffffu) < p.f_ts2;
-        if (MODE != MODE_S) any = any | ((accM & 0xffffu) < tm2);
+        bool any = (accT & 0xffffu) < bd.ts2;
+        if (MODE != MODE_S) any = any | ((accM & 0xffffu) < bd.tm2);
         if (SLOW) any = any | close;
         near |= (any ? 1u : 0u) << q;
     }
@@ -964,14 +1017,14 @@ __device__ __forceinline__ unsigned quads_fix(const PairParams &p, const Tile &t
 
 // Two pairs' bins and near flags from their fixed-point values (the near-edge
 // check repeats the loop's arithmetic with them); bin -1: discarded.
-template <int MODE>
-__device__ __forceinline__ int fix_bin(const PairParams &p, float T, float M, unsigned tm2, bool &near) {
+template <int MODE, int PATH>
+__device__ __forceinline__ int fix_bin(const PairParams &p, float T, float M, const Bands &b, bool &near) {
     const unsigned t = __float_as_uint(T), m = MODE == MODE_S ? 0u : __float_as_uint(M);
-    near = (t & 0xffffu) < p.f_ts2;
-    if (MODE != MODE_S) near = near || (m & 0xffffu) < tm2;
-    if (MODE == MODE_SMU) near = near || T < p.f_close;
-    const int n = (int)((t >> 16) & 0x7f), k = (int)((m >> 16) & 0x7f);
-    return n < p.n_a && k < p.n_b ? n * p.n_b + k : -1;
+    near = (t & 0xffffu) < b.ts2;
+    if (MODE != MODE_S) near = near || (m & 0xffffu) < b.tm2;
+    if (MODE == MODE_SMU) near = near || T < b.close;
+    const int n = (int)((t >> 16) & 0x7f) - (PATH == PATH_FIX ? 0 : 1), k = (int)((m >> 16) & 0x7f);
+    return n >= 0 && n < p.n_a && k < p.n_b ? n * p.n_b + k : -1;
 }
 
 // Weighted product of a pair as the fast path added it (integer paths).
@@ -983,7 +1036,7 @@ __device__ __forceinline__ unsigned long long fast_product(const IPts<LOS, W> &I
 
 // Check n queued near-edge quads with the binary64 definition, one per lane.
 // An entry is {first of its four j-points, source lane | own block << 5 |
-// segment << 6 | mu band << 13}.  The lane repeats the quad's FP32 arithmetic
+// segment << 6 | the batch's bound (fix_bands) << 13}.  The lane repeats the quad's FP32 arithmetic
 // on the same operands, so it sees the same bins and the same near pairs, and
 // corrects the global histogram where the binary64 bin differs from the one
 // counted.  With a rescue queue (pc_opts.rescue_capacity > 0) the fast count is
@@ -993,8 +1046,8 @@ __device__ __noinline__ void check_near(const PairParams &p, const uint2 *queue,
                                         int cell, int start, int count, unsigned copy, const float2 *s_lut) {
     const int lane = threadIdx.x & 31;
     const TaskDev &T = p.tasks[task];
-    Ctx<MODE, LOS, PATH == PATH_FIX ? PATH_LIN : PATH> c;
-    if (PATH != PATH_FIX) c.init(p, s_lut, copy);
+    Ctx<MODE, LOS, is_fix(PATH) ? PATH_LIN : PATH> c;
+    if (!is_fix(PATH)) c.init(p, s_lut, copy);
     unsigned m8 = 0u;         // near pairs: bit 4 r + j
     int b8[8];                // the bins they were counted in (-1: none)
     int i0 = 0, j0 = 0, img = 13;
@@ -1002,7 +1055,6 @@ __device__ __noinline__ void check_near(const PairParams &p, const uint2 *queue,
         const uint2 e = queue[lane];
         const int src = (int)(e.y & 31u);
         const bool own = (e.y >> 5) & 1u;
-        const unsigned band = e.y >> 13;
         j0 = (int)e.x;
         i0 = start + 2 * src;
         int4 sg = make_int4(start, start + count, TREE ? -1 : 0, 13);
@@ -1024,9 +1076,8 @@ __device__ __noinline__ void check_near(const PairParams &p, const uint2 *queue,
             else s[j] = own ? make_float3(q.x, q.y, q.z)
                             : stage_grid(p, q, T.gj.cx[j0 + j], ax, sg.z, img);
         }
-        const float cf1 = MODE == MODE_SIGPI ? p.f_cfp : fmaf((float)band, 1.0f / 65536.0f, 128.0f);
-        const float2 cfm = make_float2(cf1, cf1);
-        const unsigned tm2 = MODE == MODE_SIGPI ? p.f_tp2 : 2u * band;
+        const Bands bd = fix_bands<MODE, PATH>(p, e.y >> 13);
+        const float2 cfm = make_float2(bd.cfm, bd.cfm);
         IPts<LOS, W> I;
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
@@ -1043,14 +1094,14 @@ __device__ __noinline__ void check_near(const PairParams &p, const uint2 *queue,
                 const bool v1 = iok && (vm >> (j + 1) & 1u) && !(own && j0 + j + 1 <= i0 + r);
                 float2 s2;
                 bool n0, n1;
-                if (PATH == PATH_FIX) {
-                    const Fix2 f = fix2<MODE, LOS>(p, dx, dy, dz, cfm, I.xa[r], I.ya[r], I.za[r], s2);
-                    b8[4 * r + j] = fix_bin<MODE>(p, f.T.x, f.M.x, tm2, n0);
-                    b8[4 * r + j + 1] = fix_bin<MODE>(p, f.T.y, f.M.y, tm2, n1);
+                if (is_fix(PATH)) {
+                    const Fix2 f = fix2<MODE, LOS, PATH>(p, dx, dy, dz, bd.cfs, cfm, I.xa[r], I.ya[r], I.za[r], s2);
+                    b8[4 * r + j] = fix_bin<MODE, PATH>(p, f.T.x, f.M.x, bd, n0);
+                    b8[4 * r + j + 1] = fix_bin<MODE, PATH>(p, f.T.y, f.M.y, bd, n1);
                 } else {
                     const float2 qq = __ffma2_rn(dy, dy, __fmul2_rn(dx, dx));
                     s2 = __ffma2_rn(dz, dz, qq);
-                    const Pair2 b = bin2<MODE, LOS, PATH == PATH_FIX ? PATH_LIN : PATH>(
+                    const Pair2 b = bin2<MODE, LOS, is_fix(PATH) ? PATH_LIN : PATH>(
                         p, c, dx, dy, dz, qq, s2, I.xa[r], I.ya[r], I.za[r]);
                     n0 = b.n0;
                     n1 = b.n1;
@@ -1365,6 +1416,7 @@ __device__ __forceinline__ int ring_round(const PairParams &p, const TaskDev &T,
         keep = g2 < p.r2prune;
         if (MODE == MODE_SIGPI && LOS == LOS_Z)   // the reach is a cylinder
             keep = keep && gq < p.q2prune && gz < p.zprune;
+        if (MODE == MODE_SIGPI) g2 = LOS == LOS_Z ? gq : 0.f;
         const unsigned long long np2 =
             (unsigned long long)(min(sg.y, p0 + 8) - max(sg.x, p0)) * (unsigned)count;
         cand += np2;
@@ -1373,7 +1425,7 @@ __device__ __forceinline__ int ring_round(const PairParams &p, const TaskDev &T,
     const unsigned who = __ballot_sync(FULL, keep);
     if (keep)
         ring[(tail + __popc(who & ((1u << lane) - 1u))) & (RING - 1)] =
-            make_int4(p0, lo, __float_as_int(g2), 0);
+            make_int4(p0, lo, __float_as_int(g2), 0);   // (sigma, pi): the gap across the line of sight
     __syncwarp();
     return tail + __popc(who);
 }
@@ -1419,8 +1471,8 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
             p.wfold_buf[(size_t)blockIdx.x * p.nbins * 2 + b] = 0ull;
     if (threadIdx.x == 0) s_range = RangeShared{0, 0, 0, 0, -1};
     const unsigned copy = 4u * (unsigned)(lane & (p.hist_k - 1));
-    Ctx<MODE, LOS, PATH == PATH_FIX ? PATH_LIN : PATH> c;
-    if (PATH != PATH_FIX) c.init(p, s_lut, copy);
+    Ctx<MODE, LOS, is_fix(PATH) ? PATH_LIN : PATH> c;
+    if (!is_fix(PATH)) c.init(p, s_lut, copy);
     const unsigned wbase = (unsigned)__cvta_generic_to_shared(smem + p.sm_whist);
     const float far = p.far;
 
@@ -1436,7 +1488,7 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
     // counter, and flushes (counts with the weights) only past a quarter of the
     // bound; what is in flight during a flush, at most 16 slots of a lane and
     // warp, is taken off the quarter
-    constexpr bool SCAN = !(PATH == PATH_FIX && MODE == MODE_S);
+    constexpr bool SCAN = !(is_fix(PATH) && MODE == MODE_S);
     constexpr unsigned wmax = W == 3 ? WINT_LIMIT / 2 : WINT_LIMIT;
     const unsigned wlimit = (SCAN ? wmax / 4 * 3 : wmax) / (unsigned)nw;
     const int wfull = (int)(wmax / 4) - 16 * nw * (32 / p.hist_k);
@@ -1475,7 +1527,7 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
             if (2 * lane + r < it.count) {
                 const int i = it.start + 2 * lane + r;
                 load_i<MODE, LOS, W>(T.gi, i, I, r);
-                if (PATH == PATH_FIX && !(fabsf(I.x[r]) + fabsf(I.y[r]) + fabsf(I.z[r]) < 1e16f)) {
+                if (is_fix(PATH) && !(fabsf(I.x[r]) + fabsf(I.y[r]) + fabsf(I.z[r]) < 1e16f)) {
                     I.x[r] = -far;      // not a number: no pair
                     I.y[r] = I.z[r] = 0.f;
                 }
@@ -1509,7 +1561,7 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
                 // one batch: the block's own points, or up to eight octs
                 const int m = own ? (it.count + 7) >> 3 : min(JO, tail - head);
                 unsigned near = 0u;
-                unsigned band = 0u;
+                unsigned key = 0u;   // bound of the batch's separations (fix_bands)
                 if (m > 0) {
                     float g2 = INFINITY;
 #pragma unroll
@@ -1538,7 +1590,7 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
                                 }
                             }
                         }
-                        if (PATH == PATH_FIX && !(fabsf(s.x) + fabsf(s.y) + fabsf(s.z) < 1e16f))
+                        if (is_fix(PATH) && !(fabsf(s.x) + fabsf(s.y) + fabsf(s.z) < 1e16f))
                             s = make_float3(far, 0.f, 0.f);   // not a number: no pair
                         tx[sl] = s.x; ty[sl] = s.y; tz[sl] = s.z;
                         if (W == 1) tw[sl] = v ? T.gj.xw[pj].w : 0.0;
@@ -1562,23 +1614,21 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
                             wterms = wper * (unsigned)nq;
                         }
                     }
-                    if constexpr (PATH == PATH_FIX) {
-                        float cfm = p.f_cfp;
-                        unsigned tm2 = p.f_tp2;
+                    if constexpr (is_fix(PATH)) {
                         bool slow = own;
-                        if (MODE == MODE_SMU) {
-                            // the mu band at the batch's smallest separation
+                        if (MODE == MODE_SMU || PATH == PATH_FIXLOG) {
+                            // the batch's smallest separation: the smallest gap less the
+                            // box tests' rounding
                             g2 = own ? 0.f : __uint_as_float(__reduce_min_sync(FULL, __float_as_uint(g2)));
-                            slow = g2 < p.f_sf2;
-                            band = __float2uint_ru(fmaf(p.f_mA, rsqrt_fast(fmaxf(g2, p.f_sf2)), p.f_mB));
-                            cfm = fmaf((float)band, 1.0f / 65536.0f, 128.0f);
-                            tm2 = 2u * band;
+                            const float g = fmaxf(g2 * rsqrt_fast(fmaxf(g2, 1e-30f)) - p.f_gm, 0.f);
+                            key = __float_as_uint(g * g) >> 16;
+                            slow = own || (MODE == MODE_SMU && __uint_as_float(key << 16) < p.f_sf2);
                         }
+                        const Bands bd = fix_bands<MODE, PATH>(p, key);
                         if (slow)
-                            near = quads_fix<MODE, LOS, W, true>(p, tile, nq, I, smem, cfm, tm2,
-                                                                 own ? 0 : 2 * BI);
+                            near = quads_fix<MODE, LOS, W, PATH, true>(p, tile, nq, I, smem, bd, own ? 0 : 2 * BI);
                         else
-                            near = quads_fix<MODE, LOS, W, false>(p, tile, nq, I, smem, cfm, tm2, 0);
+                            near = quads_fix<MODE, LOS, W, PATH, false>(p, tile, nq, I, smem, bd, 0);
                     } else {
                         const size_t hbase = (size_t)T.hist * p.nbins;
                         if (own)
@@ -1595,11 +1645,11 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
                     if (near) {
                         const int q = __ffs(near) - 1;
                         near &= near - 1;
-                        uint2 e = make_uint2((unsigned)(it.start + 4 * q), (unsigned)lane | 32u | band << 13);
+                        uint2 e = make_uint2((unsigned)(it.start + 4 * q), (unsigned)lane | 32u | key << 13);
                         if (!own) {
                             const int4 o = ring[(head + (q >> 1)) & (RING - 1)];
                             e = make_uint2((unsigned)(o.x + 4 * (q & 1)),
-                                           (unsigned)lane | (unsigned)o.y << 6 | band << 13);
+                                           (unsigned)lane | (unsigned)o.y << 6 | key << 13);
                         }
                         queue[qn + __popc(who & ((1u << lane) - 1u))] = e;
                     }
@@ -1916,7 +1966,7 @@ using PairKernel = void (*)(PairParams);
 template <int MODE, int LOS, int PATH, bool TREE>
 PairKernel<MODE, LOS> pick_w(const PairParams &p) {
     if (!p.weighted) return k_pairs_f32<MODE, LOS, 0, PATH, TREE>;
-    if constexpr (PATH == PATH_FIX)   // integer weight products only
+    if constexpr (is_fix(PATH))   // integer weight products only
         return p.wcorr ? k_pairs_f32<MODE, LOS, 3, PATH, TREE> : k_pairs_f32<MODE, LOS, 2, PATH, TREE>;
     else {
     if constexpr (PATH != PATH_LUT && PATH != PATH_GLOBAL) {
@@ -1934,9 +1984,11 @@ PairKernel<MODE, LOS> pick_f32(const PairParams &p) {
     if (!p.smem_hist_ok) return pick_w<MODE, LOS, PATH_GLOBAL, TREE>(p);
     if constexpr (MODE != MODE_SIGPI) {
         if (p.path == PATH_LINOFF) return pick_w<MODE, LOS, PATH_LINOFF, TREE>(p);
+        if (p.path == PATH_FIXOFF) return pick_w<MODE, LOS, PATH_FIXOFF, TREE>(p);
         if (p.path == PATH_LOG) return pick_w<MODE, LOS, PATH_LOG, TREE>(p);
     }
     if (p.path == PATH_FIX) return pick_w<MODE, LOS, PATH_FIX, TREE>(p);
+    if (p.path == PATH_FIXLOG) return pick_w<MODE, LOS, PATH_FIXLOG, TREE>(p);
     if (p.path == PATH_LIN) return pick_w<MODE, LOS, PATH_LIN, TREE>(p);
     return pick_w<MODE, LOS, PATH_LUT, TREE>(p);
 }

@@ -132,15 +132,18 @@ struct PairParams {
     // threshold, minus the bytes of a row and of a column
     float2 c_23, c_p, c_m1, c_invA, c_offA, c_thrA, c_nmS, c_invB, c_nmB, c_cB, c_nrow, c_ncol;
     float c_kA;              // counter address constant without the lane copy
-    // fixed-point floors (PATH_FIX, see the kernel): 1e-30; 128 + band of the
-    // first axis and (sigma, pi) of the second; the clamps; twice the bands in
-    // units of 2^-16; t below which a pair is always near, its separation
-    // squared; mu band in units, f_mA / s + f_mB
+    // fixed-point floors (PATH_FIX and following, see the kernel): 1e-30; the
+    // first axis's constant (with its band, but for logarithms) and pi's; the
+    // clamps; twice the bands in units of 2^-16; bands in units that grow as
+    // 1 / s, f_mA / s + f_mB (mu) and f_sA / s + f_sC (logarithms), and the
+    // squared separations they stop growing at; t (without its band) below which
+    // a pair is always near; the box tests' rounding; the scales
     float2 f_tiny, f_cfs;
-    float f_cfp, f_lim, f_limB, f_close, f_sf2, f_mA, f_mB;
+    float f_cfp, f_lim, f_limB, f_close, f_sf2, f_mA, f_mB, f_se2, f_sA, f_sC, f_gm, f_inv, f_invB;
     unsigned f_ts2, f_tp2;
+    int row0;                // 1: a discarded row before the first bin
     unsigned f_coef;         // weighted LAY_ROWS: bytes {hist_k, hs hist_k} (entry from the two bins)
-    int fix;                 // the plan allows PATH_FIX
+    int fix;                 // 0, or the PATH_FIX* the plan allows
     int layout;              // of the shared histogram (LAY_*)
     float L32[3];            // periodic box sides (0: none)
     // shared histogram: entry (a, b) = a hs + b, the columns n_b .. hs - 1 and

@@ -1,7 +1,8 @@
 """The pair kernel's fixed-point floors (CPU, emulated): for bins evenly spaced
 from zero a scaled value t is summed once in binary32 onto 128 + B 2^-16 (a grid
-of 2^-16), the bin is the sum's third byte and the pair is near an edge iff its
-low half is below 2 B.  On the kernel's own binary32 separations (cell-relative
+of 2^-16; offset and logarithmic edges: 129 + B 2^-16 less the first edge's t),
+the bin is the sum's third byte and the pair is near an edge iff its low half is
+below 2 B.  On the kernel's own binary32 separations (cell-relative
 coordinates, both ends of the reciprocal root's error) every pair that is not
 near must sit in the bin of its binary64 value, for s (band of the whole count)
 and mu (band at a lower bound of the pair's separation), with the bands as the
@@ -60,6 +61,58 @@ def test_fixed_floors_decide_like_binary64(L, ng, lo, R, periodic, na, nb):
         far = keep & (frac >= 2 * bm)
         assert np.array_equal(m[far], j_true[far])
         seen += int(far.sum())
+    assert seen > 0
+
+
+@pytest.mark.parametrize("L,ng,lo,R,periodic", fb.GEOMETRIES)
+@pytest.mark.parametrize("e0,na,log", [(0.3, 125, False), (0.02, 7, False), (1e-3, 40, True), (0.2, 125, True),
+                                       (0.02, 1, True)])
+def test_offset_and_log_floors_decide_like_binary64(L, ng, lo, R, periodic, e0, na, log):
+    """First edge e0 R: bins below (row 0) and past the last are discarded."""
+    rng = np.random.default_rng(na + ng)
+    c, xi, xj, idi, idj, dxc = fb._pairs(rng, 200_000, L, ng, lo, R, periodic)
+    o = fb._oracle_values(xi, xj, L, periodic)
+    e0 = e0 * R
+    X, Lm = max(abs(lo), abs(lo + ng * c)), L if periodic else 0.0
+    tiny = 2.0 ** -48 * (X + Lm + R)
+    s = o["s"]
+    low = np.maximum(s * rng.choice([1.0, 0.7], s.shape), 0.5 * e0)   # a batch's smallest separation
+    if log:
+        lq = np.log2(R / e0) / na
+        A, B = 0.5 / lq, -np.log2(e0) / lq
+        Lmax = max(abs(np.log2(R * R)), abs(np.log2(0.25 * e0 * e0)))
+        C = 129.0 + B
+        common = (A * 2.0 ** -21 * max(1.0, Lmax) + U * (A * Lmax + abs(B) + na + 130.0) * 2.0 + 1e-6 + A * 2.0 ** -45)
+        sC = 2.0 * (A * 9.0 * U / np.log(2.0) * 1.01 + common) * 65536.0 + 2.0
+        sA = 4.0 * A * (4.4 * U * c + 2.0 ** -51 * (X + Lm + R)) / np.log(2.0) * 1.01 * 65536.0
+        if not (abs(C) < 250.0 and sA / (0.5 * e0) + sC < 8192.0 and
+                2.0 * U * (4.4 * c + 10.5 * R) + tiny < 0.05 * e0):
+            pytest.skip("the library keeps the tables here")
+        b = np.ceil(sA / low + sC)
+        t = np.log2(s / e0) / lq
+        inv = F32(A)
+    else:
+        D = (R - e0) / na
+        C = 129.0 - e0 / D
+        if abs(C) >= 250.0:
+            pytest.skip("the library keeps the packed floors here")
+        b = np.full(s.shape, np.ceil(((1.25 * U * (4.34 * c + 8.7 * R) + tiny) / D + 1e-9) * 65536.0 + 1.5))
+        t = (s - e0) / D
+        inv = F32(1.0 / D)
+    k_true = np.where(s < e0, -1, np.minimum(np.floor(t), na)).astype(np.int64)
+    cst = (F32(C) + (b / 65536.0).astype(F32)).astype(F32)
+    seen = 0
+    with np.errstate(all="ignore"):
+        values = fb._kernel_values(c, lo, xi, xj, idi, idj, dxc)
+    for kv in values:
+        s2 = kv["s2"]
+        for v, r in ([(lg, np.full(s2.shape, inv)) for lg in fb._lg2_ends(np.maximum(s2, F32(1e-30)))] if log
+                     else [(s2, kv["rs"] * inv)]):
+            T = fb.fma32(v, r, cst)
+            T = np.clip(np.where(np.isnan(T), F32(128.5), T), F32(128.5), F32(129.5 + na)).view(np.uint32)
+            far = (T & 0xFFFF) >= 2 * b
+            assert np.array_equal(((T >> 16) & 0x7F).astype(np.int64)[far] - 1, k_true[far])
+            seen += int(far.sum())
     assert seen > 0
 
 

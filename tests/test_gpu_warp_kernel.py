@@ -57,6 +57,29 @@ def test_bin_counts_around_the_fixed_point_limit(mode, na, nb, weights):
     _check(x, w=w, mode=mode, edges_a=ea, edges_b=eb)
 
 
+@pytest.mark.parametrize("na", [1, 7, 125, 126])
+@pytest.mark.parametrize("e0,spacing", [(3.0, "even"), (24.0, "even"), (0.004, "log"), (0.5, "log"), (20.0, "log")])
+@pytest.mark.parametrize("mode,los", [("s", "z"), ("smu", "z"), ("sigpi", "z"), ("smu", "mid"), ("sigpi", "mid")])
+def test_first_edges_above_zero(mode, los, e0, spacing, na):
+    """Offset and logarithmic first axes (also sigma), about their limit of 125
+    bins, from one bin over orders of magnitude to narrow ones far out."""
+    rng = np.random.default_rng(na + 41)
+    ea = np.linspace(e0, 25.0, na + 1) if spacing == "even" else np.geomspace(e0, 25.0, na + 1)
+    eb = {"s": None, "smu": np.linspace(0.0, 1.0, 13), "sigpi": np.linspace(0.0, 20.0, 21)}[mode]
+    x = _points(2500, 42)
+    box = dict(box=L, periodic=True)
+    if los == "mid":
+        x, box = x + 400.0, {}
+    w = 0.3 + 0.7 * rng.random(x.shape[0])
+    want, wantw = oracle.count(x, w1=w, mode=mode, los=los, edges_a=ea, edges_b=eb, method="brute", **box)
+    for f in (P.count, P.count_tree):
+        for v in (None, w, w.astype(np.float32)):
+            got, gotw = f(x, w1=v, mode=mode, los=los, edges_a=ea, edges_b=eb, **box)
+            np.testing.assert_array_equal(got, want, err_msg=f.__name__)
+            if v is w:
+                np.testing.assert_allclose(gotw, wantw, rtol=1e-10, atol=0.0, err_msg=f.__name__)
+
+
 @pytest.mark.parametrize("n1,n2", [(40, 5000), (5000, 40), (1, 300), (300, 1)])
 def test_cross_counts_either_way_round(n1, n2):
     x, y = _points(n1, 21), _points(n2, 22)

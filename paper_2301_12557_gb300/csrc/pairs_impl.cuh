@@ -802,7 +802,7 @@ __device__ __forceinline__ unsigned pair_quads(const PairParams &p, const Tile &
 // cycles each); measured on the loop alone, (s, mu) 40 x 100: 161 against 224
 // cycles a quad and scheduler, one axis 121 against 147.
 // Whole kernel: 300,001 points, 40 logarithmic s bins x 100 mu bins 4.44 -> 3.40
-// ms against the packed floors; 10^6 points, 20 logarithmic sigma x 40 pi bins
+// ms against the packed floors; 10^6 points, 20 logarithmic sigma x 60 pi bins
 // 4.58 -> 2.70 ms against the tables.
 __device__ __forceinline__ unsigned prmt(unsigned a, unsigned b, unsigned s) {
     unsigned d;

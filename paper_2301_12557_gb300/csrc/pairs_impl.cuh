@@ -4,16 +4,18 @@
 // Work decomposition of the FP32 kernel (grid traversal of Sect. 2.1 with the
 // half-shell duplicate removal of Sect. 3.1): every warp works on its own,
 // with no barrier among the warps of a CTA, which share only the histogram.
-// A warp takes up to 64 consecutive points of one cell (the i-points, two a
-// lane, in registers) and walks the candidate j-points of the neighbouring
+// A warp takes up to 64 consecutive points of one cell (the i-points, in
+// registers: a lane holds one of either half) and walks the candidate j-points of the neighbouring
 // cells.  Neighbours are visited row by row: for a stencil row (dy, dz) the
 // cells (ax + xlo .. ax + xhi, ay + dy, az + dz) are contiguous in the
 // cell-sorted arrays, so each row is one index range (split at most in three
 // by periodic wrapping).  Periodic images are handled by shifting whole cells
 // (Sect. 3.1), never by testing each pair.  The build stores the bounding box
 // of every run of eight points (an oct); the warp tests 32 octs at a time
-// against the box of its i-points and stages only those that can reach it,
-// eight octs a batch, in its own slice of shared memory.
+// against the boxes of its two halves and keeps three lists, octs that reach
+// both or only one, staged a batch at a time in its own slice of shared memory.
+// Batches of one list need no test in the loop; one half's run with one i-point
+// a lane, at half the instructions.
 //
 // FP32 arithmetic: the j-point is staged as its offset from the i-cell centre,
 // rel_j + delta * c, so a pair costs three subtractions and three
@@ -29,12 +31,19 @@
 // one, so the integer counts equal the binary64 definition exactly.
 //
 // What bounds it (2M clustered points, (s, mu) 40 x 100, 6.70e10 pairs in
-// range): issue slots (70 % used; the FMA and integer pipes at 52 %, shared
-// memory at 62 %).  139 warp instructions per 64 x 4 pairs, 113 of them the loop
-// itself; 18 % of the pairs are empty lanes and the ends of octs.  80.7 ms
-// against 154.7 ms for CTAs of 128 threads that staged every candidate tile
-// behind a barrier (138 instructions per 64 x 2 pairs in range, issued on 60 % of
-// the cycles) and queued near-edge pairs for a second kernel.
+// range): issue slots (82 % used; the FMA and integer pipes at 51 and 54 %, shared
+// memory at 61 %).  1.52 pairs are evaluated for each in range, against 1.70 with
+// one list for the 64 points along a Morton curve; 113 of about 135 warp
+// instructions per 64 x 4 pairs are the loop itself.  68.2 ms against 154.7 ms for
+// CTAs of 128 threads that staged every candidate tile behind a barrier and queued
+// near-edge pairs for a second kernel (138 instructions per 64 x 2 pairs, issued
+// on 60 % of the cycles).
+//
+// The warps of an SM are spread over all of this code, so its size counts: with a
+// second loop body (two quads unrolled) for one half, unrolled staging and an
+// unrolled near-edge check, warps waited for instructions longer than for anything
+// else (stall 0.1 -> 5.5 an instruction, 312k points 3.2 -> 4.6 ms).  Loops that
+// run rarely are rolled.
 #pragma once
 
 #include "pc_internal.cuh"
@@ -54,10 +63,9 @@ __host__ __device__ inline size_t align_up(size_t x, size_t a) { return (x + a -
 // ---------------------------------------------------------------------------
 // FP32 kernel: shared memory
 // ---------------------------------------------------------------------------
-constexpr int BI = 64;        // i-points per warp (two a lane)
-constexpr int JB = 64;        // j-points per staged batch (eight octs)
-constexpr int JO = JB / 8;
-constexpr int RING = 64;      // octs kept for staging (ring): up to JO - 1 + 32
+constexpr int BI = 64;        // i-points per warp: two halves of 32, one point of each a lane
+constexpr int JB_COUNTS = 128;   // j-points per staged batch, counts only (64: 4 % slower; weights bound a
+                                 // batch by the records' range)
 constexpr int QCAP = 64;      // near-edge quads kept by a warp before it checks them
 constexpr int FIX_TOP = 126;  // most bins per axis of the fixed-point floors (125 with an offset)
 constexpr int SEG_G = 97;     // j-segments of a chunk: 32 stencil rows, <= 3 each, and the own cell
@@ -65,17 +73,22 @@ constexpr int SEG_T = 33;     // 32 listed tree nodes and the own node
 
 // Byte offsets of a warp's slice: segments, their offsets (tree), the staged
 // batch (FP64: coordinates and weight, and the images' shifts), its weights, the
-// near-edge queue, the ring and the octs before each segment.
+// near-edge queue, the octs to stage, the halves' boxes and the octs before each
+// segment.
 template <bool TREE, bool WEIGHTED, bool F64>
 struct WarpOff {
     enum {
+        jb = WEIGHTED || F64 ? 64 : JB_COUNTS,               // j-points per staged batch
+        jo = jb / 8,
+        list = jo + 32,                                      // octs kept per class: jo - 1 and a round
         nseg = TREE ? SEG_T : SEG_G,
         soff = nseg * 16,                                    // int4[nseg] before it
         tile = soff + (TREE ? SEG_T * 16 : 0),               // float4[nseg]
-        tw = tile + (F64 ? JB * 7 * 8 : 3 * JB * 4),         // x, y, z (+ w, shifts)
-        queue = tw + (WEIGHTED && !F64 ? JB * 8 : 0),        // 8 B a point
-        ring = queue + (F64 ? 0 : QCAP * 8),                 // uint2[QCAP]
-        pref = ring + RING * 16,                             // int4[RING]
+        tw = tile + (F64 ? jb * 7 * 8 : 3 * jb * 4),         // x, y, z (+ w, shifts)
+        queue = tw + (WEIGHTED && !F64 ? jb * 8 : 0),        // 8 B a point
+        ring = (queue + (F64 ? 0 : QCAP * 8) + 15) / 16 * 16,   // uint2[QCAP]
+        ibox = ring + 3 * list * 8,                          // uint2[3][list]
+        pref = ibox + 64,                                    // IBox[2]
         total = (pref + (nseg + 1) * 4 + 15) / 16 * 16       // int[nseg + 1]
     };
 };
@@ -641,7 +654,7 @@ __device__ __forceinline__ Pair2 bin2(const PairParams &p, const Ctx<MODE, LOS, 
     return o;
 }
 
-// A warp's i-points: lane l holds the block's points 2 l and 2 l + 1.
+// A warp's i-points: lane l holds point l of either half of the block.
 template <int LOS, int W>
 struct IPts {
     float x[2], y[2], z[2];        // offsets from the i-cell centre (far away if unused)
@@ -650,6 +663,20 @@ struct IPts {
     unsigned wm[2];                // W >= 2: packed integer weight
     unsigned wb[2];                // W == 3: wm halved and the next 31 bits
 };
+
+// The second half's points where the first's are (batches of that half alone).
+template <int MODE, int LOS, int W>
+__device__ __forceinline__ IPts<LOS, W> half_points(const IPts<LOS, W> &I, bool second) {
+    IPts<LOS, W> o = I;
+    if (second) {
+        o.x[0] = I.x[1]; o.y[0] = I.y[1]; o.z[0] = I.z[1];
+        if (LOS == LOS_MID && MODE != MODE_S) { o.xa[0] = I.xa[1]; o.ya[0] = I.ya[1]; o.za[0] = I.za[1]; }
+        if (W == 1) o.w[0] = I.w[1];
+        if (W >= 2) o.wm[0] = I.wm[1];
+        if (W == 3) o.wb[0] = I.wb[1];
+    }
+    return o;
+}
 
 // One i-point's registers from its record (the midpoint sums start from 2 x_i:
 // doubling is exact, so 2 x_i + d rounds once, as a fused multiply-add would).
@@ -687,7 +714,7 @@ __device__ __forceinline__ float4 tree_offset(const PairParams &p, int inode, in
                        __double2float_rn(__dsub_rn(__dadd_rn(cj[2], __dmul_rn(sz, p.g.L[2])), ci[2])), 0.f);
 }
 
-// The staged batch of JB j-points in a warp's slice.
+// The staged batch of j-points in a warp's slice.
 struct Tile {
     const float *x, *y, *z;
     const double *w;               // W == 1
@@ -696,15 +723,15 @@ struct Tile {
 };
 
 // All pairs of the warp's i-points with nq quads of staged j-points: per
-// iteration four j-points x two i-points a lane, in packed FP32, every
+// iteration four j-points x R i-points a lane, in packed FP32, every
 // counter updated by the full warp (pairs outside the histogram go to the
 // discarded counter).  Returns a bit per quad: some pair of this lane is near
 // an edge.  MASK: the tile holds points jbase, jbase + 1, ... of the i-block
 // itself and only pairs j > i count.
-template <int MODE, int LOS, int W, int PATH, bool MASK>
+template <int MODE, int LOS, int W, int PATH, bool MASK, int R>
 __device__ __forceinline__ unsigned pair_quads(const PairParams &p, const Tile &t, int nq,
                                                const IPts<LOS, W> &I, const Ctx<MODE, LOS, PATH> &c,
-                                               unsigned char *hist, unsigned wbase, int jbase,
+                                               unsigned char *hist, unsigned wbase, int jbase, int me,
                                                size_t hbase) {
     const int lane = threadIdx.x & 31;
     unsigned near = 0u;
@@ -720,14 +747,14 @@ __device__ __forceinline__ unsigned pair_quads(const PairParams &p, const Tile &
             const float2 Yh = h ? make_float2(Y.z, Y.w) : make_float2(Y.x, Y.y);
             const float2 Zh = h ? make_float2(Z.z, Z.w) : make_float2(Z.x, Z.y);
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
+            for (int r = 0; r < R; ++r) {
                 float2 dx = __fadd2_rn(Xh, make_float2(-I.x[r], -I.x[r]));
                 const float2 dy = __fadd2_rn(Yh, make_float2(-I.y[r], -I.y[r]));
                 const float2 dz = __fadd2_rn(Zh, make_float2(-I.z[r], -I.z[r]));
                 if (MASK) {   // masked pairs: far out of range
                     const int jj = jbase + 4 * q + 2 * h;
-                    if (jj <= 2 * lane + r) dx.x = p.far;
-                    if (jj + 1 <= 2 * lane + r) dx.y = p.far;
+                    if (jj <= me) dx.x = p.far;
+                    if (jj + 1 <= me) dx.y = p.far;
                 }
                 const float2 qq = __ffma2_rn(dy, dy, __fmul2_rn(dx, dx));
                 const float2 s2 = __ffma2_rn(dz, dz, qq);
@@ -920,17 +947,17 @@ __device__ __forceinline__ Fix2 fix2(const PairParams &p, float2 dx, float2 dy, 
 // mu band is taken at (T below f_close: near), and the block's own points (the
 // tile holds its points from jbase on, pairs j <= i are masked; jbase past any
 // i: none is).
-template <int MODE, int LOS, int W, int PATH, bool SLOW>
+template <int MODE, int LOS, int W, int PATH, bool SLOW, int R>
 __device__ __forceinline__ unsigned quads_fix(const PairParams &p, const Tile &t, int nq, const IPts<LOS, W> &I,
-                                              unsigned char *smem, const Bands &bd, int jbase) {
+                                              unsigned char *smem, const Bands &bd, int jbase, int me) {
     const int lane = threadIdx.x & 31;
     const float2 cfm = make_float2(bd.cfm, bd.cfm);
     const unsigned copy = 4u * (unsigned)lane;                 // LAY_BYTES
     const unsigned kc = (unsigned)(lane & (p.hist_k - 1));    // LAY_ROWS
     unsigned *hist = reinterpret_cast<unsigned *>(smem);
     unsigned near = 0u;
-    // two quads an iteration where the body stays small in the instruction cache
-    constexpr int UNROLL = SLOW || W || (LOS == LOS_MID && MODE != MODE_S) ? 1 : 2;
+    // two quads an iteration only where the code stays small (instruction cache)
+    constexpr int UNROLL = R == 1 || W || (LOS == LOS_MID && MODE != MODE_S) ? 1 : 2;
 #pragma unroll UNROLL
     for (int q = 0; q < nq; ++q) {
         const float4 X = reinterpret_cast<const float4 *>(t.x)[q];
@@ -944,14 +971,14 @@ __device__ __forceinline__ unsigned quads_fix(const PairParams &p, const Tile &t
             const float2 Yh = h ? make_float2(Y.z, Y.w) : make_float2(Y.x, Y.y);
             const float2 Zh = h ? make_float2(Z.z, Z.w) : make_float2(Z.x, Z.y);
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
+            for (int r = 0; r < R; ++r) {
                 float2 dx = __fadd2_rn(Xh, make_float2(-I.x[r], -I.x[r]));
                 const float2 dy = __fadd2_rn(Yh, make_float2(-I.y[r], -I.y[r]));
                 const float2 dz = __fadd2_rn(Zh, make_float2(-I.z[r], -I.z[r]));
                 if (SLOW) {   // masked pairs: far out of range
                     const int jj = jbase + 4 * q + 2 * h;
-                    if (jj <= 2 * lane + r) dx.x = p.far;
-                    if (jj + 1 <= 2 * lane + r) dx.y = p.far;
+                    if (jj <= me) dx.x = p.far;
+                    if (jj + 1 <= me) dx.y = p.far;
                 }
                 float2 s2;
                 const Fix2 f = fix2<MODE, LOS, PATH>(p, dx, dy, dz, bd.cfs, cfm, I.xa[r], I.ya[r], I.za[r], s2);
@@ -1039,92 +1066,103 @@ __device__ __forceinline__ unsigned long long fast_product(const IPts<LOS, W> &I
 // segment << 6 | the batch's bound (fix_bands) << 13}.  The lane repeats the quad's FP32 arithmetic
 // on the same operands, so it sees the same bins and the same near pairs, and
 // corrects the global histogram where the binary64 bin differs from the one
-// counted.  With a rescue queue (pc_opts.rescue_capacity > 0) the fast count is
+// counted.  (Pairs of a half that the batch left out are repeated too: they are
+// beyond the last edge by more than the error bands, bin -1 both ways.)  With a
+// rescue queue (pc_opts.rescue_capacity > 0) the fast count is
 // undone instead and the pair queued while there is room.
 template <int MODE, int LOS, int W, int PATH, bool TREE>
 __device__ __noinline__ void check_near(const PairParams &p, const uint2 *queue, const int4 *seg, int n, int task,
-                                        int cell, int start, int count, unsigned copy, const float2 *s_lut) {
+                                        int cell, int start, int count, int half, unsigned copy, const float2 *s_lut) {
     const int lane = threadIdx.x & 31;
     const TaskDev &T = p.tasks[task];
     Ctx<MODE, LOS, is_fix(PATH) ? PATH_LIN : PATH> c;
     if (!is_fix(PATH)) c.init(p, s_lut, copy);
-    unsigned m8 = 0u;         // near pairs: bit 4 r + j
-    int b8[8];                // the bins they were counted in (-1: none)
-    int i0 = 0, j0 = 0, img = 13;
+    // The lane's quad: segment, image, i-points and the batch's bands.
+    int i0 = 0, j0 = 0, img = 13, meta = 0;
+    unsigned vm = 0u, key = 0u;   // its j-points that are there; fix_bands
+    bool own = false;
     if (lane < n) {
         const uint2 e = queue[lane];
         const int src = (int)(e.y & 31u);
-        const bool own = (e.y >> 5) & 1u;
+        own = (e.y >> 5) & 1u;
+        key = e.y >> 13;
         j0 = (int)e.x;
-        i0 = start + 2 * src;
+        i0 = start + src;
         int4 sg = make_int4(start, start + count, TREE ? -1 : 0, 13);
         if (!own) sg = seg[(e.y >> 6) & 127u];
+        meta = sg.z;
         img = sg.w;
-        unsigned vm = 0u;
 #pragma unroll
         for (int j = 0; j < 4; ++j) vm |= (j0 + j >= sg.x && j0 + j < sg.y) ? 1u << j : 0u;
-        float3 s[4];
-        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (TREE && sg.z >= 0) o = tree_offset(p, cell, sg.z, img);
-        const int ax = TREE ? 0 : cell % p.g.ng[0];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            s[j] = make_float3(0.f, 0.f, 0.f);
-            if (!(vm >> j & 1u)) continue;
-            const float4 q = T.gj.rel[j0 + j];
-            if (TREE) s[j] = own ? make_float3(q.x, q.y, q.z) : make_float3(o.x + q.x, o.y + q.y, o.z + q.z);
-            else s[j] = own ? make_float3(q.x, q.y, q.z)
-                            : stage_grid(p, q, T.gj.cx[j0 + j], ax, sg.z, img);
-        }
-        const Bands bd = fix_bands<MODE, PATH>(p, e.y >> 13);
-        const float2 cfm = make_float2(bd.cfm, bd.cfm);
+        vm |= (src < half ? 1u << 8 : 0u) | (src < count - half ? 1u << 9 : 0u);
+    }
+    const Bands bd = fix_bands<MODE, PATH>(p, key);
+    const float2 cfm = make_float2(bd.cfm, bd.cfm);
+    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (TREE && meta >= 0 && !own && lane < n) o = tree_offset(p, cell, meta, img);
+    const int ax = TREE ? 0 : cell % p.g.ng[0];
+    auto stage = [&](int j) -> float3 {
+        const float4 q = T.gj.rel[j];
+        if (own) return make_float3(q.x, q.y, q.z);
+        if (TREE) return make_float3(o.x + q.x, o.y + q.y, o.z + q.z);
+        return stage_grid(p, q, T.gj.cx[j], ax, meta, img);
+    };
+    // Pass 1, a pair of j-points and an i-point at a time (rolled: this function
+    // runs once in thousands of quads and shares the instruction cache with the
+    // loops): which are near (bit 4 r + j), and the bins they were counted in,
+    // two 16-bit words each (0xffff: none)
+    unsigned m8 = 0u;
+    unsigned b0 = 0u, b1 = 0u, b2 = 0u, b3 = 0u;
+#pragma unroll 1
+    for (int u = 0; u < 4; ++u) {
+        const int r = u >> 1, j = j0 + 2 * (u & 1), i = i0 + r * half;
+        const unsigned v = (vm >> 8 >> r & 1u) ? vm >> (2 * (u & 1)) & 3u : 0u;
+        if (!v) continue;
+        const float3 s0 = (v & 1u) ? stage(j) : make_float3(0.f, 0.f, 0.f);
+        const float3 s1 = (v & 2u) ? stage(j + 1) : make_float3(0.f, 0.f, 0.f);
         IPts<LOS, W> I;
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            I.x[r] = I.y[r] = I.z[r] = I.xa[r] = I.ya[r] = I.za[r] = 0.f;
-            if (2 * src + r < count) load_i<MODE, LOS, W>(T.gi, i0 + r, I, r);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const float2 dx = __fadd2_rn(make_float2(s[2 * h].x, s[2 * h + 1].x), make_float2(-I.x[r], -I.x[r]));
-                const float2 dy = __fadd2_rn(make_float2(s[2 * h].y, s[2 * h + 1].y), make_float2(-I.y[r], -I.y[r]));
-                const float2 dz = __fadd2_rn(make_float2(s[2 * h].z, s[2 * h + 1].z), make_float2(-I.z[r], -I.z[r]));
-                const int j = 2 * h;
-                const bool iok = 2 * src + r < count;
-                const bool v0 = iok && (vm >> j & 1u) && !(own && j0 + j <= i0 + r);
-                const bool v1 = iok && (vm >> (j + 1) & 1u) && !(own && j0 + j + 1 <= i0 + r);
-                float2 s2;
-                bool n0, n1;
-                if (is_fix(PATH)) {
-                    const Fix2 f = fix2<MODE, LOS, PATH>(p, dx, dy, dz, bd.cfs, cfm, I.xa[r], I.ya[r], I.za[r], s2);
-                    b8[4 * r + j] = fix_bin<MODE, PATH>(p, f.T.x, f.M.x, bd, n0);
-                    b8[4 * r + j + 1] = fix_bin<MODE, PATH>(p, f.T.y, f.M.y, bd, n1);
-                } else {
-                    const float2 qq = __ffma2_rn(dy, dy, __fmul2_rn(dx, dx));
-                    s2 = __ffma2_rn(dz, dz, qq);
-                    const Pair2 b = bin2<MODE, LOS, is_fix(PATH) ? PATH_LIN : PATH>(
-                        p, c, dx, dy, dz, qq, s2, I.xa[r], I.ya[r], I.za[r]);
-                    n0 = b.n0;
-                    n1 = b.n1;
-                    b8[4 * r + j] = b8[4 * r + j + 1] = -1;   // tables: near pairs are not counted
-                    if (PATH != PATH_LUT && PATH != PATH_GLOBAL) {
-                        if (b.a0 < c.trash) b8[4 * r + j] = entry_bin(p, (int)((b.a0 - copy) / c.hk4));
-                        if (b.a1 < c.trash) b8[4 * r + j + 1] = entry_bin(p, (int)((b.a1 - copy) / c.hk4));
-                    }
-                }
-                if (v0 && n0 && s2.x < p.r2cut) m8 |= 1u << (4 * r + j);
-                if (v1 && n1 && s2.y < p.r2cut) m8 |= 1u << (4 * r + j + 1);
+        I.xa[0] = I.ya[0] = I.za[0] = 0.f;
+        load_i<MODE, LOS, W>(T.gi, i, I, 0);
+        const float2 dx = __fadd2_rn(make_float2(s0.x, s1.x), make_float2(-I.x[0], -I.x[0]));
+        const float2 dy = __fadd2_rn(make_float2(s0.y, s1.y), make_float2(-I.y[0], -I.y[0]));
+        const float2 dz = __fadd2_rn(make_float2(s0.z, s1.z), make_float2(-I.z[0], -I.z[0]));
+        float2 s2;
+        bool n0, n1;
+        int f0 = -1, f1 = -1;   // tables: near pairs are not counted
+        if (is_fix(PATH)) {
+            const Fix2 f = fix2<MODE, LOS, PATH>(p, dx, dy, dz, bd.cfs, cfm, I.xa[0], I.ya[0], I.za[0], s2);
+            f0 = fix_bin<MODE, PATH>(p, f.T.x, f.M.x, bd, n0);
+            f1 = fix_bin<MODE, PATH>(p, f.T.y, f.M.y, bd, n1);
+        } else {
+            const float2 qq = __ffma2_rn(dy, dy, __fmul2_rn(dx, dx));
+            s2 = __ffma2_rn(dz, dz, qq);
+            const Pair2 b = bin2<MODE, LOS, is_fix(PATH) ? PATH_LIN : PATH>(p, c, dx, dy, dz, qq, s2, I.xa[0],
+                                                                           I.ya[0], I.za[0]);
+            n0 = b.n0;
+            n1 = b.n1;
+            if (PATH != PATH_LUT && PATH != PATH_GLOBAL) {
+                if (b.a0 < c.trash) f0 = entry_bin(p, (int)((b.a0 - copy) / c.hk4));
+                if (b.a1 < c.trash) f1 = entry_bin(p, (int)((b.a1 - copy) / c.hk4));
             }
         }
+        if ((v & 1u) && !(own && j <= i) && n0 && s2.x < p.r2cut) m8 |= 1u << (2 * u);
+        if ((v & 2u) && !(own && j + 1 <= i) && n1 && s2.y < p.r2cut) m8 |= 2u << (2 * u);
+        const unsigned w = (unsigned)f0 & 0xffffu | (unsigned)f1 << 16;
+        b0 = u == 0 ? w : b0;
+        b1 = u == 1 ? w : b1;
+        b2 = u == 2 ? w : b2;
+        b3 = u == 3 ? w : b3;
     }
+    // Pass 2: the near pairs, one a lane
     unsigned done = 0u;
     while (__any_sync(FULL, m8 != 0u)) {
         if (m8) {
             const int k = __ffs(m8) - 1;
             m8 &= m8 - 1;
-            int fast = b8[0];
-#pragma unroll
-            for (int q = 1; q < 8; ++q) fast = k == q ? b8[q] : fast;
-            const int i = i0 + (k >> 2), j = j0 + (k & 3);
+            const unsigned w = k < 4 ? (k < 2 ? b0 : b1) : (k < 6 ? b2 : b3);
+            const unsigned fb = (k & 1) ? w >> 16 : w & 0xffffu;   // below 2^16 - 1: 4 bytes each fit shared memory
+            const int fast = fb == 0xffffu ? -1 : (int)fb;
+            const int i = i0 + half * (k >> 2), j = j0 + (k & 3);
             const size_t hb = (size_t)T.hist * p.nbins;
             unsigned long long slot = ~0ull;
             if (p.qcap) slot = atomicAdd(p.qcount, 1ull);
@@ -1168,8 +1206,10 @@ __device__ __noinline__ void check_near(const PairParams &p, const uint2 *queue,
 // work items, candidate segments and box tests (both precisions)
 // ---------------------------------------------------------------------------
 // Work items: (block, 64-point part of the block, slice of its octs).  Slices
-// (S > 1) split the i-points' candidates among warps, for about 24 items a
-// warp of the grid, so that the last items do not leave the chip half empty.
+// (S > 1) split the i-points' candidates among warps, for about 12 items a
+// warp of the grid, so that the last items do not leave the chip half empty (24:
+// a warp starts over too often, 312k points 2.97 -> 3.32 ms; 6: within 2 %, but
+// 3 to 4 % slower where a batch of items takes long).
 // One histogram: each warp takes items from the global counter until none are
 // left.  Several (batches): the CTA takes ranges of items of one histogram and
 // flushes between them.
@@ -1182,7 +1222,7 @@ struct Items {
     __device__ __forceinline__ void init(const PairParams &p, int nw) {
         const int nblocks = *p.nblocks;
         const long long units = max((long long)nblocks, p.npts_i / BI + 1);
-        const long long want = 24ll * gridDim.x * nw;
+        const long long want = 12ll * gridDim.x * nw;
         S = 1;
         if (units < want) S = (int)min(32ll, (want + units - 1) / units);
         per_block = p.nsub * S;
@@ -1245,18 +1285,27 @@ __device__ __forceinline__ long long next_item(const PairParams &p, const Items 
 struct Item {
     Block B;
     int start, count, part;
+    int half;                // points of the first half: lane l holds points l and half + l
     int ax, ay, az;          // grid: the i-cell
     int ts0, ntl, own_end;   // list (tree) or stencil rows; end of the own cell (auto)
 };
 template <bool TREE>
 __device__ __forceinline__ bool open_item(const PairParams &p, const Items &W, long long it, Item &I) {
-    I.B = p.blocks[it / W.per_block];
-    const int rem = (int)(it % W.per_block), sub = rem / W.S;
+    const unsigned blk = (unsigned)it / (unsigned)W.per_block;   // (the counter of the items is an int)
+    I.B = p.blocks[blk];
+    const int rem = (int)((unsigned)it - blk * (unsigned)W.per_block), sub = rem / W.S;
     I.part = rem - sub * W.S;
     const int k = (I.B.count + BI - 1) / BI;
     if (sub >= k) return false;
-    I.start = I.B.start + (int)((long long)I.B.count * sub / k);
-    I.count = I.B.start + (int)((long long)I.B.count * (sub + 1) / k) - I.start;
+    if (TREE) {   // equal parts: close to the k-d tree's own cuts
+        I.start = I.B.start + (int)((long long)I.B.count * sub / k);
+        I.count = I.B.start + (int)((long long)I.B.count * (sub + 1) / k) - I.start;
+        I.half = (I.count + 1) / 2;
+    } else {      // full parts: a rest of up to 32 points leaves the second half out
+        I.start = I.B.start + BI * sub;
+        I.count = min(BI, I.B.count - BI * sub);
+        I.half = min(32, I.count);
+    }
     const TaskDev &T = p.tasks[I.B.task];
     const int nx = p.g.ng[0], ny = p.g.ng[1];
     I.ax = TREE ? 0 : I.B.cell % nx;
@@ -1278,7 +1327,8 @@ __device__ __forceinline__ bool open_item(const PairParams &p, const Items &W, l
     return true;
 }
 
-// Bounding box of the warp's i-points, relative to the j-grid's origin.
+// Bounding box of a half of the warp's i-points, relative to the j-grid's origin
+// (no points: infinitely far from everything).
 struct IBox {
     float lx, ly, lz, hx, hy, hz;
     __device__ __forceinline__ void clear() {
@@ -1296,6 +1346,12 @@ struct IBox {
                     ogz = (float)(T.gj.org[2] - T.gi.org[2]);
         lx = warp_minf(lx) - ogx; ly = warp_minf(ly) - ogy; lz = warp_minf(lz) - ogz;
         hx = warp_maxf(hx) - ogx; hy = warp_maxf(hy) - ogy; hz = warp_maxf(hz) - ogz;
+    }
+    __device__ __forceinline__ void store(float4 *b) const {
+        if ((threadIdx.x & 31) == 0) {
+            b[0] = make_float4(lx, ly, lz, 0.f);
+            b[1] = make_float4(hx, hy, hz, 0.f);
+        }
     }
 };
 
@@ -1378,19 +1434,21 @@ __device__ __forceinline__ int build_chunk(const PairParams &p, const TaskDev &T
     return noct;
 }
 
-// One round: octs 32 rd .. 32 rd + 31 of the chunk, those whose box can reach
-// the i-points' box appended to the ring {first point, segment, squared gap}.
-// Boxes are rounded outward, and r2prune carries the rounding of this test
-// (host side), so a dropped pair is at least rcut apart.
-template <int MODE, int LOS>
-__device__ __forceinline__ int ring_round(const PairParams &p, const TaskDev &T, int rd, int noct, int nseg,
-                                          const int4 *seg, const int *pref, const IBox &b, int count, int4 *ring,
-                                          int tail, unsigned long long &cand, unsigned long long &pruned) {
+// One round: octs 32 rd .. 32 rd + 31 of the chunk.  Those whose box can reach
+// both halves of the i-points, or only the first or the second, are appended to
+// that class's list {first point, segment | upper half of the squared gap << 16}
+// and its length n[] grows.  Boxes are rounded outward, and r2prune carries the
+// rounding of this test (host side), so a dropped pair is at least rcut apart.
+template <int MODE, int LOS, class O>
+__device__ __forceinline__ void ring_round(const PairParams &p, const TaskDev &T, int rd, int noct, int nseg,
+                                           const int4 *seg, const int *pref, const float4 *ibox, int count, int half,
+                                           uint2 *ring, int (&n)[3], unsigned long long &cand,
+                                           unsigned long long &pruned) {
     const int lane = threadIdx.x & 31;
     const int f = rd * 32 + lane;
-    bool keep = false;
+    bool keep[2] = {false, false};
     int lo = 0, p0 = 0;
-    float g2 = 0.f;
+    float g2 = INFINITY;
     if (f < noct) {
         int hi = nseg;
         while (hi - lo > 1) {
@@ -1408,26 +1466,46 @@ __device__ __forceinline__ int ring_round(const PairParams &p, const TaskDev &T,
             bl.x += sx; bl.y += sy; bl.z += sz;
             bh.x += sx; bh.y += sy; bh.z += sz;
         }
-        const float gx = fmaxf(fmaxf(bl.x - b.hx, b.lx - bh.x), 0.f);
-        const float gy = fmaxf(fmaxf(bl.y - b.hy, b.ly - bh.y), 0.f);
-        const float gz = fmaxf(fmaxf(bl.z - b.hz, b.lz - bh.z), 0.f);
-        const float gq = fmaf(gy, gy, gx * gx);
-        g2 = fmaf(gz, gz, gq);
-        keep = g2 < p.r2prune;
-        if (MODE == MODE_SIGPI && LOS == LOS_Z)   // the reach is a cylinder
-            keep = keep && gq < p.q2prune && gz < p.zprune;
-        if (MODE == MODE_SIGPI) g2 = LOS == LOS_Z ? gq : 0.f;
-        const unsigned long long np2 =
-            (unsigned long long)(min(sg.y, p0 + 8) - max(sg.x, p0)) * (unsigned)count;
-        cand += np2;
-        if (!keep) pruned += np2;
+        const unsigned nj = (unsigned)(min(sg.y, p0 + 8) - max(sg.x, p0));
+        cand += (unsigned long long)(nj * (unsigned)count);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const float4 l = ibox[2 * r], h = ibox[2 * r + 1];
+            const float gx = fmaxf(fmaxf(bl.x - h.x, l.x - bh.x), 0.f);
+            const float gy = fmaxf(fmaxf(bl.y - h.y, l.y - bh.y), 0.f);
+            const float gz = fmaxf(fmaxf(bl.z - h.z, l.z - bh.z), 0.f);
+            const float gq = fmaf(gy, gy, gx * gx), g = fmaf(gz, gz, gq);
+            keep[r] = g < p.r2prune;
+            if (MODE == MODE_SIGPI && LOS == LOS_Z)   // the reach is a cylinder
+                keep[r] = keep[r] && gq < p.q2prune && gz < p.zprune;
+            // (sigma, pi): the gap across the line of sight
+            if (keep[r]) g2 = fminf(g2, MODE != MODE_SIGPI ? g : (LOS == LOS_Z ? gq : 0.f));
+            else pruned += (unsigned long long)(nj * (unsigned)(r ? count - half : half));
+        }
     }
-    const unsigned who = __ballot_sync(FULL, keep);
-    if (keep)
-        ring[(tail + __popc(who & ((1u << lane) - 1u))) & (RING - 1)] =
-            make_int4(p0, lo, __float_as_int(g2), 0);   // (sigma, pi): the gap across the line of sight
+    const uint2 e = make_uint2((unsigned)p0, (unsigned)lo | (__float_as_uint(g2) & 0xffff0000u));
+    const unsigned below = (1u << lane) - 1u;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const bool in = c == 0 ? keep[0] && keep[1] : (c == 1 ? keep[0] && !keep[1] : !keep[0] && keep[1]);
+        const unsigned who = __ballot_sync(FULL, in);
+        if (in) ring[c * O::list + n[c] + __popc(who & below)] = e;
+        n[c] += __popc(who);
+    }
     __syncwarp();
-    return tail + __popc(who);
+}
+
+// The class of the next batch: one with a full batch, else (rounds over) any with
+// octs left; the batch takes the last of its list.  -1: none.
+template <class O>
+__device__ __forceinline__ int next_class(const int (&n)[3], bool over) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        if (n[c] >= O::jo) return c;
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        if (over && n[c] > 0) return c;
+    return -1;
 }
 
 // ---------------------------------------------------------------------------
@@ -1452,12 +1530,13 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
     int4 *seg = reinterpret_cast<int4 *>(ws);
     float4 *soff = reinterpret_cast<float4 *>(ws + O::soff);
     float *tx = reinterpret_cast<float *>(ws + O::tile);
-    float *ty = tx + JB, *tz = ty + JB;
+    float *ty = tx + O::jb, *tz = ty + O::jb;
     double *tw = reinterpret_cast<double *>(ws + O::tw);
     unsigned *twm = reinterpret_cast<unsigned *>(tw);
-    unsigned *twl = twm + JB;
+    unsigned *twl = twm + O::jb;
     uint2 *queue = reinterpret_cast<uint2 *>(ws + O::queue);
-    int4 *ring = reinterpret_cast<int4 *>(ws + O::ring);
+    uint2 *ring = reinterpret_cast<uint2 *>(ws + O::ring);
+    float4 *ibox = reinterpret_cast<float4 *>(ws + O::ibox);
     int *pref = reinterpret_cast<int *>(ws + O::pref);
     const Tile tile{tx, ty, tz, tw, twm, twl};
     const float2 *s_lut = reinterpret_cast<const float2 *>(smem + p.sm_lut);
@@ -1488,6 +1567,10 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
     // counter, and flushes (counts with the weights) only past a quarter of the
     // bound; what is in flight during a flush, at most 16 slots of a lane and
     // warp, is taken off the quarter
+    // one loop body for both halves in turn where a body of two i-points a lane is
+    // too large to share the instruction cache with the rest: (s, mu) along the
+    // midpoint with binary64 weights, 140k points, 21.8 -> 16.4 ms
+    constexpr bool TWO = !(W == 3 && LOS == LOS_MID && MODE != MODE_S);
     constexpr bool SCAN = !(is_fix(PATH) && MODE == MODE_S);
     constexpr unsigned wmax = W == 3 ? WINT_LIMIT / 2 : WINT_LIMIT;
     const unsigned wlimit = (SCAN ? wmax / 4 * 3 : wmax) / (unsigned)nw;
@@ -1514,18 +1597,19 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
         const TaskDev &T = p.tasks[it.B.task];
 
         IPts<LOS, W> I;
-        IBox box;
-        box.clear();
+        __syncwarp();
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
+            IBox box;
+            box.clear();
             I.x[r] = -far;      // unused: out of range of every j-point
             I.y[r] = I.z[r] = 0.f;
             I.xa[r] = I.ya[r] = I.za[r] = 0.f;
             I.w[r] = 0.0;
             I.wm[r] = 0u;
             I.wb[r] = 0u;
-            if (2 * lane + r < it.count) {
-                const int i = it.start + 2 * lane + r;
+            if (lane < (r ? it.count - it.half : it.half)) {
+                const int i = it.start + lane + r * it.half;
                 load_i<MODE, LOS, W>(T.gi, i, I, r);
                 if (is_fix(PATH) && !(fabsf(I.x[r]) + fabsf(I.y[r]) + fabsf(I.z[r]) < 1e16f)) {
                     I.x[r] = -far;      // not a number: no pair
@@ -1533,8 +1617,9 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
                 }
                 box.add(T.gi, T.gi.xw[i]);
             }
+            box.finish(T);
+            box.store(ibox + 2 * r);
         }
-        box.finish(T);
 
         // pairs inside the block (j > i) first
         bool own = T.is_auto && it.part == 0;
@@ -1551,21 +1636,30 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
             // this slice's rounds: global round number = part (mod S)
             int rd = (it.part - round0 % items.S + items.S) % items.S;
             round0 += nround;
-            int head = 0, tail = 0;
+            int left[3] = {0, 0, 0};   // octs to stage: for both halves, the first, the second
             for (;;) {
-                while (!own && tail - head < JO && rd < nround) {
-                    tail = ring_round<MODE, LOS>(p, T, rd, noct, nseg, seg, pref, box, it.count, ring, tail, cand,
-                                                 pruned);
+                while (!own && next_class<O>(left, false) < 0 && rd < nround) {
+                    ring_round<MODE, LOS, O>(p, T, rd, noct, nseg, seg, pref, ibox, it.count, it.half, ring, left, cand,
+                                             pruned);
                     rd += items.S;
                 }
-                // one batch: the block's own points, or up to eight octs
-                const int m = own ? (it.count + 7) >> 3 : min(JO, tail - head);
+                // one batch: the block's own points, or up to eight octs of a class
+                const int cls = own ? 0 : next_class<O>(left, true);
+                int m = (it.count + 7) >> 3;
+                if (!own) {
+                    const int nc = cls == 1 ? left[1] : (cls == 2 ? left[2] : left[0]);
+                    m = cls < 0 ? 0 : min((int)O::jo, nc);
+#pragma unroll
+                    for (int c = 0; c < 3; ++c)
+                        if (c == cls) left[c] -= m;
+                }
+                const uint2 *list = ring + (cls == 1 ? O::list + left[1] : (cls == 2 ? 2 * O::list + left[2] : left[0]));
                 unsigned near = 0u;
                 unsigned key = 0u;   // bound of the batch's separations (fix_bands)
                 if (m > 0) {
-                    float g2 = INFINITY;
-#pragma unroll
-                    for (int h = 0; h < JB / 32; ++h) {
+                    unsigned kmin = 0x7f80u;
+#pragma unroll 2
+                    for (int h = 0; h < (m + 3) >> 2; ++h) {
                         const int sl = lane + 32 * h, oc = sl >> 3;
                         float3 s = make_float3(far, 0.f, 0.f);
                         float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1575,15 +1669,16 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
                             q = T.gj.rel[pj];
                             s = make_float3(q.x, q.y, q.z);
                         } else if (!own && oc < m) {
-                            const int4 e = ring[(head + oc) & (RING - 1)];
-                            const int4 sg = seg[e.y];
-                            g2 = fminf(g2, __int_as_float(e.z));
-                            pj = e.x + (lane & 7);
+                            const uint2 e = list[oc];
+                            const unsigned es = e.y & 0xffffu;
+                            const int4 sg = seg[es];
+                            kmin = min(kmin, e.y >> 16);
+                            pj = (int)e.x + (lane & 7);
                             v = pj >= sg.x && pj < sg.y;
                             if (v) {
                                 q = T.gj.rel[pj];
                                 if (TREE) {
-                                    const float4 o = soff[e.y];
+                                    const float4 o = soff[es];
                                     s = make_float3(o.x + q.x, o.y + q.y, o.z + q.z);
                                 } else {
                                     s = stage_grid(p, q, T.gj.cx[pj], it.ax, sg.z, sg.w);
@@ -1619,27 +1714,45 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
                         if (MODE == MODE_SMU || PATH == PATH_FIXLOG) {
                             // the batch's smallest separation: the smallest gap less the
                             // box tests' rounding
-                            g2 = own ? 0.f : __uint_as_float(__reduce_min_sync(FULL, __float_as_uint(g2)));
+                            const float g2 = own ? 0.f : __uint_as_float(__reduce_min_sync(FULL, kmin) << 16);
                             const float g = fmaxf(g2 * rsqrt_fast(fmaxf(g2, 1e-30f)) - p.f_gm, 0.f);
                             key = __float_as_uint(g * g) >> 16;
                             slow = own || (MODE == MODE_SMU && __uint_as_float(key << 16) < p.f_sf2);
                         }
                         const Bands bd = fix_bands<MODE, PATH>(p, key);
-                        if (slow)
-                            near = quads_fix<MODE, LOS, W, PATH, true>(p, tile, nq, I, smem, bd, own ? 0 : 2 * BI);
-                        else
-                            near = quads_fix<MODE, LOS, W, PATH, false>(p, tile, nq, I, smem, bd, 0);
+                        if (slow) {
+#pragma unroll 1
+                            for (int r = cls == 2; r < (cls == 1 ? 1 : 2); ++r)
+                                near |= quads_fix<MODE, LOS, W, PATH, true, 1>(
+                                    p, tile, nq, half_points<MODE, LOS, W>(I, r), smem, bd, own ? 0 : BI,
+                                    lane + r * it.half);
+                        } else if (TWO && cls == 0) {
+                            near = quads_fix<MODE, LOS, W, PATH, false, TWO ? 2 : 1>(p, tile, nq, I, smem, bd, 0, 0);
+                        } else {
+#pragma unroll 1
+                            for (int r = cls == 2; r < (TWO || cls == 1 ? 1 + (cls == 2) : 2); ++r)
+                                near |= quads_fix<MODE, LOS, W, PATH, false, 1>(
+                                    p, tile, nq, half_points<MODE, LOS, W>(I, r), smem, bd, 0, 0);
+                        }
                     } else {
                         const size_t hbase = (size_t)T.hist * p.nbins;
-                        if (own)
-                            near = pair_quads<MODE, LOS, W, PATH, true>(p, tile, nq, I, c, smem, wbase, 0, hbase);
-                        else
-                            near = pair_quads<MODE, LOS, W, PATH, false>(p, tile, nq, I, c, smem, wbase, 0, hbase);
+                        if (own) {
+#pragma unroll 1
+                            for (int r = 0; r < 2; ++r)
+                                near |= pair_quads<MODE, LOS, W, PATH, true, 1>(
+                                    p, tile, nq, half_points<MODE, LOS, W>(I, r), c, smem, wbase, 0,
+                                    lane + r * it.half, hbase);
+                        } else if (cls == 0) {
+                            near = pair_quads<MODE, LOS, W, PATH, false, 2>(p, tile, nq, I, c, smem, wbase, 0, 0, hbase);
+                        } else {
+                            near = pair_quads<MODE, LOS, W, PATH, false, 1>(
+                                p, tile, nq, half_points<MODE, LOS, W>(I, cls == 2), c, smem, wbase, 0, 0, hbase);
+                        }
                     }
                 }
                 // queue the near quads, check them 32 at a time (and, before the
                 // segments change, the rest)
-                const bool last = rd >= nround && (own ? tail == head && nround == 0 : tail - head == m);
+                const bool last = rd >= nround && left[0] + left[1] + left[2] == 0 && !(own && nround > 0);
                 for (;;) {
                     const unsigned who = __ballot_sync(FULL, near != 0u);
                     if (near) {
@@ -1647,9 +1760,9 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
                         near &= near - 1;
                         uint2 e = make_uint2((unsigned)(it.start + 4 * q), (unsigned)lane | 32u | key << 13);
                         if (!own) {
-                            const int4 o = ring[(head + (q >> 1)) & (RING - 1)];
-                            e = make_uint2((unsigned)(o.x + 4 * (q & 1)),
-                                           (unsigned)lane | (unsigned)o.y << 6 | key << 13);
+                            const uint2 o = list[q >> 1];
+                            e = make_uint2(o.x + 4u * (unsigned)(q & 1),
+                                           (unsigned)lane | (o.y & 0xffffu) << 6 | key << 13);
                         }
                         queue[qn + __popc(who & ((1u << lane) - 1u))] = e;
                     }
@@ -1658,7 +1771,7 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
                     if (qn >= 32 || (rest && qn > 0)) {
                         const int n = min(qn, 32);
                         __syncwarp();
-                        check_near<MODE, LOS, W, PATH, TREE>(p, queue, seg, n, it.B.task, it.B.cell, it.start, it.count, copy,
+                        check_near<MODE, LOS, W, PATH, TREE>(p, queue, seg, n, it.B.task, it.B.cell, it.start, it.count, it.half, copy,
                                                              s_lut);
                         __syncwarp();
                         qn -= n;
@@ -1670,7 +1783,6 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
                     __syncwarp();
                     if (who == 0u && qn < 32 && !(last && qn > 0)) break;
                 }
-                if (!own) head += m;
                 own = false;
                 if (last) break;
             }
@@ -1779,7 +1891,8 @@ __global__ void __maxnreg__(96) k_pairs_f64(const __grid_constant__ PairParams p
     unsigned char *ws = smem + p.sm_warp + (size_t)warp * O::total;
     int4 *seg = reinterpret_cast<int4 *>(ws);
     double *tile = reinterpret_cast<double *>(ws + O::tile);   // {x, y, z, w, shift x, y, z} by point
-    int4 *ring = reinterpret_cast<int4 *>(ws + O::ring);
+    uint2 *ring = reinterpret_cast<uint2 *>(ws + O::ring);
+    float4 *ibox = reinterpret_cast<float4 *>(ws + O::ibox);
     int *pref = reinterpret_cast<int *>(ws + O::pref);
     double *sEa = reinterpret_cast<double *>(smem + p.sm_lut), *sEb = sEa + p.n_a + 1;
     float *sF = reinterpret_cast<float *>(sEb + p.n_b + 1);
@@ -1823,20 +1936,22 @@ __global__ void __maxnreg__(96) k_pairs_f64(const __grid_constant__ PairParams p
         const TaskDev &T = p.tasks[it.B.task];
         const size_t hbase = (size_t)T.hist * p.nbins;
         double a[2][3], wi[2];
-        IBox box;
-        box.clear();
+        __syncwarp();
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
+            IBox box;
+            box.clear();
             a[r][0] = a[r][1] = a[r][2] = __longlong_as_double(0x7ff8000000000000ll);   // no point: not a number
             wi[r] = 0.0;
-            if (2 * lane + r < it.count) {
-                const double4_32a q = T.gi.xw[it.start + 2 * lane + r];
+            if (lane < (r ? it.count - it.half : it.half)) {
+                const double4_32a q = T.gi.xw[it.start + lane + r * it.half];
                 a[r][0] = q.x; a[r][1] = q.y; a[r][2] = q.z;
                 wi[r] = q.w;
                 box.add(T.gi, q);
             }
+            box.finish(T);
+            box.store(ibox + 2 * r);
         }
-        box.finish(T);
         bool own = T.is_auto && it.part == 0;
         if (own && lane == 0) cand += (unsigned long long)it.count * (unsigned)(it.count - 1) / 2;
         const int nchunk = max(1, (it.ntl + 31) / 32);
@@ -1849,25 +1964,34 @@ __global__ void __maxnreg__(96) k_pairs_f64(const __grid_constant__ PairParams p
             const int nround = (noct + 31) / 32;
             int rd = (it.part - round0 % items.S + items.S) % items.S;
             round0 += nround;
-            int head = 0, tail = 0;
+            int left[3] = {0, 0, 0};   // octs to stage: for both halves, the first, the second
             for (;;) {
-                while (!own && tail - head < JO && rd < nround) {
-                    tail = ring_round<MODE, LOS>(p, T, rd, noct, nseg, seg, pref, box, it.count, ring, tail, cand,
-                                                 pruned);
+                while (!own && next_class<O>(left, false) < 0 && rd < nround) {
+                    ring_round<MODE, LOS, O>(p, T, rd, noct, nseg, seg, pref, ibox, it.count, it.half, ring, left, cand,
+                                             pruned);
                     rd += items.S;
                 }
-                const int m = own ? (it.count + 7) >> 3 : min(JO, tail - head);
+                const int cls = own ? 0 : next_class<O>(left, true);
+                int m = (it.count + 7) >> 3;
+                if (!own) {
+                    const int nc = cls == 1 ? left[1] : (cls == 2 ? left[2] : left[0]);
+                    m = cls < 0 ? 0 : min((int)O::jo, nc);
+#pragma unroll
+                    for (int c = 0; c < 3; ++c)
+                        if (c == cls) left[c] -= m;
+                }
                 if (m == 0) break;
+                const uint2 *list = ring + (cls == 1 ? O::list + left[1] : (cls == 2 ? 2 * O::list + left[2] : left[0]));
                 bool shifted = false;
 #pragma unroll
-                for (int h = 0; h < JB / 32; ++h) {
+                for (int h = 0; h < O::jb / 32; ++h) {
                     const int sl = lane + 32 * h, oc = sl >> 3;
                     int pj = it.start + sl, img = 13;
                     bool v = own && sl < it.count;
                     if (!own && oc < m) {
-                        const int4 e = ring[(head + oc) & (RING - 1)];
-                        const int4 sg = seg[e.y];
-                        pj = e.x + (lane & 7);
+                        const uint2 e = list[oc];
+                        const int4 sg = seg[e.y & 0xffffu];
+                        pj = (int)e.x + (lane & 7);
                         v = pj >= sg.x && pj < sg.y;
                         img = sg.w;
                     }
@@ -1893,6 +2017,7 @@ __global__ void __maxnreg__(96) k_pairs_f64(const __grid_constant__ PairParams p
                     const double *t = tile + 7 * j;
 #pragma unroll
                     for (int r = 0; r < 2; ++r) {
+                        if (cls == 2 - r) continue;   // the other half's batch
                         double d0 = __dsub_rn(t[0], a[r][0]), d1 = __dsub_rn(t[1], a[r][1]),
                                d2 = __dsub_rn(t[2], a[r][2]);
                         if (shifted) {
@@ -1903,7 +2028,7 @@ __global__ void __maxnreg__(96) k_pairs_f64(const __grid_constant__ PairParams p
                         const double s2 =
                             __dadd_rn(__dadd_rn(__dmul_rn(d0, d0), __dmul_rn(d1, d1)), __dmul_rn(d2, d2));
                         bool in = s2 < reach2;
-                        if (own) in = in && j > 2 * lane + r;
+                        if (own) in = in && j > lane + r * it.half;
                         if (in) {
                             const int b = bin64<MODE, LOS>(d0, d1, d2, s2, a[r], t, E, p.n_a, p.n_b);
                             if (b >= 0) {
@@ -1918,7 +2043,6 @@ __global__ void __maxnreg__(96) k_pairs_f64(const __grid_constant__ PairParams p
                         }
                     }
                 }
-                if (!own) head += m;
                 own = false;
                 __syncwarp();
             }

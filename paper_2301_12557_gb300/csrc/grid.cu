@@ -513,13 +513,7 @@ extern "C" pc_status pc_aabb(const double *xyz, long long n, void *stream, doubl
 
 static void grid_release(pc_grid *g) {
     if (!g) return;
-    cudaFree(g->rel);
-    cudaFree(g->cx);
-    cudaFree(g->xw);
-    cudaFree(g->cell_start);
-    cudaFree(g->perm);
-    cudaFree(g->wlo);
-    cudaFree(g->obox);
+    cudaFree(g->arrays);
     delete g;
 }
 
@@ -703,13 +697,28 @@ extern "C" pc_status pc_build_grid(const double *xyz, const void *w, int w_is_f3
     // device arrays
     cudaError_t e = cudaSuccess;
     size_t nn = std::max<long long>(n, 1);
-    e = ::pc::alloc_dev(&g->rel, sizeof(float4) * nn);
-    if (e == cudaSuccess) e = ::pc::alloc_dev(&g->cx, sizeof(uint16_t) * nn);
-    if (e == cudaSuccess) e = ::pc::alloc_dev(&g->xw, sizeof(double4_32a) * nn);
-    if (e == cudaSuccess) e = ::pc::alloc_dev(&g->cell_start, sizeof(int) * (g->ncell + 1));
-    if (e == cudaSuccess) e = ::pc::alloc_dev(&g->perm, sizeof(int) * nn);
-    if (e == cudaSuccess) e = ::pc::alloc_dev(&g->obox, obox_bytes((long long)nn));
-    if (e == cudaSuccess && g->wcorr) e = ::pc::alloc_dev(&g->wlo, sizeof(unsigned) * nn);
+    {   // one allocation: each call costs as much as a small count
+        size_t total = 0;
+        auto place = [&](size_t bytes) {
+            const size_t at = total;
+            total += (bytes + 255) / 256 * 256;
+            return at;
+        };
+        const size_t xw = place(sizeof(double4_32a) * nn), rel = place(sizeof(float4) * nn),
+                     obox = place(obox_bytes((long long)nn)), start = place(sizeof(int) * ((size_t)g->ncell + 1)),
+                     perm = place(sizeof(int) * nn), cx = place(sizeof(uint16_t) * nn),
+                     wlo = g->wcorr ? place(sizeof(unsigned) * nn) : 0;
+        e = ::pc::alloc_dev(&g->arrays, total);
+        if (e == cudaSuccess) {
+            g->xw = reinterpret_cast<double4_32a *>(g->arrays + xw);
+            g->rel = reinterpret_cast<float4 *>(g->arrays + rel);
+            g->obox = reinterpret_cast<float4 *>(g->arrays + obox);
+            g->cell_start = reinterpret_cast<int *>(g->arrays + start);
+            g->perm = reinterpret_cast<int *>(g->arrays + perm);
+            g->cx = reinterpret_cast<uint16_t *>(g->arrays + cx);
+            if (g->wcorr) g->wlo = reinterpret_cast<unsigned *>(g->arrays + wlo);
+        }
+    }
     if (e != cudaSuccess) {
         cleanup();
         grid_release(g);
@@ -722,11 +731,9 @@ extern "C" pc_status pc_build_grid(const double *xyz, const void *w, int w_is_f3
     int sub_bits = per_cell >= 2048.0 ? 4 : (per_cell >= 256.0 ? 3 : (per_cell >= 32.0 ? 2 : (per_cell >= 4.0 ? 1 : 0)));
     while (sub_bits > 0 && ((long long)g->ncell << (3 * sub_bits)) > (1LL << 28)) --sub_bits;
     const int nkey = g->ncell << (3 * sub_bits);
-    int *counts = nullptr, *cell = nullptr, *slot = nullptr, *key_start = nullptr;
-    e = ::pc::alloc_dev_async(&counts, sizeof(int) * nkey, st);
-    if (e == cudaSuccess) e = ::pc::alloc_dev_async(&key_start, sizeof(int) * ((size_t)nkey + 1), st);
-    if (e == cudaSuccess) e = ::pc::alloc_dev_async(&cell, sizeof(int) * nn, st);
-    if (e == cudaSuccess) e = ::pc::alloc_dev_async(&slot, sizeof(int) * nn, st);
+    int *counts = nullptr;   // with the keys' starts, the points' keys and slots after them
+    e = ::pc::alloc_dev_async(&counts, sizeof(int) * (2 * (size_t)nkey + 1 + 2 * nn), st);
+    int *key_start = counts + nkey, *cell = key_start + nkey + 1, *slot = cell + nn;
     if (e == cudaSuccess) e = cudaMemsetAsync(counts, 0, sizeof(int) * nkey, st);
     if (e == cudaSuccess && n > 0) {
         int blocks = (int)((n + 255) / 256);
@@ -751,10 +758,7 @@ extern "C" pc_status pc_build_grid(const double *xyz, const void *w, int w_is_f3
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = make_obox(g->xw, (int)n, G.lo, g->obox, st);
-    if (key_start) cudaFreeAsync(key_start, st);
     if (counts) cudaFreeAsync(counts, st);
-    if (cell) cudaFreeAsync(cell, st);
-    if (slot) cudaFreeAsync(slot, st);
     cleanup();
     cudaError_t e2 = cudaStreamSynchronize(st);
     if (e == cudaSuccess) e = e2;

@@ -24,6 +24,7 @@ struct pc_grid {
     // 32 in wlo (wcorr)
     int wint = 0, wemax = 0, wemin = 0;
     int wcorr = 0;
+    unsigned char *arrays;         // the allocation that holds the arrays below
     unsigned *wlo = nullptr;       // cell order: remainders (GridDev::wlo), or null
     float4 *rel;
     uint16_t *cx;

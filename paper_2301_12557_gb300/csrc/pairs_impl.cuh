@@ -64,8 +64,9 @@ __host__ __device__ inline size_t align_up(size_t x, size_t a) { return (x + a -
 // FP32 kernel: shared memory
 // ---------------------------------------------------------------------------
 constexpr int BI = 64;        // i-points per warp: two halves of 32, one point of each a lane
-constexpr int JB_COUNTS = 128;   // j-points per staged batch, counts only (64: 4 % slower; weights bound a
-                                 // batch by the records' range)
+// j-points per staged batch: 128 (64 is 4 % slower), or 64 where the range of the
+// weights' records bounds a batch (bytes: LAY_BYTES) and in the FP64 kernel
+__host__ __device__ constexpr int batch_points(int w, bool bytes) { return w == 0 || (w == 2 && bytes) ? 128 : 64; }
 constexpr int QCAP = 64;      // near-edge quads kept by a warp before it checks them
 constexpr int FIX_TOP = 126;  // most bins per axis of the fixed-point floors (125 with an offset)
 constexpr int SEG_G = 97;     // j-segments of a chunk: 32 stencil rows, <= 3 each, and the own cell
@@ -75,10 +76,10 @@ constexpr int SEG_T = 33;     // 32 listed tree nodes and the own node
 // batch (FP64: coordinates and weight, and the images' shifts), its weights, the
 // near-edge queue, the octs to stage, the halves' boxes and the octs before each
 // segment.
-template <bool TREE, bool WEIGHTED, bool F64>
+template <bool TREE, bool WEIGHTED, bool F64, int JB>
 struct WarpOff {
     enum {
-        jb = WEIGHTED || F64 ? 64 : JB_COUNTS,               // j-points per staged batch
+        jb = JB,
         jo = jb / 8,
         list = jo + 32,                                      // octs kept per class: jo - 1 and a round
         nseg = TREE ? SEG_T : SEG_G,
@@ -92,10 +93,14 @@ struct WarpOff {
         total = (pref + (nseg + 1) * 4 + 15) / 16 * 16       // int[nseg + 1]
     };
 };
+enum { LAY_ROWS = 0, LAY_SKEW = 1, LAY_BYTES = 2 };   // see below
 inline size_t warp_slice(const PairParams &p) {
-    int n = p.weighted ? (int)WarpOff<false, true, false>::total : (int)WarpOff<false, false, false>::total;
-    if (p.tree) n = p.weighted ? (int)WarpOff<true, true, false>::total : (int)WarpOff<true, false, false>::total;
-    if (p.f64) n = (int)WarpOff<false, false, true>::total;
+    const bool wide = batch_points(!p.weighted ? 0 : (p.wint ? 2 + p.wcorr : 1), p.layout == LAY_BYTES) == 128;
+    int n = 0;
+    if (p.f64) n = (int)WarpOff<false, false, true, 64>::total;
+    else if (!p.weighted) n = p.tree ? (int)WarpOff<true, false, false, 128>::total : (int)WarpOff<false, false, false, 128>::total;
+    else if (wide) n = p.tree ? (int)WarpOff<true, true, false, 128>::total : (int)WarpOff<false, true, false, 128>::total;
+    else n = p.tree ? (int)WarpOff<true, true, false, 64>::total : (int)WarpOff<false, true, false, 64>::total;
     return (size_t)n;
 }
 
@@ -105,9 +110,10 @@ inline size_t warp_slice(const PairParams &p) {
 //             index, or records of three u32 at 3 x the word
 //  LAY_SKEW   word w + w / 32, w = 256 n + m: the bytes of the two fixed-point
 //             floors side by side; the skew puts rows 8 banks apart (counts only)
-//  LAY_BYTES  word 64 n + k, 32 copies (one axis); weights: the pieces of a
-//             product at + 32 words and, past the last row, at + 0 and + 32
-enum { LAY_ROWS = 0, LAY_SKEW = 1, LAY_BYTES = 2 };
+//  LAY_BYTES  word 64 n + k, 32 copies (one axis); weights: the count and a
+//             product's lowest piece share that word (the count in its upper 12
+//             bits), the next 20 bits add up at + 32 words and the top ones past
+//             the last row
 
 __host__ __device__ inline int hist_words(const PairParams &p) {
     if (p.layout == LAY_SKEW) {
@@ -197,6 +203,7 @@ __device__ __forceinline__ int hist_word(const PairParams &p, int e, int k, int 
 
 static __device__ __noinline__ void flush_counts(const PairParams &p, int off, int first, int nw, int h) {
     extern __shared__ __align__(16) unsigned char smem[];
+    if (p.weighted && p.layout == LAY_BYTES) return;   // flush_bytes takes them along
     const int lane = threadIdx.x & 31, K = p.hist_k, words = hist_entries(p) * K;
     int *hist = reinterpret_cast<int *>(smem + off);
     for (int w0 = first * 32; w0 < words; w0 += nw * 32) {
@@ -212,12 +219,54 @@ static __device__ __noinline__ void flush_counts(const PairParams &p, int off, i
     }
 }
 
+// LAY_BYTES with weights: counts and products of the bins whose fullest record
+// holds more than `above` of them (-1: all), four bins a step dealt to warps first,
+// first + nw, ...  A lane's records fill unevenly (128 neighbouring j-points are at
+// much the same distance): flushing all bins for the fullest of 1,280 records took
+// 50 of 340 ms.  Pieces are summed as integers (FP64 shuffles are slow here).
+static __device__ __noinline__ void flush_bytes(const PairParams &p, int above, int first, int nw, int h,
+                                                double wscale) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int lane = threadIdx.x & 31;
+    unsigned *hist = reinterpret_cast<unsigned *>(smem) + 64 * p.row0;
+    unsigned *top = reinterpret_cast<unsigned *>(smem + p.sm_whist) + 64 * p.row0;
+    for (int g = first; 4 * g < p.n_a; g += nw) {
+        const int bin = 4 * g + (lane >> 3);
+        bool full = false;
+        if (bin < p.n_a) {
+            const uint4 v = reinterpret_cast<const uint4 *>(hist + 64 * bin)[lane & 7];
+            full = (int)(max(max(v.x, v.y), max(v.z, v.w)) >> 20) > above;
+        }
+        unsigned who = __ballot_sync(FULL, full);
+        while (who) {
+            const int k = (__ffs(who) - 1) >> 3;
+            who &= ~(0xffu << (8 * k));
+            const int b = 4 * g + k, word = 64 * b + lane;
+            const unsigned v = atomicExch(&hist[word], 0u), mid = atomicExch(&hist[word + 32], 0u),
+                           hi = atomicExch(&top[word], 0u);
+            const unsigned cnt = __reduce_add_sync(FULL, v >> 20), lo = __reduce_add_sync(FULL, v & 0xFFFFFu);
+            const unsigned m0 = __reduce_add_sync(FULL, mid & 0xFFFFu), m1 = __reduce_add_sync(FULL, mid >> 16);
+            const unsigned h0 = __reduce_add_sync(FULL, hi & 0xFFFFu), h1 = __reduce_add_sync(FULL, hi >> 16);
+            if (lane == 0 && (cnt | lo | m0 | m1 | h0 | h1)) {
+                if (cnt) atomicAdd(&p.hist[(size_t)h * p.nbins + b], (unsigned long long)cnt);
+                const int sh = 8 + p.wcorr;   // bits of the lowest piece
+                const unsigned long long m = m0 + ((unsigned long long)m1 << 16),
+                                         t = h0 + ((unsigned long long)h1 << 16);
+                // m 2^sh + lo below 2^47 and t 2^20 below 2^58, added as binary64 numbers
+                const double w = (double)(t << 20) * (double)(1u << sh) + (double)((m << sh) + lo);
+                atomicAdd(&p.whist[(size_t)h * p.nbins + b], w * wscale);
+            }
+        }
+    }
+}
+
 // Weighted sums: binary64 (wint = 0), or the exact sums of the integer
 // products' pieces, either scaled into the global histogram or (fold mode)
 // added to the CTA's exact 128-bit sums in wfold_buf.
 static __device__ __noinline__ void flush_weights(const PairParams &p, int woff, int first, int nw, int h,
                                                   double wscale) {
     extern __shared__ __align__(16) unsigned char smem[];
+    if (p.layout == LAY_BYTES) return flush_bytes(p, -1, first, nw, h, wscale);
     unsigned char *wbase = smem + woff;
     const int lane = threadIdx.x & 31, K = p.hist_k, words = hist_entries(p) * K;
     for (int w0 = first * 32; w0 < words; w0 += nw * 32) {
@@ -228,18 +277,9 @@ static __device__ __noinline__ void flush_weights(const PairParams &p, int woff,
             const int word = hist_word(p, idx / K, idx & (K - 1), b);
             if (p.wint) {
                 unsigned *r = reinterpret_cast<unsigned *>(wbase);
-                unsigned *r0, *r1, *r2;
-                if (p.layout == LAY_BYTES) {
-                    r0 = reinterpret_cast<unsigned *>(smem) + word + 32;
-                    r1 = r + word;
-                    r2 = r1 + 32;
-                } else {
-                    r0 = r + 3 * (size_t)word;
-                    r1 = r0 + 1;
-                    r2 = r0 + 2;
-                }
-                const unsigned long long lo = atomicExch(r0, 0u), mid = atomicExch(r1, 0u),
-                                         hi = atomicExch(r2, 0u);
+                r += 3 * (size_t)word;
+                const unsigned long long lo = atomicExch(r, 0u), mid = atomicExch(r + 1, 0u),
+                                         hi = atomicExch(r + 2, 0u);
                 t = lo + (mid << 16) + (hi << 32);
             } else {
                 t = atomicExch(reinterpret_cast<unsigned long long *>(wbase) + word, 0ull);
@@ -852,6 +892,18 @@ __device__ __forceinline__ void add_pieces(unsigned char *a0, unsigned char *a1,
     atomicAdd(reinterpret_cast<unsigned *>(a2), v.z);
 }
 
+// The words of a LAY_BYTES record that a product adds to: 1 << 20 | its lowest 8
+// bits (of P >> 16; 9 of V), the next 20 bits, the top 20.  Three shared additions
+// a pair instead of four, for 4,095 products a record between flushes (2,047).
+__device__ __forceinline__ uint3 packed_p(unsigned long long P) {
+    const unsigned lo = (unsigned)P, hi = (unsigned)(P >> 32);
+    return make_uint3(prmt(lo, 0x00100000u, 0x7642), __funnelshift_r(lo, hi, 24) & 0xFFFFFu, hi >> 12);
+}
+__device__ __forceinline__ uint3 packed_v(unsigned long long V) {
+    const unsigned lo = (unsigned)V, hi = (unsigned)(V >> 32);
+    return make_uint3((lo & 0x1FFu) | 0x100000u, __funnelshift_r(lo, hi, 9) & 0xFFFFFu, __funnelshift_r(lo, hi, 29));
+}
+
 // A batch's constants, from a 16-bit lower bound of its separations' square (the
 // upper half of the FP32 number; 0: none).
 struct Bands {
@@ -989,8 +1041,10 @@ __device__ __forceinline__ unsigned quads_fix(const PairParams &p, const Tile &t
                 if (MODE == MODE_S) {
                     // byte 1: the bin, byte 0: this lane's copy
                     const unsigned a0 = prmt(t0, copy, 0x5524), a1 = prmt(t1, copy, 0x5524);
-                    atomicAdd(reinterpret_cast<unsigned *>(smem + a0), 1u);
-                    atomicAdd(reinterpret_cast<unsigned *>(smem + a1), 1u);
+                    if (W == 0) {
+                        atomicAdd(reinterpret_cast<unsigned *>(smem + a0), 1u);
+                        atomicAdd(reinterpret_cast<unsigned *>(smem + a1), 1u);
+                    }
                     P0 = a0;
                     P1 = a1;
                 } else {
@@ -1014,18 +1068,22 @@ __device__ __forceinline__ unsigned quads_fix(const PairParams &p, const Tile &t
                     // P = M_i M_j 2^(16 - k_i - k_j), and the product is P >> 16
                     // (truncation < 2^(k_i + k_j - 46) relative, below 2^48)
                     const uint2 wj = *reinterpret_cast<const uint2 *>(t.wm + 4 * q + 2 * h);
-                    uint3 v0, v1;   // 16-bit pieces, lowest first
+                    uint3 v0, v1;   // pieces, lowest first
                     if (W == 2) {
-                        v0 = pieces((unsigned long long)I.wm[r] * wj.x);
-                        v1 = pieces((unsigned long long)I.wm[r] * wj.y);
+                        const unsigned long long p0 = (unsigned long long)I.wm[r] * wj.x,
+                                                 p1 = (unsigned long long)I.wm[r] * wj.y;
+                        v0 = MODE == MODE_S ? packed_p(p0) : pieces(p0);
+                        v1 = MODE == MODE_S ? packed_p(p1) : pieces(p1);
                     } else {
                         const uint2 lj = *reinterpret_cast<const uint2 *>(t.wl + 4 * q + 2 * h);
-                        v0 = pieces_v(corrected_product(I.wm[r], I.wb[r], wj.x, lj.x));
-                        v1 = pieces_v(corrected_product(I.wm[r], I.wb[r], wj.y, lj.y));
+                        const unsigned long long p0 = corrected_product(I.wm[r], I.wb[r], wj.x, lj.x),
+                                                 p1 = corrected_product(I.wm[r], I.wb[r], wj.y, lj.y);
+                        v0 = MODE == MODE_S ? packed_v(p0) : pieces_v(p0);
+                        v1 = MODE == MODE_S ? packed_v(p1) : pieces_v(p1);
                     }
                     if (MODE == MODE_S) {
-                        add_pieces(smem + P0 + 128, smem + P0 + p.sm_whist, smem + P0 + p.sm_whist + 128, v0);
-                        add_pieces(smem + P1 + 128, smem + P1 + p.sm_whist, smem + P1 + p.sm_whist + 128, v1);
+                        add_pieces(smem + P0, smem + P0 + 128, smem + P0 + p.sm_whist, v0);
+                        add_pieces(smem + P1, smem + P1 + 128, smem + P1 + p.sm_whist, v1);
                     } else {
                         unsigned char *r0 = smem + p.sm_whist + 12 * P0, *r1 = smem + p.sm_whist + 12 * P1;
                         add_pieces(r0, r0 + 4, r0 + 8, v0);
@@ -1525,7 +1583,8 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ RangeShared s_range;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
-    using O = WarpOff<TREE, W != 0, false>;
+    constexpr bool BYTES = is_fix(PATH) && MODE == MODE_S;   // LAY_BYTES
+    using O = WarpOff<TREE, W != 0, false, batch_points(W, BYTES)>;
     unsigned char *ws = smem + p.sm_warp + (size_t)warp * O::total;
     int4 *seg = reinterpret_cast<int4 *>(ws);
     float4 *soff = reinterpret_cast<float4 *>(ws + O::soff);
@@ -1561,20 +1620,19 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
     unsigned since = 0, wterms = 0;            // quads, products per copy since this warp's flushes
     const unsigned flush_quads = (unsigned)(FLUSH_LIMIT / 256 / nw);
     // Integer weights: no record may take more than `wmax` products between
-    // flushes.  One axis (LAY_BYTES, 32 copies): each warp flushes after its
-    // share of that bound.  Otherwise a copy's share is used up in a batch or
-    // two while its bins hold little: each warp then looks for the largest
-    // counter, and flushes (counts with the weights) only past a quarter of the
-    // bound; what is in flight during a flush, at most 16 slots of a lane and
-    // warp, is taken off the quarter
+    // flushes.  A copy's share of that is used up in a few batches while its bins
+    // hold little: each warp then looks for the largest counter, and flushes (counts
+    // with the weights) only past a quarter of the bound (LAY_BYTES: bin by bin, past
+    // half); what is in flight during a flush, at most 16 slots of a lane and warp,
+    // is taken off that
+    constexpr unsigned wmax = (BYTES ? 4095u : WINT_LIMIT) / (W == 3 ? 2u : 1u);
     // one loop body for both halves in turn where a body of two i-points a lane is
     // too large to share the instruction cache with the rest: (s, mu) along the
     // midpoint with binary64 weights, 140k points, 21.8 -> 16.4 ms
     constexpr bool TWO = !(W == 3 && LOS == LOS_MID && MODE != MODE_S);
-    constexpr bool SCAN = !(is_fix(PATH) && MODE == MODE_S);
-    constexpr unsigned wmax = W == 3 ? WINT_LIMIT / 2 : WINT_LIMIT;
-    const unsigned wlimit = (SCAN ? wmax / 4 * 3 : wmax) / (unsigned)nw;
-    const int wfull = (int)(wmax / 4) - 16 * nw * (32 / p.hist_k);
+    constexpr unsigned wkeep = BYTES ? wmax / 2 : wmax / 4;   // what a look may leave in a record
+    const unsigned wlimit = (wmax - wkeep) / (unsigned)nw;
+    const int wfull = (int)wkeep - 16 * nw * (32 / p.hist_k);
     const unsigned wper = W >= 2 ? 8u * (unsigned)(32 / p.hist_k) : 0u;   // products per copy and quad
     __syncthreads();
 
@@ -1697,15 +1755,18 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
                     since += nq;
                     if (since > flush_quads && PATH != PATH_GLOBAL) {
                         flush_counts(p, 0, 0, 1, T.hist);
-                        if (SCAN && W >= 2) flush_weights(p, p.sm_whist, 0, 1, T.hist, T.wscale);
+                        if (W >= 2) flush_weights(p, p.sm_whist, 0, 1, T.hist, T.wscale);
                         since = nq;
                     }
                     if (W >= 2) {
                         wterms += wper * (unsigned)nq;
                         if (wterms > wlimit) {
-                            const bool full = !SCAN || most_counted(p) > wfull;
-                            if (SCAN && full) flush_counts(p, 0, 0, 1, T.hist);
-                            if (full) flush_weights(p, p.sm_whist, 0, 1, T.hist, T.wscale);
+                            if (BYTES) {
+                                flush_bytes(p, wfull, 0, 1, T.hist, T.wscale);
+                            } else if (most_counted(p) > wfull) {
+                                flush_counts(p, 0, 0, 1, T.hist);
+                                flush_weights(p, p.sm_whist, 0, 1, T.hist, T.wscale);
+                            }
                             wterms = wper * (unsigned)nq;
                         }
                     }
@@ -1887,7 +1948,7 @@ __global__ void __maxnreg__(96) k_pairs_f64(const __grid_constant__ PairParams p
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ RangeShared s_range;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
-    using O = WarpOff<false, false, true>;
+    using O = WarpOff<false, false, true, 64>;
     unsigned char *ws = smem + p.sm_warp + (size_t)warp * O::total;
     int4 *seg = reinterpret_cast<int4 *>(ws);
     double *tile = reinterpret_cast<double *>(ws + O::tile);   // {x, y, z, w, shift x, y, z} by point

@@ -80,6 +80,27 @@ def test_first_edges_above_zero(mode, los, e0, spacing, na):
                 np.testing.assert_allclose(gotw, wantw, rtol=1e-10, atol=0.0, err_msg=f.__name__)
 
 
+@pytest.mark.parametrize("wtype", ["f32", "f64"])
+@pytest.mark.parametrize("mode", ["s", "smu"])
+def test_weight_records_that_fill(mode, wtype):
+    """All pairs in one or a few bins, weights just below the scale's top: the
+    integer weight records are flushed long before a piece or count overflows."""
+    n = 5003
+    rng = np.random.default_rng(51)
+    x = 50.0 + rng.normal(0.0, 0.2, (n, 3))
+    w = 1.0 - 1e-6 * rng.random(n)
+    if wtype == "f32":
+        w = w.astype(np.float32)
+    kw = dict(mode=mode, edges_a=np.linspace(0.0, 25.0, 6))
+    if mode == "smu":
+        kw["edges_b"] = np.linspace(0.0, 1.0, 3)
+    want, wantw = oracle.count(x, w1=w.astype(np.float64), box=L, periodic=True, method="grid", **kw)
+    for f in (P.count, P.count_tree):
+        got, gotw = f(x, w1=w, box=L, periodic=True, **kw)
+        np.testing.assert_array_equal(got, want, err_msg=f.__name__)
+        np.testing.assert_allclose(gotw, wantw, rtol=1e-10, atol=0.0, err_msg=f.__name__)
+
+
 @pytest.mark.parametrize("n1,n2", [(40, 5000), (5000, 40), (1, 300), (300, 1)])
 def test_cross_counts_either_way_round(n1, n2):
     x, y = _points(n1, 21), _points(n2, 22)

@@ -135,6 +135,8 @@ static cudaError_t radix_sort(unsigned long long *ka, unsigned *va, unsigned lon
 // per-level node statistics
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ double canon_t(double x, double L) {
+    // in [0, L) already (-0, negative numbers and not-a-number compare above)
+    if ((unsigned long long)__double_as_longlong(x) < (unsigned long long)__double_as_longlong(L)) return x;
     double y = __dsub_rn(x, __dmul_rn(L, floor(__ddiv_rn(x, L))));
     if (y < 0.0) y = __dadd_rn(y, L);
     if (y >= L) y = __dsub_rn(y, L);
@@ -316,14 +318,21 @@ __global__ void k_node_finish(const NodeAcc *__restrict__ acc, int level, const 
 // Along the positions the node ids (the keys' high bits) never decrease, so
 // the stable sort of all keys only reorders the keys of each node among
 // themselves.  Once every node of a level fits a chunk, one CTA per chunk of
-// q whole nodes sorts its keys on (key, position) in shared memory (a bitonic
-// network over the next power of two, the padding after every key) and
+// q whole nodes sorts each node's keys on (key, position) in shared memory (a
+// bitonic network over 2^seg keys a node, the padding after every key) and
 // writes the values back in that order: the radix sort's result, from one
 // read and one write of the level's values.  With acc given it then takes
 // the next level's node statistics as k_node_stats would (the children's
 // ranges are the halves of each sorted node): one warp per child, its sums
 // reduced in registers and stored once, with no atomics.
-constexpr int CS_SMALL = 4096;    // chunk capacities (keys)
+//
+// Bound by shared memory and the barriers of the network's steps: seg (seg + 1) / 2
+// of them, the ones within runs of 64 keys without a barrier.  2M points, the nine
+// levels of 7,813 points a node and less: 1.77 ms against 2.31 for one network over the
+// whole chunk with a barrier a step and at least 4,096 keys a CTA (2,048 leave room
+// for seven CTAs an SM, one wave).
+constexpr int CS_MINI = 2048;     // chunk capacities (keys)
+constexpr int CS_SMALL = 4096;
 constexpr int CS_LARGE = 16384;
 
 template <int CAP, int NTH, class R>
@@ -335,51 +344,68 @@ __global__ void __launch_bounds__(NTH) k_chunk_sort(const unsigned long long *__
     unsigned long long *sk = reinterpret_cast<unsigned long long *>(cs_sm);
     unsigned *sv = reinterpret_cast<unsigned *>(sk + CAP);
     unsigned short *si = reinterpret_cast<unsigned short *>(sv + CAP);
-    const int2 rg = r.range(blockIdx.x);
-    const int len = min(rg.y - rg.x, CAP);   // the host sizes chunks to CAP
-    int P = 1;
-    while (P < len) P <<= 1;
+    const int P = r.q << r.seg;   // at most CAP
     for (int t = threadIdx.x; t < P; t += NTH) {
-        if (t < len) {
-            sk[t] = keys[rg.x + t];
-            sv[t] = vals[rg.x + t];
-        } else {
-            sk[t] = ~0ull;
-        }
+        const int2 nd = r.node(blockIdx.x, t >> r.seg);
+        const int o = t & ((1 << r.seg) - 1);
+        sk[t] = o < nd.y ? keys[nd.x + o] : ~0ull;
+        if (o < nd.y) sv[t] = vals[nd.x + o];
         si[t] = (unsigned short)t;
     }
     __syncthreads();
-    for (int k = 2; k <= P; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int t = threadIdx.x; t < (P >> 1); t += NTH) {
-                const int i = ((t & ~(j - 1)) << 1) | (t & (j - 1));   // bit j clear
-                const int l = i + j;
-                const unsigned long long a = sk[i], b = sk[l];
-                const unsigned short ia = si[i], ib = si[l];
-                const bool gt = a > b || (a == b && ia > ib);
-                if (gt == ((i & k) == 0)) {   // ascending where bit k of i is clear
-                    sk[i] = b;
-                    sk[l] = a;
-                    si[i] = ib;
-                    si[l] = ia;
-                }
-            }
+    // compare-exchange t of step (k, j)
+    auto step = [&](int t, int k, int j) {
+        const int i = ((t & ~(j - 1)) << 1) | (t & (j - 1));   // bit j clear
+        const int l = i + j;
+        const unsigned long long a = sk[i], b = sk[l];
+        const unsigned short ia = si[i], ib = si[l];
+        const bool gt = a > b || (a == b && ia > ib);
+        if (gt == ((i & k) == 0 || k == 1 << r.seg)) {   // ascending where bit k of i is clear; last: all
+            sk[i] = b;
+            sk[l] = a;
+            si[i] = ib;
+            si[l] = ia;
+        }
+    };
+    for (int k = 2; k <= 1 << r.seg; k <<= 1) {
+        for (int j = k >> 1; j > 32; j >>= 1) {
+            for (int t = threadIdx.x; t < (P >> 1); t += NTH) step(t, k, j);
             __syncthreads();
         }
+        // the rest of the stage stays inside runs of 64, one warp's
+        for (int t0 = threadIdx.x & ~31; t0 < (P >> 1); t0 += NTH) {
+            const int t = t0 + (threadIdx.x & 31);
+            for (int j = min(k >> 1, 32); j > 0; j >>= 1) {
+                if (t < (P >> 1)) step(t, k, j);
+                __syncwarp();
+            }
+        }
+        __syncthreads();
     }
-    for (int t = threadIdx.x; t < len; t += NTH) vals[rg.x + t] = sv[si[t]];
+    for (int t = threadIdx.x; t < P; t += NTH) {
+        const int2 nd = r.node(blockIdx.x, t >> r.seg);
+        const int o = t & ((1 << r.seg) - 1);
+        if (o < nd.y) vals[nd.x + o] = sv[si[t]];
+    }
     if (!acc) return;
     const int lane = threadIdx.x & 31;
     const double3 sh3 = r.shift(blockIdx.x);
     const double sh[3] = {sh3.x, sh3.y, sh3.z};
-    for (int c = threadIdx.x >> 5; c < 2 * r.q; c += NTH / 32) {
-        const int2 nd = r.node(blockIdx.x, c >> 1);     // {first position, count}
-        const int half = nd.y / 2;
-        const int b0 = nd.x - rg.x + ((c & 1) ? half : 0);
-        const int b1 = nd.x - rg.x + ((c & 1) ? nd.y : half);
+    // a child holds at most 2^(seg - 1) points: as many lanes, up to a warp, share it
+    // (the lanes left out would add zeros: the same sums)
+    const int G = r.seg <= 1 ? 1 : min(32, 1 << (r.seg - 1)), per = 32 / G, own = lane & (G - 1);
+    for (int c0 = (threadIdx.x >> 5) * per; c0 < 2 * r.q; c0 += NTH / 32 * per) {
+        const int c = c0 + lane / G;
+        int b0 = 0, b1 = 0;
+        if (c < 2 * r.q) {
+            const int2 nd = r.node(blockIdx.x, c >> 1);     // {first position, count}
+            const int half = nd.y / 2, at = (c >> 1) << r.seg;
+            b0 = at + ((c & 1) ? half : 0);
+            b1 = at + ((c & 1) ? nd.y : half);
+        }
         double s[3] = {0, 0, 0}, q[3] = {0, 0, 0};
         long long mn[3] = {LLONG_MAX, LLONG_MAX, LLONG_MAX}, mx[3] = {LLONG_MIN, LLONG_MIN, LLONG_MIN};
-        for (int t = b0 + lane; t < b1; t += 32) {
+        for (int t = b0 + own; t < b1; t += G) {
             const unsigned pidx = sv[si[t]];
             for (int d = 0; d < 3; ++d) {
                 const double v = x[3 * (size_t)pidx + d];
@@ -390,14 +416,14 @@ __global__ void __launch_bounds__(NTH) k_chunk_sort(const unsigned long long *__
                 mx[d] = max(mx[d], okey(v));
             }
         }
-        for (int o = 16; o > 0; o >>= 1)
+        for (int o = G / 2; o > 0; o >>= 1)
             for (int d = 0; d < 3; ++d) {
                 s[d] += __shfl_xor_sync(0xffffffffu, s[d], o);
                 q[d] += __shfl_xor_sync(0xffffffffu, q[d], o);
                 mn[d] = min(mn[d], __shfl_xor_sync(0xffffffffu, mn[d], o));
                 mx[d] = max(mx[d], __shfl_xor_sync(0xffffffffu, mx[d], o));
             }
-        if (lane == 0) {
+        if (own == 0 && c < 2 * r.q) {
             NodeAcc A;
             for (int d = 0; d < 3; ++d) {
                 A.s[d] = s[d];
@@ -417,11 +443,7 @@ struct ChunksOne {
     const int2 *vnode;
     int level, q;
     double3 centre;
-    __device__ int2 range(int c) const {
-        const long long h0 = (1LL << level) - 1 + (long long)c * q;
-        const int2 a = vnode[h0], b = vnode[h0 + q - 1];
-        return make_int2(a.x, b.x + b.y);
-    }
+    int seg = 0;
     __device__ int2 node(int c, int j) const {
         return vnode[(1LL << level) - 1 + (long long)c * q + j];
     }
@@ -453,13 +475,17 @@ template <class R>
 static bool chunk_sort_level(const unsigned long long *keys, unsigned *vals, R r, int level,
                              long long nodes, long long maxsize, const double *x, NodeAcc *acc,
                              cudaStream_t st, cudaError_t *err) {
-    const int cap = maxsize <= CS_SMALL ? CS_SMALL : (maxsize <= CS_LARGE ? CS_LARGE : 0);
+    const int cap = maxsize <= CS_MINI ? CS_MINI : maxsize <= CS_SMALL ? CS_SMALL : (maxsize <= CS_LARGE ? CS_LARGE : 0);
     if (cap == 0) return false;
+    int seg = 0;
+    while ((1LL << seg) < maxsize) ++seg;
     long long q = 1;
-    while (q < (1LL << level) && 2 * q * maxsize <= cap) q *= 2;
+    while (q < (1LL << level) && (2 * q) << seg <= cap) q *= 2;
     r.level = level;
     r.q = (int)q;
-    *err = cap == CS_SMALL ? launch_chunk_sort<CS_SMALL, 256>(keys, vals, r, nodes / q, x, acc, st)
+    r.seg = seg;
+    *err = cap == CS_MINI ? launch_chunk_sort<CS_MINI, 256>(keys, vals, r, nodes / q, x, acc, st)
+           : cap == CS_SMALL ? launch_chunk_sort<CS_SMALL, 256>(keys, vals, r, nodes / q, x, acc, st)
                            : launch_chunk_sort<CS_LARGE, 1024>(keys, vals, r, nodes / q, x, acc, st);
     return true;
 }
@@ -1272,13 +1298,7 @@ struct ChunksForest {
     const FTree *ft;
     int level, q;
     const double3 *centres;
-    __device__ int2 range(int c) const {
-        const long long g0 = (long long)c * q;
-        const FTree &T = ft[g0 >> level];
-        const long long h0 = (1LL << level) - 1 + (g0 & ((1LL << level) - 1));
-        const int2 a = T.vnode[h0], b = T.vnode[h0 + q - 1];
-        return make_int2((int)(T.pos + a.x), (int)(T.pos + b.x + b.y));
-    }
+    int seg = 0;
     __device__ int2 node(int c, int j) const {
         const long long g = (long long)c * q + j;
         const FTree &T = ft[g >> level];

@@ -700,7 +700,7 @@ struct DevBufs {
     unsigned long long *hist = nullptr;
     double *whist = nullptr;
     unsigned long long *ctr = nullptr;   // [0] candidates, [1] inline rescues, [2] queue count,
-                                         // [3] pairs pruned by group bounds
+                                         // [3] pairs pruned by the octs' boxes
     int *sc = nullptr;                   // [0] work counter, [1] number of blocks
     uint3 *queue = nullptr;
     Block *blocks = nullptr;

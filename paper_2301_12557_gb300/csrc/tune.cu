@@ -5,9 +5,9 @@
 // sample of the point blocks -- the block-shard mechanism of the multi-GPU
 // path with one shard -- first for 2 and 4 i-points per thread at that side,
 // then at cell sides in quarter-octave steps from 0.7 to 2 times it, then
-// with one count copy per warp, then with the near-edge pairs evaluated
-// inside the pair kernel instead of queued, and returns the fastest
-// combination.
+// with priv 1 (binary64 weight sums), then with rescue_capacity -1 (the
+// near-edge pairs checked in the pair kernel, which is also the default's
+// path), and returns the fastest combination.
 #include <math.h>
 #include <string.h>
 
@@ -227,9 +227,9 @@ extern "C" pc_status pc_tune(const double *xyz, const void *w, int w_is_f32, lon
             out->priv = 1;
         }
     }
-    // near-edge pairs evaluated inside the pair kernel (no queue, no rescue
-    // kernel: the binary64 work interleaves with the FP32 pairs of other
-    // warps) at the best options, unless the caller fixed the queue size
+    // rescue_capacity -1 (no queue, as by default: the binary64 work interleaves
+    // with the FP32 pairs of other warps) at the best options, unless the caller
+    // fixed the queue size
     if (fp32 && o.rescue_capacity == 0 && std::isfinite(best_ms)) {
         pc_opts oc = *out;
         pc_grid *g = nullptr;

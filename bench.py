@@ -518,7 +518,7 @@ def run_ours(args, emit=True):
               "ms_per_step": statistics.mean(kd_ms), "steps": args.tree_steps,
               "step": "tree build + dual-tree traversal + pair and rescue kernels",
               "list_cap": cap_kd or "auto", "ipt": o_kd.ipt, "n_leaf": args.n_leaf,
-              "rescue": "inline" if o_kd.rescue_capacity < 0 else "queued",
+              "rescue": "inline" if o_kd.rescue_capacity <= 0 else "queued",
               "tuning_seconds": tune_s,
               "counts_identical_to_grid": bool(torch.equal(out_kd, out))}
 
@@ -586,7 +586,7 @@ def run_ours(args, emit=True):
                                      "traversal" % (args.n_leaf, list_cap or "auto"))
                                     if tree else "regular grid",
                        "cell_size": s0.cell_size, "ipt": opts.ipt, "priv": opts.priv,
-                       "rescue": ("inline in the pair kernel" if opts.rescue_capacity < 0 else
+                       "rescue": ("inline in the pair kernel" if opts.rescue_capacity <= 0 else
                                   "queued for the rescue kernel"),
                        "tuning": tuning,
                        "tree": ({"node_pairs": int(s0.tree_pairs), "blocks": int(s0.blocks),
@@ -1245,7 +1245,7 @@ def run_sets(args, extra=None):
                        "structure": ("k-d tree (leaf capacity %d, list nodes %s), dual-tree traversal"
                                      % (args.n_leaf, list_cap or "auto")) if tree else "regular grid",
                        "cell_size": s0.cell_size, "ipt": opts.ipt, "priv": opts.priv,
-                       "rescue": ("inline in the pair kernel" if opts.rescue_capacity < 0 else
+                       "rescue": ("inline in the pair kernel" if opts.rescue_capacity <= 0 else
                                   "queued for the rescue kernel"),
                        "weight_sums": {0: "none", 1: "binary64 products",
                                        2: "exact integer products of binary32 significands",

@@ -34,7 +34,7 @@
 // range): issue slots (82 % used; the FMA and integer pipes at 51 and 54 %, shared
 // memory at 61 %).  1.52 pairs are evaluated for each in range, against 1.70 with
 // one list for the 64 points along a Morton curve; 113 of about 135 warp
-// instructions per 64 x 4 pairs are the loop itself.  68.2 ms against 154.7 ms for
+// instructions per 64 x 4 pairs are the loop itself.  65.4 ms against 154.7 ms for
 // CTAs of 128 threads that staged every candidate tile behind a barrier and queued
 // near-edge pairs for a second kernel (138 instructions per 64 x 2 pairs, issued
 // on 60 % of the cycles).

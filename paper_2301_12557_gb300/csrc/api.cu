@@ -951,8 +951,8 @@ static pc_status fit_params(int prec, int opt_priv, int dev, bool weighted, bool
                  (p.mode == PC_BIN_S ? 0.0f : 0.5f * col);
     }
     // 8 warps at most with weights: a copy's products between a warp's flushes
-    // must hold one batch (64 x 64 products to one lane copy, WINT_LIMIT / 2 / 8; on
-    // one axis 8 a quad and copy, 32 quads, against 4095 * 3 / 4 / 8)
+    // must hold one batch (64 x 64 products to one lane copy, of WINT_LIMIT 3 / 4 / 8; on
+    // one axis 8 a quad and copy, 32 quads, of 4095 / 2 / 8)
     int best_warps = 0, best_nw = 0;
     for (int nw : {1, 2, 4, 8, 12, 16}) {
         if (nw < nw_min || (p.wint && nw > 8)) continue;

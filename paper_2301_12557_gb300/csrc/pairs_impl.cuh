@@ -51,12 +51,11 @@
 namespace pc {
 
 constexpr unsigned long long FLUSH_LIMIT = 1ull << 30;
-// integer weight path: products (each < 2^48) per lane copy between flushes;
-// each of its three u32 piece sums then adds less than 2^16 pieces of 16
-// bits, and the copy's recombined sum stays below 2^64.  With binary64
-// weights (W == 3) a product may reach 2^48, its top piece 2^16, and half as
-// many are allowed.
-constexpr unsigned WINT_LIMIT = 1u << 16;
+// integer weight path: most products (each at most 2^48) in one lane copy's
+// record: each of its three u32 piece sums then adds at most 65,535 pieces of
+// 16 bits (the top one at most 2^16, with binary64 weights), and the record's
+// recombined sum stays below 2^64.
+constexpr unsigned WINT_LIMIT = 65535;
 
 __host__ __device__ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -201,11 +200,10 @@ __device__ __forceinline__ int hist_word(const PairParams &p, int e, int k, int 
     return (e + p.row0 * p.hs) * p.hist_k + k;
 }
 
-static __device__ __noinline__ void flush_counts(const PairParams &p, int off, int first, int nw, int h) {
+static __device__ __noinline__ void flush_counts(const PairParams &p, int first, int nw, int h) {
     extern __shared__ __align__(16) unsigned char smem[];
-    if (p.weighted && p.layout == LAY_BYTES) return;   // flush_bytes takes them along
     const int lane = threadIdx.x & 31, K = p.hist_k, words = hist_entries(p) * K;
-    int *hist = reinterpret_cast<int *>(smem + off);
+    int *hist = reinterpret_cast<int *>(smem);
     for (int w0 = first * 32; w0 < words; w0 += nw * 32) {
         const int idx = w0 + lane;
         int v = 0, b = -1;
@@ -260,33 +258,45 @@ static __device__ __noinline__ void flush_bytes(const PairParams &p, int above, 
     }
 }
 
-// Weighted sums: binary64 (wint = 0), or the exact sums of the integer
-// products' pieces, either scaled into the global histogram or (fold mode)
-// added to the CTA's exact 128-bit sums in wfold_buf.
-static __device__ __noinline__ void flush_weights(const PairParams &p, int woff, int first, int nw, int h,
-                                                  double wscale) {
+// LAY_ROWS with integer weights: every entry's counter and record of products, the
+// exact sum of whose pieces is either scaled into the global histogram or (fold
+// mode) added to the CTA's exact 128-bit sums in wfold_buf.
+//
+// Other warps keep adding meanwhile, and may look for full records or flush them
+// as well.  A counter must never say less than its record holds (but for the quad
+// that each warp is in): it is marked by CLAIM, the record is taken, and only then
+// are the mark and the counts that stood there taken off.  Of several warps at an
+// entry the first takes the counts; each takes the record, which is thus empty for
+// whoever has flushed.  (Taking all counters first and the records after them left
+// full records beside counters of zero: a warp that looked then added another
+// share, and the sums could wrap.)
+constexpr int CLAIM = 1 << 24;   // above any count between flushes
+static __device__ __noinline__ void flush_records(const PairParams &p, int first, int nw, int h, double wscale) {
     extern __shared__ __align__(16) unsigned char smem[];
-    if (p.layout == LAY_BYTES) return flush_bytes(p, -1, first, nw, h, wscale);
-    unsigned char *wbase = smem + woff;
     const int lane = threadIdx.x & 31, K = p.hist_k, words = hist_entries(p) * K;
+    int *hist = reinterpret_cast<int *>(smem);
     for (int w0 = first * 32; w0 < words; w0 += nw * 32) {
         const int idx = w0 + lane;
         unsigned long long t = 0ull;
-        int b = -1;
+        int b = -1, n = 0;
         if (idx < words) {
             const int word = hist_word(p, idx / K, idx & (K - 1), b);
-            if (p.wint) {
-                unsigned *r = reinterpret_cast<unsigned *>(wbase);
-                r += 3 * (size_t)word;
+            if (b >= 0 && *reinterpret_cast<volatile int *>(hist + word) != 0) {
+                n = atomicAdd(&hist[word], CLAIM);
+                if (n >= CLAIM) n = 0;   // another warp's
+                __threadfence_block();
+                unsigned *r = reinterpret_cast<unsigned *>(smem + p.sm_whist) + 3 * (size_t)word;
                 const unsigned long long lo = atomicExch(r, 0u), mid = atomicExch(r + 1, 0u),
                                          hi = atomicExch(r + 2, 0u);
                 t = lo + (mid << 16) + (hi << 32);
-            } else {
-                t = atomicExch(reinterpret_cast<unsigned long long *>(wbase) + word, 0ull);
+                __threadfence_block();
+                atomicSub(&hist[word], CLAIM + n);
             }
         }
         const bool head = b >= 0 && (lane & (K - 1)) == 0;
-        if (p.wint && p.wfold) {
+        for (int o = 1; o < K; o <<= 1) n += __shfl_xor_sync(FULL, n, o);
+        if (head && n) atomicAdd(&p.hist[(size_t)h * p.nbins + b], (unsigned long long)n);
+        if (p.wfold) {
             unsigned long long hi = 0ull;
             for (int o = 1; o < K; o <<= 1) {
                 const unsigned long long l2 = __shfl_xor_sync(FULL, t, o), h2 = __shfl_xor_sync(FULL, hi, o);
@@ -301,16 +311,45 @@ static __device__ __noinline__ void flush_weights(const PairParams &p, int woff,
                 if (hi) atomicAdd(&f[1], hi);
             }
         } else {
-            double w = p.wint ? (double)t : __longlong_as_double((long long)t);
+            double w = (double)t;
             for (int o = 1; o < K; o <<= 1) w += __shfl_xor_sync(FULL, w, o);
-            if (head && w != 0.0) atomicAdd(&p.whist[(size_t)h * p.nbins + b], p.wint ? w * wscale : w);
+            if (head && w != 0.0) atomicAdd(&p.whist[(size_t)h * p.nbins + b], w * wscale);
         }
     }
 }
 
-// Largest counter of a LAY_ROWS histogram: with counts and weights flushed
-// together, no record of the integer weights has taken more products since
-// (but for additions in flight while they were flushed).
+// Binary64 weighted sums.
+static __device__ __noinline__ void flush_weights(const PairParams &p, int first, int nw, int h) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int lane = threadIdx.x & 31, K = p.hist_k, words = hist_entries(p) * K;
+    unsigned long long *sums = reinterpret_cast<unsigned long long *>(smem + p.sm_whist);
+    for (int w0 = first * 32; w0 < words; w0 += nw * 32) {
+        const int idx = w0 + lane;
+        double w = 0.0;
+        int b = -1;
+        if (idx < words) {
+            const int word = hist_word(p, idx / K, idx & (K - 1), b);
+            w = __longlong_as_double((long long)atomicExch(&sums[word], 0ull));
+        }
+        for (int o = 1; o < K; o <<= 1) w += __shfl_xor_sync(FULL, w, o);
+        if (b >= 0 && (lane & (K - 1)) == 0 && w != 0.0) atomicAdd(&p.whist[(size_t)h * p.nbins + b], w);
+    }
+}
+
+// Everything a CTA has added, by warps first, first + nw, ...  W as in the kernels.
+template <int W>
+__device__ __forceinline__ void flush_all(const PairParams &p, int first, int nw, int h, double wscale) {
+    if (W >= 2) {
+        if (p.layout == LAY_BYTES) flush_bytes(p, -1, first, nw, h, wscale);
+        else flush_records(p, first, nw, h, wscale);
+    } else {
+        flush_counts(p, first, nw, h);
+        if (W) flush_weights(p, first, nw, h);
+    }
+}
+
+// Largest counter of a LAY_ROWS histogram with integer weights: no record holds
+// more products (but for the quads in flight, flush_records).
 static __device__ __noinline__ int most_counted(const PairParams &p) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, rows = p.n_a + p.row0;
@@ -321,12 +360,13 @@ static __device__ __noinline__ int most_counted(const PairParams &p) {
         for (int k = lane; k < rows * p.hist_k; k += 32)
             hist[((k / p.hist_k) * p.hs + p.n_b) * p.hist_k + (k & (p.hist_k - 1))] = 0;
     for (int k = lane; k < p.row0 * p.hs * p.hist_k; k += 32) hist[k] = 0;
+    constexpr int counts = CLAIM - 1;   // without the marks of warps that flush
     int m = 0;
     for (int k = lane; k < n4; k += 32) {
         const int4 v = reinterpret_cast<const int4 *>(hist)[k];
-        m = max(max(m, max(v.x, v.y)), max(v.z, v.w));
+        m = max(max(m, max(v.x & counts, v.y & counts)), max(v.z & counts, v.w & counts));
     }
-    if (4 * n4 + lane < words) m = max(m, hist[4 * n4 + lane]);
+    if (4 * n4 + lane < words) m = max(m, hist[4 * n4 + lane] & counts);
     return __reduce_max_sync(FULL, m);
 }
 
@@ -1619,18 +1659,22 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
     unsigned long long cand = 0, pruned = 0;   // per lane
     unsigned since = 0, wterms = 0;            // quads, products per copy since this warp's flushes
     const unsigned flush_quads = (unsigned)(FLUSH_LIMIT / 256 / nw);
-    // Integer weights: no record may take more than `wmax` products between
-    // flushes.  A copy's share of that is used up in a few batches while its bins
-    // hold little: each warp then looks for the largest counter, and flushes (counts
-    // with the weights) only past a quarter of the bound (LAY_BYTES: bin by bin, past
-    // half); what is in flight during a flush, at most 16 slots of a lane and warp,
-    // is taken off that
-    constexpr unsigned wmax = (BYTES ? 4095u : WINT_LIMIT) / (W == 3 ? 2u : 1u);
+    // Integer weights: no record may hold more than `wmax` products.  Each warp adds
+    // at most `wlimit` to any (a batch or more), then looks for the largest counter,
+    // and flushes (counts with the weights) only past a quarter of the bound
+    // (LAY_BYTES: bin by bin, past half).  After the latest look of any warp a record
+    // holds at most what that look leaves, wkeep: the counter and the quad (eight
+    // pairs a lane, taken as 16) that each warp is in; and each warp has added at most
+    // wlimit since, so wkeep + nwarps wlimit <= wmax is the bound
+    constexpr unsigned wmax = BYTES ? (W == 3 ? 2047u : 4095u) : WINT_LIMIT;
     // one loop body for both halves in turn where a body of two i-points a lane is
     // too large to share the instruction cache with the rest: (s, mu) along the
     // midpoint with binary64 weights, 140k points, 21.8 -> 16.4 ms
     constexpr bool TWO = !(W == 3 && LOS == LOS_MID && MODE != MODE_S);
     constexpr unsigned wkeep = BYTES ? wmax / 2 : wmax / 4;   // what a look may leave in a record
+    constexpr unsigned wbatch = 8u * (BYTES ? 1u : 32u) * O::jb / 4u;   // largest batch to one record
+    static_assert(W < 2 || 8u * wbatch <= wmax - wkeep, "a batch of each of 8 warps fits");
+    static_assert(W < 2 || wkeep > 16u * 8u * (BYTES ? 1u : 32u), "the quads in flight fit");
     const unsigned wlimit = (wmax - wkeep) / (unsigned)nw;
     const int wfull = (int)wkeep - 16 * nw * (32 / p.hist_k);
     const unsigned wper = W >= 2 ? 8u * (unsigned)(32 / p.hist_k) : 0u;   // products per copy and quad
@@ -1639,10 +1683,7 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
     for (;;) {
         auto flush = [&](int old) {
             const int h = p.tasks[old].hist;
-            if (PATH != PATH_GLOBAL) {
-                flush_counts(p, 0, warp, nw, h);
-                if (W) flush_weights(p, p.sm_whist, warp, nw, h, p.tasks[old].wscale);
-            }
+            if (PATH != PATH_GLOBAL) flush_all<W>(p, warp, nw, h, p.tasks[old].wscale);
             __syncthreads();
             if (W >= 2 && p.wfold) flush_folded(p, h, p.tasks[old].wscale);
             since = wterms = 0;
@@ -1754,19 +1795,15 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
                     const int nq = 2 * m;
                     since += nq;
                     if (since > flush_quads && PATH != PATH_GLOBAL) {
-                        flush_counts(p, 0, 0, 1, T.hist);
-                        if (W >= 2) flush_weights(p, p.sm_whist, 0, 1, T.hist, T.wscale);
+                        if (W >= 2) flush_all<W>(p, 0, 1, T.hist, T.wscale);
+                        else flush_counts(p, 0, 1, T.hist);
                         since = nq;
                     }
                     if (W >= 2) {
                         wterms += wper * (unsigned)nq;
                         if (wterms > wlimit) {
-                            if (BYTES) {
-                                flush_bytes(p, wfull, 0, 1, T.hist, T.wscale);
-                            } else if (most_counted(p) > wfull) {
-                                flush_counts(p, 0, 0, 1, T.hist);
-                                flush_weights(p, p.sm_whist, 0, 1, T.hist, T.wscale);
-                            }
+                            if (BYTES) flush_bytes(p, wfull, 0, 1, T.hist, T.wscale);
+                            else if (most_counted(p) > wfull) flush_records(p, 0, 1, T.hist, T.wscale);
                             wterms = wper * (unsigned)nq;
                         }
                     }
@@ -1852,10 +1889,7 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
     __syncthreads();
     if (!p.multi) {   // batches have flushed after their last range
         const double wscale = p.tasks[0].wscale;
-        if (PATH != PATH_GLOBAL) {
-            flush_counts(p, 0, warp, nw, 0);
-            if (W) flush_weights(p, p.sm_whist, warp, nw, 0, wscale);
-        }
+        if (PATH != PATH_GLOBAL) flush_all<W>(p, warp, nw, 0, wscale);
         if (W >= 2 && p.wfold) {
             __syncthreads();
             flush_folded(p, 0, wscale);
@@ -1983,10 +2017,7 @@ __global__ void __maxnreg__(96) k_pairs_f64(const __grid_constant__ PairParams p
 
     for (;;) {
         auto flush = [&](int old) {
-            if (p.smem_hist_ok) {
-                flush_counts(p, 0, warp, nw, p.tasks[old].hist);
-                if (W) flush_weights(p, p.sm_whist, warp, nw, p.tasks[old].hist, 0.0);
-            }
+            if (p.smem_hist_ok) flush_all<W ? 1 : 0>(p, warp, nw, p.tasks[old].hist, 0.0);
             since = 0;
             __syncthreads();
         };
@@ -2071,7 +2102,7 @@ __global__ void __maxnreg__(96) k_pairs_f64(const __grid_constant__ PairParams p
                 __syncwarp();
                 since += 8 * m;
                 if (since > flush_j && p.smem_hist_ok) {
-                    flush_counts(p, 0, 0, 1, T.hist);
+                    flush_counts(p, 0, 1, T.hist);
                     since = 8 * m;
                 }
                 for (int j = 0; j < 8 * m; ++j) {
@@ -2110,10 +2141,7 @@ __global__ void __maxnreg__(96) k_pairs_f64(const __grid_constant__ PairParams p
         }
     }
     __syncthreads();
-    if (!p.multi && p.smem_hist_ok) {
-        flush_counts(p, 0, warp, nw, 0);
-        if (W) flush_weights(p, p.sm_whist, warp, nw, 0, 0.0);
-    }
+    if (!p.multi && p.smem_hist_ok) flush_all<W ? 1 : 0>(p, warp, nw, 0, 0.0);
     cand = warp_sum_u64(cand);
     pruned = warp_sum_u64(pruned);
     if (lane == 0 && cand) atomicAdd(&p.counters[0], cand);

@@ -1,0 +1,97 @@
+"""The bound on the integer weight records (CPU, a model of the protocol): no lane
+copy's record may hold more than 65,535 products.  Eight warps add batches of up
+to 4,096 products to one record (one lane copy, every pair in one bin), each looks
+at the record's counter when another batch would take it past its share, and
+flushes when the counter says more than is left over.  A scheduler that may stop
+any warp between any two of its shared-memory operations for as long as it likes
+must not bring a record past the bound; taking the counters of all entries before
+their records, as a flush in two passes does, must."""
+
+import random
+
+import pytest
+
+LIMIT, WARPS, QUAD, BATCH_QUADS = 65535, 8, 256, 16      # one lane copy: 32 lanes x 8 pairs a quad
+KEEP = LIMIT // 4                                        # what a look may leave
+SHARE = (LIMIT - KEEP) // WARPS
+FULL = KEEP - 2 * QUAD * WARPS                           # flush past it (16 slots a lane in flight)
+CLAIM = 1 << 24
+
+
+class Cta:
+    def __init__(self):
+        self.count = self.record = self.most = 0
+        self.counts_out = self.products_out = 0
+
+
+def _warp(c, two_passes):
+    """One step per yield: a quad's counters, a quad's products, a look, and the
+    operations of a flush."""
+    share = 0
+    while True:
+        share += QUAD * BATCH_QUADS
+        if share > SHARE:
+            look = c.count & (CLAIM - 1)
+            yield
+            if look > FULL:
+                if two_passes:
+                    n, c.count = c.count, 0
+                    for _ in range(100):                  # the other entries' counters
+                        yield
+                    c.products_out += c.record
+                    c.record = 0
+                    c.counts_out += n
+                else:
+                    n = c.count
+                    c.count += CLAIM
+                    n = 0 if n >= CLAIM else n
+                    yield
+                    c.products_out += c.record
+                    c.record = 0
+                    yield
+                    c.count -= CLAIM + n
+                    c.counts_out += n
+                yield
+            share = QUAD * BATCH_QUADS
+        for _ in range(BATCH_QUADS):
+            c.count += QUAD
+            yield
+            c.record += QUAD
+            c.most = max(c.most, c.record)
+            yield
+
+
+def _run(seed, two_passes, steps=60_000):
+    rng = random.Random(seed)
+    c = Cta()
+    warps = [_warp(c, two_passes) for _ in range(WARPS)]
+    asleep = [0] * WARPS
+    for t in range(steps):
+        w = rng.randrange(WARPS)
+        while asleep[w] > t and any(a <= t for a in asleep):
+            w = (w + 1) % WARPS
+        next(warps[w])
+        if rng.random() < 0.02:
+            asleep[w] = t + int(rng.expovariate(1.0 / 400.0))
+    return c
+
+
+@pytest.mark.parametrize("seed", range(12))
+def test_no_record_passes_the_bound(seed):
+    c = _run(seed, two_passes=False)
+    assert c.most <= LIMIT
+    assert c.products_out > 20 * LIMIT                     # it flushed many times
+    # what was taken out and what is left agree, but for the quads in flight
+    assert abs((c.counts_out + (c.count & (CLAIM - 1))) - (c.products_out + c.record)) <= QUAD * WARPS + LIMIT
+
+
+def test_the_bound_of_the_constants():
+    assert BATCH_QUADS * QUAD <= SHARE and KEEP + WARPS * SHARE <= LIMIT
+    assert LIMIT * 0xFFFF < 2 ** 32                        # 16-bit pieces
+    assert LIMIT * 2 ** 16 < 2 ** 32                       # top piece of products up to 2^48
+    assert LIMIT * 2 ** 48 < 2 ** 64                       # the record's sum
+    assert LIMIT + WARPS * 2 * QUAD < CLAIM
+
+
+def test_counters_taken_before_the_records_pass_it():
+    assert max(_run(seed, two_passes=True).most for seed in range(12)) > LIMIT

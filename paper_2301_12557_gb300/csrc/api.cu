@@ -85,16 +85,16 @@ struct Buf {
 
 struct Workspace {
     Buf hist, whist, counters, scalars, queue, blocks, tmp_cnt, tmp_off, tmp_tot, tasks, stencil, lut,
-        ea, eb, fold;
+        ea, eb, wsums;
 };
 
-// Fold mode (PairParams::wfold): each of the launch's `grid` CTAs gets its
-// own 128-bit sums per bin in the workspace.
-static pc_status attach_fold(Workspace &W, PairParams &p, int grid) {
-    if (!p.wfold) return PC_OK;
-    PC_CUDA(W.fold.ensure(sizeof(unsigned long long) * 2 * (size_t)p.nbins *
-                          (size_t)std::max(grid, 1)));
-    p.wfold_buf = (unsigned long long *)W.fold.p;
+// Integer weight products: each of the launch's `grid` CTAs gets its own exact
+// sums per bin in the workspace (PairParams::wsums).
+static pc_status attach_wsums(Workspace &W, PairParams &p, int grid) {
+    if (!p.wint) return PC_OK;
+    PC_CUDA(W.wsums.ensure(sizeof(unsigned long long) * 2 * (size_t)p.nbins *
+                           (size_t)std::max(grid, 1)));
+    p.wsums = (unsigned long long *)W.wsums.p;
     return PC_OK;
 }
 
@@ -930,7 +930,6 @@ static pc_status fit_params(int prec, int opt_priv, int dev, bool weighted, bool
         p.nent = nent0;
         fit(false);
     }
-    p.wfold = (p.wint && p.hist_k < 16) ? 1 : 0;
     {   // the floor paths' pair constants
         auto two = [](float v) { return make_float2(v, v); };
         const float row = 4.0f * p.hist_k * p.hs, col = 4.0f * p.hist_k;
@@ -1020,10 +1019,7 @@ static pc_status make_params(const CountJob &J, const CountSetup &S, const DevBu
     for (auto &t : J.tasks) p.npts_i += t.gi.n;
     p.npts_i /= p.shard_count;
     // integer weight products need floor bins, every weight packable and
-    // shared histograms with one count copy per CTA; with fewer than 16 lane
-    // copies (more than a few hundred bins) a copy would be flushed every few
-    // hundred j-points, so its records are folded into the CTA's exact sums
-    // instead (fold mode)
+    // shared histograms
     const bool wint_try = S.weighted && (p.path != PLAN_LUT || p.fix) && J.wint_ok && S.prec == PC_PREC_F32_RESCUE;
     int per_sm = 0;
     pc_status s = fit_params(S.prec, S.o.priv, S.dev, S.weighted, wint_try, J.wcorr, p, smem, per_sm);
@@ -1119,7 +1115,7 @@ static pc_status run_count(const CountJob &J, const pc_bins *b, const pc_opts *o
     int grid = 0;
     size_t smem = 0;
     s = make_params(J, S, B, p, grid, smem);
-    if (s == PC_OK) s = attach_fold(workspace(S.dev), p, grid);
+    if (s == PC_OK) s = attach_wsums(workspace(S.dev), p, grid);
     if (s != PC_OK) return s;
     S.wsum = p.wint ? (p.wcorr ? 3 : 2) : (S.weighted ? 1 : 0);
     Events ev(stats != nullptr);
@@ -1176,7 +1172,7 @@ struct GraphEntry {
         cudaFreeHost(h_ctr);
         cudaFreeHost(h_blocks);
         for (Buf *b : {&W.hist, &W.whist, &W.counters, &W.scalars, &W.queue, &W.blocks, &W.tmp_cnt,
-                       &W.tmp_off, &W.tmp_tot, &W.tasks, &W.stencil, &W.lut, &W.ea, &W.eb, &W.fold})
+                       &W.tmp_off, &W.tmp_tot, &W.tasks, &W.stencil, &W.lut, &W.ea, &W.eb, &W.wsums})
             if (b->p) cudaFree(b->p);
     }
 };
@@ -1239,7 +1235,7 @@ static pc_status run_count_graph(const CountJob &J, const std::vector<const pc_g
         int grid = 0;
         size_t smem = 0;
         s = make_params(J, N->S, N->B, p, grid, smem);
-        if (s == PC_OK) s = attach_fold(N->W, p, grid);
+        if (s == PC_OK) s = attach_wsums(N->W, p, grid);
         if (s != PC_OK) return s;
         N->S.wsum = p.wint ? (p.wcorr ? 3 : 2) : (N->S.weighted ? 1 : 0);
         const size_t hb = N->S.hist_n;
@@ -1501,7 +1497,7 @@ extern "C" pc_status pc_count_tree(const pc_tree *t1, const pc_tree *t2, const p
     int grid = 0;
     size_t smem = 0;
     s = make_params(J, S, B, p, grid, smem);
-    if (s == PC_OK) s = attach_fold(workspace(S.dev), p, grid);
+    if (s == PC_OK) s = attach_wsums(workspace(S.dev), p, grid);
     if (s != PC_OK) return s;
     S.wsum = p.wint ? (p.wcorr ? 3 : 2) : (S.weighted ? 1 : 0);
     Events ev(stats != nullptr);
@@ -1620,7 +1616,7 @@ extern "C" pc_status pc_count_tree_batch(const pc_tree *const *ts, int m, const 
     int grid = 0;
     size_t smem = 0;
     s = make_params(J, S, B, p, grid, smem);
-    if (s == PC_OK) s = attach_fold(workspace(S.dev), p, grid);
+    if (s == PC_OK) s = attach_wsums(workspace(S.dev), p, grid);
     if (s != PC_OK) return s;
     S.wsum = p.wint ? (p.wcorr ? 3 : 2) : (S.weighted ? 1 : 0);
     Events ev(stats != nullptr);
@@ -2036,7 +2032,7 @@ extern "C" pc_status pc_count_auto_noalloc(const pc_grid *g, const pc_bins *b, c
     int sms = 0, per_sm = 0;
     size_t smem = 0;
     PC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, cur));
-    // binary64 weight sums here (fold mode's sums would need an allocation)
+    // binary64 weight sums here (the exact sums of integer products would need an allocation)
     s = fit_params(prec, o.priv, cur, wcounts != nullptr, false, false, p, smem, per_sm);
     if (s != PC_OK) return s;
     if (per_sm <= 0) return fail(PC_ECUDA, "pair kernel cannot be resident");

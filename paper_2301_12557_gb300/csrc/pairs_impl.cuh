@@ -217,13 +217,38 @@ static __device__ __noinline__ void flush_counts(const PairParams &p, int first,
     }
 }
 
+// Integer weights: a CTA's exact sums of its products by bin (PairParams::wsums),
+// two words of value low + high 2^32, both signed, so that additions need no carry
+// and return nothing.  A flush adds less than 2^32 to the low word: 2^31 flushes of
+// tens of thousands of products fit.  They are converted and scaled once, when the
+// CTA is done with a histogram: adding every flush's sum to the binary64 totals
+// instead cost 3.9e-12 where 2e10 pairs of equal weights fall in one bin (their
+// partial sums round alike), against 3e-16.
+__device__ __forceinline__ void add_exact(const PairParams &p, int b, unsigned long long lo, unsigned long long hi) {
+    unsigned long long *f = p.wsums + ((size_t)blockIdx.x * p.nbins + b) * 2;
+    atomicAdd(&f[0], lo & 0xffffffffull);
+    hi += lo >> 32;
+    if (hi) atomicAdd(&f[1], hi);
+}
+
+// The CTA's exact sums into the global histogram (after a barrier that follows the
+// last flush).
+__device__ __forceinline__ void flush_exact(const PairParams &p, int h, double wscale) {
+    for (int b = threadIdx.x; b < p.nbins; b += blockDim.x) {
+        unsigned long long *f = p.wsums + ((size_t)blockIdx.x * p.nbins + b) * 2;
+        const long long lo = (long long)atomicExch(&f[0], 0ull);
+        const long long hi = (long long)atomicExch(&f[1], 0ull) + (lo >> 32);
+        const double w = fma((double)hi, 4294967296.0, (double)(lo & 0xffffffffll));
+        if (w != 0.0) atomicAdd(&p.whist[(size_t)h * p.nbins + b], w * wscale);
+    }
+}
+
 // LAY_BYTES with weights: counts and products of the bins whose fullest record
 // holds more than `above` of them (-1: all), four bins a step dealt to warps first,
 // first + nw, ...  A lane's records fill unevenly (128 neighbouring j-points are at
 // much the same distance): flushing all bins for the fullest of 1,280 records took
 // 50 of 340 ms.  Pieces are summed as integers (FP64 shuffles are slow here).
-static __device__ __noinline__ void flush_bytes(const PairParams &p, int above, int first, int nw, int h,
-                                                double wscale) {
+static __device__ __noinline__ void flush_bytes(const PairParams &p, int above, int first, int nw, int h) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31;
     unsigned *hist = reinterpret_cast<unsigned *>(smem) + 64 * p.row0;
@@ -250,17 +275,14 @@ static __device__ __noinline__ void flush_bytes(const PairParams &p, int above, 
                 const int sh = 8 + p.wcorr;   // bits of the lowest piece
                 const unsigned long long m = m0 + ((unsigned long long)m1 << 16),
                                          t = h0 + ((unsigned long long)h1 << 16);
-                // m 2^sh + lo below 2^47 and t 2^20 below 2^58, added as binary64 numbers
-                const double w = (double)(t << 20) * (double)(1u << sh) + (double)((m << sh) + lo);
-                atomicAdd(&p.whist[(size_t)h * p.nbins + b], w * wscale);
+                // m 2^sh + lo (below 2^47) + t 2^(20 + sh)
+                add_exact(p, b, ((m << sh) + lo) + ((t << (20 + sh)) & 0xffffffffull), t >> (12 - sh));
             }
         }
     }
 }
 
-// LAY_ROWS with integer weights: every entry's counter and record of products, the
-// exact sum of whose pieces is either scaled into the global histogram or (fold
-// mode) added to the CTA's exact 128-bit sums in wfold_buf.
+// LAY_ROWS with integer weights: every entry's counter and record of products.
 //
 // Other warps keep adding meanwhile, and may look for full records or flush them
 // as well.  A counter must never say less than its record holds (but for the quad
@@ -271,13 +293,13 @@ static __device__ __noinline__ void flush_bytes(const PairParams &p, int above, 
 // full records beside counters of zero: a warp that looked then added another
 // share, and the sums could wrap.)
 constexpr int CLAIM = 1 << 24;   // above any count between flushes
-static __device__ __noinline__ void flush_records(const PairParams &p, int first, int nw, int h, double wscale) {
+static __device__ __noinline__ void flush_records(const PairParams &p, int first, int nw, int h) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, K = p.hist_k, words = hist_entries(p) * K;
     int *hist = reinterpret_cast<int *>(smem);
     for (int w0 = first * 32; w0 < words; w0 += nw * 32) {
         const int idx = w0 + lane;
-        unsigned long long t = 0ull;
+        unsigned long long lo = 0ull, hi = 0ull;   // of the record's sum: lower 32 bits and upper
         int b = -1, n = 0;
         if (idx < words) {
             const int word = hist_word(p, idx / K, idx & (K - 1), b);
@@ -286,34 +308,22 @@ static __device__ __noinline__ void flush_records(const PairParams &p, int first
                 if (n >= CLAIM) n = 0;   // another warp's
                 __threadfence_block();
                 unsigned *r = reinterpret_cast<unsigned *>(smem + p.sm_whist) + 3 * (size_t)word;
-                const unsigned long long lo = atomicExch(r, 0u), mid = atomicExch(r + 1, 0u),
-                                         hi = atomicExch(r + 2, 0u);
-                t = lo + (mid << 16) + (hi << 32);
+                const unsigned long long r0 = atomicExch(r, 0u), r1 = atomicExch(r + 1, 0u),
+                                         r2 = atomicExch(r + 2, 0u);
+                lo = r0 + ((r1 & 0xffffull) << 16);
+                hi = r2 + (r1 >> 16);
                 __threadfence_block();
                 atomicSub(&hist[word], CLAIM + n);
             }
         }
-        const bool head = b >= 0 && (lane & (K - 1)) == 0;
-        for (int o = 1; o < K; o <<= 1) n += __shfl_xor_sync(FULL, n, o);
-        if (head && n) atomicAdd(&p.hist[(size_t)h * p.nbins + b], (unsigned long long)n);
-        if (p.wfold) {
-            unsigned long long hi = 0ull;
-            for (int o = 1; o < K; o <<= 1) {
-                const unsigned long long l2 = __shfl_xor_sync(FULL, t, o), h2 = __shfl_xor_sync(FULL, hi, o);
-                const unsigned long long s = t + l2;
-                hi += h2 + (s < t ? 1ull : 0ull);
-                t = s;
-            }
-            if (head && (t | hi)) {
-                unsigned long long *f = p.wfold_buf + ((size_t)blockIdx.x * p.nbins + b) * 2;
-                const unsigned long long old = atomicAdd(&f[0], t);
-                if (old + t < old) ++hi;
-                if (hi) atomicAdd(&f[1], hi);
-            }
-        } else {
-            double w = (double)t;
-            for (int o = 1; o < K; o <<= 1) w += __shfl_xor_sync(FULL, w, o);
-            if (head && w != 0.0) atomicAdd(&p.whist[(size_t)h * p.nbins + b], w * wscale);
+        for (int o = 1; o < K; o <<= 1) {
+            n += __shfl_xor_sync(FULL, n, o);
+            lo += __shfl_xor_sync(FULL, lo, o);
+            hi += __shfl_xor_sync(FULL, hi, o);
+        }
+        if (b >= 0 && (lane & (K - 1)) == 0) {
+            if (n) atomicAdd(&p.hist[(size_t)h * p.nbins + b], (unsigned long long)n);
+            if (lo | hi) add_exact(p, b, lo, hi);
         }
     }
 }
@@ -338,10 +348,10 @@ static __device__ __noinline__ void flush_weights(const PairParams &p, int first
 
 // Everything a CTA has added, by warps first, first + nw, ...  W as in the kernels.
 template <int W>
-__device__ __forceinline__ void flush_all(const PairParams &p, int first, int nw, int h, double wscale) {
+__device__ __forceinline__ void flush_all(const PairParams &p, int first, int nw, int h) {
     if (W >= 2) {
-        if (p.layout == LAY_BYTES) flush_bytes(p, -1, first, nw, h, wscale);
-        else flush_records(p, first, nw, h, wscale);
+        if (p.layout == LAY_BYTES) flush_bytes(p, -1, first, nw, h);
+        else flush_records(p, first, nw, h);
     } else {
         flush_counts(p, first, nw, h);
         if (W) flush_weights(p, first, nw, h);
@@ -368,18 +378,6 @@ static __device__ __noinline__ int most_counted(const PairParams &p) {
     }
     if (4 * n4 + lane < words) m = max(m, hist[4 * n4 + lane] & counts);
     return __reduce_max_sync(FULL, m);
-}
-
-// Fold mode: the CTA's exact sums, converted once (after a barrier that
-// follows the last fold).
-__device__ __forceinline__ void flush_folded(const PairParams &p, int h, double wscale) {
-    for (int b = threadIdx.x; b < p.nbins; b += blockDim.x) {
-        unsigned long long *f = p.wfold_buf + ((size_t)blockIdx.x * p.nbins + b) * 2;
-        const unsigned long long lo = atomicExch(&f[0], 0ull), hi = atomicExch(&f[1], 0ull);
-        if (lo | hi)
-            atomicAdd(&p.whist[(size_t)h * p.nbins + b],
-                      ((double)hi * 18446744073709551616.0 + (double)lo) * wscale);
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1644,9 +1642,9 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
     for (int k = threadIdx.x; k < p.sm_lut / 4; k += blockDim.x) reinterpret_cast<unsigned *>(smem)[k] = 0u;
     for (int k = threadIdx.x; k < p.lut_total; k += blockDim.x)
         reinterpret_cast<float2 *>(smem + p.sm_lut)[k] = p.lut[k];
-    if (W >= 2 && p.wfold)
+    if (W >= 2)
         for (int b = threadIdx.x; b < 2 * p.nbins; b += blockDim.x)
-            p.wfold_buf[(size_t)blockIdx.x * p.nbins * 2 + b] = 0ull;
+            p.wsums[(size_t)blockIdx.x * p.nbins * 2 + b] = 0ull;
     if (threadIdx.x == 0) s_range = RangeShared{0, 0, 0, 0, -1};
     const unsigned copy = 4u * (unsigned)(lane & (p.hist_k - 1));
     Ctx<MODE, LOS, is_fix(PATH) ? PATH_LIN : PATH> c;
@@ -1683,9 +1681,9 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
     for (;;) {
         auto flush = [&](int old) {
             const int h = p.tasks[old].hist;
-            if (PATH != PATH_GLOBAL) flush_all<W>(p, warp, nw, h, p.tasks[old].wscale);
+            if (PATH != PATH_GLOBAL) flush_all<W>(p, warp, nw, h);
             __syncthreads();
-            if (W >= 2 && p.wfold) flush_folded(p, h, p.tasks[old].wscale);
+            if (W >= 2) flush_exact(p, h, p.tasks[old].wscale);
             since = wterms = 0;
             __syncthreads();
         };
@@ -1795,15 +1793,15 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
                     const int nq = 2 * m;
                     since += nq;
                     if (since > flush_quads && PATH != PATH_GLOBAL) {
-                        if (W >= 2) flush_all<W>(p, 0, 1, T.hist, T.wscale);
+                        if (W >= 2) flush_all<W>(p, 0, 1, T.hist);
                         else flush_counts(p, 0, 1, T.hist);
                         since = nq;
                     }
                     if (W >= 2) {
                         wterms += wper * (unsigned)nq;
                         if (wterms > wlimit) {
-                            if (BYTES) flush_bytes(p, wfull, 0, 1, T.hist, T.wscale);
-                            else if (most_counted(p) > wfull) flush_records(p, 0, 1, T.hist, T.wscale);
+                            if (BYTES) flush_bytes(p, wfull, 0, 1, T.hist);
+                            else if (most_counted(p) > wfull) flush_records(p, 0, 1, T.hist);
                             wterms = wper * (unsigned)nq;
                         }
                     }
@@ -1888,11 +1886,10 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
     }
     __syncthreads();
     if (!p.multi) {   // batches have flushed after their last range
-        const double wscale = p.tasks[0].wscale;
-        if (PATH != PATH_GLOBAL) flush_all<W>(p, warp, nw, 0, wscale);
-        if (W >= 2 && p.wfold) {
+        if (PATH != PATH_GLOBAL) flush_all<W>(p, warp, nw, 0);
+        if (W >= 2) {
             __syncthreads();
-            flush_folded(p, 0, wscale);
+            flush_exact(p, 0, p.tasks[0].wscale);
         }
     }
     cand = warp_sum_u64(cand);
@@ -2017,7 +2014,7 @@ __global__ void __maxnreg__(96) k_pairs_f64(const __grid_constant__ PairParams p
 
     for (;;) {
         auto flush = [&](int old) {
-            if (p.smem_hist_ok) flush_all<W ? 1 : 0>(p, warp, nw, p.tasks[old].hist, 0.0);
+            if (p.smem_hist_ok) flush_all<W ? 1 : 0>(p, warp, nw, p.tasks[old].hist);
             since = 0;
             __syncthreads();
         };
@@ -2141,7 +2138,7 @@ __global__ void __maxnreg__(96) k_pairs_f64(const __grid_constant__ PairParams p
         }
     }
     __syncthreads();
-    if (!p.multi && p.smem_hist_ok) flush_all<W ? 1 : 0>(p, warp, nw, 0, 0.0);
+    if (!p.multi && p.smem_hist_ok) flush_all<W ? 1 : 0>(p, warp, nw, 0);
     cand = warp_sum_u64(cand);
     pruned = warp_sum_u64(pruned);
     if (lane == 0 && cand) atomicAdd(&p.counters[0], cand);

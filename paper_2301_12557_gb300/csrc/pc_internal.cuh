@@ -162,19 +162,14 @@ struct PairParams {
     // weighted sums from exact integer products of the packed binary32 weights
     // (significand product shifted by both exponent offsets, below 2^48),
     // accumulated as three 16-bit pieces in a record of three u32 sums per bin
-    // and lane copy, recombined exactly per copy and flushed as binary64 times
-    // the task's wscale
+    // and lane copy, flushed into exact sums per bin and CTA (wsums) and
+    // converted once per CTA to binary64 times the task's wscale
     int wint;
     // integer weight path with binary64 weights (some grid carries wlo): each
     // pair's product gains the cross terms of the next 31 bits and is rounded
     // to the accumulators' unit instead of truncated
     int wcorr;
-    // integer weights with fewer than 16 lane copies (large histograms): each
-    // copy reaches its product limit often, so the records are folded into
-    // exact 128-bit sums per bin held for each CTA in wfold_buf (two u64 per
-    // bin, low word first: gridDim x nbins x 2) instead of being flushed
-    int wfold;
-    unsigned long long *wfold_buf;
+    unsigned long long *wsums;   // gridDim x nbins x 2 words (add_exact)
     // k-d tree path (Alg. 3): each i-block (a tree node at the block level)
     // pairs with the j-blocks listed for it by the dual-tree traversal
     int tree;

@@ -45,3 +45,36 @@ def test_all_pairs_in_one_bin(form, mode, nb, wtype):
     # products truncated below 2^-34 of their value each
     assert abs(gotw[b] - want) <= 2.0 ** -34 * want
     assert np.count_nonzero(gotw) == 1
+
+
+def _unit_product(w, wtype):
+    """A pair's integer product of two weights w in [0.5, 1), in units of 2^-48."""
+    a = int(w * 2.0 ** 32)                                 # the packed 32 bits
+    if wtype == "f32":
+        return (a * a) >> 16
+    b = int((w * 2.0 ** 32 - a) * 2.0 ** 31)               # and the next 31
+    t = ((((a >> 1) * b) >> 32) + ((((a & 1) << 30 | b >> 1) * a) >> 32) + 0x2000) * 2
+    return (t + (a >> 1) * a) >> 15
+
+
+@pytest.mark.parametrize("wtype", ["f32", "f64"])
+@pytest.mark.parametrize("mode", ["s", "sigpi"])
+def test_sums_are_exact_but_for_one_conversion_a_cta(mode, wtype):
+    """5.0e9 pairs of equal weights in one bin: every product is the same integer,
+    so their exact sum is known.  A CTA's part is exact until it is converted (two
+    roundings) and added (one): at most three halves of 2^-52 of the sum a CTA."""
+    torch = pytest.importorskip("torch")
+    n, w = 100003, float(np.float32(0.7853981))
+    if wtype == "f64":
+        w += 1.23e-10
+    x = 50.0 + np.random.default_rng(1).uniform(-0.25, 0.25, (n, 3))
+    weights = np.full(n, w, np.float32 if wtype == "f32" else np.float64)
+    eb = np.linspace(0.0, 30.0, 41) if mode == "sigpi" else None
+    bins = P.Bins(mode, "z", np.linspace(0.0, 30.0, 31 if mode == "s" else 41), eb)
+    g = P.pc_build_grid(x, weights, box=P.make_box(L, True), r_max=bins.r_max)
+    got, gotw, st = P.pc_count_auto(g, bins, opts=P.make_opts(grid_ctas_per_sm=1), weighted=True)
+    assert st.wsum == (2 if wtype == "f32" else 3)
+    assert got[0] == n * (n - 1) // 2
+    want = int(got[0]) * _unit_product(w, wtype) / 2 ** 48
+    ctas = torch.cuda.get_device_properties(0).multi_processor_count
+    assert abs(gotw[0] - want) <= 3 * ctas * 2.0 ** -53 * want

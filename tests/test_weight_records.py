@@ -8,6 +8,7 @@ must not bring a record past the bound; taking the counters of all entries befor
 their records, as a flush in two passes does, must."""
 
 import random
+from fractions import Fraction
 
 import pytest
 
@@ -95,3 +96,26 @@ def test_the_bound_of_the_constants():
 
 def test_counters_taken_before_the_records_pass_it():
     assert max(_run(seed, two_passes=True).most for seed in range(12)) > LIMIT
+
+
+def test_exact_sums_without_carries():
+    """A CTA's sums: low + high 2^32 in two 64-bit words that wrap on their own;
+    products may be taken off again.  The conversion rounds at most twice."""
+    m64, rng = 2 ** 64 - 1, random.Random(3)
+
+    def signed(v):
+        return v - 2 ** 64 if v >> 63 else v
+
+    for _ in range(200):
+        f, exact = [0, 0], 0
+        for _ in range(rng.randint(1, 400)):
+            t = rng.randint(0, LIMIT * 2 ** 48 * 32 if rng.random() < 0.5 else 2 ** 48)
+            sign = -1 if t < 2 ** 48 and exact > t and rng.random() < 0.5 else 1
+            lo, hi = t & 0xFFFFFFFF, t >> 32
+            f[0], f[1] = (f[0] + sign * lo) & m64, (f[1] + sign * hi) & m64
+            exact += sign * t
+        lo = signed(f[0])
+        hi = signed(f[1]) + (lo >> 32)
+        assert hi >= 0 and (hi << 32) + (lo & 0xFFFFFFFF) == exact
+        w = Fraction(float(Fraction(float(hi)) * 2 ** 32 + (lo & 0xFFFFFFFF)))
+        assert abs(w - exact) <= Fraction(exact, 2 ** 52)

@@ -231,6 +231,15 @@ __device__ __forceinline__ void add_exact(const PairParams &p, int b, unsigned l
     if (hi) atomicAdd(&f[1], hi);
 }
 
+// A product that this CTA has added is taken off again.  (Taken off the binary64
+// totals, it left their rounding behind: up to 4e-10 in a bin without pairs, for
+// 90,000 products of about 0.6 just below its edge.)
+__device__ __forceinline__ void sub_exact(const PairParams &p, int b, unsigned long long v) {
+    unsigned long long *f = p.wsums + ((size_t)blockIdx.x * p.nbins + b) * 2;
+    atomicAdd(&f[0], 0ull - (v & 0xffffffffull));
+    atomicAdd(&f[1], 0ull - (v >> 32));
+}
+
 // The CTA's exact sums into the global histogram (after a barrier that follows the
 // last flush).
 __device__ __forceinline__ void flush_exact(const PairParams &p, int h, double wscale) {
@@ -1161,8 +1170,8 @@ __device__ __forceinline__ unsigned long long fast_product(const IPts<LOS, W> &I
 // An entry is {first of its four j-points, source lane | own block << 5 |
 // segment << 6 | the batch's bound (fix_bands) << 13}.  The lane repeats the quad's FP32 arithmetic
 // on the same operands, so it sees the same bins and the same near pairs, and
-// corrects the global histogram where the binary64 bin differs from the one
-// counted.  (Pairs of a half that the batch left out are repeated too: they are
+// corrects the global histogram (integer weights: the CTA's exact sums) where the
+// binary64 bin differs from the one counted.  (Pairs of a half that the batch left out are repeated too: they are
 // beyond the last edge by more than the error bands, bin -1 both ways.)  With a
 // rescue queue (pc_opts.rescue_capacity > 0) the fast count is
 // undone instead and the pair queued while there is room.
@@ -1280,8 +1289,7 @@ __device__ __noinline__ void check_near(const PairParams &p, const uint2 *queue,
                         load_i<MODE, LOS, W>(T.gi, i, I, 0);
                         const unsigned wj = __float_as_uint(T.gj.rel[j].w);
                         const unsigned lj = (W == 3 && T.gj.wlo) ? T.gj.wlo[j] : 0u;
-                        atomicAdd(&p.whist[hb + (size_t)fast],
-                                  -((double)fast_product<LOS, W>(I, 0, wj, lj) * T.wscale));
+                        sub_exact(p, fast, fast_product<LOS, W>(I, 0, wj, lj));
                     }
                 }
                 if (bin >= 0) {

@@ -78,3 +78,29 @@ def test_sums_are_exact_but_for_one_conversion_a_cta(mode, wtype):
     want = int(got[0]) * _unit_product(w, wtype) / 2 ** 48
     ctas = torch.cuda.get_device_properties(0).multi_processor_count
     assert abs(gotw[0] - want) <= 3 * ctas * 2.0 ** -53 * want
+
+
+@pytest.mark.parametrize("capacity", [0, 1 << 20])
+@pytest.mark.parametrize("wtype", ["f32", "f64"])
+@pytest.mark.parametrize("mode", ["s", "smu", "sigpi"])
+def test_pairs_taken_out_of_a_bin_leave_nothing(mode, wtype, capacity):
+    """90,000 pairs 1e-9 (relative) below an edge are counted past it in binary32
+    and put right: a bin without pairs has a weighted sum of exactly zero."""
+    rng = np.random.default_rng(2)
+    n = 300
+    a = np.array([20.0, 30.0, 40.0]) + 1e-10 * rng.random((n, 3))
+    d = {"s": [3.0, 0.0, 4.0], "smu": [3.0, 0.0, 4.0], "sigpi": [3.0, 4.0, 2.0]}[mode]   # s or sigma = 5
+    x = np.concatenate([a, a + np.array(d) * (1.0 - 1e-9)])
+    w = 0.5 + 0.5 * rng.random(2 * n)
+    v = w.astype(np.float32) if wtype == "f32" else w
+    eb = {"s": None, "smu": np.linspace(0.0, 1.0, 101), "sigpi": np.linspace(0.0, 30.0, 41)}[mode]
+    bins = P.Bins(mode, "z", np.linspace(0.0, 25.0, 6), eb)
+    g = P.pc_build_grid(x, v, box=P.make_box(L, True), r_max=bins.r_max)
+    got, gotw, st = P.pc_count_auto(g, bins, opts=P.make_opts(rescue_capacity=capacity), weighted=True)
+    assert st.wsum == (2 if wtype == "f32" else 3) and st.rescued >= n * n
+    row = got.reshape(5, -1).sum(1)
+    assert row[1] == 0 and got.sum() == n * (2 * n - 1)
+    assert not np.any(gotw[got == 0])
+    y = v.astype(np.longdouble)
+    want = float((y.sum() ** 2 - (y * y).sum()) / 2)
+    assert abs(gotw.sum() - want) <= 2.0 ** -34 * want

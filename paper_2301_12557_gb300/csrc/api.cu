@@ -844,7 +844,10 @@ static void set_fp32_params(const Geom &g, const double *lo, const double *hi, c
     // that takes four more roundings of at most 2^-24 x 3 X, so a computed gap
     // exceeds the true one by less than 2^-20 X (2^-50 of the absolute
     // coordinates for the subtraction of the origin); squares and sums add a
-    // relative 2^-22.  The limits carry twice that.
+    // relative 2^-22.  The limits carry twice that, and seven of the smallest
+    // numbers for squares that underflow; they are infinite where a square in reach
+    // may overflow, and the tests then drop nothing (catalogues in metres: the FP64
+    // kernel counts those as it does any).
     double X = 0.0, A = 0.0, c = 0.0;
     for (int a = 0; a < 3; ++a) {
         X = std::max(X, (hi[a] - lo[a]) + g.L[a]);
@@ -854,7 +857,7 @@ static void set_fp32_params(const Geom &g, const double *lo, const double *hi, c
     const double m = ldexp(X, -19) + ldexp(A, -49);
     p.f_gm = nextafterf((float)m, INFINITY);
     auto up = [&](double r) {
-        const double v = (r + m) * (r + m) * (1.0 + ldexp(1.0, -20));
+        const double v = (r + m) * (r + m) * (1.0 + ldexp(1.0, -20)) + 1e-44;
         return v < 1e38 ? nextafterf((float)v, INFINITY) : INFINITY;
     };
     p.r2prune = up(P.rcut);
@@ -862,7 +865,7 @@ static void set_fp32_params(const Geom &g, const double *lo, const double *hi, c
     if (P.mode == PC_BIN_SIGPI) {   // along z: sigma and pi each stay below their last edge
         const double slack = P.rcut - P.reff;
         p.q2prune = up(P.ea[P.na] + slack);
-        p.zprune = nextafterf((float)((P.eb[P.nb] + slack + m) * (1.0 + ldexp(1.0, -20))), INFINITY);
+        p.zprune = nextafterf((float)((P.eb[P.nb] + slack + m) * (1.0 + ldexp(1.0, -20)) + 1e-44), INFINITY);
     }
     // absent points: beyond the reach of every point of a neighbouring cell
     // (node), whose offset is at most rcut + 3 c, and small enough for exact floors

@@ -1579,9 +1579,9 @@ __device__ __forceinline__ void ring_round(const PairParams &p, const TaskDev &T
             const float gy = fmaxf(fmaxf(bl.y - h.y, l.y - bh.y), 0.f);
             const float gz = fmaxf(fmaxf(bl.z - h.z, l.z - bh.z), 0.f);
             const float gq = fmaf(gy, gy, gx * gx), g = fmaf(gz, gz, gq);
-            keep[r] = g < p.r2prune;
+            keep[r] = g <= p.r2prune;                 // (an infinite limit keeps gaps that overflow)
             if (MODE == MODE_SIGPI && LOS == LOS_Z)   // the reach is a cylinder
-                keep[r] = keep[r] && gq < p.q2prune && gz < p.zprune;
+                keep[r] = keep[r] && gq <= p.q2prune && gz <= p.zprune;
             // (sigma, pi): the gap across the line of sight
             if (keep[r]) g2 = fminf(g2, MODE != MODE_SIGPI ? g : (LOS == LOS_Z ? gq : 0.f));
             else pruned += (unsigned long long)(nj * (unsigned)(r ? count - half : half));

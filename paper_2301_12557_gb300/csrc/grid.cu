@@ -475,29 +475,38 @@ cudaError_t make_blocks_into(const TaskDev *tasks_dev, int ntasks, int ncell, in
 // ---------------------------------------------------------------------------
 using namespace pc;
 
-// Default cell side of a periodic box: about 160 points a cell, between a
-// quarter of the reach and the reach.  The pair kernel's warps take 64 points of
-// one cell (fewer points leave lanes empty, larger cells add candidate boxes and
-// widen the error bands) and prune by boxes of eight, so the side matters little
-// around the best: 100k clustered points, reach 200: 0.75 ms here (cells of 125)
-// against 0.87 at the cost model's 200; 2M, reach 60: 3.2 against 3.8; 3.7M
-// weighted, reach 200: 360 (50) against 376 (40); 12 mocks: 121 against 133;
-// 200k to 2M, reach 200: within 2 %.  The model's side stays where either grid
-// leaves the limits of the allocation-free count, so that it takes the same
-// catalogues, and without a box: the points' bounds say little of their density
-// (survey shell, 500k points: 26 ms at the model's 200, 28 at 120).
+// Default cell side of a periodic box: the cost model's 4 r_max / k, brought to
+// between a quarter of the reach and the reach, about 160 points a cell.  The pair
+// kernel's warps take 64 points of one cell (fewer points leave lanes empty, larger
+// cells add candidate boxes and widen the error bands) and prune by boxes of eight,
+// so the side matters little around the best: 100k clustered points, reach 200:
+// 0.75 ms in cells of 125 against 0.87 at the model's 200; 2M, reach 60: 3.2 against
+// 3.8; 3.7M weighted, reach 200: 360 (50) against 376 (40).
+//
+// A function of k alone: catalogues whose sizes give one model side share their
+// default grid, so that cross counts and batches take them (a side that followed the
+// density cut the boxes of 50k and 100k points differently).  k = 4 stands for 108 to
+// 1,028 and 2,048 to 2,309 points in a cube of the reach, 7 and 8 for two ranges,
+// larger k for one within 1.5.  Against the cube root of 160 / density, 20k to 1.2M
+// points at reaches of 60 to 200: within 3 %, but for 60 from 650k points (a side of
+// 42 instead of 60: 1.79 -> 1.97 ms); 1M projected, reach 85: 2.92 -> 2.76 ms.
+// The model's side stays where either grid has many cells, so that the
+// allocation-free count takes the same catalogues (where this side is the smaller,
+// 65,536 cells leave room for the blocks of any catalogue it took), and without a
+// box: the points' bounds say little of their density (survey shell, 500k points:
+// 26 ms at the model's 200, 28 at 120).
 static double default_cell_side(long long n, const double L[3], double vol, double r_max, bool periodic) {
     const double model = pc_suggest_cell_size(n, vol, r_max, 1);
     if (n < 1 || !periodic) return model;
-    const double c = std::min(std::max(cbrt(160.0 * vol / (double)n), 0.25 * r_max), r_max);
+    const double k = 4.0 * r_max / model;
+    const double c = r_max * (k < 3.5 ? 1.0 : k < 6.5 ? 0.7 : k < 8.5 ? 3.4 / k : std::max(0.25, 3.42 / (k - 0.5)));
     auto cells = [&](double side) {
         double t = 1.0;
         for (int a = 0; a < 3; ++a) t *= std::max(1.0, floor(L[a] / side));
         return t;
     };
-    const double most = 250000.0;   // (cells added for the stencil's reach not counted)
-    if (cells(c) > most || cells(model) > most || cells(c) + (double)n / 128.0 > 500000.0) return model;
-    return c;
+    // (cells added for the stencil's reach not counted)
+    return cells(c) > 65536.0 || cells(model) > 250000.0 ? model : c;
 }
 
 extern "C" pc_status pc_aabb(const double *xyz, long long n, void *stream, double *lo,

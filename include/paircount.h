@@ -456,11 +456,12 @@ pc_status pc_stencil(const double cell[3], double r_max, int half, int max_rows,
  *   5 fp32_ok 1 when the FP32 path's bound holds (else counts run in FP64)
  *   6 lin     1 when the bins are found by a floor instead of tables
  *   7 r2cut   the FP32 cut the kernel compares s^2 against
- *   8..15     floor-based bins (when lin): t = s * invA + offA and bin =
+ *   8..15     packed floors (when lin): t = s * invA + offA and bin =
  *             floor(t), not near an edge iff |frac(t) - 1/2| < thrA (offA
- *             carries +1 when the s range is tested, the bin then floor(t) -
- *             1); mu bins t_mu = mu * nB, not near iff |frac(t_mu) - 1/2| <
- *             cB - mA / s; then norange (1: e_0 = 0 and no range test) and
+ *             carries +1 unless norange, the bin then floor(t) - 1); mu bins
+ *             t_mu = mu * nB, not near iff |frac(t_mu) - 1/2| < cB - mA / s
+ *             (lin is 0 for mu along the midpoint, whose floors
+ *             pc_fp32_floors gives); then norange (1: e_0 = 0) and
  *             log (1: logarithmic s edges, t from log2(s^2)):
  *             invA, offA, thrA, nB, mA, cB, norange, log (with log, t =
  *             log2(s^2) * invA + offA and the band is thrA - mS / s, mS in
@@ -475,6 +476,36 @@ pc_status pc_stencil(const double cell[3], double r_max, int half, int max_rows,
 pc_status pc_fp32_bands(const pc_bins *b, const double cell[3], const double lo[3],
                         const double hi[3], const double L[3], int periodic, double rmin,
                         double out[19]);
+
+/* The constants that the FP32 kernel of the same count receives (host-only), as
+ * binary32 values; fixed-point floors add a value t = v inv to c + B 2^-16 in
+ * one fused multiply-add: byte 2 of the sum is the bin (c = 128, or 129 less
+ * the first edge's t with a discarded bin 0), and its low half is below 2 B
+ * near an edge.  out[0..31]:
+ *    0 path     0 tables, 1 floors from zero, 2 from any edge, 3 of logarithms
+ *    1 fix      5, 6, 7: floors 1, 2, 3 in fixed point (126 bins an axis at
+ *               most; 0: not); wider histograms and binary64 weight sums take
+ *               `path`
+ *    2, 3       inv, inv_b: scales of the axes (logarithms: of log2 of the square)
+ *    4, 5       c + B 2^-16 of the first axis (logarithms: c) and 2 B
+ *    6, 7       the same of pi
+ *    8, 9       largest sums of the axes (past the last bin, not near)
+ *   10..12      mu: B = ceil(mA / s + mB) at a lower bound of the batch's s, and
+ *               the square that this bound starts at
+ *   13..15      logarithms: B = ceil(sA / s + sC), and the square it starts at
+ *   16          sums of the first axis, less 2 B 2^-16, below which a pair is near
+ *               whatever its mu
+ *   17          added to the squares
+ *   18          coordinate of absent points
+ *   19..22      box tests: what a gap may exceed the true one by, the largest
+ *               squared gap kept, and for (sigma, pi) along z that of the gap
+ *               across the line of sight and the largest gap along it
+ *   23..31      packed floors: invA, offA, thrA, mS, nB, mA, cB, invB, thrB as
+ *               in pc_fp32_bands (offA with + 1)
+ * Errors as pc_fp32_bands. */
+pc_status pc_fp32_floors(const pc_bins *b, const double cell[3], const double lo[3],
+                         const double hi[3], const double L[3], int periodic, double rmin,
+                         double out[32]);
 
 /* The lookup tables the FP32 path stages for the same count as
  * pc_fp32_bands (host-only).  lut receives n_entries pairs {edge, bin

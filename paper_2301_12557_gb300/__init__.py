@@ -76,7 +76,7 @@ EXPORTS = ["pc_build_grid", "pc_free_grid", "pc_grid_info", "pc_count_auto", "pc
            "pc_version", "pc_launch_count", "pc_count_auto_noalloc", "pc_tune",
            "pc_build_tree", "pc_free_tree", "pc_tree_info", "pc_tree_export", "pc_count_tree",
            "pc_tune_tree", "pc_hist_s2", "pc_count_tree_batch", "pc_stencil", "pc_fp32_bands",
-           "pc_fp32_tables", "pc_fp_peak", "pc_alloc_count", "pc_build_tree_batch"]
+           "pc_fp32_floors", "pc_fp32_tables", "pc_fp_peak", "pc_alloc_count", "pc_build_tree_batch"]
 
 
 def library_path() -> str:
@@ -165,6 +165,8 @@ def lib():
     L.pc_fp32_bands.argtypes = [POINTER(pc_bins), POINTER(c_double), POINTER(c_double),
                                 POINTER(c_double), POINTER(c_double), c_int, c_double,
                                 POINTER(c_double)]
+    L.pc_fp32_floors.restype = c_int
+    L.pc_fp32_floors.argtypes = L.pc_fp32_bands.argtypes
     L.pc_fp32_tables.restype = c_int
     L.pc_fp32_tables.argtypes = [POINTER(pc_bins), POINTER(c_double), POINTER(c_double),
                                  POINTER(c_double), POINTER(c_double), c_int, c_double,
@@ -682,6 +684,22 @@ def pc_fp32_bands(bins: "Bins", cell, lo, hi, L=None, periodic: bool = False,
     keys = ("eps_a", "eps_b", "mu_A", "mu_B", "rcut", "fp32_ok", "lin", "r2cut",
             "lin_invA", "lin_offA", "lin_thrA", "lin_nB", "lin_mA", "lin_cB", "lin_norange",
             "lin_log", "lin_invB", "lin_thrB", "lin_mS")
+    return dict(zip(keys, (float(v) for v in out)))
+
+
+def pc_fp32_floors(bins: "Bins", cell, lo, hi, L=None, periodic: bool = False,
+                   rmin: float = 0.0) -> dict:
+    """The constants the FP32 kernel of a count receives (host-only)."""
+    def v3(a):
+        return (c_double * 3)(*np.broadcast_to(np.asarray(a, dtype=np.float64), (3,)))
+    out = (c_double * 32)()
+    _check(lib().pc_fp32_floors(ctypes.byref(bins.s), v3(cell), v3(lo), v3(hi),
+                                v3(L) if L is not None else None, int(bool(periodic)),
+                                float(rmin), out), "pc_fp32_floors")
+    keys = ("path", "fix", "inv", "inv_b", "c_a", "near_a", "c_pi", "near_pi", "max_a", "max_b",
+            "mu_A", "mu_B", "mu_s2", "log_A", "log_C", "log_s2", "close", "tiny", "far", "gap_error",
+            "gap2", "gap2_across", "gap_along", "lin_invA", "lin_offA", "lin_thrA", "lin_mS", "lin_nB",
+            "lin_mA", "lin_cB", "lin_invB", "lin_thrB")
     return dict(zip(keys, (float(v) for v in out)))
 
 

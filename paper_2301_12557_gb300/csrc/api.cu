@@ -1728,7 +1728,7 @@ extern "C" pc_status pc_fp32_bands(const pc_bins *b, const double cell[3], const
     out[5] = P.fp32_ok;
     out[6] = P.lin;
     out[7] = P.r2cut;
-    // floor-based bins, as the kernel receives them
+    // packed floors (pc_fp32_floors has what a kernel receives)
     out[8] = P.lin_invA;
     out[9] = P.lin_norange ? P.lin_offA : P.lin_offA1;
     out[10] = P.lin_thrA;
@@ -1740,6 +1740,46 @@ extern "C" pc_status pc_fp32_bands(const pc_bins *b, const double cell[3], const
     out[16] = P.lin_invB2;
     out[17] = P.lin_thrB;
     out[18] = P.lin_mS;
+    return PC_OK;
+}
+
+// Host-only view of the constants the FP32 kernel of the same count receives.
+extern "C" pc_status pc_fp32_floors(const pc_bins *b, const double cell[3], const double lo[3],
+                                    const double hi[3], const double L[3], int periodic,
+                                    double rmin, double out[32]) {
+    if (!b || !cell || !lo || !hi || !out || (periodic && !L))
+        return fail(PC_EINVAL, "pc_fp32_floors: bad arguments");
+    Geom g;
+    memset(&g, 0, sizeof(g));
+    g.periodic = periodic ? 1 : 0;
+    for (int a = 0; a < 3; ++a) {
+        if (!(cell[a] > 0.0) || !std::isfinite(cell[a]) || !std::isfinite(lo[a]) ||
+            !std::isfinite(hi[a]) || hi[a] < lo[a])
+            return fail(PC_EINVAL, "pc_fp32_floors: bad cell sides or bounds");
+        if (periodic && (!(L[a] > 0.0) || !std::isfinite(L[a])))
+            return fail(PC_EINVAL, "pc_fp32_floors: periodic box needs L > 0");
+        g.c[a] = cell[a];
+        g.c32[a] = (float)cell[a];
+        g.ng[a] = 1;
+        g.lo[a] = lo[a];
+        g.L[a] = periodic ? L[a] : 0.0;
+        g.hL[a] = 0.5 * g.L[a];
+    }
+    Plan P;
+    pc_status s = make_plan(b, g, lo, hi, rmin, false, P, false);
+    if (s != PC_OK) return s;
+    PairParams p;
+    memset(static_cast<void *>(&p), 0, sizeof(p));
+    p.mode = P.mode;
+    p.los = P.los;
+    p.n_a = P.na;
+    p.n_b = P.nb;
+    set_fp32_params(g, lo, hi, P, P.fp32_ok ? PC_PREC_F32_RESCUE : PC_PREC_F64, p);
+    const double v[32] = {(double)p.path, (double)p.fix, p.f_inv, p.f_invB, p.f_cfs.x, (double)p.f_ts2, p.f_cfp,
+                          (double)p.f_tp2, p.f_lim, p.f_limB, p.f_mA, p.f_mB, p.f_sf2, p.f_sA, p.f_sC, p.f_se2,
+                          p.f_close, p.f_tiny.x, p.far, p.f_gm, p.r2prune, p.q2prune, p.zprune, p.lin_invA,
+                          p.lin_offA, p.lin_thrA, p.lin_mS, p.lin_nB, p.lin_mA, p.lin_cB, p.lin_invB2, p.lin_thrB};
+    for (int k = 0; k < 32; ++k) out[k] = v[k];
     return PC_OK;
 }
 

@@ -1709,7 +1709,10 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
             box.clear();
             I.x[r] = -far;      // unused: out of range of every j-point
             I.y[r] = I.z[r] = 0.f;
-            I.xa[r] = I.ya[r] = I.za[r] = 0.f;
+            // (midpoint: l = 2 x_i + d across d, else mu = 1 and sigma = 0 are near an
+            // edge and every quad of such a lane is queued)
+            I.xa[r] = I.za[r] = 0.f;
+            I.ya[r] = LOS == LOS_MID ? far : 0.f;
             I.w[r] = 0.0;
             I.wm[r] = 0u;
             I.wb[r] = 0u;

@@ -11,7 +11,8 @@ shows here.
     band (the check that sees a band cut short although no planted pair does).
   * Packed floors of mu along the midpoint (more than 126 bins).
   * The box tests: no pair in range is dropped, whatever box of eight and half of
-    the i-points it is in."""
+    the i-points it is in.
+  * Points that are not there: near an edge no more often than others."""
 
 import importlib.util
 import os
@@ -378,3 +379,27 @@ def test_box_tests_keep_every_pair_in_range(mode, L, ng, lo, R, periodic):
     root = np.maximum(np.sqrt((gq if mode == "sigpi" else g2).astype(F64)) * (1 - 2.0 ** -21) - k["gap_error"], 0.0)
     least = np.sqrt((q2 if mode == "sigpi" else s2).reshape(s2.shape[0], -1).min(1))
     assert np.all(root <= least)
+
+
+@pytest.mark.parametrize("mode", ["smu", "sigpi"])
+def test_absent_points_are_seldom_near_an_edge(mode):
+    """An i-point that is not there stands at x = -far with 2 x_i = (0, far, 0) along
+    the midpoint: l is not parallel to d, so sigma and pi lie past the last edge and
+    mu is near one as often as any value, 2 B 2^-16.  (With 2 x_i = 0, l = d: mu = 1
+    and sigma = 0, always near.)"""
+    rng = np.random.default_rng(9)
+    ea, eb = EVEN[mode]
+    c = 200.0
+    k = P.pc_fp32_floors(P.Bins(mode, "mid", ea, eb), c, np.full(3, -2000.0), np.full(3, 2000.0), None, False, 1000.0)
+    assert int(k["fix"]) == FIX
+    far, n = F32(k["far"]), 100_000
+    xj = rng.uniform(-400.0, 400.0, (n, 3)).astype(F32)
+    dd = xj - np.array([-far, 0, 0], F32)
+    for y in (far, F32(0.0)):
+        v = _separations(dd, np.tile(np.array([0, y, 0], F32), (n, 1)), k, "mid")
+        with np.errstate(divide="ignore", invalid="ignore"):
+            b = _bands(mode, "mid", k, np.zeros(n), np.zeros(n))
+            for t, m in _sums(mode, "mid", k, v, b):
+                near = ((t.view(np.uint32) & 0xFFFF) < b["ts2"]) | ((m.view(np.uint32) & 0xFFFF) < b["tm2"])
+                usual = (b["ts2"][0] + b["tm2"][0]) / 65536.0
+                assert near.mean() < 1.5 * usual if y else near.mean() > 0.99

@@ -233,21 +233,18 @@ pc_status pc_count_auto_noalloc(const pc_grid *g, const pc_bins *b, const pc_opt
 /* One configuration timed by pc_tune. */
 typedef struct {
     double cell_size;   /* requested cell side */
-    int ipt;            /* i-points per thread */
-    int priv;           /* replication: 0 automatic, 1 one count copy per warp */
+    int ipt;            /* blocks of 128 ipt points */
+    int priv;           /* as in pc_opts: 0 automatic, 1 binary64 weight sums */
     float ms;           /* device time of the sampled pair and rescue kernels */
 } pc_tune_trial;
 
 /* Measured autotuner for the options of a count (the cost model of Appendix
  * B.1 gives the starting cell side).  Times the pair and rescue kernels on an
- * evenly spaced sample of the point blocks: 2 and 4 i-points per thread at
- * the model's cell side, then the better of those at cell sides in
- * quarter-octave steps from 0.7 to 2 times it (distinct grids only), then one
- * count copy per warp at the best, then (unless base fixes rescue_capacity)
- * the near-edge pairs evaluated inside the pair kernel (rescue_capacity -1)
- * instead of queued for the rescue kernel; writes the fastest options to
- * *out (base's other fields are kept).  pc_tune_trial of the last trial
- * carries the options it ran with.
+ * evenly spaced sample of the point blocks: ipt 2 and 4 at the model's cell
+ * side, then the better of those at cell sides in quarter-octave steps from
+ * 0.7 to 2 times it (distinct grids only), then, with weights, binary64
+ * weight sums (priv 1) at the best; writes the fastest options to *out
+ * (base's other fields are kept).
  *   xyz, w, w_is_f32, n, box   the catalogue, as for pc_build_grid
  *   b                          the bins the counts will use
  *   base                       starting options (NULL = defaults); priv 1 or
@@ -373,14 +370,12 @@ pc_status pc_count_tree_batch(const pc_tree *const *ts, int m, const pc_bins *b,
 /* Measured options of the k-d tree path for the auto count of a catalogue:
  * builds the tree (leaf capacity n_leaf) with the automatic list level and
  * with list nodes of at most 512, 1024, 2048 and 4096 points (distinct levels
- * only), times the pair and rescue kernels for 2 and 4 i-points per thread
- * on every S-th block (S as in pc_tune), and writes the fastest: out->ipt
- * (base's other fields kept) and *list_cap for pc_build_tree; the automatic
- * level with 2 i-points is kept unless another option is more than 3 %
- * faster.  A last trial (unless base fixes rescue_capacity) evaluates the
- * near-edge pairs inside the pair kernel (out->rescue_capacity -1 when
- * faster; its record has priv -1).  trials (cell_size holds the list_cap
- * tried, 0 = automatic) and n_trials as for pc_tune.
+ * only), times the pair and rescue kernels for ipt 2 and 4 on every S-th
+ * block (S as in pc_tune), and writes the fastest: out->ipt (base's other
+ * fields kept) and *list_cap for pc_build_tree; the automatic level with
+ * ipt 2 is kept unless another option is more than 3 % faster.  trials
+ * (cell_size holds the list_cap tried, 0 = automatic) and n_trials as for
+ * pc_tune.
  * Errors as pc_build_tree and pc_count_tree. */
 pc_status pc_tune_tree(const double *xyz, const void *w, int w_is_f32, long long n,
                        const pc_box *box, const pc_bins *b, int n_leaf, const pc_opts *base,

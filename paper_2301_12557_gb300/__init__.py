@@ -361,8 +361,8 @@ def pc_build_grid(xyz, w=None, *, box: pc_box, r_max: float, opts: pc_opts | Non
 
 def pc_tune(xyz, w=None, *, box: pc_box, bins: Bins, opts: pc_opts | None = None, stream=None,
             max_trials: int = 32):
-    """Measured autotuning of cell side, i-points per thread and histogram
-    privatisation; returns (tuned pc_opts, list of (cell_size, ipt, priv, ms))."""
+    """Measured autotuning of cell side, points of a block and, with weights, the
+    form of the weighted sums; returns (tuned pc_opts, list of (cell_size, ipt, priv, ms))."""
     px, keep_x, n = _ptr(xyz, np.float64, 3)
     w_is_f32 = 0
     pw, keep_w = None, None
@@ -544,7 +544,7 @@ def pc_build_tree_batch(xyzs, ws=None, *, box: pc_box, n_leaf: int = 32, list_ca
 
 def pc_tune_tree(xyz, w=None, *, box: pc_box, bins: Bins, n_leaf: int = 32,
                  opts: pc_opts | None = None, stream=None, max_trials: int = 16):
-    """Measured list level and i-points per thread of the tree path; returns
+    """Measured list level and points of a block of the tree path; returns
     (pc_opts with ipt, list_cap, list of (list_cap, ipt, ms))."""
     px, keep_x, n = _ptr(xyz, np.float64, 3)
     pw, keep_w, w_is_f32 = _weights_arg(w, n)

@@ -1,13 +1,14 @@
-// Measured autotuner: cell side, i-points per thread and histogram privatisation.
+// Measured autotuner: cell side, points of a block and, with weights, the form of
+// the weighted sums.
 //
 // The cost model of Appendix B.1 (pc_suggest_cell_size) gives a starting cell
 // side; the tuner times the FP32 pair kernel (plus rescue) on an evenly spaced
 // sample of the point blocks -- the block-shard mechanism of the multi-GPU
-// path with one shard -- first for 2 and 4 i-points per thread at that side,
-// then at cell sides in quarter-octave steps from 0.7 to 2 times it, then
-// with priv 1 (binary64 weight sums), then with rescue_capacity -1 (the
-// near-edge pairs checked in the pair kernel, which is also the default's
-// path), and returns the fastest combination.
+// path with one shard -- first for blocks of 256 and 512 points (ipt 2 and 4) at
+// that side, then at cell sides in quarter-octave steps from 0.7 to 2 times it,
+// then, with weights, with priv 1 (binary64 weight sums), and returns the fastest
+// combination.  (Without weights priv 1 is the automatic choice, and
+// rescue_capacity -1 is the default's own path: neither is timed.)
 #include <math.h>
 #include <string.h>
 
@@ -150,7 +151,7 @@ extern "C" pc_status pc_tune(const double *xyz, const void *w, int w_is_f32, lon
             out->ipt = ipt;
         }
     };
-    // 1. i-points per thread at the model's cell side
+    // 1. points of a block at the model's cell side
     int ipt_best = 2;
     {
         pc_opts oc = o;
@@ -200,9 +201,9 @@ extern "C" pc_status pc_tune(const double *xyz, const void *w, int w_is_f32, lon
         if (s != PC_OK) return s;
         record(c, ipt_best, ms);
     }
-    // histogram replication (automatic vs one copy per warp) at the best cell
-    // side and i-tile, unless the caller fixed it
-    if (!fixed_priv && std::isfinite(best_ms)) {
+    // binary64 weight sums (priv 1) at the best cell side and block, unless the
+    // caller fixed priv
+    if (w && !fixed_priv && std::isfinite(best_ms)) {
         pc_opts oc = *out;
         pc_grid *g = nullptr;
         pc_status s = pc_build_grid(xyz, w, w_is_f32, n, box, reach, &oc, stream, &g);
@@ -227,41 +228,13 @@ extern "C" pc_status pc_tune(const double *xyz, const void *w, int w_is_f32, lon
             out->priv = 1;
         }
     }
-    // rescue_capacity -1 (no queue, as by default: the binary64 work interleaves
-    // with the FP32 pairs of other warps) at the best options, unless the caller
-    // fixed the queue size
-    if (fp32 && o.rescue_capacity == 0 && std::isfinite(best_ms)) {
-        pc_opts oc = *out;
-        pc_grid *g = nullptr;
-        pc_status s = pc_build_grid(xyz, w, w_is_f32, n, box, reach, &oc, stream, &g);
-        if (s != PC_OK) return s;
-        pc_opts ot = oc;
-        ot.rescue_capacity = -1;
-        ot.shard_index = 0;
-        ot.shard_count = S;
-        float ms = INFINITY;
-        for (int rep = 0; rep < 2 && s == PC_OK; ++rep) {
-            pc_stats sts;
-            s = pc_count_auto(g, b, &ot, stream, (long long *)dc.p, (double *)dw.p, &sts);
-            if (s == PC_OK) ms = std::min(ms, sts.ms_pairs + sts.ms_rescue);
-            if (ms > 4.f * TRIAL_MS) break;
-        }
-        pc_free_grid(g);
-        if (s != PC_OK) return s;
-        if (nt < max_trials) trials[nt] = pc_tune_trial{out->cell_size, out->ipt, out->priv, ms};
-        ++nt;
-        if (ms < best_ms) {
-            best_ms = ms;
-            out->rescue_capacity = -1;
-        }
-    }
     if (n_trials) *n_trials = std::min(nt, max_trials);
     PC_CUDA(cudaStreamSynchronize(st));
     return PC_OK;
 }
 
 // Measured choice of the k-d tree path's options: the list level (through
-// the list-node capacity of pc_build_tree) and the i-points per thread,
+// the list-node capacity of pc_build_tree) and the points of a block (ipt),
 // timed like pc_tune on every S-th point block of the catalogue's auto count.
 // (pc_tune_trial.cell_size carries the list-node capacity tried.)
 extern "C" pc_status pc_tune_tree(const double *xyz, const void *w, int w_is_f32, long long n,
@@ -316,7 +289,7 @@ extern "C" pc_status pc_tune_tree(const double *xyz, const void *w, int w_is_f32
         return s;
     };
     // list-node capacities: automatic, then 512 .. 4096 (distinct levels only);
-    // another option replaces the automatic level with 2 i-points only when
+    // another option replaces the automatic level with ipt 2 only when
     // it is faster by more than the trials' run-to-run spread (3 %)
     float ms_default = INFINITY;
     std::vector<int> seen_levels;
@@ -359,23 +332,6 @@ extern "C" pc_status pc_tune_tree(const double *xyz, const void *w, int w_is_f32
     if (std::isfinite(ms_default) && best_ms > 0.97f * ms_default) {
         out->ipt = 2;
         *list_cap = 0;
-        best_ms = ms_default;
-    }
-    // near-edge pairs evaluated inside the pair kernel, at the chosen options
-    if (o.rescue_capacity == 0 && o.prec == PC_PREC_F32_RESCUE && std::isfinite(best_ms)) {
-        pc_tree *t = nullptr;
-        pc_status s = pc_build_tree(xyz, w, w_is_f32, n, box, n_leaf, *list_cap, stream, &t);
-        if (s != PC_OK) return s;
-        pc_opts keep = o;
-        o.rescue_capacity = -1;
-        float ms = INFINITY;
-        s = run(t, out->ipt, ms);
-        o = keep;
-        pc_free_tree(t);
-        if (s != PC_OK) return s;
-        if (nt < max_trials) trials[nt] = pc_tune_trial{(double)*list_cap, out->ipt, -1, ms};
-        ++nt;
-        if (ms < best_ms) out->rescue_capacity = -1;
     }
     if (n_trials) *n_trials = std::min(nt, max_trials);
     PC_CUDA(cudaStreamSynchronize(st));

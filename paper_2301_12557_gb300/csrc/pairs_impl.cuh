@@ -1675,8 +1675,9 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
     constexpr unsigned wmax = BYTES ? (W == 3 ? 2047u : 4095u) : WINT_LIMIT;
     // one loop body for both halves in turn where a body of two i-points a lane is
     // too large to share the instruction cache with the rest: (s, mu) along the
-    // midpoint with binary64 weights, 140k points, 21.8 -> 16.4 ms
-    constexpr bool TWO = !(W == 3 && LOS == LOS_MID && MODE != MODE_S);
+    // midpoint with binary64 weights (500k survey randoms 15.9 -> 12.1 ms; (sigma, pi)
+    // there takes the two-point body, 100k x 2M points 32.1 -> 30.8)
+    constexpr bool TWO = !(W == 3 && LOS == LOS_MID && MODE == MODE_SMU);
     constexpr unsigned wkeep = BYTES ? wmax / 2 : wmax / 4;   // what a look may leave in a record
     constexpr unsigned wbatch = 8u * (BYTES ? 1u : 32u) * O::jb / 4u;   // largest batch to one record
     static_assert(W < 2 || 8u * wbatch <= wmax - wkeep, "a batch of each of 8 warps fits");

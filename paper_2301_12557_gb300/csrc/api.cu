@@ -106,9 +106,6 @@ static Workspace &workspace(int dev) {
 // ---------------------------------------------------------------------------
 // plan: bins, error bands, lookup tables, stencil
 // ---------------------------------------------------------------------------
-enum { PLAN_LUT = 0, PLAN_LIN = 1, PLAN_LINOFF = 2, PLAN_LOG = 3,   // PATH_* of the kernel
-       PLAN_FIX = 5, PLAN_FIXOFF = 6, PLAN_FIXLOG = 7 };
-
 struct Plan {
     int mode = 0, los = 0, na = 0, nb = 1, nbins = 0;
     std::vector<double> ea, eb;   // edges
@@ -131,8 +128,8 @@ struct Plan {
     // the pair kernel's choice: tables, or floors from zero, from any edge or
     // of logarithms (the lin fields; also for mu along the midpoint line of
     // sight, which lin leaves out)
-    int path = PLAN_LUT;
-    // fixed-point floors (fix: PLAN_FIX*, or 0): scales, the first axis's constant
+    int path = PATH_LUT;
+    // fixed-point floors (fix: PATH_FIX*, or 0): scales, the first axis's constant
     // without its band, bands in units of 2^-16 (first axis, fx_sA / s for
     // logarithms; pi of (sigma, pi); mu, fx_mA / s + fx_mB), and the separation the
     // mu band stops growing at
@@ -482,7 +479,7 @@ static pc_status make_plan(const pc_bins *b, const Geom &g, const double *pts_lo
             }
         }
     }
-    P.path = !P.lin ? PLAN_LUT : (P.lin_log ? PLAN_LOG : (P.ea[0] == 0.0 ? PLAN_LIN : PLAN_LINOFF));
+    P.path = !P.lin ? PATH_LUT : (P.lin_log ? PATH_LOG : (P.ea[0] == 0.0 ? PATH_LIN : PATH_LINOFF));
     if (mid_mu) P.lin = P.lin_log = P.lin_norange = 0;
     // ---- (sigma, pi) with evenly spaced edges from 0: floors of both ------
     // t_sigma = sigma / D_a, t_pi = pi / D_b, sigma and pi formed as on the
@@ -507,7 +504,7 @@ static pc_status make_plan(const pc_bins *b, const Geom &g, const double *pts_lo
             P.lin_invB2 = (float)(1.0 / Db);
             P.lin_thrB = nextafterf((float)(0.5 - etb), 0.0f);
             P.lin_norange = 0;
-            P.path = PLAN_LIN;
+            P.path = PATH_LIN;
         }
     }
     // ---- fixed-point floors (PATH_FIX*) ---------------------------------------
@@ -521,8 +518,8 @@ static pc_status make_plan(const pc_bins *b, const Geom &g, const double *pts_lo
     {
         const double one = 65536.0;
         const double na = P.na, nb = P.nb;
-        int kind = P.path == PLAN_LIN ? PLAN_FIX : (P.path == PLAN_LINOFF ? PLAN_FIXOFF
-                                                    : (P.path == PLAN_LOG ? PLAN_FIXLOG : 0));
+        int kind = P.path == PATH_LIN ? PATH_FIX : (P.path == PATH_LINOFF ? PATH_FIXOFF
+                                                    : (P.path == PATH_LOG ? PATH_FIXLOG : 0));
         const double D = (P.ea[P.na] - P.ea[0]) / na;
         bool ok = true;
         // edges evenly spaced from zero (second axis of (sigma, pi)), and
@@ -536,13 +533,13 @@ static pc_status make_plan(const pc_bins *b, const Geom &g, const double *pts_lo
                 lq = log2(P.ea[P.na] / P.ea[0]) / na;
                 double dev = 0.0;
                 for (int k = 0; k <= P.na; ++k) dev = std::max(dev, fabs(log2(P.ea[k] / P.ea[0]) / lq - k));
-                if (dev <= 1e-6 && eps_sig < 0.05 * P.ea[0]) kind = PLAN_FIXLOG;
+                if (dev <= 1e-6 && eps_sig < 0.05 * P.ea[0]) kind = PATH_FIXLOG;
             }
             P.fx_invB = 1.0 / Db;
             P.fx_p = ceil((eps_z / Db + 1e-9 + 4.0 * u * nb) * one + 0.5);
             ok = ok && P.fx_p < 8192.0;
         }
-        if (kind == PLAN_FIXLOG) {
+        if (kind == PATH_FIXLOG) {
             const double e0 = P.ea[0];
             if (lq == 0.0) lq = log2(P.ea[P.na] / e0) / na;
             const double ln2 = log(2.0), A = 1.0 / (2.0 * lq), B = -log2(e0) / lq;
@@ -559,15 +556,15 @@ static pc_status make_plan(const pc_bins *b, const Geom &g, const double *pts_lo
                 P.fx_s = 2.0 * (A * 9.0 * u / ln2 * 1.01 + common) * one + 2.0;
             }
             P.fx_sA *= 1.001;
-            ok = ok && e0 > 1e-9 && eps_s < 0.05 * e0 && fabs(P.fx_c) < 250.0 && P.fx_sA / (0.5 * e0) + P.fx_s < 8192.0 && na <= 125;
+            ok = ok && e0 > 1e-9 && eps_s < 0.05 * e0 && fabs(P.fx_c) < 250.0 && P.fx_sA / (0.5 * e0) + P.fx_s < 8192.0 && na < FIX_TOP;
         } else if (kind) {
             const double es = P.mode == PC_BIN_SIGPI
                                   ? eps_sig / D + 1e-9 + 4.0 * u * na
                                   : (1.25 * u * (4.34 * c + 8.7 * Rb) + tiny) / D + 1e-9;
             P.fx_inv = 1.0 / D;
-            P.fx_c = kind == PLAN_FIX ? 128.0 : 129.0 - P.ea[0] / D;
-            P.fx_s = ceil(es * one + (kind == PLAN_FIX ? 0.5 : 1.5));
-            ok = ok && P.fx_s < 8192.0 && (kind == PLAN_FIX || (na <= 125 && fabs(P.fx_c) < 250.0));
+            P.fx_c = kind == PATH_FIX ? 128.0 : 129.0 - P.ea[0] / D;
+            P.fx_s = ceil(es * one + (kind == PATH_FIX ? 0.5 : 1.5));
+            ok = ok && P.fx_s < 8192.0 && (kind == PATH_FIX || (na < FIX_TOP && fabs(P.fx_c) < 250.0));
         }
         if (P.mode == PC_BIN_SMU) {
             const double mA = P.los == PC_LOS_Z ? 1.25 * 6.9 * u * c + tiny : muA;
@@ -580,7 +577,7 @@ static pc_status make_plan(const pc_bins *b, const Geom &g, const double *pts_lo
         }
         // no FP32 square may overflow (the kernel's indices rely on it), and the
         // constant 1e-30 in the squares must stay far inside the first band
-        ok = ok && X + Lm + R0 + c < 1e15 && std::min({D, Db, P.ea[1]}) > 1e-9 && na <= 126 && nb <= 126;
+        ok = ok && X + Lm + R0 + c < 1e15 && std::min({D, Db, P.ea[1]}) > 1e-9 && na <= FIX_TOP && nb <= FIX_TOP;
         P.fix = ok ? kind : 0;
     }
     // ---- stencil -------------------------------------------------------------
@@ -621,7 +618,7 @@ static void choose_replication(int mode, int nbins, bool weighted, int &hist_k) 
 // entry past them.  The (sigma, pi) floors send pi past its last bin to a
 // discarded column.
 static void set_hist_rows(PairParams &p, const Plan &P) {
-    p.hs = P.nb + (P.mode == PC_BIN_SIGPI && p.path == PLAN_LIN ? 1 : 0);
+    p.hs = P.nb + (P.mode == PC_BIN_SIGPI && p.path == PATH_LIN ? 1 : 0);
     p.nent = P.na * p.hs + 1;
 }
 
@@ -797,7 +794,7 @@ static pc_status upload_tables(const CountJob &J, const CountSetup &S, const Dev
 // The FP32 path's constants from the plan, and the box tests' limits.
 static void set_fp32_params(const Geom &g, const double *lo, const double *hi, const Plan &P, int prec,
                             PairParams &p) {
-    p.path = (prec == PC_PREC_F32_RESCUE) ? P.path : PLAN_LUT;
+    p.path = (prec == PC_PREC_F32_RESCUE) ? P.path : PATH_LUT;
     p.lin_invA = P.lin_invA;
     // the floors with an offset take t_s + 1 (exact floors down to t_s = -1)
     p.lin_offA = P.lin_offA1;
@@ -814,11 +811,11 @@ static void set_fp32_params(const Geom &g, const double *lo, const double *hi, c
         const double one = 65536.0;
         p.fix = prec == PC_PREC_F32_RESCUE ? P.fix : 0;
         p.row0 = 0;
-        const bool off = P.fix == PLAN_FIXOFF || P.fix == PLAN_FIXLOG;
+        const bool off = P.fix == PATH_FIXOFF || P.fix == PATH_FIXLOG;
         p.f_inv = (float)P.fx_inv;
         p.f_invB = (float)P.fx_invB;
         p.f_tiny = two(1e-30f);
-        p.f_cfs = two((float)(P.fx_c + (P.fix == PLAN_FIXLOG ? 0.0 : P.fx_s / one)));
+        p.f_cfs = two((float)(P.fx_c + (P.fix == PATH_FIXLOG ? 0.0 : P.fx_s / one)));
         p.f_ts2 = 2 * (unsigned)ceil(P.fx_s);
         p.f_cfp = (float)(128.0 + P.fx_p / one);
         p.f_tp2 = 2 * (unsigned)P.fx_p;
@@ -833,7 +830,7 @@ static void set_fp32_params(const Geom &g, const double *lo, const double *hi, c
         // edge: they are out of range)
         p.f_sf2 = (float)(P.fx_sf * P.fx_sf);
         double tsf = P.fx_sf * (1.0 + 1e-6);
-        if (P.fix == PLAN_FIXLOG) tsf = tsf > P.ea[0] ? 2.0 * log2(tsf) * P.fx_inv : -1e3;
+        if (P.fix == PATH_FIXLOG) tsf = tsf > P.ea[0] ? 2.0 * log2(tsf) * P.fx_inv : -1e3;
         else tsf *= P.fx_inv;
         p.f_close = (float)(P.fx_c + tsf + 0.01);
         if (off && p.f_close < 129.0f) p.f_close = 0.0f;
@@ -889,17 +886,17 @@ static pc_status fit_params(int prec, int opt_priv, int dev, bool weighted, bool
         p.wint = wint ? 1 : 0;
         p.wcorr = (wint && wcorr) ? 1 : 0;
         p.path = path0;
-        p.layout = 0;
+        p.layout = LAY_ROWS;
         p.row0 = 0;
         choose_replication(opt_priv, p.nbins, weighted && !wint, p.hist_k);
         if (p.fix && (wint || !weighted)) {   // fixed-point floors (not for binary64 weight sums)
             p.path = p.fix;
-            p.row0 = p.fix == PLAN_FIX ? 0 : 1;
+            p.row0 = p.fix == PATH_FIX ? 0 : 1;
             if (p.mode == PC_BIN_S) {
-                p.layout = 2;
+                p.layout = LAY_BYTES;
                 p.hist_k = 32;
             } else if (!weighted) {
-                p.layout = 1;
+                p.layout = LAY_SKEW;
                 p.hist_k = 1;
             } else {   // mu = 1 (pi past its last bin) needs a column of its own
                 p.hs = p.n_b + 1;
@@ -910,15 +907,15 @@ static pc_status fit_params(int prec, int opt_priv, int dev, bool weighted, bool
         for (;;) {
             p.smem_hist_ok = 1;
             // the floor bins need no tables
-            p.lut_total = (p.path != PLAN_LUT || f64) ? 0 : lut_size;
+            p.lut_total = (p.path != PATH_LUT || f64) ? 0 : lut_size;
             if (pairs_smem(p, nw_min) + static_smem <= (size_t)smem_optin) break;
-            if (p.layout == 0 && p.hist_k > 1) {   // fewer lane copies, then the global histogram
+            if (p.layout == LAY_ROWS && p.hist_k > 1) {   // fewer lane copies, then the global histogram
                 p.hist_k /= 2;
                 continue;
             }
             p.smem_hist_ok = 0;
-            p.path = PLAN_LUT;
-            p.layout = 0;
+            p.path = PATH_LUT;
+            p.layout = LAY_ROWS;
             p.row0 = 0;
             p.lut_total = f64 ? 0 : lut_size;
             p.hist_k = 1;
@@ -940,16 +937,16 @@ static pc_status fit_params(int prec, int opt_priv, int dev, bool weighted, bool
         p.c_23 = two(8388608.0f);
         p.c_p = two(8388607.5f);
         p.c_m1 = two(-1.0f);
-        p.c_invA = two(p.path >= PLAN_FIX ? p.f_inv : p.lin_invA);
+        p.c_invA = two(p.path >= PATH_FIX ? p.f_inv : p.lin_invA);
         p.c_offA = two(p.lin_offA);
         p.c_thrA = two(p.lin_thrA);
         p.c_nmS = two(-p.lin_mS);
-        p.c_invB = two(p.path >= PLAN_FIX ? p.f_invB : (p.mode == PC_BIN_SIGPI ? p.lin_invB2 : p.lin_nB));
+        p.c_invB = two(p.path >= PATH_FIX ? p.f_invB : (p.mode == PC_BIN_SIGPI ? p.lin_invB2 : p.lin_nB));
         p.c_nmB = two(-p.lin_mA);
         p.c_cB = two(p.mode == PC_BIN_SIGPI ? p.lin_thrB : p.lin_cB);
         p.c_nrow = two(-row);
         p.c_ncol = two(-col);
-        p.c_kA = 8388608.0f - (p.path == PLAN_LIN ? 0.5f : 1.5f) * row -
+        p.c_kA = 8388608.0f - (p.path == PATH_LIN ? 0.5f : 1.5f) * row -
                  (p.mode == PC_BIN_S ? 0.0f : 0.5f * col);
     }
     // 8 warps at most with weights: a copy's products between a warp's flushes
@@ -1023,7 +1020,7 @@ static pc_status make_params(const CountJob &J, const CountSetup &S, const DevBu
     p.npts_i /= p.shard_count;
     // integer weight products need floor bins, every weight packable and
     // shared histograms
-    const bool wint_try = S.weighted && (p.path != PLAN_LUT || p.fix) && J.wint_ok && S.prec == PC_PREC_F32_RESCUE;
+    const bool wint_try = S.weighted && (p.path != PATH_LUT || p.fix) && J.wint_ok && S.prec == PC_PREC_F32_RESCUE;
     int per_sm = 0;
     pc_status s = fit_params(S.prec, S.o.priv, S.dev, S.weighted, wint_try, J.wcorr, p, smem, per_sm);
     if (s != PC_OK) return s;
@@ -2083,10 +2080,6 @@ extern "C" pc_status pc_count_auto_noalloc(const pc_grid *g, const pc_bins *b, c
     cudaError_t e = (prec == PC_PREC_F64) ? launch_pairs_f64(p, sms * per_sm, smem, st)
                                           : launch_pairs_f32(p, sms * per_sm, smem, st);
     if (e != cudaSuccess) return cuda_fail(e, "pair kernel launch");
-    if (p.qcap) {
-        e = launch_rescue(p, st);
-        if (e != cudaSuccess) return cuda_fail(e, "rescue kernel launch");
-    }
     if (counts) {
         cudaMemcpyKind k = is_device_ptr(counts) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
         PC_CUDA(cudaMemcpyAsync(counts, hist, sizeof(long long) * hist_n, k, st));

@@ -439,7 +439,7 @@ __global__ void k_block_emit(const TaskDev *tasks, int ntasks, int ncell, const 
     int s = cs[c], nc = cs[c + 1] - s;
     // cut at multiples of 64, the points of a warp's item: only a cell's last item
     // is not full (equal blocks left a rest in each: 2M clustered points 68.2 ->
-    // 65.4 ms, 140k survey randoms in cells of 200 16.5 -> 13.3)
+    // 65.4 ms, 500k survey randoms in cells of 200 16.5 -> 13.3)
     const long long units = (nc + 63) / 64;
     for (int k = 0; k < nb; ++k) {
         const int b0 = (int)(units * k / nb) * 64, b1 = min(nc, (int)(units * (k + 1) / nb) * 64);

@@ -67,7 +67,6 @@ constexpr int BI = 64;        // i-points per warp: two halves of 32, one point 
 // weights' records bounds a batch (bytes: LAY_BYTES) and in the FP64 kernel
 __host__ __device__ constexpr int batch_points(int w, bool bytes) { return w == 0 || (w == 2 && bytes) ? 128 : 64; }
 constexpr int QCAP = 64;      // near-edge quads kept by a warp before it checks them
-constexpr int FIX_TOP = 126;  // most bins per axis of the fixed-point floors (125 with an offset)
 constexpr int SEG_G = 97;     // j-segments of a chunk: 32 stencil rows, <= 3 each, and the own cell
 constexpr int SEG_T = 33;     // 32 listed tree nodes and the own node
 
@@ -92,7 +91,6 @@ struct WarpOff {
         total = (pref + (nseg + 1) * 4 + 15) / 16 * 16       // int[nseg + 1]
     };
 };
-enum { LAY_ROWS = 0, LAY_SKEW = 1, LAY_BYTES = 2 };   // see below
 inline size_t warp_slice(const PairParams &p) {
     const bool wide = batch_points(!p.weighted ? 0 : (p.wint ? 2 + p.wcorr : 1), p.layout == LAY_BYTES) == 128;
     int n = 0;
@@ -564,13 +562,6 @@ __device__ __forceinline__ void red_shared_f64_if(unsigned addr, double v, bool 
         ::"r"(addr), "d"(v), "r"((unsigned)on));
 }
 
-// How the bins are found: lookup tables, floors (evenly spaced from 0; evenly
-// spaced from any edge; logarithmic s), or tables into the global histogram
-// when it does not fit shared memory.  PATH_FIX, PATH_FIXOFF and
-// PATH_FIXLOG: the first three floors (logarithmic also for sigma) in fixed
-// point, for up to FIX_TOP bins an axis.
-enum { PATH_LUT = 0, PATH_LIN = 1, PATH_LINOFF = 2, PATH_LOG = 3, PATH_GLOBAL = 4,
-       PATH_FIX = 5, PATH_FIXOFF = 6, PATH_FIXLOG = 7 };
 __host__ __device__ constexpr bool is_fix(int path) { return path >= PATH_FIX; }
 
 // Two pairs' outcome: byte offset of the counter in the shared histogram

@@ -23,6 +23,18 @@ constexpr int WINT_MAX_SPAN = 12;
 
 enum { MODE_S = 0, MODE_SMU = 1, MODE_SIGPI = 2 };
 
+// How the FP32 kernel finds bins: lookup tables, floors (evenly spaced from 0;
+// evenly spaced from any edge; logarithmic), or tables into the global histogram
+// when it does not fit shared memory.  PATH_FIX, PATH_FIXOFF and PATH_FIXLOG: the
+// first three floors (logarithmic also for sigma) in fixed point, for up to FIX_TOP
+// bins an axis (one fewer on a first axis with a discarded row before it).
+enum { PATH_LUT = 0, PATH_LIN = 1, PATH_LINOFF = 2, PATH_LOG = 3, PATH_GLOBAL = 4,
+       PATH_FIX = 5, PATH_FIXOFF = 6, PATH_FIXLOG = 7 };
+constexpr int FIX_TOP = 126;
+
+// Layouts of the shared histogram (described with the pair kernel)
+enum { LAY_ROWS = 0, LAY_SKEW = 1, LAY_BYTES = 2 };
+
 // Packed integer weight: w 2^(158 - emax), emax the largest biased binary32
 // exponent of the catalogue's weights' binary32 roundings (exponents spanning at
 // most 8 binades), as 32 bits, and the next 31.  A binary32 value w = M 2^(e -

@@ -344,7 +344,7 @@ def run_ours(args, emit=True):
     if tree and (args.list_cap > 0 or args.ipt > 0):
         opts = P.make_opts("f32", 0.0, args.ipt or 2)
     elif tree:
-        # measured list level and i-points per thread, once, before the timed steps
+        # measured list level and points of a block, once, before the timed steps
         t0 = time.perf_counter()
         opts, list_cap, trials = P.pc_tune_tree(D, box=box, bins=bins, n_leaf=args.n_leaf,
                                                 stream=stream)
@@ -531,7 +531,7 @@ def run_ours(args, emit=True):
     evaluated = cand - stats[0].pruned       # pairs the kernel separated one by one
     flops_ev = FLOPS_PER_CANDIDATE * evaluated + FLOPS_PER_IN_RANGE * inr_step
     ach_ev = flops_ev / (ms_pairs * 1e-3) / 1e12
-    trec = traffic_record(w.name, tree, opts.rescue_capacity < 0)
+    trec = traffic_record(w.name, tree, opts.rescue_capacity <= 0)
     roofline = {"bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
                 "frac": achieved / fp32_peak,
                 "traffic": trec["bytes_per_launch"] if trec else None,
@@ -649,7 +649,7 @@ def run_batch(args):
         opts = P.make_opts("f32", 0.0, args.ipt or 2)
         cell = 0.0
     elif tree:
-        # measured list level and i-points per thread, on the mock of median size
+        # measured list level and points of a block, on the mock of median size
         t0 = time.perf_counter()
         opts, list_cap, trials = P.pc_tune_tree(X[med], box=box, bins=bins, n_leaf=args.n_leaf,
                                                 stream=stream)
@@ -1188,7 +1188,7 @@ def run_sets(args, extra=None):
     flops_ev = FLOPS_PER_CANDIDATE * evaluated + FLOPS_PER_IN_RANGE * inr_d
     ach_ev = flops_ev / (ms_pairs * 1e-3) / 1e12
     fp32_peak = peaks["fp32_tflops"]
-    trec = traffic_record(w.name, tree, opts.rescue_capacity < 0)
+    trec = traffic_record(w.name, tree, opts.rescue_capacity <= 0)
     kname = {"s": "S", "smu": "SMU", "sigpi": "SIGPI"}[w.mode]
     wkind = {0: "", 1: ", binary64 weight products", 2: ", integer weight products"}.get(sd.wsum, "")
     roofline = {"bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",

@@ -31,8 +31,8 @@
 // one, so the integer counts equal the binary64 definition exactly.
 //
 // What bounds it (2M clustered points, (s, mu) 40 x 100, 6.70e10 pairs in
-// range): issue slots (82 % used; the FMA and integer pipes at 51 and 54 %, shared
-// memory at 61 %).  1.52 pairs are evaluated for each in range, against 1.70 with
+// range): issue slots (76 % of the cycles issue; the FMA and integer pipes at 51 and
+// 53 %, the shared-memory pipe at 62 %).  1.52 pairs are evaluated for each in range, against 1.70 with
 // one list for the 64 points along a Morton curve; 113 of about 135 warp
 // instructions per 64 x 4 pairs are the loop itself.  65.4 ms against 154.7 ms for
 // CTAs of 128 threads that staged every candidate tile behind a barrier and queued
@@ -310,11 +310,13 @@ static __device__ __noinline__ void flush_records(const PairParams &p, int first
         int b = -1, n = 0;
         if (idx < words) {
             const int word = hist_word(p, idx / K, idx & (K - 1), b);
-            if (b >= 0 && *reinterpret_cast<volatile int *>(hist + word) != 0) {
+            unsigned *r = reinterpret_cast<unsigned *>(smem + p.sm_whist) + 3 * (size_t)word;
+            // (a record may hold the products of a quad whose counts an earlier flush took)
+            volatile const unsigned *v = r;
+            if (b >= 0 && (*reinterpret_cast<volatile int *>(hist + word) || (v[0] | v[1] | v[2]))) {
                 n = atomicAdd(&hist[word], CLAIM);
                 if (n >= CLAIM) n = 0;   // another warp's
                 __threadfence_block();
-                unsigned *r = reinterpret_cast<unsigned *>(smem + p.sm_whist) + 3 * (size_t)word;
                 const unsigned long long r0 = atomicExch(r, 0u), r1 = atomicExch(r + 1, 0u),
                                          r2 = atomicExch(r + 2, 0u);
                 lo = r0 + ((r1 & 0xffffull) << 16);

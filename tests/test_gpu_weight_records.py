@@ -104,3 +104,32 @@ def test_pairs_taken_out_of_a_bin_leave_nothing(mode, wtype, capacity):
     y = v.astype(np.longdouble)
     want = float((y.sum() ** 2 - (y * y).sum()) / 2)
     assert abs(gotw.sum() - want) <= 2.0 ** -34 * want
+
+
+@pytest.mark.parametrize("wtype", ["f32", "f64"])
+@pytest.mark.parametrize("mode", ["s", "sigpi", "smu"])
+@pytest.mark.parametrize("form", ["grid", "tree"])
+def test_no_product_is_lost_while_others_fill(form, mode, wtype):
+    """1.8e9 pairs of equal weights in a clump, bins from crowded ones, for which the
+    records are flushed all the time, to rare ones: every bin's sum is its count
+    times one product, to the conversions of the CTAs (three halves of 2^-52 each) and
+    to a unit of 2^-48 for each pair that its binary64 check moved."""
+    torch = pytest.importorskip("torch")
+    n, w = 60001, float(np.float32(0.7853981))
+    if wtype == "f64":
+        w += 1.23e-10
+    x = 50.0 + np.random.default_rng(4).normal(0.0, 0.5, (n, 3))
+    weights = np.full(n, w, np.float32 if wtype == "f32" else np.float64)
+    eb = {"s": None, "sigpi": np.linspace(0.0, 30.0, 41), "smu": np.linspace(0.0, 1.0, 101)}[mode]
+    bins = P.Bins(mode, "z", np.linspace(0.0, 30.0, 41), eb)
+    box, v = P.make_box(L, True), _unit_product(w, wtype)
+    if form == "grid":
+        g = P.pc_build_grid(x, weights, box=box, r_max=bins.r_max)
+        got, gotw, st = P.pc_count_auto(g, bins, weighted=True)
+    else:
+        t = P.pc_build_tree(x, weights, box=box)
+        got, gotw, st = P.pc_count_tree(t, None, bins, weighted=True)
+    assert st.wsum == (2 if wtype == "f32" else 3) and got.sum() == n * (n - 1) // 2
+    want = np.array([int(c) * v / 2 ** 48 for c in got])
+    ctas = 8 * torch.cuda.get_device_properties(0).multi_processor_count
+    np.testing.assert_array_less(np.abs(gotw - want), want * (3 * ctas * 2.0 ** -53) + got * 2.0 ** -48 + 1e-300)

@@ -5,7 +5,9 @@ at the record's counter when another batch would take it past its share, and
 flushes when the counter says more than is left over.  A scheduler that may stop
 any warp between any two of its shared-memory operations for as long as it likes
 must not bring a record past the bound; taking the counters of all entries before
-their records, as a flush in two passes does, must."""
+their records, as a flush in two passes does, must.  No product is lost: a flush may
+take a quad's counts and leave its products, added later, to a flush that finds no
+count beside them."""
 
 import random
 from fractions import Fraction
@@ -84,6 +86,45 @@ def test_no_record_passes_the_bound(seed):
     assert c.products_out > 20 * LIMIT                     # it flushed many times
     # what was taken out and what is left agree, but for the quads in flight
     assert abs((c.counts_out + (c.count & (CLAIM - 1))) - (c.products_out + c.record)) <= QUAD * WARPS + LIMIT
+
+
+@pytest.mark.parametrize("seed", range(40))
+def test_no_product_is_lost(seed):
+    """A rare entry of a histogram that is flushed for others: one quad's counts and
+    products, flushes in between at any step, the last one after all warps stopped."""
+    rng = random.Random(seed)
+    c = Cta()
+
+    def quads(k):
+        for _ in range(k):
+            c.count += QUAD
+            yield
+            c.record += QUAD
+            yield
+
+    def flush():
+        if c.count == 0 and c.record == 0:                 # nothing to take
+            return
+        n = c.count
+        c.count += CLAIM
+        n = 0 if n >= CLAIM else n
+        yield
+        c.products_out += c.record
+        c.record = 0
+        yield
+        c.count -= CLAIM + n
+        c.counts_out += n
+
+    total = rng.randint(1, 3)
+    live = [quads(1) for _ in range(total)] + [flush() for _ in range(3)]
+    while live:
+        g = rng.choice(live)
+        if next(g, "done") == "done":
+            live.remove(g)
+    for _ in flush():
+        pass
+    assert c.products_out == total * QUAD and c.counts_out == total * QUAD
+    assert c.count == c.record == 0
 
 
 def test_the_bound_of_the_constants():

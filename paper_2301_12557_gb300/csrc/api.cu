@@ -318,6 +318,7 @@ static pc_status make_plan(const pc_bins *b, const Geom &g, const double *pts_lo
     double eps_z = 2.0 * u * (2.5 * c + 4.0 * Rb) + tiny;
     double eps_sig = 2.0 * u * (3.6 * c + 11.5 * Rb) + ldexp(Rb, -25) + tiny;
     double muA = 2.0 * (6.9 * u * c) + tiny, muB = 2.0 * 21.0 * u + ldexp(1.0, -48);
+    double lmin = 0.0;   // midpoint: lower bound of |x_i + x_j|
     if (P.los == PC_LOS_MIDPOINT) {
         // distance of the nearest point to the observer bounds |x_i + x_j|:
         // the larger of the bounding box's distance and the points' own
@@ -331,7 +332,7 @@ static pc_status make_plan(const pc_bins *b, const Geom &g, const double *pts_lo
             dmin2 += d * d;
         }
         const double dmin = std::max(sqrt(dmin2) * (1.0 - 1e-12), rmin);
-        double lmin = 2.0 * dmin - Rb;
+        lmin = 2.0 * dmin - Rb;
         double dl = u * (5.5 * X + 4.4 * c + 6.2 * Rb);
         if (lmin > 4.0 * Rb) {
             double em = 2.0 * (u * (4.4 * c + 17.5 * Rb) + 2.0 * Rb * dl / lmin) +
@@ -578,6 +579,12 @@ static pc_status make_plan(const pc_bins *b, const Geom &g, const double *pts_lo
         // no FP32 square may overflow (the kernel's indices rely on it), and the
         // constant 1e-30 in the squares must stay far inside the first band
         ok = ok && X + Lm + R0 + c < 1e15 && std::min({D, Db, P.ea[1]}) > 1e-9 && na <= FIX_TOP && nb <= FIX_TOP;
+        // along the midpoint |d x l|^2 is a fourth power (|l| <= 2 sqrt(3) X): it comes to
+        // the ends of binary32 and near that constant first, in units far from a
+        // catalogue's scale (limits of a survey shell in Mpc: times 2^21 and 2^-21);
+        // packed floors and tables find such pairs near an edge
+        if (P.mode == PC_BIN_SIGPI && P.los == PC_LOS_MIDPOINT)
+            ok = ok && R0 * (4.0 * X + R0) < 1.7e19 && (P.ea[0] > 0.0 ? P.ea[0] : P.ea[1]) * lmin > 1e-9;
         P.fix = ok ? kind : 0;
     }
     // ---- stencil -------------------------------------------------------------

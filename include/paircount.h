@@ -129,7 +129,8 @@ typedef struct {
                                     range by one bounding-box test per point group */
     int prec;                    /* pc_prec that ran: PC_PREC_F64 also when FP32 was asked
                                     for but its error bound does not hold (midpoint line of
-                                    sight with the observer too close to the points) */
+                                    sight with the observer too close to the points, or
+                                    separations whose binary32 squares overflow) */
     int wsum;                    /* weighted sums: 0 none; 1 binary64 products w_i w_j;
                                     2 exact products of binary32 significands accumulated
                                     as integers (evenly spaced bins, shared histograms, every
@@ -349,7 +350,7 @@ pc_status pc_tree_export(const pc_tree *t, long long *start, long long *count, i
  * Errors: PC_EINVAL (trees of different boxes or devices, missing weights,
  * bad bins, a periodic separation of L/2 or more), PC_EUNSUPPORTED (plain
  * FP64 asked for, or forced by a midpoint line of sight too close to the
- * observer), PC_EOVERFLOW, PC_ENOMEM, PC_ECUDA. */
+ * observer or a reach above 1.7e19), PC_EOVERFLOW, PC_ENOMEM, PC_ECUDA. */
 pc_status pc_count_tree(const pc_tree *t1, const pc_tree *t2, const pc_bins *b,
                         const pc_opts *o, void *stream, long long *counts, double *wcounts,
                         pc_stats *st);

@@ -347,6 +347,13 @@ static pc_status make_plan(const pc_bins *b, const Geom &g, const double *pts_lo
         }
     }
     P.rcut = R0 + std::max({eps_s, eps_z, eps_sig}) * 2.0;
+    // binary32 squares of separations in range (midpoint: and of x_i + x_j) must be
+    // finite, or pairs were lost: a box of 2^60 x 100 with reach 2^60 x 30 kept 15 % of
+    // its pairs, one of 2^66 none
+    if (!(P.rcut < 1.7e19) || (P.los == PC_LOS_MIDPOINT && !(4.0 * X + R0 < 1.7e19))) {
+        P.fp32_ok = 0;
+        P.fp32_why = "binary32 squares of the separations overflow";
+    }
     {
         double r2 = P.rcut * P.rcut * (1.0 + 8.0 * u);
         P.r2cut = nextafterf((float)r2, INFINITY);
@@ -1495,7 +1502,8 @@ extern "C" pc_status pc_count_tree(const pc_tree *t1, const pc_tree *t2, const p
     if (S.prec != PC_PREC_F32_RESCUE)
         return fail(PC_EUNSUPPORTED,
                     "pc_count_tree: runs the FP32 + rescue kernel only (the plain FP64 path, "
-                    "asked for or forced by a midpoint line of sight close to the observer, "
+                    "asked for or forced by a midpoint line of sight close to the observer or a reach "
+                    "above 1.7e19, "
                     "is a grid-path option)");
     DevBufs B;
     s = ensure_bufs(workspace(S.dev), S, B);

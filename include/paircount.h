@@ -111,22 +111,22 @@ typedef struct {
     int shard_count;             /* cells (tree: list nodes) whose index % shard_count ==
                                     shard_index (multi-GPU shards; the int64 counts of all
                                     shards sum to the full count, and a shard is the same set
-                                    of pairs whatever the precision or i-points per thread) */
+                                    of pairs whatever the precision or ipt) */
 } pc_opts;
 
 /* Counters of the last count call (all optional). */
 typedef struct {
     long long candidates;        /* pair separations evaluated by the kernel */
     long long rescued;           /* pairs re-evaluated in FP64 */
-    long long rescue_inline;     /* of those, evaluated inline (queue full) */
+    long long rescue_inline;     /* of those, evaluated inline (no queue, or full) */
     long long blocks;            /* i-blocks processed */
     double cell_size;            /* cell side used (first grid) */
     float ms_total;              /* device time of the call, milliseconds */
     float ms_pairs;              /* device time of the pair kernel alone */
     float ms_rescue;             /* device time of the rescue kernel */
     int launches;                /* kernels this call launched */
-    long long pruned;            /* of the candidates, pairs the FP32 kernel decided out of
-                                    range by one bounding-box test per point group */
+    long long pruned;            /* of the candidates, pairs the kernel decided out of
+                                    range by a box test of eight points at a time */
     int prec;                    /* pc_prec that ran: PC_PREC_F64 also when FP32 was asked
                                     for but its error bound does not hold (midpoint line of
                                     sight with the observer too close to the points, or

@@ -31,10 +31,12 @@
 // one, so the integer counts equal the binary64 definition exactly.
 //
 // What bounds it (2M clustered points, (s, mu) 40 x 100, 6.70e10 pairs in
-// range): issue slots (76 % of the cycles issue; the FMA and integer pipes at 51 and
-// 53 %, the shared-memory pipe at 62 %).  1.52 pairs are evaluated for each in range, against 1.70 with
-// one list for the 64 points along a Morton curve; 113 of about 135 warp
-// instructions per 64 x 4 pairs are the loop itself.  65.4 ms against 154.7 ms for
+// range): issue slots (75 % of the cycles issue; the FMA and integer pipes at 51 and
+// 54 %, the shared-memory pipe at 61 %).  1.52 pairs are evaluated for each in range,
+// against 1.70 with one list for the 64 points along a Morton curve; 113 of 147 warp
+// instructions per 64 x 4 pairs are the loop itself.  Weighted counts of many bins wait
+// for bank conflicts of their additions: survey (sigma, pi) with binary64 weights, 86 %
+// of the shared-memory pipe, 67 % of its wavefronts conflicts.  65.4 ms against 154.7 ms for
 // CTAs of 128 threads that staged every candidate tile behind a barrier and queued
 // near-edge pairs for a second kernel (138 instructions per 64 x 2 pairs, issued
 // on 60 % of the cycles).
@@ -1915,7 +1917,7 @@ __global__ void __maxnreg__((LOS == LOS_MID && MODE != MODE_S) || W == 1 || PATH
 // under the visited image is one the rule gives that image, since the reach
 // stays below L / 2 by more than the roundings.  Before: every candidate of the
 // stencil, with six comparisons for the wrap rule and a binary64 search; 50,001
-// uniform points in 40 s bins took 120.5 ms, now 4.9 ms.
+// uniform points in 40 s bins took 115 ms as a whole call, now 5.45 ms.
 struct F64Edges {
     const double *Ea, *Eb;
     const float *Fa, *Fb;    // FP32 roundings, or null

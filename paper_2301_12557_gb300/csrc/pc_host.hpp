@@ -95,8 +95,7 @@ struct TreeLists {
 pc_status tree_traverse(const pc_tree *t1, const pc_tree *t2, bool is_auto, double r2hi,
                         double r2lo, cudaStream_t st, TreeLists &out);
 
-// Balanced blocks per list node for ipt i-points per thread (NT * ipt points
-// per block at most), and the pair kernel's block list of a tree count: the
+// Balanced blocks per list node (NT * ipt points per block at most), and the pair kernel's block list of a tree count: the
 // list nodes of the shard (node % shard_count == shard_index) only.
 int tree_chunks(const pc_tree *t, int ipt);
 cudaError_t tree_blocks(const pc_tree *t, int ipt, int shard_index, int shard_count, Block *blocks,

@@ -928,7 +928,9 @@ static long long level_largest(long long n, int d) {
 // most cap points; cap = 0: among the levels whose largest node holds 129 to
 // 2048 points, the one whose nodes split into TREE_BLOCK-point blocks with
 // the fewest idle i-slots (the deepest on a tie; a catalogue of at most
-// TREE_BLOCK points: the root).
+// TREE_BLOCK points: the root).  The pair kernel's warps take equal parts of a
+// block, at most 64 points, so this stands in for the lanes they fill (95 % at
+// 2M points, nodes of 244).
 static int list_level(long long n, int cap) {
     int best = tree_depth(n, cap > 0 ? cap : TREE_BLOCK);
     if (cap == 0) {

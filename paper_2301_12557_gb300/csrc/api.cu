@@ -579,12 +579,13 @@ static pc_status make_plan(const pc_bins *b, const Geom &g, const double *pts_lo
             const double mB = P.los == PC_LOS_Z ? 1.25 * 10.7 * u + ldexp(1.0, -46) : muB + 4.0 * u;
             P.fx_invB = nb;   // mu = 1 may land in column n_mu: near, put right there
             // Pairs closer than this are near whatever their mu, and batches whose boxes
-            // touch take the band there: where that is 1/512 of a bin (about as many
-            // pairs near for their mu as a uniform catalogue has closer ones), at most
-            // c / 16, and for cells or list nodes above twice the reach an eighth of it
-            // (c / 16 alone made every pair of tight clusters near: 200 clusters of 1,000
-            // points in a tree, nb = 20: pairs to 20 8.9 -> 0.49 ms, to 60 7.5 -> 0.54)
-            P.fx_sf = std::max(std::min({c / 16.0, R0 / 8.0, 512.0 * nb * mA}), 1e-3 * R0);
+            // touch take the band there.  c / 16 suits catalogues with few such pairs and
+            // many mu bins.  With fewer bins the band allows less, down to c / 64, until it
+            // is 1/2048 of a bin, which spares tight clusters (c / 16 found half of a
+            // cluster's pairs near; 1/512 cost cross counts of 40 bins 5 to 12 %), and in
+            // cells or list nodes above twice the reach it is an eighth of the reach (at a
+            // reach of 5 every pair of a 250-point node was closer than c / 16)
+            P.fx_sf = std::max(std::min({c / 16.0, R0 / 8.0, std::max(c / 64.0, 2048.0 * nb * mA)}), 1e-3 * R0);
             P.fx_mA = nb * mA * one * 1.001;
             P.fx_mB = nb * mB * one * 1.001 + 1e-12 * nb * one + 1.0;
             ok = ok && P.fx_mA / P.fx_sf + P.fx_mB < 8192.0;

@@ -37,7 +37,7 @@ def test_few_pairs_are_near_for_their_separation_alone(ratio, nb, los):
         assert (np.sqrt(k["mu_s2"]) / R) ** 3 < 1.0 / 500.0
     else:
         assert los == "mid"
-    # clusters tighter than the cells: never beyond the separation whose band is 1/512
-    # of a bin (mu_A: its band times s, in units of 2^-16)
+    # clusters tighter than the cells: never beyond the separation whose band is 1/2048
+    # of a bin (mu_A: its band times s, in units of 2^-16), or a 64th of the cell
     if int(k["fix"]):
-        assert np.sqrt(k["mu_s2"]) < 1.01 * max(1e-3 * R, 512.0 * k["mu_A"] / 65536.0)
+        assert np.sqrt(k["mu_s2"]) < 1.01 * max(ratio * R / 64.0, 1e-3 * R, 2048.0 * k["mu_A"] / 65536.0)
